@@ -294,15 +294,15 @@ mbd_status mbd_set_real_space_method(mbd_system *sys, int32_t method);
 /* ---- autotuning ----
  * Times the candidate launch choices for this system at n_probes probes on the
  * system's stream and keeps the fastest.  The candidates are the FP32 FFT tile
- * width (32 or 16 complex columns), the tile width of the fused
- * spreading + first FFT pass (32 or 16), and the field kernel's atoms per
+ * width (32 or 16 complex columns) and the field kernel's atoms per
  * block (the occupancy-derived value, half and twice it, and four blocks per
  * SM).  The choices hold for later calls with the same probe width and until
- * the next mbd_autotune or mbd_set_launch_choices.  The tile widths do not
+ * the next mbd_autotune or mbd_set_launch_choices.  The tile width does not
  * change any result.  The
  * atoms per block change the summation order of the a_k reductions (last-bit
  * differences).  choices (host [4], may be NULL) receives the probe width,
- * the atoms per block, the FFT tile and the spreading tile (0: not
+ * the atoms per block, the FFT tile and the spreading tile (one width, 32
+ * columns, where the probes fill it; kept for saved choices; 0: not
  * applicable). */
 mbd_status mbd_autotune(mbd_system *sys, int32_t n_probes, int32_t choices[4]);
 

@@ -282,7 +282,7 @@ mbd_status build_neighbors(mbd_system *s) {
 // the host and the kernels agree exactly.
 mbd_status build_bins(mbd_system *s) {
     const int N = s->N;
-    int bs[3], nb[3], ncand[3];
+    int bs[3], nb[3];
     for (int a = 0; a < 3; ++a) {
         const int K = s->K[a];
         const int pref[5] = {4, 5, 3, 2, 1};
@@ -293,7 +293,6 @@ mbd_status build_bins(mbd_system *s) {
                 break;
             }
         nb[a] = K / bs[a];
-        ncand[a] = std::min(nb[a], 1 + (bs[a] + s->p - 2) / bs[a]);
     }
     const int nbins = nb[0] * nb[1] * nb[2];
     MBD_TRY(s->bin_start_d.ensure(sizeof(int) * (nbins + 1)));
@@ -309,9 +308,6 @@ mbd_status build_bins(mbd_system *s) {
     B.bs1 = bs[0];
     B.bs2 = bs[1];
     B.bs3 = bs[2];
-    B.nc1 = ncand[0];
-    B.nc2 = ncand[1];
-    B.nc3 = ncand[2];
     B.start = s->bin_start_d.as<int>();
     B.atoms = s->bin_atoms_d.as<int>();
     MBD_TRY(launch_bin_atoms(N, s->top_d.as<int>(), B, s->bin_of_d.as<int>(), s->scan_cnt.as<int>(),
@@ -390,7 +386,7 @@ template <class T> mbd_status setup_geometry(mbd_system *s) {
     MBD_TRY(launch_pair_tensors<T>(s, s->stream));
     MBD_TRY(launch_splines<T>(s, s->stream));
     MBD_TRY(build_bins(s));
-    MBD_TRY(build_spread_matrix<T>(s));
+    MBD_TRY(build_spread_records<T>(s));
     int head[2] = {0, 0};
     MBD_CUDA_TRY(cudaMemcpyAsync(&head[0], s->row_d.as<int>() + s->N, sizeof(int), cudaMemcpyDeviceToHost,
                                  s->stream));
@@ -536,16 +532,16 @@ struct Lz {
     int R, ld, m, rows, nblk;
 };
 
-mbd_status lanczos_workspace(mbd_system *s, int R, int m, int rows, int field_nblk, Lz &z) {
+mbd_status lanczos_workspace(mbd_system *s, int R, int ld_, int m, int rows, int field_nblk, Lz &z) {
     z.R = R;
-    z.ld = probe_ld(R);
+    z.ld = ld_;
     z.m = m;
     z.rows = rows;
     // prologue blocks per probe chunk: one per SM (fewer, fuller blocks keep the
     // two-level norm reduction short), at least 16 rows each; vectors of more
     // than 2^22 values take two to four per SM, so that enough loads are in
     // flight to stream them from HBM
-    const long long vals = (long long)rows * probe_ld(R);
+    const long long vals = (long long)rows * z.ld;
     const int per_sm = vals >= (1LL << 24) ? 4 : (vals >= (1LL << 22) ? 2 : 1);
     z.nblk = std::max(1, std::min((rows + 15) / 16, per_sm * std::max(1, s->num_sms)));
     const size_t ld = z.ld;
@@ -600,7 +596,7 @@ template <class T> mbd_status ensure_mesh(mbd_system *s, int ld) {
 // Workspace for an m-step run with R probes (allocations only: eager).
 template <class T> mbd_status prepare_lanczos(mbd_system *s, int R, int m, Lz &z, bool full) {
     const int rows = 3 * s->N;
-    MBD_TRY(lanczos_workspace(s, R, m, rows, field_blocks(s, probe_ld(R)), z));
+    MBD_TRY(lanczos_workspace(s, R, probe_ld<T>(R), m, rows, field_blocks(s, probe_ld<T>(R)), z));
     MBD_TRY(ensure_mesh<T>(s, z.ld));
     if (full) MBD_TRY(s->work2.ensure(sizeof(double) * (size_t)m * z.ld));
     return MBD_OK;
@@ -619,8 +615,7 @@ mbd_status enqueue_steps(mbd_system *s, int R, int m, uint64_t seed, const uint6
     fo.out = nullptr;
     fo.xin = nullptr;
     fo.lz = z.v;
-    // the fused spread + k3 pass exists for the specialised sizes with whole probe-pair tiles
-    const bool fuse3 = spread_fft3_supported(s, z.ld, (int)sizeof(T));
+    const bool fuse3 = spread_fft3_supported(s);
     const bool real_cl = real_on_clusters(s, z.ld, (int)sizeof(T));
     for (int k = 0; k < m; ++k) {
         MBD_STAGE(s, MBD_STAGE_PROLOGUE, 1,
@@ -725,7 +720,7 @@ mbd_status forces_impl(mbd_system *s, int R, int m, uint64_t seed, double *energ
     // w_l = C^{-1/2} v_l = sum_k c_lk y_lk with c = Delta^{-1/2} e_1 from the quadrature kernel
     MBD_TRY(run_lanczos<T>(s, R, m, seed, z, true));
     PrecData<T> &P = prec<T>(s);
-    const int ld2 = 2 * R;
+    const int ld2 = probe_ld<T>(2 * R);
     const size_t npts = (size_t)s->K[0] * s->K[1] * s->K[2];
     MBD_TRY(P.d.ensure(sizeof(T) * 3 * (size_t)s->N * std::max(ld2, z.ld)));
     MBD_TRY(P.mesh.ensure(sizeof(T) * npts * std::max(ld2, z.ld)));
@@ -748,14 +743,14 @@ mbd_status forces_impl(mbd_system *s, int R, int m, uint64_t seed, double *energ
                   launch_force_dipoles_t<T>(s, z.v.Y, s->work2.as<double>(), z.v.length, R, z.ld, m,
                                             P.d.template as<T>(), ld2));
     }
-    const bool fuse3 = spread_fft3_supported(s, ld2, (int)sizeof(T));
+    const bool fuse3 = spread_fft3_supported(s);
     if (fuse3) {
         MBD_STAGE(s, MBD_STAGE_FORCE_SPREAD, 1,
-                  launch_spread_fft3<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), ld2, ld2));
+                  launch_spread_fft3<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), 2 * R, ld2));
         MBD_STAGE(s, MBD_STAGE_FORCE_FFT, 4, launch_convolve<T>(s, P.mesh.template as<T>(), ld2, true));
     } else {
         MBD_STAGE(s, MBD_STAGE_FORCE_SPREAD, 1,
-                  launch_spread<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), ld2, ld2));
+                  launch_spread<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), 2 * R, ld2));
         MBD_STAGE(s, MBD_STAGE_FORCE_FFT, 5, launch_convolve<T>(s, P.mesh.template as<T>(), ld2));
     }
     const double scale = 0.25 * (3.0 * s->N) / R;
@@ -767,7 +762,7 @@ mbd_status forces_impl(mbd_system *s, int R, int m, uint64_t seed, double *energ
 
 template <class T> mbd_status apply_impl(mbd_system *s, int nvec, const double *x, double *y, int terms, bool field) {
     const int rows = 3 * s->N;
-    const int ld = probe_ld(nvec);
+    const int ld = probe_ld<T>(nvec);
     MBD_TRY(ensure_mesh<T>(s, ld));
     MBD_TRY(s->L.ensure(sizeof(double) * (size_t)rows * ld));
     MBD_TRY(s->work2.ensure(sizeof(double) * (size_t)rows * ld));
@@ -783,8 +778,11 @@ template <class T> mbd_status apply_impl(mbd_system *s, int nvec, const double *
                   launch_gscale<T>(xt, s->g_d.as<double>(), P.d.template as<T>(), rows, ld, s->stream));
     }
     if (terms & MBD_TERM_RECIP) {
-        MBD_STAGE(s, MBD_STAGE_SPREAD, 1, launch_spread<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), nvec, ld));
-        MBD_STAGE(s, MBD_STAGE_FFT, 5, launch_convolve<T>(s, P.mesh.template as<T>(), ld));
+        const bool fuse3 = spread_fft3_supported(s);
+        MBD_STAGE(s, MBD_STAGE_SPREAD, 1,
+                  fuse3 ? launch_spread_fft3<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), nvec, ld)
+                        : launch_spread<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), nvec, ld));
+        MBD_STAGE(s, MBD_STAGE_FFT, fuse3 ? 4 : 5, launch_convolve<T>(s, P.mesh.template as<T>(), ld, fuse3));
     }
     FieldOut<T> fo;
     fo.mode = field ? kFieldOut : kFieldApply;
@@ -805,7 +803,7 @@ template <class T> mbd_status apply_impl(mbd_system *s, int nvec, const double *
 
 template <class T> mbd_status spread_impl(mbd_system *s, int nvec, const double *d, double *mesh_out) {
     const int rows = 3 * s->N;
-    const int ld = probe_ld(nvec);
+    const int ld = probe_ld<T>(nvec);
     MBD_TRY(ensure_mesh<T>(s, ld));
     MBD_TRY(s->L.ensure(sizeof(double) * (size_t)rows * ld));
     double *xt = s->L.as<double>();
@@ -821,7 +819,7 @@ template <class T> mbd_status spread_impl(mbd_system *s, int nvec, const double 
 }
 
 template <class T> mbd_status convolve_impl(mbd_system *s, int nvec, const double *in, double *out) {
-    const int ld = probe_ld(nvec);
+    const int ld = probe_ld<T>(nvec);
     MBD_TRY(ensure_mesh<T>(s, ld));
     PrecData<T> &P = prec<T>(s);
     const size_t npts = (size_t)s->K[0] * s->K[1] * s->K[2];
@@ -932,7 +930,7 @@ template <class T> mbd_status capture_batch(mbd_batch *b, int R, int m) {
 // Time each candidate launch choice for probe width ld on the system's stream
 // (CUDA events, one untimed launch then three timed) and keep the fastest.
 template <class T> mbd_status autotune_impl(mbd_system *s, int R, int32_t *out) {
-    const int ld = probe_ld(R);
+    const int ld = probe_ld<T>(R);
     const size_t rows = 3 * (size_t)s->N;
     const size_t npts = (size_t)s->K[0] * s->K[1] * s->K[2];
     PrecData<T> &P = prec<T>(s);
@@ -943,7 +941,7 @@ template <class T> mbd_status autotune_impl(mbd_system *s, int R, int32_t *out) 
     MBD_CUDA_TRY(cudaMemsetAsync(P.mesh.ptr, 0, sizeof(T) * npts * ld, s->stream));
     MBD_CUDA_TRY(cudaMemsetAsync(s->L.ptr, 0, sizeof(double) * rows * ld, s->stream));
     if (s->real_clusters) MBD_CUDA_TRY(cudaMemsetAsync(P.ereal.ptr, 0, sizeof(T) * rows * ld, s->stream));
-    s->tune_ld = ld;
+    s->tune_ld = R + (R & 1);
     s->tune_field_apb = s->tune_fft_w = s->tune_sf3_w = 0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     MBD_CUDA_TRY(cudaEventCreate(&e0));
@@ -973,18 +971,8 @@ template <class T> mbd_status autotune_impl(mbd_system *s, int R, int32_t *out) 
                 if (bw == 0 || ms < best) bw = w, best = ms;
             }
             s->tune_fft_w = bw;
-            // tile width of the fused spreading + k3 pass
-            if (fft_ct_size(s->K[2]) && (ld / 2) % 32 == 0) {
-                bw = 0;
-                for (int w : {32, 16}) {
-                    s->tune_sf3_w = w;
-                    MBD_TRY(timed([&] {
-                        return launch_spread_fft3<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), R, ld);
-                    }, &ms));
-                    if (bw == 0 || ms < best) bw = w, best = ms;
-                }
-                s->tune_sf3_w = bw;
-            }
+            // the fused spreading has one tile width; reported where it fills whole tiles
+            s->tune_sf3_w = fft_ct_size(s->K[2]) && s->tune_ld / 2 % 32 == 0 ? 32 : 0;
         }
         // atoms per block of the field kernel
         const int a0 = field_apb(s, ld);
@@ -1018,7 +1006,7 @@ template <class T> mbd_status autotune_impl(mbd_system *s, int R, int32_t *out) 
         return st;
     }
     if (out) {
-        out[0] = ld;
+        out[0] = s->tune_ld;
         out[1] = s->tune_field_apb;
         out[2] = s->tune_fft_w;
         out[3] = s->tune_sf3_w;
@@ -1350,7 +1338,7 @@ mbd_status mbd_lanczos_energy_dense(int32_t dim, const double *c_dev, double ome
         if (cudaMallocHost(&s->host_scal, 16 * sizeof(double)) != cudaSuccess) return MBD_ERR_OOM;
         if (cudaMallocHost(&s->host_status, 4 * sizeof(int)) != cudaSuccess) return MBD_ERR_OOM;
         Lz z;
-        MBD_TRY(lanczos_workspace(s, R, m, dim, 1, z));
+        MBD_TRY(lanczos_workspace(s, R, probe_ld<double>(R), m, dim, 1, z));
         MBD_TRY(s->f64.d.ensure(sizeof(double) * (size_t)dim * z.ld));
         MBD_TRY(s->g_d.ensure(sizeof(double) * ((size_t)dim / 3 + 1)));
         // g = 1 so that the prologue's d output is y* itself (unused by the dense operator)

@@ -20,72 +20,58 @@ template <class T> struct FFTArgs {
     int nst;
     unsigned long long radices;   // stage s radix = (radices >> 4 s) & 15
     int V;               // complex probe pairs per mesh point (fused pass: G index = e / V)
-    int sign;            // -1 forward, +1 inverse (unfused passes)
     int early;           // compile-time passes: programmatic dependent launch (1) or plain (0)
-    int sms;             // multiprocessors (persistent compile-time passes; 0: not persistent)
+    int sms;             // multiprocessors
 };
 
-// Compile-time passes for the smooth sizes listed below (fft_sizes_*.cu).
-// Return 1 when launched, 0 when the launch could not be configured, -1 when
-// there is no compile-time pass for the size or tile width asked for.
-//   a.W: the tile width; float passes exist for W = 32 and 16, double
-//   passes for W = 16.
-template <class T> int launch_fft_ct_sized(const FFTArgs<T> &a, bool fused, unsigned grid, cudaStream_t st);
-//   W: the tile width of the fused spreading (float 32 or 16, double 16).
-template <class T>
-int launch_sf3_sized(int K3, int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *row,
-                     const SpreadRec<T> *rec, const typename Cplx<T>::type *tw, cudaStream_t st);
+// Compile-time passes for the smooth sizes listed below (fft_sizes_*.cu) over
+// [outer][K][inner]; mode 0 forward, 1 inverse, 2 forward x G inverse (outer =
+// 1).  Return 1 when launched, 0 when the launch could not be configured, -1
+// when there is no compile-time pass for the size.
+//   a.W: the tile width in complex columns of float passes, 32 or 16 (double
+//   passes have one width).
+template <class T> int launch_fft_ct_sized(const FFTArgs<T> &a, int mode, unsigned outer, cudaStream_t st);
 bool fft_ct_size(int K);
-//   The same fused pass with spreading by pencil records (spline order 6):
-//   W = 32 or 16 for float, 16 for double.
-template <class T>
-int launch_spp_sized(int K3, int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *prow,
-                     const PencilRec<T> *prec, const T *k3w, const typename Cplx<T>::type *tw, cudaStream_t st);
+
+// Arguments of the spreading by pencil records (PencilRec) into the mesh.
+template <class T> struct SpreadArgs {
+    const T *d;          // dipoles [N][3][ld]
+    T *mesh;             // [K1][K2][K3][ld]
+    int R, ld;           // probes (the rest of ld is written as zero)
+    int K1, K2, K3, p;
+    const int *prow;     // [K1 K2 K3 + 1] records by point (k1, k2, top3)
+    const PencilRec<T> *prec;
+    const T *k3w;        // [N][2p] M3, M3'
+    const typename Cplx<T>::type *tw;   // twiddles of k3
+};
+// Spreading fused with the forward transform along k3; same return values.
+template <class T> int launch_spp_sized(const SpreadArgs<T> &a, cudaStream_t st);
 
 // Sizes with a compile-time pass and their radices (first stage first), in
 // groups of one translation unit each.
-#define MBD_FFT_GROUP0(X) X(16, 4, 4) X(18, 3, 3, 2) X(20, 5, 4) X(24, 8, 3) X(25, 5, 5) X(27, 3, 3, 3) X(30, 5, 3, 2)
-#define MBD_FFT_GROUP1(X) X(32, 8, 4) X(36, 4, 3, 3) X(40, 8, 5) X(45, 5, 3, 3) X(48, 4, 4, 3) X(50, 5, 5, 2) \
-    X(54, 3, 3, 3, 2)
-#define MBD_FFT_GROUP2(X) X(60, 5, 4, 3) X(64, 8, 8) X(72, 8, 3, 3) X(75, 5, 5, 3) X(80, 5, 4, 4) \
-    X(81, 3, 3, 3, 3) X(90, 5, 3, 3, 2)
-#define MBD_FFT_GROUP3(X) X(96, 8, 4, 3) X(100, 5, 5, 4) X(108, 4, 3, 3, 3) X(120, 8, 5, 3) X(125, 5, 5, 5) \
-    X(128, 8, 8, 2) X(135, 5, 3, 3, 3)
-#define MBD_FFT_GROUP4(X) X(144, 4, 4, 3, 3) X(150, 5, 5, 3, 2) X(160, 8, 5, 4) X(162, 3, 3, 3, 3, 2) \
-    X(180, 5, 4, 3, 3) X(192, 8, 8, 3) X(200, 8, 5, 5)
-#define MBD_FFT_GROUP5(X) X(216, 8, 3, 3, 3) X(225, 5, 5, 3, 3) X(240, 5, 4, 4, 3) X(243, 3, 3, 3, 3, 3) \
-    X(250, 5, 5, 5, 2) X(256, 8, 8, 4)
+#define MBD_FFT_GROUP0(X) X(16, 4, 4) X(18, 6, 3) X(20, 5, 4) X(24, 6, 4) X(25, 5, 5) X(27, 9, 3) X(30, 6, 5)
+#define MBD_FFT_GROUP1(X) X(32, 8, 4) X(36, 6, 6) X(40, 8, 5) X(45, 9, 5) X(48, 8, 6) X(50, 10, 5) X(54, 9, 6)
+#define MBD_FFT_GROUP2(X) X(60, 10, 6) X(64, 8, 8) X(72, 9, 8) X(75, 15, 5) X(80, 10, 8) X(81, 9, 9) X(90, 10, 9)
+#define MBD_FFT_GROUP3(X) X(96, 12, 8) X(100, 10, 10) X(108, 12, 9) X(120, 12, 10) X(125, 5, 5, 5) X(128, 16, 8) \
+    X(135, 15, 9)
+#define MBD_FFT_GROUP4(X) X(144, 12, 12) X(150, 15, 10) X(160, 16, 10) X(162, 9, 6, 3) X(180, 15, 12) \
+    X(192, 16, 12) X(200, 10, 5, 4)
+#define MBD_FFT_GROUP5(X) X(216, 6, 6, 6) X(225, 15, 15) X(240, 16, 15) X(243, 9, 9, 3) X(250, 10, 5, 5) \
+    X(256, 16, 16)
 #define MBD_FFT_NUM_GROUPS 6
 
-template <class T> int launch_fft_ct_group0(const FFTArgs<T> &, bool, unsigned, cudaStream_t);
-template <class T> int launch_fft_ct_group1(const FFTArgs<T> &, bool, unsigned, cudaStream_t);
-template <class T> int launch_fft_ct_group2(const FFTArgs<T> &, bool, unsigned, cudaStream_t);
-template <class T> int launch_fft_ct_group3(const FFTArgs<T> &, bool, unsigned, cudaStream_t);
-template <class T> int launch_fft_ct_group4(const FFTArgs<T> &, bool, unsigned, cudaStream_t);
-template <class T> int launch_fft_ct_group5(const FFTArgs<T> &, bool, unsigned, cudaStream_t);
-#define MBD_SF3_DECL(g)                                                                                          \
-    template <class T>                                                                                           \
-    int launch_sf3_group##g(int K3, int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *row, \
-                            const SpreadRec<T> *rec, const typename Cplx<T>::type *tw, cudaStream_t st);
-MBD_SF3_DECL(0)
-MBD_SF3_DECL(1)
-MBD_SF3_DECL(2)
-MBD_SF3_DECL(3)
-MBD_SF3_DECL(4)
-MBD_SF3_DECL(5)
-#undef MBD_SF3_DECL
-#define MBD_SPP_DECL(g)                                                                                          \
-    template <class T>                                                                                           \
-    int launch_spp_group##g(int K3, int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *prow, \
-                            const PencilRec<T> *prec, const T *k3w, const typename Cplx<T>::type *tw,            \
-                            cudaStream_t st);
-MBD_SPP_DECL(0)
-MBD_SPP_DECL(1)
-MBD_SPP_DECL(2)
-MBD_SPP_DECL(3)
-MBD_SPP_DECL(4)
-MBD_SPP_DECL(5)
-#undef MBD_SPP_DECL
+template <class T> int launch_fft_ct_group0(const FFTArgs<T> &, int, unsigned, cudaStream_t);
+template <class T> int launch_fft_ct_group1(const FFTArgs<T> &, int, unsigned, cudaStream_t);
+template <class T> int launch_fft_ct_group2(const FFTArgs<T> &, int, unsigned, cudaStream_t);
+template <class T> int launch_fft_ct_group3(const FFTArgs<T> &, int, unsigned, cudaStream_t);
+template <class T> int launch_fft_ct_group4(const FFTArgs<T> &, int, unsigned, cudaStream_t);
+template <class T> int launch_fft_ct_group5(const FFTArgs<T> &, int, unsigned, cudaStream_t);
+template <class T> int launch_spp_group0(const SpreadArgs<T> &, cudaStream_t);
+template <class T> int launch_spp_group1(const SpreadArgs<T> &, cudaStream_t);
+template <class T> int launch_spp_group2(const SpreadArgs<T> &, cudaStream_t);
+template <class T> int launch_spp_group3(const SpreadArgs<T> &, cudaStream_t);
+template <class T> int launch_spp_group4(const SpreadArgs<T> &, cudaStream_t);
+template <class T> int launch_spp_group5(const SpreadArgs<T> &, cudaStream_t);
 
 namespace {
 
@@ -145,677 +131,772 @@ template <class T, int VEC> __device__ __forceinline__ void vstore(T *p, const T
 }
 
 // ---------------------------------------------------------------- FFT
-template <class C> __device__ __forceinline__ C cmul(C a, C b) {
-    return C{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+// Complex values Cx<F>: F = float or double holds one complex probe pair, F =
+// float2 two of them, (x0, x1) in x and (y0, y1) in y, on which every
+// operation is one packed instruction (add, multiply, FMA of two floats).
+// FP32 meshes hold a multiple of four probes per point, and four consecutive
+// probes p0 .. p3 are read as the two complex pairs p0 + i p2 and p1 + i p3,
+// which needs no shuffle and half the FP32 instructions of the scalar form.
+// Any pairing of the probes gives the same convolution (the influence function
+// is real and even); every pass of one mesh uses the same pairing.
+template <class F> struct __align__(2 * sizeof(F)) Cx {
+    F x, y;
+};
+// The packed form of a real type's columns.
+template <class T> struct PackOf { using type = T; };
+template <> struct PackOf<float> { using type = float2; };
+template <class F> struct Scal { using type = F; };
+template <> struct Scal<float2> { using type = float; };
+
+__device__ __forceinline__ float fadd(float a, float b) { return a + b; }
+__device__ __forceinline__ double fadd(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 fadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float fsub(float a, float b) { return a - b; }
+__device__ __forceinline__ double fsub(double a, double b) { return a - b; }
+__device__ __forceinline__ float2 fsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float fmulc(float a, float c) { return a * c; }
+__device__ __forceinline__ double fmulc(double a, double c) { return a * c; }
+__device__ __forceinline__ float2 fmulc(float2 a, float c) { return __fmul2_rn(a, make_float2(c, c)); }
+// a c + b with a scalar c
+__device__ __forceinline__ float fmac(float a, float c, float b) { return fmaf(a, c, b); }
+__device__ __forceinline__ double fmac(double a, double c, double b) { return fma(a, c, b); }
+__device__ __forceinline__ float2 fmac(float2 a, float c, float2 b) { return __ffma2_rn(a, make_float2(c, c), b); }
+
+template <class F> __device__ __forceinline__ Cx<F> cadd(Cx<F> a, Cx<F> b) { return {fadd(a.x, b.x), fadd(a.y, b.y)}; }
+template <class F> __device__ __forceinline__ Cx<F> csub(Cx<F> a, Cx<F> b) { return {fsub(a.x, b.x), fsub(a.y, b.y)}; }
+// a + s i b and a - s i b, s = -1 (forward transforms) or +1 (INV)
+template <bool INV, class F> __device__ __forceinline__ Cx<F> cadd_i(Cx<F> a, Cx<F> b) {
+    if constexpr (INV) return {fsub(a.x, b.y), fadd(a.y, b.x)};
+    else return {fadd(a.x, b.y), fsub(a.y, b.x)};
 }
-template <class C> __device__ __forceinline__ C cadd(C a, C b) { return C{a.x + b.x, a.y + b.y}; }
-template <class C> __device__ __forceinline__ C csub(C a, C b) { return C{a.x - b.x, a.y - b.y}; }
-// multiply by -i*sign... rot(a) = sign * i * a, with sign = -1 (forward) or +1 (inverse)
-template <class C> __device__ __forceinline__ C rot(C a, int sign) {
-    return sign < 0 ? C{a.y, -a.x} : C{-a.y, a.x};
+template <bool INV, class F> __device__ __forceinline__ Cx<F> csub_i(Cx<F> a, Cx<F> b) { return cadd_i<!INV>(a, b); }
+// a c + b, a scalar c; and b + s i c a
+template <class F, class S> __device__ __forceinline__ Cx<F> cfma(Cx<F> a, S c, Cx<F> b) {
+    return {fmac(a.x, c, b.x), fmac(a.y, c, b.y)};
+}
+template <bool INV, class F, class S> __device__ __forceinline__ Cx<F> cfma_i(Cx<F> a, S c, Cx<F> b) {
+    const S d = INV ? c : -c;
+    return {fmac(a.y, -d, b.x), fmac(a.x, d, b.y)};
+}
+// a (c + s i t) for constants c, t (the twiddle exp(s i angle) with c = cos, t = sin)
+template <bool INV, class F, class S> __device__ __forceinline__ Cx<F> crot(Cx<F> a, S c, S t) {
+    const S d = INV ? t : -t;
+    return {fmac(a.y, -d, fmulc(a.x, c)), fmac(a.x, d, fmulc(a.y, c))};
 }
 
-// In-register R-point DFT  X_t = sum_q x_q exp(sign 2 pi i q t / R), R in {2,3,4,5,8}.
-template <class T, class C> __device__ __forceinline__ void dft2(C *v) {
-    const C a = v[0], b = v[1];
-    v[0] = cadd(a, b);
-    v[1] = csub(a, b);
-}
-template <class T, class C> __device__ __forceinline__ void dft4(C *v, int sign) {
-    const C s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
-    const C s13 = cadd(v[1], v[3]), d13 = rot(csub(v[1], v[3]), sign);
-    v[0] = cadd(s02, s13);
-    v[2] = csub(s02, s13);
-    v[1] = cadd(d02, d13);
-    v[3] = csub(d02, d13);
-}
-template <class T, class C> __device__ __forceinline__ void dft8(C *v, int sign) {
-    const T h = T(0.70710678118654752440);
-    C e[4] = {v[0], v[2], v[4], v[6]};
-    C o[4] = {v[1], v[3], v[5], v[7]};
-    dft4<T>(e, sign);
-    dft4<T>(o, sign);
-    // twiddles exp(sign 2 pi i t / 8), t = 0..3
-    const C o1 = C{h * (o[1].x - T(sign) * o[1].y), h * (o[1].y + T(sign) * o[1].x)};
-    const C o2 = rot(o[2], sign);
-    const C o3 = C{h * (-o[3].x - T(sign) * o[3].y), h * (-o[3].y + T(sign) * o[3].x)};
-    v[0] = cadd(e[0], o[0]);
-    v[4] = csub(e[0], o[0]);
-    v[1] = cadd(e[1], o1);
-    v[5] = csub(e[1], o1);
-    v[2] = cadd(e[2], o2);
-    v[6] = csub(e[2], o2);
-    v[3] = cadd(e[3], o3);
-    v[7] = csub(e[3], o3);
-}
-template <class T, class C> __device__ __forceinline__ void dft3(C *v, int sign) {
-    const T c = T(-0.5), s = T(sign) * T(0.86602540378443864676);
-    const C a = v[0], b = v[1], d = v[2];
-    const C t = cadd(b, d);
-    const C u = csub(b, d);
-    v[0] = cadd(a, t);
-    const C m = C{a.x + c * t.x, a.y + c * t.y};
-    const C n = C{-s * u.y, s * u.x};   // i s (b - d)
-    v[1] = cadd(m, n);
-    v[2] = csub(m, n);
-}
-template <class T, class C> __device__ __forceinline__ void dft5(C *v, int sign) {
-    // cos/sin of 2 pi / 5 and 4 pi / 5
-    const T c1 = T(0.30901699437494742410), c2 = T(-0.80901699437494742410);
-    const T s1 = T(sign) * T(0.95105651629515357212), s2 = T(sign) * T(0.58778525229247312917);
-    const C a = v[0];
-    const C t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
-    const C u1 = csub(v[1], v[4]), u2 = csub(v[2], v[3]);
-    v[0] = C{a.x + t1.x + t2.x, a.y + t1.y + t2.y};
-    const C m1 = C{a.x + c1 * t1.x + c2 * t2.x, a.y + c1 * t1.y + c2 * t2.y};
-    const C m2 = C{a.x + c2 * t1.x + c1 * t2.x, a.y + c2 * t1.y + c1 * t2.y};
-    // i (s1 u1 + s2 u2) and i (s2 u1 - s1 u2)
-    const C n1 = C{-(s1 * u1.y + s2 * u2.y), s1 * u1.x + s2 * u2.x};
-    const C n2 = C{-(s2 * u1.y - s1 * u2.y), s2 * u1.x - s1 * u2.x};
-    v[1] = cadd(m1, n1);
-    v[4] = csub(m1, n1);
-    v[2] = cadd(m2, n2);
-    v[3] = csub(m2, n2);
-}
+// In-register R-point DFTs  X_t = sum_q x_q exp(s 2 pi i q t / R), natural
+// order in and out.
+template <class F, int R, bool INV> struct Dft;
+template <class F, bool INV> struct Dft<F, 2, INV> {
+    static __device__ __forceinline__ void run(Cx<F> *v) {
+        const Cx<F> a = v[0], b = v[1];
+        v[0] = cadd(a, b);
+        v[1] = csub(a, b);
+    }
+};
+template <class F, bool INV> struct Dft<F, 3, INV> {
+    static __device__ __forceinline__ void run(Cx<F> *v) {
+        using S = typename Scal<F>::type;
+        const Cx<F> t = cadd(v[1], v[2]), u = csub(v[1], v[2]);
+        const Cx<F> m = cfma(t, S(-0.5), v[0]);
+        v[0] = cadd(v[0], t);
+        v[1] = cfma_i<INV>(u, S(0.86602540378443864676), m);
+        v[2] = cfma_i<!INV>(u, S(0.86602540378443864676), m);
+    }
+};
+template <class F, bool INV> struct Dft<F, 4, INV> {
+    static __device__ __forceinline__ void run(Cx<F> *v) {
+        const Cx<F> s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
+        const Cx<F> s13 = cadd(v[1], v[3]), d13 = csub(v[1], v[3]);
+        v[0] = cadd(s02, s13);
+        v[2] = csub(s02, s13);
+        v[1] = cadd_i<INV>(d02, d13);
+        v[3] = csub_i<INV>(d02, d13);
+    }
+};
+template <class F, bool INV> struct Dft<F, 5, INV> {
+    static __device__ __forceinline__ void run(Cx<F> *v) {
+        using S = typename Scal<F>::type;
+        // cos and sin of 2 pi / 5 and 4 pi / 5
+        const S c1 = S(0.30901699437494742410), c2 = S(-0.80901699437494742410);
+        const S s1 = S(0.95105651629515357212), s2 = S(0.58778525229247312917);
+        const Cx<F> a = v[0];
+        const Cx<F> t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+        const Cx<F> u1 = csub(v[1], v[4]), u2 = csub(v[2], v[3]);
+        v[0] = cadd(cadd(a, t1), t2);
+        const Cx<F> m1 = cfma(t2, c2, cfma(t1, c1, a)), m2 = cfma(t2, c1, cfma(t1, c2, a));
+        v[1] = cfma_i<INV>(u2, s2, cfma_i<INV>(u1, s1, m1));
+        v[4] = cfma_i<!INV>(u2, s2, cfma_i<!INV>(u1, s1, m1));
+        v[2] = cfma_i<!INV>(u2, s1, cfma_i<INV>(u1, s2, m2));
+        v[3] = cfma_i<INV>(u2, s1, cfma_i<!INV>(u1, s2, m2));
+    }
+};
+template <class F, bool INV> struct Dft<F, 8, INV> {
+    static __device__ __forceinline__ void run(Cx<F> *v) {
+        using S = typename Scal<F>::type;
+        const S h = S(0.70710678118654752440);
+        Cx<F> e[4] = {v[0], v[2], v[4], v[6]};
+        Cx<F> o[4] = {v[1], v[3], v[5], v[7]};
+        Dft<F, 4, INV>::run(e);
+        Dft<F, 4, INV>::run(o);
+        // odd outputs times exp(s 2 pi i t / 8) = h (1 + s i), s i, h (-1 + s i)
+        const Cx<F> p1 = cadd_i<INV>(o[1], o[1]), p3 = csub_i<INV>(o[3], o[3]);
+        v[0] = cadd(e[0], o[0]);
+        v[4] = csub(e[0], o[0]);
+        v[1] = cfma(p1, h, e[1]);
+        v[5] = cfma(p1, -h, e[1]);
+        v[2] = cadd_i<INV>(e[2], o[2]);
+        v[6] = csub_i<INV>(e[2], o[2]);
+        v[3] = cfma(p3, -h, e[3]);
+        v[7] = cfma(p3, h, e[3]);
+    }
+};
+// R = A B with A, B coprime: two dimensions of DFTs and no twiddles.  Input
+// n = (B a + A b) mod R, output k with k mod A = ka and k mod B = kb.
+template <class F, int A, int B, bool INV> struct DftCoprime {
+    static constexpr int out(int ka, int kb) {
+        for (int k = 0; k < A * B; ++k)
+            if (k % A == ka && k % B == kb) return k;
+        return 0;
+    }
+    static __device__ __forceinline__ void run(Cx<F> *v) {
+        Cx<F> t[A * B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            Cx<F> u[A];
+#pragma unroll
+            for (int a = 0; a < A; ++a) u[a] = v[(B * a + A * b) % (A * B)];
+            Dft<F, A, INV>::run(u);
+#pragma unroll
+            for (int a = 0; a < A; ++a) t[a * B + b] = u[a];
+        }
+#pragma unroll
+        for (int a = 0; a < A; ++a) {
+            Dft<F, B, INV>::run(t + a * B);
+#pragma unroll
+            for (int b = 0; b < B; ++b) v[out(a, b)] = t[a * B + b];
+        }
+    }
+};
+template <class F, bool INV> struct Dft<F, 6, INV> : DftCoprime<F, 2, 3, INV> {};
+template <class F, bool INV> struct Dft<F, 10, INV> : DftCoprime<F, 2, 5, INV> {};
+template <class F, bool INV> struct Dft<F, 12, INV> : DftCoprime<F, 4, 3, INV> {};
+template <class F, bool INV> struct Dft<F, 15, INV> : DftCoprime<F, 3, 5, INV> {};
+// 9 = 3 x 3 and 16 = 4 x 4: x[B a + b] -> DFT over a, twiddle exp(s 2 pi i b ka / R), DFT over b -> k = ka + A kb
+template <class F, bool INV> struct Dft<F, 9, INV> {
+    static __device__ __forceinline__ void run(Cx<F> *v) {
+        using S = typename Scal<F>::type;
+        Cx<F> t[3][3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            Cx<F> u[3] = {v[b], v[3 + b], v[6 + b]};
+            Dft<F, 3, INV>::run(u);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) t[a][b] = u[a];
+        }
+        // cos and sin of 40, 80 and 160 degrees
+        const S c2 = S(0.17364817766693034885), s2 = S(0.98480775301220805937);
+        t[1][1] = crot<INV>(t[1][1], S(0.76604444311897803520), S(0.64278760968653932632));
+        t[1][2] = crot<INV>(t[1][2], c2, s2);
+        t[2][1] = crot<INV>(t[2][1], c2, s2);
+        t[2][2] = crot<INV>(t[2][2], S(-0.93969262078590838405), S(0.34202014332566873304));
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            Dft<F, 3, INV>::run(t[a]);
+#pragma unroll
+            for (int b = 0; b < 3; ++b) v[a + 3 * b] = t[a][b];
+        }
+    }
+};
+template <class F, bool INV> struct Dft<F, 16, INV> {
+    static __device__ __forceinline__ void run(Cx<F> *v) {
+        using S = typename Scal<F>::type;
+        Cx<F> t[4][4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            Cx<F> u[4] = {v[b], v[4 + b], v[8 + b], v[12 + b]};
+            Dft<F, 4, INV>::run(u);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) t[a][b] = u[a];
+        }
+        const S h = S(0.70710678118654752440), c = S(0.92387953251128675613), d = S(0.38268343236508977173);
+        t[1][1] = crot<INV>(t[1][1], c, d);
+        t[1][2] = crot<INV>(t[1][2], h, h);
+        t[1][3] = crot<INV>(t[1][3], d, c);
+        t[2][1] = crot<INV>(t[2][1], h, h);
+        t[2][2] = crot<INV>(t[2][2], S(0), S(1));
+        t[2][3] = crot<INV>(t[2][3], -h, h);
+        t[3][1] = crot<INV>(t[3][1], d, c);
+        t[3][2] = crot<INV>(t[3][2], -h, h);
+        t[3][3] = crot<INV>(t[3][3], -c, -d);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            Dft<F, 4, INV>::run(t[a]);
+#pragma unroll
+            for (int b = 0; b < 4; ++b) v[a + 4 * b] = t[a][b];
+        }
+    }
+};
 
-
-
-template <class T, class C, int R> __device__ __forceinline__ void dft(C *v, int sign) {
-    if constexpr (R == 2) dft2<T>(v);
-    else if constexpr (R == 3) dft3<T>(v, sign);
-    else if constexpr (R == 4) dft4<T>(v, sign);
-    else if constexpr (R == 5) dft5<T>(v, sign);
-    else dft8<T>(v, sign);
+// Twiddles exp(-2 pi i n / K) in shared memory: as complex values, or for the
+// packed form with each component doubled.
+template <class F> struct TwOf { using type = Cx<F>; };
+template <> struct TwOf<float2> { using type = float4; };
+__device__ __forceinline__ void tw_set(Cx<float> &t, float2 w) { t = {w.x, w.y}; }
+__device__ __forceinline__ void tw_set(Cx<double> &t, double2 w) { t = {w.x, w.y}; }
+__device__ __forceinline__ void tw_set(float4 &t, float2 w) { t = make_float4(w.x, w.x, w.y, w.y); }
+// v times the twiddle (its conjugate for INV)
+template <bool INV> __device__ __forceinline__ Cx<float> ctw(Cx<float> v, Cx<float> w) {
+    const float wy = INV ? -w.y : w.y;
+    return {fmaf(v.x, w.x, -(v.y * wy)), fmaf(v.x, wy, v.y * w.x)};
+}
+template <bool INV> __device__ __forceinline__ Cx<double> ctw(Cx<double> v, Cx<double> w) {
+    const double wy = INV ? -w.y : w.y;
+    return {fma(v.x, w.x, -(v.y * wy)), fma(v.x, wy, v.y * w.x)};
+}
+template <bool INV> __device__ __forceinline__ Cx<float2> ctw(Cx<float2> v, float4 w) {
+    const float2 wx = make_float2(w.x, w.y), wy = make_float2(w.z, w.w), nwy = make_float2(-w.z, -w.w);
+    return {__ffma2_rn(v.x, wx, __fmul2_rn(v.y, INV ? wy : nwy)), __ffma2_rn(v.x, INV ? nwy : wy, __fmul2_rn(v.y, wx))};
+}
+template <class F> __device__ __forceinline__ Cx<F> cld(const Cx<F> *p) {
+    if constexpr (sizeof(Cx<F>) == 16) {
+        union {
+            float4 v;
+            Cx<F> c;
+        } u;
+        u.v = *reinterpret_cast<const float4 *>(p);
+        return u.c;
+    } else {
+        return *p;
+    }
+}
+template <class F> __device__ __forceinline__ void cst(Cx<F> *p, Cx<F> c) {
+    if constexpr (sizeof(Cx<F>) == 16) {
+        union {
+            float4 v;
+            Cx<F> c;
+        } u;
+        u.c = c;
+        *reinterpret_cast<float4 *>(p) = u.v;
+    } else {
+        *p = c;
+    }
 }
 
 // ---------------------------------------------------------------- compile-time passes
-// Threads of a compile-time pass: enough for the stage with the most
-// butterflies (K / smallest radix rows x W columns), at most 256.
-template <int R> constexpr int ct_rmin() { return R; }
-template <int R, int S, int... RS> constexpr int ct_rmin() {
-    return R < ct_rmin<S, RS...>() ? R : ct_rmin<S, RS...>();
-}
-template <int K, int W, int... RS> constexpr int ct_threads() {
-    return (K / ct_rmin<RS...>()) * W >= 256 ? 256 : (((K / ct_rmin<RS...>()) * W + 31) / 32) * 32;
+// A transform of K = r_1 r_2 ... r_n rows, in place on a K x W tile in shared
+// memory.  Forward (decimation in frequency): stage s splits every block of
+// B = r_s M rows into r_s-point DFTs over the rows m + M q, multiplied by the
+// twiddles exp(-2 pi i m q / B), leaving r_s blocks of M rows; the last stage
+// (M = 1) leaves the row of frequency k at the digit-reversed place, so its
+// thread writes the frequencies it holds straight to their rows of the mesh.
+// A butterfly is read and written by one thread, so a stage needs no second
+// buffer and one barrier follows it: for almost all sizes n = 2 (radices up
+// to 16), that is a tile written once, read, written and read.  The pass fused
+// with the influence function multiplies the frequencies that a thread of the
+// last stage holds by G, transforms them back at once (inverse r_n-point DFT)
+// and runs the remaining stages backwards (decimation in time) in the same
+// places: three exchanges instead of the six of a forward and an inverse pass.
+template <int... RS> struct Plan {
+    static constexpr int n = sizeof...(RS);
+    static constexpr int r[n] = {RS...};
+    static constexpr int K = (RS * ... * 1);
+    static constexpr int M(int s) {          // rows of the blocks that stage s leaves
+        int m = 1;
+        for (int t = s + 1; t < n; ++t) m *= r[t];
+        return m;
+    }
+    static constexpr int last() { return r[n - 1]; }
+    static constexpr int rmin() {
+        int m = r[0];
+        for (int t = 1; t < n; ++t) m = r[t] < m ? r[t] : m;
+        return m;
+    }
+    static constexpr int before(int s) {     // product of the radices before stage s
+        int m = 1;
+        for (int t = 0; t < s; ++t) m *= r[t];
+        return m;
+    }
+    // lowest frequency of the last stage's block `blk`: digits k_1 .. k_{n-1}, first digit fastest
+    template <int S = n - 2> static __device__ __forceinline__ int rev(int blk) {
+        constexpr int R = r[S], mult = before(S);
+        if constexpr (S == 0) return blk;
+        else return (blk % R) * mult + rev<S - 1>(blk / R);
+    }
+};
+
+// Threads of a pass: one butterfly each in the stage with the most, at most 256.
+template <class P, int W> constexpr int ct_threads() {
+    constexpr int t = ((P::K / P::rmin()) * W + 31) / 32 * 32;
+    return t < 256 ? t : 256;
 }
 
-// One radix-R Stockham stage over the K rows of a K x W tile with K, W, the
-// stage's stride NS and the block size NT compile-time, so the index
-// arithmetic folds away and each butterfly stays in registers.  The stage reads
-// the global tile (IN_G, columns >= wc read as zero) or shared memory, and
-// writes the global tile (OUT_G, columns < wc only) or shared memory,
-// multiplying by G on the way out (MULG; G index row * gstride + (c0 + col) / V).
-// A thread takes CV adjacent columns of a row (CV = 2: float tiles, one
-// 16-byte access for both and one twiddle for both; the caller guarantees
-// whole column pairs, 16-byte alignment and an even V).
-template <class T, class C, int R, int K, int W, int NT, int CV, int NS, bool IN_G, bool OUT_G, bool MULG>
-__device__ __forceinline__ void ct_stage(const C *__restrict__ in_s, const C *__restrict__ in_g, C *__restrict__ out_s,
-                                         C *__restrict__ out_g, size_t gs, int wc, const C *__restrict__ tw, int sign,
-                                         const T *__restrict__ G, size_t gstride, int c0, int V) {
-    static_assert(CV == 1 || (CV == 2 && sizeof(T) == 4 && W % 2 == 0), "column pairs are float tiles");
-    constexpr int nb = K / R;
-    constexpr int step = K / (NS * R);
-    constexpr int WG = W / CV;
-    constexpr int total = nb * WG;
+// Stage S (not the last) of the forward transform in place, and the same stage
+// of the inverse (twiddles first) in place or, for S = 0, to the rows of the
+// mesh column gout (row stride gs) of a valid column.
+template <class P, int S, class F, int W, int NT, bool INV>
+__device__ __forceinline__ void ct_fwd_stage(Cx<F> *tile, const typename TwOf<F>::type *tw) {
+    constexpr int R = P::r[S], M = P::M(S), K = P::K, B = R * M, NB = K / R;
+    const int col = threadIdx.x % W;
 #pragma unroll
-    for (int it = 0; it < (total + NT - 1) / NT; ++it) {
-        const int idx = it * NT + (int)threadIdx.x;
-        if (total % NT != 0 && idx >= total) break;
-        const int j = idx / WG, col = (idx % WG) * CV;
-        C v[CV][R];
+    for (int it = 0; it < (NB * W + NT - 1) / NT; ++it) {
+        const int j = it * (NT / W) + (int)threadIdx.x / W;
+        if (NB % (NT / W) != 0 && j >= NB) break;
+        const int m = j % M;
+        Cx<F> *t = tile + ((j / M) * B + m) * W + col;
+        Cx<F> v[R];
 #pragma unroll
-        for (int q = 0; q < R; ++q) {
-            if constexpr (CV == 1) {
-                if (IN_G)
-                    v[0][q] = col < wc ? in_g[(size_t)(j + q * nb) * gs + col] : C{T(0), T(0)};
-                else
-                    v[0][q] = in_s[(j + q * nb) * W + col];
-            } else {
-                float4 x;
-                if (IN_G)
-                    x = col < wc ? *reinterpret_cast<const float4 *>(in_g + (size_t)(j + q * nb) * gs + col)
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-                else
-                    x = *reinterpret_cast<const float4 *>(in_s + (j + q * nb) * W + col);
-                v[0][q] = C{x.x, x.y};
-                v[1][q] = C{x.z, x.w};
+        for (int q = 0; q < R; ++q) v[q] = cld(t + q * M * W);
+        Dft<F, R, INV>::run(v);
+        cst(t, v[0]);
+#pragma unroll
+        for (int q = 1; q < R; ++q) cst(t + q * M * W, ctw<INV>(v[q], tw[(K / B) * m * q]));
+    }
+}
+template <class P, int S, class F, int W, int NT>
+__device__ __forceinline__ void ct_inv_stage(Cx<F> *tile, const typename TwOf<F>::type *tw, Cx<F> *gout, size_t gs,
+                                             bool valid) {
+    constexpr int R = P::r[S], M = P::M(S), K = P::K, B = R * M, NB = K / R;
+    const int col = threadIdx.x % W;
+#pragma unroll
+    for (int it = 0; it < (NB * W + NT - 1) / NT; ++it) {
+        const int j = it * (NT / W) + (int)threadIdx.x / W;
+        if (NB % (NT / W) != 0 && j >= NB) break;
+        const int m = j % M;
+        Cx<F> *t = tile + ((j / M) * B + m) * W + col;
+        Cx<F> v[R];
+        v[0] = cld(t);
+#pragma unroll
+        for (int q = 1; q < R; ++q) v[q] = ctw<true>(cld(t + q * M * W), tw[(K / B) * m * q]);
+        Dft<F, R, true>::run(v);
+        if constexpr (S == 0) {
+            if (valid) {
+#pragma unroll
+                for (int q = 0; q < R; ++q) cst(gout + (size_t)(m + M * q) * gs, v[q]);
             }
-        }
-        const int jm = j % NS;
-        if (NS > 1 && jm != 0) {
+        } else {
 #pragma unroll
-            for (int q = 1; q < R; ++q) {
-                C t = tw[q * jm * step];
-                if (sign > 0) t.y = -t.y;
-#pragma unroll
-                for (int u = 0; u < CV; ++u) v[u][q] = cmul(v[u][q], t);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < CV; ++u) dft<T, C, R>(v[u], sign);
-        const int base = (j / NS) * NS * R + jm;
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-            const int row = base + q * NS;
-            if (MULG && col < wc) {
-                const T gv = G[(size_t)row * gstride + (c0 + col) / V];
-#pragma unroll
-                for (int u = 0; u < CV; ++u) {
-                    v[u][q].x *= gv;
-                    v[u][q].y *= gv;
-                }
-            }
-            if constexpr (CV == 1) {
-                if (OUT_G) {
-                    if (col < wc) out_g[(size_t)row * gs + col] = v[0][q];
-                } else {
-                    out_s[row * W + col] = v[0][q];
-                }
-            } else {
-                const float4 x = make_float4(v[0][q].x, v[0][q].y, v[1][q].x, v[1][q].y);
-                if (OUT_G) {
-                    if (col < wc) *reinterpret_cast<float4 *>(out_g + (size_t)row * gs + col) = x;
-                } else {
-                    *reinterpret_cast<float4 *>(out_s + row * W + col) = x;
-                }
-            }
+            for (int q = 0; q < R; ++q) cst(t + q * M * W, v[q]);
         }
     }
 }
+// The last stage of a pass: frequencies to the mesh column gout.
+template <class P, class F, int W, int NT, bool INV>
+__device__ __forceinline__ void ct_last_stage(const Cx<F> *tile, Cx<F> *gout, size_t gs, bool valid) {
+    constexpr int R = P::r[P::n - 1], K = P::K, NB = K / R;
+    const int col = threadIdx.x % W;
+#pragma unroll
+    for (int it = 0; it < (NB * W + NT - 1) / NT; ++it) {
+        const int j = it * (NT / W) + (int)threadIdx.x / W;
+        if (NB % (NT / W) != 0 && j >= NB) break;
+        const Cx<F> *t = tile + j * R * W + col;
+        Cx<F> v[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = cld(t + q * W);
+        Dft<F, R, INV>::run(v);
+        if (valid) {
+            Cx<F> *o = gout + (size_t)P::template rev<>(j) * gs;
+#pragma unroll
+            for (int q = 0; q < R; ++q) cst(o + (size_t)(q * NB) * gs, v[q]);
+        }
+    }
+}
+// The G of one butterfly of the mid stage: rows rev(j) + NB q of the column.
+template <class P, class S> __device__ __forceinline__ void ct_load_g(const S *__restrict__ gcol, size_t gstride, int j,
+                                                                      S *g) {
+    constexpr int R = P::r[P::n - 1], NB = P::K / R;
+    const S *gr = gcol + (size_t)P::template rev<>(j) * gstride;
+#pragma unroll
+    for (int q = 0; q < R; ++q) g[q] = gr[(size_t)(q * NB) * gstride];
+}
+// Whether a thread has one butterfly of the mid stage per tile, whose G it then
+// loads before it waits for the tile.
+template <class P, int W, int NT> constexpr bool ct_g_early() { return (P::K / P::r[P::n - 1]) * W <= NT; }
 
-// A run of stages: the first reads the global tile (IN_G) or shared buffer
-// sin, intermediate results ping-pong between the shared buffers, the last
-// writes the global tile (OUT_G) or shared memory, multiplying by G (MULG).
-// Returns the shared buffer holding the result when it stays in shared memory.
-template <class T, class C, int K, int W, int NT, int CV, int NS, bool IN_G, bool OUT_G, bool MULG, int R, int... RS>
-__device__ __forceinline__ C *ct_pipe(const C *gin, C *gout, size_t gs, int wc, C *sin, C *sout, const C *tw, int sign,
-                                      const T *G, size_t gstride, int c0, int V) {
-    constexpr bool last = sizeof...(RS) == 0;
-    ct_stage<T, C, R, K, W, NT, CV, NS, IN_G, last && OUT_G, last && MULG>(sin, gin, sout, gout, gs, wc, tw, sign, G,
-                                                                           gstride, c0, V);
-    if constexpr (last) {
-        return sout;
-    } else {
+// The last forward stage, the product with G (gcol: G of the column, row
+// stride gstride; g: the values already loaded, ct_g_early) and the first
+// inverse stage, in place.
+template <class P, class F, int W, int NT>
+__device__ __forceinline__ void ct_mid_stage(Cx<F> *tile, const typename Scal<F>::type *__restrict__ gcol,
+                                             size_t gstride, const typename Scal<F>::type *gearly) {
+    using S = typename Scal<F>::type;
+    constexpr int R = P::r[P::n - 1], K = P::K, NB = K / R;
+    const int col = threadIdx.x % W;
+#pragma unroll
+    for (int it = 0; it < (NB * W + NT - 1) / NT; ++it) {
+        const int j = it * (NT / W) + (int)threadIdx.x / W;
+        if (NB % (NT / W) != 0 && j >= NB) break;
+        Cx<F> *t = tile + j * R * W + col;
+        S g[R];
+        if constexpr (ct_g_early<P, W, NT>()) {
+#pragma unroll
+            for (int q = 0; q < R; ++q) g[q] = gearly[q];
+        } else {
+            ct_load_g<P>(gcol, gstride, j, g);
+        }
+        Cx<F> v[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = cld(t + q * W);
+        Dft<F, R, false>::run(v);
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = {fmulc(v[q].x, g[q]), fmulc(v[q].y, g[q])};
+        Dft<F, R, true>::run(v);
+#pragma unroll
+        for (int q = 0; q < R; ++q) cst(t + q * W, v[q]);
+    }
+}
+template <class P, int S, class F, int W, int NT, bool INV>
+__device__ __forceinline__ void ct_forward(Cx<F> *tile, const typename TwOf<F>::type *tw) {
+    if constexpr (S < P::n - 1) {
+        ct_fwd_stage<P, S, F, W, NT, INV>(tile, tw);
         __syncthreads();
-        return ct_pipe<T, C, K, W, NT, CV, NS * R, false, OUT_G, MULG, RS...>(gin, gout, gs, wc, sout, sin, tw, sign,
-                                                                               G, gstride, c0, V);
+        ct_forward<P, S + 1, F, W, NT, INV>(tile, tw);
     }
 }
-
-// One 1D pass along the middle axis of [outer][K][inner] (complex) with
-// compile-time K, W and radices (at least two stages): a block owns one
-// K x W tile.  The first stage loads the global tile straight into registers
-// and the last one stores straight from registers, so shared memory carries
-// only the exchanges between stages; the fused pass (forward, x G, inverse)
-// multiplies by G in the last forward stage.
-template <class T, bool FUSED, int K, int W, int NT, int CV, int... RS>
-__global__ void __launch_bounds__(NT) k_fft_ct(FFTArgs<T> a) {
-    using C = typename Cplx<T>::type;
-    static_assert(sizeof...(RS) >= 2, "single-stage sizes would read and write the same global tile");
-    extern __shared__ __align__(16) unsigned char smem_ct[];
-    C *buf0 = reinterpret_cast<C *>(smem_ct), *buf1 = buf0 + K * W;
-    C *tw = buf1 + K * W;
-    pdl_launch_dependents();
-    for (int i = threadIdx.x; i < K; i += NT) tw[i] = a.tw[i];   // set up once per system
-    pdl_wait();
-    __syncthreads();
-    const int ncb = (a.inner + W - 1) / W;
-    const size_t outer = blockIdx.x / ncb;
-    const int c0 = (int)(blockIdx.x % ncb) * W;
-    const int wc = min(W, a.inner - c0);
-    C *base = a.data + outer * (size_t)K * a.inner + c0;
-    const size_t gstride = (size_t)(a.inner / a.V);
-    if (FUSED) {
-        // G of this block's slab: G[outer][row][(c0 + col) / V]
-        const T *Gb = a.G + outer * (size_t)K * gstride;
-        C *res = ct_pipe<T, C, K, W, NT, CV, 1, true, false, true, RS...>(base, base, a.inner, wc, buf0, buf1, tw,
-                                                                           -1, Gb, gstride, c0, a.V);
+template <class P, int S, class F, int W, int NT>
+__device__ __forceinline__ void ct_inverse(Cx<F> *tile, const typename TwOf<F>::type *tw, Cx<F> *gout, size_t gs,
+                                           bool valid) {
+    ct_inv_stage<P, S, F, W, NT>(tile, tw, gout, gs, valid);
+    if constexpr (S > 0) {
         __syncthreads();
-        C *other = (res == buf0) ? buf1 : buf0;
-        ct_pipe<T, C, K, W, NT, CV, 1, false, true, false, RS...>(base, base, a.inner, wc, res, other, tw, +1, a.G,
-                                                                   gstride, c0, a.V);
-    } else {
-        ct_pipe<T, C, K, W, NT, CV, 1, true, true, false, RS...>(base, base, a.inner, wc, buf0, buf1, tw, a.sign,
-                                                                  a.G, gstride, c0, a.V);
+        ct_inverse<P, S - 1, F, W, NT>(tile, tw, gout, gs, valid);
     }
 }
+// The unfused transform of a tile already in shared memory (visible to every
+// thread), to the mesh column gout.
+template <class P, class F, int W, int NT, bool INV>
+__device__ __forceinline__ void ct_transform(Cx<F> *tile, const typename TwOf<F>::type *tw, Cx<F> *gout, size_t gs,
+                                             bool valid) {
+    ct_forward<P, 0, F, W, NT, INV>(tile, tw);
+    ct_last_stage<P, F, W, NT, INV>(tile, gout, gs, valid);
+}
 
-// 16-byte asynchronous copy from global to shared memory (cp.async, cached
-// in L2 only), and the group fences of those copies.
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+// Asynchronous copies from global to shared memory (cp.async) of one complex
+// value, and the group fences of those copies.
+template <int BYTES> __device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit16() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait16() {
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// The same pass over whole tiles with persistent blocks: a block takes tiles
-// blockIdx.x, blockIdx.x + gridDim.x, ... and, while it transforms one tile
-// (from shared memory, last stage written straight to global memory), the
-// next tile is already arriving in a second shared buffer by asynchronous
-// copies (cp.async, 16 bytes each, issued by all threads).  So the tile loads
-// overlap the arithmetic and the stage barriers of the previous tile instead
-// of stalling every warp of a block on its own load; the arithmetic per
-// element is that of k_fft_ct (bit-identical results).
-// Resident blocks of a persistent pass that its shared memory allows (three
-// tiles and the twiddles), at most three: the register bound that follows.
-template <class T, int K, int W> constexpr int ct_pipe_blocks() {
-    constexpr size_t smem = sizeof(typename Cplx<T>::type) * (3 * (size_t)K * W + K) + 1024;
-    constexpr size_t per = (227u * 1024u) / smem;
-    return per < 1 ? 1 : (per > 3 ? 3 : (int)per);
-}
-
-template <class T, bool FUSED, int K, int W, int NT, int CV, int... RS>
-__global__ void __launch_bounds__(NT, (ct_pipe_blocks<T, K, W>())) k_fft_ct_pipe(FFTArgs<T> a, unsigned ntiles) {
-    using C = typename Cplx<T>::type;
-    static_assert(sizeof...(RS) >= 2, "at least two stages");
-    static_assert((W * sizeof(C)) % 16 == 0, "tile rows of whole 16-byte chunks");
-    constexpr int CPR = (int)(W * sizeof(C) / 16);   // 16-byte chunks per tile row
-    constexpr int EPC = (int)(16 / sizeof(C));       // complex values per chunk
-    extern __shared__ __align__(16) unsigned char smem_cp[];
-    C *in0 = reinterpret_cast<C *>(smem_cp), *in1 = in0 + K * W, *wk = in1 + K * W;
-    C *tw = wk + K * W;
-    pdl_launch_dependents();
-    for (int i = threadIdx.x; i < K; i += NT) tw[i] = a.tw[i];   // set up once per system
+// One 1D pass along the middle axis of [outer][K][inner] (values Cx<F>), MODE
+// 0 forward, 1 inverse, 2 forward x G inverse.  The outer x inner columns are
+// cut into tiles of W consecutive ones (a tile may span several outer slabs,
+// so narrow rows fill tiles too; only the last tile is partial).  A block
+// takes tiles blockIdx.x, blockIdx.x + gridDim.x, ...; while it transforms one,
+// the next arrives in its second buffer by cp.async.  A thread works on one
+// column of every tile.
+// Bound: HBM (each pass reads and writes the mesh once); the FP32 issue and the
+// shared-memory exchanges are what the packed form and the two stages cut.
+template <class T, class F, class P, int MODE, int W, int NT>
+__global__ void __launch_bounds__(NT) k_fft_ct(FFTArgs<T> a, unsigned ncols, unsigned ntiles) {
+    using C = Cx<F>;
+    using TW = typename TwOf<F>::type;
+    constexpr int K = P::K, RL = P::last();
+    constexpr int TR = NT / W;                // rows copied per step
+    static_assert(P::n >= 2 && NT % W == 0, "two stages at least; whole rows of threads");
+    extern __shared__ __align__(16) unsigned char smem_ct[];
+    TW *tw = reinterpret_cast<TW *>(smem_ct);
+    C *buf = reinterpret_cast<C *>(tw + K);
+    for (int i = threadIdx.x; i < K; i += NT) tw_set(tw[i], a.tw[i]);   // set up once per system
     pdl_wait();
-    const int ncb = a.inner / W;
-    const size_t gstride = (size_t)(a.inner / a.V);
+    pdl_launch_dependents();
+    const int col = threadIdx.x % W, row0 = threadIdx.x / W;
+    C *data = reinterpret_cast<C *>(a.data);
+    const size_t gs = (size_t)a.inner;
+    auto column = [&](unsigned cg) {
+        const unsigned o = cg / (unsigned)a.inner;
+        return data + (size_t)o * K * gs + (cg - o * (unsigned)a.inner);
+    };
+    auto fetch = [&](unsigned t, C *to) {
+        const unsigned cg = t * W + col;
+        if (cg < ncols) {
+            const C *src = column(cg) + (size_t)row0 * gs;
+            for (int row = row0; row < K; row += TR, src += TR * gs) cp_async<(int)sizeof(C)>(to + row * W + col, src);
+        }
+    };
     unsigned t = blockIdx.x;
-    if (t < ntiles) {
-        const size_t outer = t / ncb;
-        const C *src = a.data + outer * (size_t)K * a.inner + (size_t)(t % ncb) * W;
-        for (int q = threadIdx.x; q < K * CPR; q += NT)
-            cp_async16(in0 + (q / CPR) * W + (q % CPR) * EPC, src + (size_t)(q / CPR) * a.inner + (q % CPR) * EPC);
-    }
-    cp_async_commit16();
+    if (t < ntiles) fetch(t, buf);
+    cp_async_commit();
     for (int b = 0; t < ntiles; t += gridDim.x, b ^= 1) {
-        C *cur = b ? in1 : in0, *nxt = b ? in0 : in1;
-        __syncthreads();                         // every thread is done with nxt (two tiles ago) and wk
-        const unsigned tn = t + gridDim.x;
-        if (tn < ntiles) {
-            const size_t outer = tn / ncb;
-            const C *src = a.data + outer * (size_t)K * a.inner + (size_t)(tn % ncb) * W;
-            for (int q = threadIdx.x; q < K * CPR; q += NT)
-                cp_async16(nxt + (q / CPR) * W + (q % CPR) * EPC,
-                           src + (size_t)(q / CPR) * a.inner + (q % CPR) * EPC);
+        C *cur = buf + b * (K * W);
+        __syncthreads();                      // every thread is done with the other buffer
+        if (t + gridDim.x < ntiles) fetch(t + gridDim.x, buf + (b ^ 1) * (K * W));
+        cp_async_commit();
+        const unsigned cg = t * W + col;
+        const bool valid = cg < ncols;
+        C *out = column(valid ? cg : 0);
+        const T *gcol = MODE == 2 ? a.G + (valid ? cg : 0) / (unsigned)a.V : nullptr;
+        const size_t gstride = MODE == 2 ? gs / a.V : 0;
+        T g[RL];
+        if constexpr (MODE == 2 && ct_g_early<P, W, NT>()) {
+            if (row0 < K / RL) ct_load_g<P>(gcol, gstride, row0, g);
         }
-        cp_async_commit16();
-        cp_async_wait16<1>();                     // this thread's copies of tile t are done
-        __syncthreads();                         // and every thread's
-        const size_t outer = t / ncb;
-        const int c0 = (int)(t % ncb) * W;
-        C *base = a.data + outer * (size_t)K * a.inner + c0;
-        if (FUSED) {
-            const T *Gb = a.G + outer * (size_t)K * gstride;
-            C *res = ct_pipe<T, C, K, W, NT, CV, 1, false, false, true, RS...>(base, base, a.inner, W, cur, wk, tw,
-                                                                                -1, Gb, gstride, c0, a.V);
+        cp_async_wait<1>();                   // this thread's copies of tile t are done
+        __syncthreads();                      // and every thread's
+        if constexpr (MODE == 2) {
+            ct_forward<P, 0, F, W, NT, false>(cur, tw);
+            ct_mid_stage<P, F, W, NT>(cur, gcol, gstride, g);
             __syncthreads();
-            C *other = (res == cur) ? wk : cur;
-            ct_pipe<T, C, K, W, NT, CV, 1, false, true, false, RS...>(base, base, a.inner, W, res, other, tw, +1, Gb,
-                                                                       gstride, c0, a.V);
+            ct_inverse<P, P::n - 2, F, W, NT>(cur, tw, out, gs, valid);
         } else {
-            ct_pipe<T, C, K, W, NT, CV, 1, false, true, false, RS...>(base, base, a.inner, W, cur, wk, tw, a.sign,
-                                                                       a.G, gstride, c0, a.V);
+            ct_transform<P, F, W, NT, MODE == 1>(cur, tw, out, gs, valid);
         }
     }
-    cp_async_wait16<0>();                         // no copy in flight at exit
+    cp_async_wait<0>();                       // no copy in flight at exit
 }
 
-template <class T, bool FUSED, int K, int W, int CV, int... RS> int launch_ct_cv(const FFTArgs<T> &a, unsigned grid,
-                                                                              cudaStream_t st) {
-    using C = typename Cplx<T>::type;
-    constexpr int NT = ct_threads<K, W / CV, RS...>();
-    if (ct_pipe_blocks<T, K, W>() >= 2 && a.inner % W == 0 && a.sms > 0) {
-        // whole tiles and room for two blocks per SM: persistent blocks with the next tile prefetched
-        auto kern = k_fft_ct_pipe<T, FUSED, K, W, NT, CV, RS...>;
-        const size_t smem = sizeof(C) * (3 * (size_t)K * W + K);
-        static int per_sm = -1;                   // resident blocks per SM (one device architecture)
-        if (per_sm < 0) {
+// Launch of one pass: a block per tile when all tiles are resident at once
+// (one buffer), persistent blocks with two buffers otherwise.
+template <class T, class F, class P, int MODE, int W> int launch_ct(const FFTArgs<T> &a, unsigned outer,
+                                                                    cudaStream_t st) {
+    constexpr int NT = ct_threads<P, W>();
+    auto kern = k_fft_ct<T, F, P, MODE, W, NT>;
+    const size_t tile = sizeof(Cx<F>) * (size_t)P::K * W, fixed = sizeof(typename TwOf<F>::type) * P::K;
+    static int per_sm[2] = {-1, -1};          // resident blocks per SM with one and two buffers (one architecture)
+    for (int k = 0; k < 2; ++k)
+        if (per_sm[k] < 0) {
+            const size_t smem = fixed + (k + 1) * tile;
             int x = 0;
-            if (smem > 48 * 1024 &&
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-                x = 0;
-            else if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, kern, NT, smem) != cudaSuccess)
+            if ((smem > 48 * 1024 &&
+                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, kern, NT, smem) != cudaSuccess)
                 x = 0;
             cudaGetLastError();
-            per_sm = x;
+            per_sm[k] = x;
         }
-        if (per_sm > 0) {
-            const unsigned pgrid = (unsigned)std::min<long long>(grid, (long long)per_sm * a.sms);
-            launch_pdl(a.early != 0, kern, dim3(pgrid), dim3(NT), smem, st, a, grid);
-            return 1;
-        }
-    }
-    const size_t smem = sizeof(C) * (2 * (size_t)K * W + K);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_fft_ct<T, FUSED, K, W, NT, CV, RS...>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-        return 0;
-    launch_pdl(a.early != 0, k_fft_ct<T, FUSED, K, W, NT, CV, RS...>, dim3(grid), dim3(NT), smem, st, a);
+    const unsigned ncols = outer * (unsigned)a.inner, ntiles = (ncols + W - 1) / W;
+    const unsigned sms = (unsigned)std::max(1, a.sms);
+    if (per_sm[0] < 1 || per_sm[1] < 1) return 0;
+    const bool once = ntiles <= per_sm[0] * sms;
+    const unsigned grid = once ? ntiles : std::min(ntiles, per_sm[1] * sms);
+    const size_t smem = fixed + (once ? 1 : 2) * tile;
+    // double passes of a few blocks per SM are bound by the FP64 units: blocks
+    // launched early land unevenly on the SMs (64 atoms, 32^3 x 16 probes: 4.2 ms
+    // per energy + forces against 3.6); one block per SM or persistent blocks
+    // are even in any case
+    const bool early = a.early != 0 && (sizeof(T) == 4 || !once || grid <= sms);
+    launch_pdl(early, kern, dim3(grid), dim3(NT), smem, st, a, ncols, ntiles);
     return 1;
 }
 
-// Float tiles take column pairs when every tile is whole (inner a multiple of
-// W), so that the pairs are 16-byte aligned, and V is even, so that the two
-// columns of a pair share their G.
-template <class T, bool FUSED, int K, int W, int... RS> int launch_ct(const FFTArgs<T> &a, unsigned grid,
-                                                                      cudaStream_t st) {
-    if constexpr (sizeof(T) == 4) {
-        if (a.inner % W == 0 && a.V % 2 == 0) return launch_ct_cv<T, FUSED, K, W, 2, RS...>(a, grid, st);
-    }
-    return launch_ct_cv<T, FUSED, K, W, 1, RS...>(a, grid, st);
+// The passes of one size: packed float tiles of 16 or 8 column pairs (a.W = 32
+// or 16 complex columns; V is even), double tiles of 8.
+template <class T, class F, class P, int W> int ct_mode(const FFTArgs<T> &a, int mode, unsigned outer, cudaStream_t st) {
+    if (mode == 0) return launch_ct<T, F, P, 0, W>(a, outer, st);
+    if (mode == 1) return launch_ct<T, F, P, 1, W>(a, outer, st);
+    return launch_ct<T, F, P, 2, W>(a, outer, st);
 }
-
-// The passes of one size: float tiles of 32 or 16 complex columns, double
-// tiles of 16.
-template <class T, int K, int... RS> int ct_size(const FFTArgs<T> &a, bool fused, unsigned grid, cudaStream_t st) {
-    if constexpr (sizeof(T) == 4) {
-        if (a.W == 32) return fused ? launch_ct<T, true, K, 32, RS...>(a, grid, st)
-                                    : launch_ct<T, false, K, 32, RS...>(a, grid, st);
-        if (a.W == 16) return fused ? launch_ct<T, true, K, 16, RS...>(a, grid, st)
-                                    : launch_ct<T, false, K, 16, RS...>(a, grid, st);
+template <class T, class P> int ct_size(const FFTArgs<T> &a, int mode, unsigned outer, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8) {
+        return ct_mode<T, double, P, 8>(a, mode, outer, st);
     } else {
-        if (a.W == 16) return fused ? launch_ct<T, true, K, 16, RS...>(a, grid, st)
-                                    : launch_ct<T, false, K, 16, RS...>(a, grid, st);
+        FFTArgs<T> q = a;
+        q.inner /= 2;
+        q.V /= 2;
+        return a.W == 32 ? ct_mode<T, float2, P, 16>(q, mode, outer, st) : ct_mode<T, float2, P, 8>(q, mode, outer, st);
     }
-    return -1;
 }
 
-// Spreading fused with the forward FFT along k3: a block owns one (k1, k2)
-// pencil of K mesh points and W complex probe-pair columns.  A lane takes CPL
-// adjacent columns (CPL = 2: float tiles of 32 columns, one 16-byte dipole
-// load per component for four probes), so a warp holds 32 CPL / W row chains.
-// The chains spread rows k3 = chain, chain + NSG, ... (two rows per
-// iteration: two independent load chains) straight into the shared-memory
-// tile, with the records and order of k_spread_csr; then the block transforms
-// the tile along k3 and writes it once.  Probe columns >= R are masked to zero.
-template <class T, int K, int W, int NT, int CPL, int... RS>
-__global__ void __launch_bounds__(NT) k_spread_fft3(const T *__restrict__ d, typename Cplx<T>::type *__restrict__ mesh,
-                                                    int R, int ld, int K2, const int *__restrict__ row,
-                                                    const SpreadRec<T> *__restrict__ rec,
-                                                    const typename Cplx<T>::type *__restrict__ twg) {
-    using C = typename Cplx<T>::type;
-    constexpr int LPC = W / CPL;              // lanes per row chain
-    static_assert(W % CPL == 0 && 32 % LPC == 0, "a warp holds whole row chains");
-    static_assert(CPL == 1 || sizeof(T) == 4, "column pairs per lane are float tiles");
-    constexpr int G = 32 / LPC;               // row chains per warp
-    constexpr int NSG = (NT / 32) * G;        // row chains per block
-    constexpr int NP = 2 * CPL;               // probes per lane
-    extern __shared__ __align__(16) unsigned char smem_sf[];
-    C *buf0 = reinterpret_cast<C *>(smem_sf);
-    C *buf1 = buf0 + K * W;
-    C *tw = buf1 + K * W;
-    pdl_launch_dependents();
-    for (int i = threadIdx.x; i < K; i += NT) tw[i] = twg[i];   // set up once per system
-    pdl_wait();
-    const int V = ld / 2;
-    const int ncb = (V + W - 1) / W;
-    const size_t pencil = blockIdx.x / ncb;              // k1 * K2 + k2
-    const int c0 = (int)(blockIdx.x % ncb) * W;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int cl = (lane % LPC) * CPL, chain = warp * G + lane / LPC;
-    const int col = c0 + cl;                             // complex columns col .. col + CPL - 1 = probes 2 col ..
-    const bool on = col < V;
-    T msk[NP];
-#pragma unroll
-    for (int e = 0; e < NP; ++e) msk[e] = (2 * col + e < R) ? T(1) : T(0);
-    for (int k3 = chain; k3 < K; k3 += 2 * NSG) {
-        const int kb = k3 + NSG;
-        const size_t pa = pencil * K + k3, pb = pencil * K + kb;
-        int qa = row[pa];
-        const int qa1 = row[pa + 1];
-        int qb = 0, qb1 = 0;
-        if (kb < K) {
-            qb = row[pb];
-            qb1 = row[pb + 1];
-        }
-        T acc_a[NP], acc_b[NP];
-#pragma unroll
-        for (int e = 0; e < NP; ++e) acc_a[e] = acc_b[e] = T(0);
-        // the next record of each row is loaded one iteration ahead, so that its
-        // latency overlaps the current record's dipole loads
-        SpreadRec<T> wa{}, wb{};
-        if (qa < qa1) wa = rec[qa];
-        if (qb < qb1) wb = rec[qb];
-        while (qa < qa1 || qb < qb1) {
-            const bool ha = qa < qa1, hb = qb < qb1;
-            SpreadRec<T> na = wa, nb = wb;
-            if (ha && qa + 1 < qa1) na = rec[qa + 1];
-            if (hb && qb + 1 < qb1) nb = rec[qb + 1];
-            if (ha) {
-                if (on) {
-                    T x[NP], y[NP], z[NP];
-                    const T *dj = d + (size_t)(3 * wa.atom) * ld + 2 * col;
-                    vload<T, NP>(dj, x);
-                    vload<T, NP>(dj + ld, y);
-                    vload<T, NP>(dj + 2 * (size_t)ld, z);
-#pragma unroll
-                    for (int e = 0; e < NP; ++e) acc_a[e] += wa.w0 * x[e] + wa.w1 * y[e] + wa.w2 * z[e];
-                }
-                ++qa;
-            }
-            if (hb) {
-                if (on) {
-                    T x[NP], y[NP], z[NP];
-                    const T *dj = d + (size_t)(3 * wb.atom) * ld + 2 * col;
-                    vload<T, NP>(dj, x);
-                    vload<T, NP>(dj + ld, y);
-                    vload<T, NP>(dj + 2 * (size_t)ld, z);
-#pragma unroll
-                    for (int e = 0; e < NP; ++e) acc_b[e] += wb.w0 * x[e] + wb.w1 * y[e] + wb.w2 * z[e];
-                }
-                ++qb;
-            }
-            wa = na;
-            wb = nb;
-        }
-#pragma unroll
-        for (int u = 0; u < CPL; ++u) {
-            buf0[k3 * W + cl + u] = on ? C{acc_a[2 * u] * msk[2 * u], acc_a[2 * u + 1] * msk[2 * u + 1]}
-                                       : C{T(0), T(0)};
-            if (kb < K)
-                buf0[kb * W + cl + u] = on ? C{acc_b[2 * u] * msk[2 * u], acc_b[2 * u + 1] * msk[2 * u + 1]}
-                                           : C{T(0), T(0)};
-        }
-    }
-    __syncthreads();
-    const int wc = min(W, V - c0);
-    C *base = mesh + pencil * (size_t)K * V + c0;
-    ct_pipe<T, C, K, W, NT, 1, 1, false, true, false, RS...>(base, base, (size_t)V, wc, buf0, buf1, tw, -1,
-                                                              (const T *)nullptr, 0, c0, V);
-}
+// ---------------------------------------------------------------- spreading by pencil records
+// Spline orders the spreading is compiled for.
+#define MBD_SPLINE_ORDERS(X) X(4) X(6) X(8) X(10)
 
-template <class T, int K, int W, int CPL, int... RS>
-int launch_sf3_cpl(const T *d, T *mesh, int R, int ld, int K1, int K2, const int *row, const SpreadRec<T> *rec,
-                   const typename Cplx<T>::type *tw, cudaStream_t st) {
-    using C = typename Cplx<T>::type;
-    constexpr int NT = ct_threads<K, W, RS...>();
-    const size_t smem = sizeof(C) * (2 * (size_t)K * W + K);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_spread_fft3<T, K, W, NT, CPL, RS...>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-        return 0;
-    const int V = ld / 2;
-    const unsigned grid = (unsigned)((size_t)K1 * K2 * ((V + W - 1) / W));
-    launch_pdl(true, k_spread_fft3<T, K, W, NT, CPL, RS...>, dim3(grid), dim3(NT), smem, st, d,
-               reinterpret_cast<C *>(mesh), R, ld, K2, row, rec, tw);
-    return 1;
-}
-
-// Float tiles of 32 columns take two columns per lane when the dipole rows
-// allow 16-byte loads (ld a multiple of 4).
-template <class T, int K, int W, int... RS>
-int launch_sf3(const T *d, T *mesh, int R, int ld, int K1, int K2, const int *row, const SpreadRec<T> *rec,
-               const typename Cplx<T>::type *tw, cudaStream_t st) {
-    if constexpr (sizeof(T) == 4 && W == 32) {
-        if (ld % 4 == 0) return launch_sf3_cpl<T, K, W, 2, RS...>(d, mesh, R, ld, K1, K2, row, rec, tw, st);
-    }
-    return launch_sf3_cpl<T, K, W, 1, RS...>(d, mesh, R, ld, K1, K2, row, rec, tw, st);
-}
-
-template <class T, int K, int... RS>
-int sf3_size(int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *row, const SpreadRec<T> *rec,
-             const typename Cplx<T>::type *tw, cudaStream_t st) {
-    if constexpr (sizeof(T) == 4) {
-        if (W == 32) return launch_sf3<T, K, 32, RS...>(d, mesh, R, ld, K1, K2, row, rec, tw, st);
-        if (W == 16) return launch_sf3<T, K, 16, RS...>(d, mesh, R, ld, K1, K2, row, rec, tw, st);
+// a c + b over the probes of a lane (packed for two floats), scalar c.
+template <class T, int PPL> __device__ __forceinline__ void lane_fma(const T *a, T c, T *b) {
+    if constexpr (PPL == 2 && sizeof(T) == 4) {
+        const float2 r = __ffma2_rn(make_float2(a[0], a[1]), make_float2(c, c), make_float2(b[0], b[1]));
+        b[0] = r.x;
+        b[1] = r.y;
     } else {
-        if (W == 16) return launch_sf3<T, K, 16, RS...>(d, mesh, R, ld, K1, K2, row, rec, tw, st);
+#pragma unroll
+        for (int e = 0; e < PPL; ++e) b[e] += a[e] * c;
     }
-    return -1;
 }
 
-// Spreading by pencil records (PencilRec, spline order P) fused with the
-// forward FFT along k3: a block owns one (k1, k2) pencil and W complex
-// probe-pair columns; lane l holds the PPL = 2W / 32 probes 2 c0 + l PPL ...
-// Warp w owns the rows [w K / NW, (w + 1) K / NW) of the pencil.  It walks the
-// records of the points (k1, k2, top3) for top3 from its first row to its
-// last row + P - 2 (mod K) in CSR order, which is the order of top3, and keeps
-// the P rows top3 - P + 1 .. top3 that a record of top3 reaches in registers:
-// each record adds M3(t3) (e0 . d_j) + M3'(t3) (e1 . d_j) to row top3 - t3.
-// When top3 moves past a row's last contributor the row is complete and goes
-// to the shared tile (rows outside the warp's range belong to a neighbour and
-// are dropped), so every row is a sum in a fixed order.  The next record is
-// loaded one iteration ahead.  The block then transforms the tile along k3 and
-// writes it once.  Probes >= R are zero.
-template <class T, int K, int W, int NT, int P, int... RS>
-__global__ void __launch_bounds__(NT) k_spread_pencil_fft3(const T *__restrict__ d,
-                                                           typename Cplx<T>::type *__restrict__ mesh, int R, int ld,
-                                                           const int *__restrict__ prow,
-                                                           const PencilRec<T> *__restrict__ prec,
-                                                           const T *__restrict__ k3w,
-                                                           const typename Cplx<T>::type *__restrict__ twg) {
-    using C = typename Cplx<T>::type;
-    constexpr int PPL = 2 * W / 32;           // probes per lane
-    static_assert(PPL == 1 || PPL == 2, "tiles of 16 or 32 complex columns");
-    static_assert(P <= 8, "k3 stencils hold at most 8 points");
-    constexpr int NW = NT / 32;
-    extern __shared__ __align__(16) unsigned char smem_spp[];
-    C *buf0 = reinterpret_cast<C *>(smem_spp);
-    C *buf1 = buf0 + K * W;
-    C *tw = buf1 + K * W;
-    int *rp = reinterpret_cast<int *>(tw + K);   // [K + 1] record starts of the pencil's points
-    pdl_launch_dependents();
-    const int V = ld / 2;
-    const int ncb = V / W;
-    const size_t pencil = blockIdx.x / ncb;      // k1 * K2 + k2
-    const int c0 = (int)(blockIdx.x % ncb) * W;
-    for (int i = threadIdx.x; i < K; i += NT) tw[i] = twg[i];   // set up once per system
-    for (int i = threadIdx.x; i <= K; i += NT) rp[i] = prow[pencil * K + i];
-    pdl_wait();
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r0 = warp * K / NW, r1 = (warp + 1) * K / NW;
-    const int pr0 = 2 * c0 + lane * PPL;        // first probe of the lane
-    T msk[PPL];
-#pragma unroll
-    for (int e = 0; e < PPL; ++e) msk[e] = pr0 + e < R ? T(1) : T(0);
-    T *tile = reinterpret_cast<T *>(buf0);      // [K][2W] reals
-    T acc[P][PPL];                              // acc[j]: row cur - P + 1 + j
+// A lane's walk along one pencil (k1, k2) for its PPL probes (d: the dipole
+// rows at those probes): the records of the points (k1, k2, t) for t = t0 ..
+// t1 - 1 in CSR order (record q0 up to q1; ends(t) the end of point t's
+// records), each adding M3(j) (e0 . d) + M3'(j) (e1 . d) to the rows t - j,
+// j < P.  Row t - P + 1 is complete after point t and goes to row_done; the
+// walk ends with the P - 1 rows still open after the last point.  The window
+// of P open rows is a register array whose origin moves with t, unrolled by P
+// so that it never shifts; each row is a sum in a fixed order.  The next
+// record is loaded one ahead.
+template <class T, int P, int PPL, class Ends, class Done>
+__device__ __forceinline__ void pencil_walk(const T *__restrict__ d, int ld, const PencilRec<T> *__restrict__ prec,
+                                            const T *__restrict__ k3w, int t0, int t1, int q0, int q1, Ends &&ends,
+                                            Done &&row_done) {
+    T acc[P][PPL];
 #pragma unroll
     for (int j = 0; j < P; ++j)
 #pragma unroll
         for (int e = 0; e < PPL; ++e) acc[j][e] = T(0);
-    int cur = r0;
-    // row cur - P + 1 is complete: to the tile if it is this warp's, then shift the window
-#define MBD_SPP_FLUSH_ADVANCE()                                                                     \
-    do {                                                                                            \
-        const int row_ = cur - P + 1;                                                               \
-        if (row_ >= r0) {                                                                           \
-            _Pragma("unroll") for (int e = 0; e < PPL; ++e) tile[row_ * 2 * W + lane * PPL + e] =   \
-                acc[0][e] * msk[e];                                                                 \
-        }                                                                                           \
-        _Pragma("unroll") for (int j = 0; j < P - 1; ++j)                                          \
-            _Pragma("unroll") for (int e = 0; e < PPL; ++e) acc[j][e] = acc[j + 1][e];             \
-        _Pragma("unroll") for (int e = 0; e < PPL; ++e) acc[P - 1][e] = T(0);                      \
-        ++cur;                                                                                      \
-    } while (0)
-    // the last (unwrapped) top3 reaching row r1 - 1; beyond K it wraps to 0..
-    const int last = r1 + P - 2;
-    for (int seg = 0; seg < 2; ++seg) {
-        const int t_lo = seg == 0 ? r0 : K, t_hi = seg == 0 ? min(last, K - 1) : last;   // top3 (+ K) range
-        if (t_hi < t_lo) continue;
-        int q = rp[t_lo - seg * K];
-        const int qe = rp[t_hi - seg * K + 1];
-        PencilRec<T> rc{};
-        if (q < qe) rc = prec[q];
-        for (; q < qe; ++q) {
-            PencilRec<T> rn = rc;
-            if (q + 1 < qe) rn = prec[q + 1];
-            T x[PPL], y[PPL], z[PPL];
-            const T *dj = d + (size_t)(3 * rc.atom) * ld + pr0;
-            vload<T, PPL>(dj, x);
-            vload<T, PPL>(dj + ld, y);
-            vload<T, PPL>(dj + 2 * (size_t)ld, z);
-            T m3[P], n3[P];
-            {
-                // the atom's row of 16 values (M3 at 0.., M3' at 8..), 16-byte loads
+    int q = q0;
+    PencilRec<T> rc{};
+    if (q < q1) rc = prec[q];
+    for (int tb = t0; tb < t1 + P - 1; tb += P) {
+#pragma unroll
+        for (int u = 0; u < P; ++u) {
+            const int t = tb + u;
+            if (t >= t1 + P - 1) break;
+            const int qe = t < t1 ? ends(t) : q;
+            while (q < qe) {
+                T x[PPL], y[PPL], z[PPL], w[2 * P];
+                const T *dj = d + (size_t)(3 * rc.atom) * ld;
+                vload<T, PPL>(dj, x);
+                vload<T, PPL>(dj + ld, y);
+                vload<T, PPL>(dj + 2 * (size_t)ld, z);
                 constexpr int U = 16 / (int)sizeof(T);
-                const T *kw = k3w + (size_t)rc.atom * 16;
-                T row[16];
+                const T *kw = k3w + (size_t)rc.atom * (2 * P);
 #pragma unroll
-                for (int b = 0; b < 16; b += U) {
-                    if (b < P || (b + U > 8 && b < 8 + P)) vload<T, U>(kw + b, row + b);
-                }
+                for (int b = 0; b < 2 * P; b += U) vload<T, U>(kw + b, w + b);
+                T fu[PPL], fv[PPL];
 #pragma unroll
-                for (int t = 0; t < P; ++t) {
-                    m3[t] = row[t];
-                    n3[t] = row[8 + t];
+                for (int e = 0; e < PPL; ++e) fu[e] = fv[e] = T(0);
+                lane_fma<T, PPL>(x, rc.e0[0], fu);
+                lane_fma<T, PPL>(y, rc.e0[1], fu);
+                lane_fma<T, PPL>(z, rc.e0[2], fu);
+                lane_fma<T, PPL>(x, rc.e1[0], fv);
+                lane_fma<T, PPL>(y, rc.e1[1], fv);
+                lane_fma<T, PPL>(z, rc.e1[2], fv);
+                if (++q < q1) rc = prec[q];
+#pragma unroll
+                for (int j = 0; j < P; ++j) {
+                    lane_fma<T, PPL>(fu, w[j], acc[(u - j + P) % P]);
+                    lane_fma<T, PPL>(fv, w[P + j], acc[(u - j + P) % P]);
                 }
             }
-            // complete the rows no record of this top3 or later reaches
-            const int tcur = rc.top3 + seg * K;
-            while (cur < tcur) MBD_SPP_FLUSH_ADVANCE();
+            T *done = acc[(u + 1) % P];
+            row_done(t - P + 1, done);
 #pragma unroll
-            for (int e = 0; e < PPL; ++e) {
-                const T u = rc.e0[0] * x[e] + rc.e0[1] * y[e] + rc.e0[2] * z[e];
-                const T v = rc.e1[0] * x[e] + rc.e1[1] * y[e] + rc.e1[2] * z[e];
-#pragma unroll
-                for (int t = 0; t < P; ++t) acc[P - 1 - t][e] += m3[t] * u + n3[t] * v;
-            }
-            rc = rn;
+            for (int e = 0; e < PPL; ++e) done[e] = T(0);
         }
     }
-    while (cur <= last) MBD_SPP_FLUSH_ADVANCE();
-#undef MBD_SPP_FLUSH_ADVANCE
-    __syncthreads();
-    // the forward k3 transform of the whole tile; float tiles take column
-    // pairs (one 16-byte access and one twiddle for two columns)
-    C *base = mesh + pencil * (size_t)K * V + c0;
-    constexpr int CV = sizeof(T) == 4 ? 2 : 1;
-    ct_pipe<T, C, K, W, NT, CV, 1, false, true, false, RS...>(base, base, (size_t)V, W, buf0, buf1, tw, -1,
-                                                               (const T *)nullptr, 0, c0, V);
 }
 
-template <class T, int K, int W, int... RS>
-int launch_spp(const T *d, T *mesh, int R, int ld, int K1, int K2, const int *prow, const PencilRec<T> *prec,
-               const T *k3w, const typename Cplx<T>::type *tw, cudaStream_t st) {
-    using C = typename Cplx<T>::type;
-    constexpr int NT = ct_threads<K, W, RS...>();
-    static_assert(NT % 32 == 0 && K >= 2 * 6, "whole warps; K >= 2p");
-    const size_t smem = sizeof(C) * (2 * (size_t)K * W + K) + sizeof(int) * (K + 1);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(k_spread_pencil_fft3<T, K, W, NT, 6, RS...>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return 0;
+// Probes per lane and complex columns per tile (a warp's width) of the spreading.
+template <class T> constexpr int spread_ppl() { return sizeof(T) == 4 ? 2 : 1; }
+template <class T> constexpr int spread_w() { return 16 * spread_ppl<T>(); }
+// Warps of a block: segments of at least P - 1 rows, at most 8.
+template <int K, int P> constexpr int spread_segs() { return K / (P - 1) < 8 ? K / (P - 1) : 8; }
+
+// Shared memory of a block whose tile touches `pens` pencils, and the blocks
+// per SM asked of the compiler: 32 warps (64 registers) in float and 24 in
+// double as far as shared memory holds them (128^3 x 128 probes: 663 -> 618 us
+// per launch against the compiler's own 92 registers; 192^3, where it holds
+// three blocks, 1139 us with 80 registers and 1255 with 64).
+template <class T, int K, int P> constexpr size_t spread_smem(int pens) {
+    return sizeof(typename TwOf<typename PackOf<T>::type>::type) * K +
+           sizeof(T) * 2 * (size_t)spread_w<T>() * (K + spread_segs<K, P>() * (P - 1)) +
+           sizeof(int) * ((size_t)pens * K + 1);
+}
+template <class T, int K, int P> constexpr int spread_blocks() {
+    constexpr int by_smem = (int)(227 * 1024 / (spread_smem<T, K, P>(2) + 1024)), by_regs = (sizeof(T) == 4 ? 32 : 24) / spread_segs<K, P>();
+    return by_smem < by_regs ? by_smem : by_regs;
+}
+
+// Spreading fused with the forward FFT along k3.  A block owns a tile of W
+// consecutive complex columns (pencil, probe pair) of the mesh: one pencil's
+// when the probes fill a warp, several pencils' otherwise; lane l holds the
+// tile's probes l PPL .. and so its own pencil.  The K points of the pencil
+// are cut into one segment per warp; a warp walks the records of its segment's
+// points once, its rows go to the shared tile, and the P - 1 rows below its
+// segment, which belong to the warp before (cyclically), to a halo that this
+// warp adds after a barrier.  Then the block transforms the tile and writes it.
+// Probes >= R are zero.
+// Bound: instruction issue and the latency of the dipole loads (L2).
+template <class T, class PL, int P>
+__global__ void __launch_bounds__(32 * spread_segs<PL::K, P>(), spread_blocks<T, PL::K, P>())
+    k_spread_pencil_fft3(const T *__restrict__ d, T *__restrict__ mesh, int R, int ld, unsigned ncols,
+                         const int *__restrict__ prow, const PencilRec<T> *__restrict__ prec,
+                         const T *__restrict__ k3w, const typename Cplx<T>::type *__restrict__ twg) {
+    using F = typename PackOf<T>::type;
+    using C = Cx<F>;
+    constexpr int K = PL::K, PPL = spread_ppl<T>(), W = spread_w<T>(), NSEG = spread_segs<K, P>(), NT = 32 * NSEG;
+    constexpr int WF = W * 2 * (int)sizeof(T) / (int)sizeof(C);
+    static_assert(NT % WF == 0 && NSEG >= 2, "whole rows of threads, two segments at least");
+    extern __shared__ __align__(16) unsigned char smem_spp[];
+    auto *tw = reinterpret_cast<typename TwOf<F>::type *>(smem_spp);
+    T *tile = reinterpret_cast<T *>(tw + K);          // [K][2W] reals
+    T *halo = tile + 2 * (size_t)K * W;               // [NSEG][P - 1][2W]
+    int *rp = reinterpret_cast<int *>(halo + 2 * (size_t)NSEG * (P - 1) * W);   // record starts of the tile's pencils
     const int V = ld / 2;
-    const unsigned grid = (unsigned)((size_t)K1 * K2 * (V / W));
-    launch_pdl(true, k_spread_pencil_fft3<T, K, W, NT, 6, RS...>, dim3(grid), dim3(NT), smem, st, d,
-               reinterpret_cast<C *>(mesh), R, ld, prow, prec, k3w, tw);
+    const unsigned c0 = blockIdx.x * W;
+    const unsigned pen0 = c0 / V, pen1 = min(c0 + W, ncols) - 1;   // first pencil, last column
+    const int nrp = (int)(pen1 / V - pen0 + 1) * K;
+    for (int i = threadIdx.x; i < K; i += NT) tw_set(tw[i], twg[i]);   // set up once per system
+    for (int i = threadIdx.x; i <= nrp; i += NT) rp[i] = prow[(size_t)pen0 * K + i];
+    pdl_wait();
+    pdl_launch_dependents();
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r0 = warp * K / NSEG, r1 = (warp + 1) * K / NSEG;
+    const unsigned cl = min(c0 + lane * PPL / 2, ncols - 1);      // the lane's column (the last one again past the end)
+    const unsigned pen = cl / V;
+    const int pr0 = 2 * (int)(cl - pen * V) + (lane * PPL & 1);   // its first probe
+    const int *rpp = rp + (pen - pen0) * K;
+    T *mine = tile + lane * PPL, *hmine = halo + (size_t)warp * (P - 1) * 2 * W + lane * PPL;
+    pencil_walk<T, P, PPL>(
+        d + pr0, ld, prec, k3w, r0, r1, rpp[r0], rpp[r1], [&](int t) { return rpp[t + 1]; },
+        [&](int row, const T *v) {
+            T o[PPL];
+#pragma unroll
+            for (int e = 0; e < PPL; ++e) o[e] = pr0 + e < R ? v[e] : T(0);
+            vstore<T, PPL>(row >= r0 ? mine + row * 2 * W : hmine + (row - r0 + P - 1) * 2 * W, o);
+        });
+    __syncthreads();
+    {
+        const T *h = halo + (size_t)((warp + 1) % NSEG) * (P - 1) * 2 * W + lane * PPL;
+        T *o = mine + (r1 - (P - 1)) * 2 * W;
+#pragma unroll
+        for (int j = 0; j < P - 1; ++j) {
+            T x[PPL], y[PPL];
+            vload<T, PPL>(h + j * 2 * W, x);
+            vload<T, PPL>(o + j * 2 * W, y);
+#pragma unroll
+            for (int e = 0; e < PPL; ++e) y[e] += x[e];
+            vstore<T, PPL>(o + j * 2 * W, y);
+        }
+    }
+    __syncthreads();
+    const unsigned VF = (unsigned)((size_t)ld * sizeof(T) / sizeof(C)), nf = ncols / V * VF;
+    const unsigned cg = blockIdx.x * WF + threadIdx.x % WF;
+    const bool valid = cg < nf;
+    const unsigned pf = (valid ? cg : 0) / VF;
+    ct_transform<PL, F, WF, NT, false>(reinterpret_cast<C *>(tile), tw,
+                                       reinterpret_cast<C *>(mesh) + (size_t)pf * K * VF + ((valid ? cg : 0) - pf * VF),
+                                       VF, valid);
+}
+
+template <class T, class PL, int P>
+int launch_spp(const SpreadArgs<T> &a, cudaStream_t st) {
+    constexpr int K = PL::K, W = spread_w<T>(), NSEG = spread_segs<K, P>();
+    auto kern = k_spread_pencil_fft3<T, PL, P>;
+    const int V = a.ld / 2;
+    const int pens = (W - 1) / V + 2;              // pencils that a tile can touch
+    const size_t smem = spread_smem<T, K, P>(pens);
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return 0;
+    const unsigned ncols = (unsigned)((size_t)a.K1 * a.K2 * V);
+    launch_pdl(true, kern, dim3((ncols + W - 1) / W), dim3(32 * NSEG), smem, st, a.d, a.mesh, a.R, a.ld, ncols, a.prow,
+               a.prec, a.k3w, a.tw);
     return 1;
 }
-
-template <class T, int K, int... RS>
-int spp_size(int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *prow, const PencilRec<T> *prec,
-             const T *k3w, const typename Cplx<T>::type *tw, cudaStream_t st) {
-    if constexpr (sizeof(T) == 4) {
-        if (W == 32) return launch_spp<T, K, 32, RS...>(d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st);
-        if (W == 16) return launch_spp<T, K, 16, RS...>(d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st);
-    } else {
-        if (W == 16) return launch_spp<T, K, 16, RS...>(d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st);
-    }
+template <class T, class PL> int spp_size(const SpreadArgs<T> &a, cudaStream_t st) {
+#define MBD_SPP_ORDER(P) \
+    case P: \
+        if constexpr (PL::K >= 2 * (P)) return launch_spp<T, PL, P>(a, st); \
+        break;
+    switch (a.p) { MBD_SPLINE_ORDERS(MBD_SPP_ORDER) }
+#undef MBD_SPP_ORDER
     return -1;
 }
 
@@ -823,36 +904,19 @@ int spp_size(int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const in
 
 // The translation unit of group g: dispatch over its sizes.
 #define MBD_CT_CASE(K, ...) \
-    case K: return ct_size<T, K, __VA_ARGS__>(a, fused, grid, st);
-#define MBD_SF3_CASE(K, ...) \
-    case K: return sf3_size<T, K, __VA_ARGS__>(W, d, mesh, R, ld, K1, K2, row, rec, tw, st);
+    case K: return ct_size<T, Plan<__VA_ARGS__>>(a, mode, outer, st);
 #define MBD_SPP_CASE(K, ...) \
-    case K: return spp_size<T, K, __VA_ARGS__>(W, d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st);
+    case K: return spp_size<T, Plan<__VA_ARGS__>>(a, st);
 #define MBD_FFT_GROUP_TU(g)                                                                                       \
-    template <class T> int launch_fft_ct_group##g(const FFTArgs<T> &a, bool fused, unsigned grid, cudaStream_t st) { \
+    template <class T> int launch_fft_ct_group##g(const FFTArgs<T> &a, int mode, unsigned outer, cudaStream_t st) { \
         switch (a.K) { MBD_FFT_GROUP##g(MBD_CT_CASE) default: return -1; }                                         \
     }                                                                                                              \
-    template <class T>                                                                                             \
-    int launch_sf3_group##g(int K3, int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *row,    \
-                            const SpreadRec<T> *rec, const typename Cplx<T>::type *tw, cudaStream_t st) {          \
-        switch (K3) { MBD_FFT_GROUP##g(MBD_SF3_CASE) default: return -1; }                                         \
+    template <class T> int launch_spp_group##g(const SpreadArgs<T> &a, cudaStream_t st) {                          \
+        switch (a.K3) { MBD_FFT_GROUP##g(MBD_SPP_CASE) default: return -1; }                                       \
     }                                                                                                              \
-    template int launch_fft_ct_group##g<float>(const FFTArgs<float> &, bool, unsigned, cudaStream_t);              \
-    template int launch_fft_ct_group##g<double>(const FFTArgs<double> &, bool, unsigned, cudaStream_t);            \
-    template int launch_sf3_group##g<float>(int, int, const float *, float *, int, int, int, int, const int *,     \
-                                            const SpreadRec<float> *, const float2 *, cudaStream_t);               \
-    template int launch_sf3_group##g<double>(int, int, const double *, double *, int, int, int, int, const int *,  \
-                                             const SpreadRec<double> *, const double2 *, cudaStream_t);           \
-    template <class T>                                                                                             \
-    int launch_spp_group##g(int K3, int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *prow,    \
-                            const PencilRec<T> *prec, const T *k3w, const typename Cplx<T>::type *tw,              \
-                            cudaStream_t st) {                                                                     \
-        switch (K3) { MBD_FFT_GROUP##g(MBD_SPP_CASE) default: return -1; }                                         \
-    }                                                                                                              \
-    template int launch_spp_group##g<float>(int, int, const float *, float *, int, int, int, int, const int *,     \
-                                            const PencilRec<float> *, const float *, const float2 *, cudaStream_t); \
-    template int launch_spp_group##g<double>(int, int, const double *, double *, int, int, int, int, const int *,  \
-                                             const PencilRec<double> *, const double *, const double2 *,          \
-                                             cudaStream_t);
+    template int launch_fft_ct_group##g<float>(const FFTArgs<float> &, int, unsigned, cudaStream_t);               \
+    template int launch_fft_ct_group##g<double>(const FFTArgs<double> &, int, unsigned, cudaStream_t);             \
+    template int launch_spp_group##g<float>(const SpreadArgs<float> &, cudaStream_t);                              \
+    template int launch_spp_group##g<double>(const SpreadArgs<double> &, cudaStream_t);
 
 }  // namespace mbd

@@ -588,8 +588,6 @@ __global__ void k_mesh_in(const double *__restrict__ in, int nvec, size_t npts, 
 
 }  // namespace
 
-int probe_ld(int R) { return R + (R & 1); }
-
 mbd_status launch_prologue_t(cudaStream_t st, const LanczosView &lz, int k, int m, uint64_t seed, int R, int ld,
                              int rows, const double *g, void *dout, int dtype_bytes, int nblk,
                              const uint64_t *seed_dev) {

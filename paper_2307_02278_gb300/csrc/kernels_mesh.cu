@@ -14,160 +14,10 @@ namespace {
 constexpr int kWarps = 8;          // warps per block in the field kernel
 
 // ---------------------------------------------------------------- spreading
-// The dipole array D(k) = sum_j d_j . grad W_j(k) (Eq. dipolarr) is a sparse
-// matrix W^T (one row per mesh point, one nonzero per atom whose stencil covers
-// the point) times the dense block of dipoles [3N][probes].  W^T is built once
-// per geometry in a fixed atom order, so every mesh value is a sum in a fixed
-// order: spreading is deterministic and writes each mesh point once.
-
-// Rows of W^T: a thread per mesh point visits the atoms of the bricks whose
-// stencils can reach it (binned by their last stencil point) in a fixed order;
-// FILL = false counts, FILL = true writes the Cartesian weights
-//   dW/dR_alpha = sum_beta C_{beta alpha} dW/du_beta,
-//   dW/du = (M'(u1) M(u2) M(u3), M(u1) M'(u2) M(u3), M(u1) M(u2) M'(u3)),
-// from FP64 stencil weights.
-template <class T, bool FILL>
-__global__ void k_spread_rows(Geom g, BinView B, const int *__restrict__ top, const double *__restrict__ w64,
-                              const double *__restrict__ dw64, int *__restrict__ cnt_or_row,
-                              SpreadRec<T> *__restrict__ rec) {
-    const size_t npts = (size_t)g.K1 * g.K2 * g.K3;
-    const size_t pt = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pt >= npts) return;
-    const int g3 = (int)(pt % g.K3), g2 = (int)((pt / g.K3) % g.K2), g1 = (int)(pt / ((size_t)g.K2 * g.K3));
-    const int bb1 = g1 / B.bs1, bb2 = g2 / B.bs2, bb3 = g3 / B.bs3;
-    const int p = g.p;
-    int c = 0;
-    const int base = FILL ? cnt_or_row[pt] : 0;
-    for (int c1 = 0; c1 < B.nc1; ++c1) {
-        const int t1 = (bb1 + c1) % B.nb1;
-        for (int c2 = 0; c2 < B.nc2; ++c2) {
-            const int t2 = (bb2 + c2) % B.nb2;
-            for (int c3 = 0; c3 < B.nc3; ++c3) {
-                const int t3 = (bb3 + c3) % B.nb3;
-                const int bin = (t1 * B.nb2 + t2) * B.nb3 + t3;
-                for (int s = B.start[bin]; s < B.start[bin + 1]; ++s) {
-                    const int j = B.atoms[s];
-                    int u1 = top[3 * j] - g1;
-                    if (u1 < 0) u1 += g.K1;
-                    int u2 = top[3 * j + 1] - g2;
-                    if (u2 < 0) u2 += g.K2;
-                    int u3 = top[3 * j + 2] - g3;
-                    if (u3 < 0) u3 += g.K3;
-                    if (u1 >= p || u2 >= p || u3 >= p) continue;
-                    if (FILL) {
-                        const double *w = w64 + (size_t)3 * p * j, *dw = dw64 + (size_t)3 * p * j;
-                        const double m1 = w[u1], m2 = w[p + u2], m3 = w[2 * p + u3];
-                        const double n1 = dw[u1], n2 = dw[p + u2], n3 = dw[2 * p + u3];
-                        const double gu0 = n1 * m2 * m3, gu1 = m1 * n2 * m3, gu2 = m1 * m2 * n3;
-                        SpreadRec<T> r;
-                        r.w0 = T(g.cmat[0] * gu0 + g.cmat[3] * gu1 + g.cmat[6] * gu2);
-                        r.w1 = T(g.cmat[1] * gu0 + g.cmat[4] * gu1 + g.cmat[7] * gu2);
-                        r.w2 = T(g.cmat[2] * gu0 + g.cmat[5] * gu1 + g.cmat[8] * gu2);
-                        r.atom = j;
-                        rec[base + c] = r;
-                    }
-                    ++c;
-                }
-            }
-        }
-    }
-    if (!FILL) cnt_or_row[pt] = c;
-}
-
-// The same rows with a block per brick: the candidate atoms of the brick's
-// points (the atoms of its nc1 x nc2 x nc3 candidate bricks, in the order the
-// per-point kernel visits them) are staged once in shared memory, with their
-// top stencil points, and a thread per point of the brick tests them there.
-// The rows are identical to k_spread_rows'.  A brick with more than
-// kRowsCap candidates reads them from global memory instead.
-constexpr int kRowsCap = 512;
-constexpr int kRowsMaxBins = 512;
-template <class T, bool FILL>
-__global__ void k_spread_rows_brick(Geom g, BinView B, const int *__restrict__ top, const double *__restrict__ w64,
-                                    const double *__restrict__ dw64, int *__restrict__ cnt_or_row,
-                                    SpreadRec<T> *__restrict__ rec) {
-    __shared__ int cj[kRowsCap], ct[kRowsCap][3];
-    __shared__ int boff[kRowsMaxBins + 1], bfirst[kRowsMaxBins];
-    const int tid = threadIdx.x;
-    const int brick = blockIdx.x;
-    const int bb1 = brick / (B.nb2 * B.nb3), bb2 = (brick / B.nb3) % B.nb2, bb3 = brick % B.nb3;
-    const int nbc = B.nc1 * B.nc2 * B.nc3;
-    for (int t = tid; t < nbc; t += blockDim.x) {
-        const int c1 = t / (B.nc2 * B.nc3), c2 = (t / B.nc3) % B.nc2, c3 = t % B.nc3;
-        const int bin = (((bb1 + c1) % B.nb1) * B.nb2 + (bb2 + c2) % B.nb2) * B.nb3 + (bb3 + c3) % B.nb3;
-        bfirst[t] = B.start[bin];
-        boff[t + 1] = B.start[bin + 1] - B.start[bin];
-    }
-    __syncthreads();
-    if (tid == 0) {
-        boff[0] = 0;
-        for (int t = 0; t < nbc; ++t) boff[t + 1] += boff[t];
-    }
-    __syncthreads();
-    const int total = boff[nbc];
-    const bool staged = total <= kRowsCap;
-    if (staged) {
-        for (int k = tid; k < total; k += blockDim.x) {
-            int lo = 0, hi = nbc - 1;   // the candidate brick holding entry k
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) / 2;
-                if (boff[mid] <= k) lo = mid;
-                else hi = mid - 1;
-            }
-            const int j = B.atoms[bfirst[lo] + (k - boff[lo])];
-            cj[k] = j;
-            ct[k][0] = top[3 * j];
-            ct[k][1] = top[3 * j + 1];
-            ct[k][2] = top[3 * j + 2];
-        }
-    }
-    __syncthreads();
-    const int npb = B.bs1 * B.bs2 * B.bs3;
-    if (tid >= npb) return;
-    const int g1 = bb1 * B.bs1 + tid / (B.bs2 * B.bs3), g2 = bb2 * B.bs2 + (tid / B.bs3) % B.bs2,
-              g3 = bb3 * B.bs3 + tid % B.bs3;
-    const size_t pt = ((size_t)g1 * g.K2 + g2) * g.K3 + g3;
-    const int p = g.p;
-    int c = 0;
-    const int base = FILL ? cnt_or_row[pt] : 0;
-    for (int k = 0; k < total; ++k) {
-        int j, tj1, tj2, tj3;
-        if (staged) {
-            j = cj[k];
-            tj1 = ct[k][0];
-            tj2 = ct[k][1];
-            tj3 = ct[k][2];
-        } else {
-            int t = 0;
-            while (boff[t + 1] <= k) ++t;
-            j = B.atoms[bfirst[t] + (k - boff[t])];
-            tj1 = top[3 * j];
-            tj2 = top[3 * j + 1];
-            tj3 = top[3 * j + 2];
-        }
-        int u1 = tj1 - g1;
-        if (u1 < 0) u1 += g.K1;
-        int u2 = tj2 - g2;
-        if (u2 < 0) u2 += g.K2;
-        int u3 = tj3 - g3;
-        if (u3 < 0) u3 += g.K3;
-        if (u1 >= p || u2 >= p || u3 >= p) continue;
-        if (FILL) {
-            const double *w = w64 + (size_t)3 * p * j, *dw = dw64 + (size_t)3 * p * j;
-            const double m1 = w[u1], m2 = w[p + u2], m3 = w[2 * p + u3];
-            const double n1 = dw[u1], n2 = dw[p + u2], n3 = dw[2 * p + u3];
-            const double gu0 = n1 * m2 * m3, gu1 = m1 * n2 * m3, gu2 = m1 * m2 * n3;
-            SpreadRec<T> r;
-            r.w0 = T(g.cmat[0] * gu0 + g.cmat[3] * gu1 + g.cmat[6] * gu2);
-            r.w1 = T(g.cmat[1] * gu0 + g.cmat[4] * gu1 + g.cmat[7] * gu2);
-            r.w2 = T(g.cmat[2] * gu0 + g.cmat[5] * gu1 + g.cmat[8] * gu2);
-            r.atom = j;
-            rec[base + c] = r;
-        }
-        ++c;
-    }
-    if (!FILL) cnt_or_row[pt] = c;
-}
+// The dipole array D(k) = sum_j d_j . grad W_j(k) (Eq. dipolarr) from the
+// pencil records, built once per geometry in a fixed atom order, so every mesh
+// value is a sum in a fixed order: spreading is deterministic and writes each
+// mesh point once.
 
 // Pencil records (PencilRec): a thread per mesh point (k1, k2, k3) finds the
 // atoms whose top stencil point is (k1 + t1, k2 + t2, k3), t1, t2 < p (mod K),
@@ -225,17 +75,14 @@ __global__ void k_pencil_rows(Geom g, BinView B, const int *__restrict__ top, co
 }
 
 // The k3 stencil of each atom for the pencil spreading: k3w[j][t] = M3(t),
-// k3w[j][8 + t] = M3'(t) (t < p <= 8), zero elsewhere.
+// k3w[j][p + t] = M3'(t).
 template <class T>
 __global__ void k_pencil_k3w(int N, int p, const double *__restrict__ w64, const double *__restrict__ dw64,
                              T *__restrict__ k3w) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 16 * N) return;
-    const int j = idx / 16, t = idx % 16;
-    const int tt = t & 7;
-    double v = 0.0;
-    if (tt < p) v = (t < 8 ? w64 : dw64)[(size_t)(3 * j + 2) * p + tt];
-    k3w[idx] = T(v);
+    if (idx >= 2 * p * N) return;
+    const int j = idx / (2 * p), t = idx % (2 * p);
+    k3w[idx] = T(t < p ? w64[(size_t)(3 * j + 2) * p + t] : dw64[(size_t)(3 * j + 2) * p + t - p]);
 }
 
 // Exclusive scan of n counts (blocks of 4096), the block sums, and the fix-up.
@@ -279,117 +126,81 @@ __global__ void k_scan_add(int *__restrict__ out, const int *__restrict__ bsum, 
     if (i < n) out[i] += bsum[i / 4096];
 }
 
-// D = W^T d.  A warp takes one mesh point (row) at a time, two rows
-// interleaved for memory-level parallelism; lane owns VEC consecutive probes.
-// Every lane reads the row's records directly (one broadcast 16-byte load per
-// record) and the dipoles with vector loads.  Rows are summed in record order
-// (fixed), so the result is deterministic.  Probe columns R..ld-1 (padding of
-// an odd probe count) are masked to zero.
-template <class T, int VEC>
-__global__ void __launch_bounds__(256) k_spread_csr(const T *__restrict__ d, T *__restrict__ mesh, int R, int ld,
-                                                    size_t npts, const int *__restrict__ row,
-                                                    const SpreadRec<T> *__restrict__ rec) {
-    constexpr int U = 2;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int r0 = (blockIdx.y * 32 + lane) * VEC;
-    const bool in_ld = r0 < ld;
-    const size_t nw = (size_t)gridDim.x * 8;
-    T mask[VEC];
+// The spreading alone, for mesh lengths without a fused pass and for the
+// stage-level call: a warp per tile of W complex columns, each lane walking its
+// pencil from top3 = 0 to K3 - 1.  The P - 1 rows below the first point are
+// kept in shared memory and added to the last rows, which they are.
+template <class T, int P>
+__global__ void __launch_bounds__(128) k_spread_pencil(SpreadArgs<T> a, unsigned ncols) {
+    constexpr int PPL = spread_ppl<T>(), W = spread_w<T>();
+    __shared__ __align__(16) T halo[4][P - 1][2 * W];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, K = a.K3, V = a.ld / 2;
+    const unsigned c = (blockIdx.x * 4 + warp) * W + lane * PPL / 2;
+    if (c >= ncols) return;
+    const unsigned pen = c / V;
+    const int pr0 = 2 * (int)(c - pen * V) + (lane * PPL & 1);
+    const int *rp = a.prow + (size_t)pen * K;
+    T *out = a.mesh + (size_t)pen * K * a.ld + pr0;
+    pencil_walk<T, P, PPL>(
+        a.d + pr0, a.ld, a.prec, a.k3w, 0, K, rp[0], rp[K], [&](int t) { return rp[t + 1]; },
+        [&](int row, const T *v) {
+            T o[PPL];
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) mask[v] = (r0 + v < R) ? T(1) : T(0);
-    for (size_t pt0 = (size_t)blockIdx.x * 8 + warp; pt0 < npts; pt0 += nw * U) {
-        int q[U], qe[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const size_t pt = pt0 + u * nw;
-            q[u] = pt < npts ? row[pt] : 0;
-            qe[u] = pt < npts ? row[pt + 1] : 0;
-        }
-        T acc[U][VEC];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) acc[u][v] = T(0);
-        bool more = true;
-        while (more) {
-            more = false;
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (q[u] < qe[u]) {
-                    const SpreadRec<T> w = rec[q[u]];
-                    ++q[u];
-                    more = more || q[u] < qe[u];
-                    if (in_ld) {
-                        T x[VEC], y[VEC], z[VEC];
-                        const T *dj = d + (size_t)(3 * w.atom) * ld + r0;
-                        vload<T, VEC>(dj, x);
-                        vload<T, VEC>(dj + ld, y);
-                        vload<T, VEC>(dj + 2 * (size_t)ld, z);
-#pragma unroll
-                        for (int v = 0; v < VEC; ++v) acc[u][v] += w.w0 * x[v] + w.w1 * y[v] + w.w2 * z[v];
-                    }
-                }
+            for (int e = 0; e < PPL; ++e) o[e] = pr0 + e < a.R ? v[e] : T(0);
+            if (row < 0) {
+                vstore<T, PPL>(&halo[warp][row + P - 1][lane * PPL], o);
+                return;
             }
-        }
-        if (in_ld) {
+            if (row >= K - (P - 1)) {
+                T h[PPL];
+                vload<T, PPL>(&halo[warp][row - (K - (P - 1))][lane * PPL], h);
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const size_t pt = pt0 + u * nw;
-                if (pt < npts) {
-                    T o[VEC];
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) o[v] = acc[u][v] * mask[v];
-                    vstore<T, VEC>(mesh + pt * ld + r0, o);
-                }
+                for (int e = 0; e < PPL; ++e) o[e] += h[e];
             }
-        }
-    }
+            vstore<T, PPL>(out + (size_t)row * a.ld, o);
+        });
 }
 
 // One radix-R Stockham stage over the K rows of a K x W tile in shared memory
 // (R compile-time, so the butterfly stays in registers).
-template <class T, class C, int R>
-__device__ __forceinline__ void stockham_stage(const C *__restrict__ in, C *__restrict__ out,
-                                               const C *__restrict__ tw, int K, int W, int Ns, int sign) {
+template <class F, int R, bool INV>
+__device__ __forceinline__ void stockham_stage(const Cx<F> *__restrict__ in, Cx<F> *__restrict__ out,
+                                               const typename TwOf<F>::type *__restrict__ tw, int K, int W, int Ns) {
     const int nb = K / R;
     const int step = K / (Ns * R);
     for (int idx = threadIdx.x; idx < nb * W; idx += blockDim.x) {
         const int j = idx / W, col = idx - j * W;
-        C v[R];
+        Cx<F> v[R];
 #pragma unroll
-        for (int q = 0; q < R; ++q) v[q] = in[(j + q * nb) * W + col];
+        for (int q = 0; q < R; ++q) v[q] = cld(in + (j + q * nb) * W + col);
         const int jm = j % Ns;
         if (jm != 0) {
 #pragma unroll
-            for (int q = 1; q < R; ++q) {
-                C t = tw[q * jm * step];
-                if (sign > 0) t.y = -t.y;
-                v[q] = cmul(v[q], t);
-            }
+            for (int q = 1; q < R; ++q) v[q] = ctw<INV>(v[q], tw[q * jm * step]);
         }
-        dft<T, C, R>(v, sign);
+        Dft<F, R, INV>::run(v);
         const int base = (j / Ns) * Ns * R + jm;
 #pragma unroll
-        for (int q = 0; q < R; ++q) out[(base + q * Ns) * W + col] = v[q];
+        for (int q = 0; q < R; ++q) cst(out + (base + q * Ns) * W + col, v[q]);
     }
 }
 
 // Mixed-radix Stockham passes over the K rows of a K x W tile held in shared
 // memory; returns the buffer that holds the result (natural order).
-template <class T, class C>
-__device__ C *stockham(C *in, C *out, const FFTArgs<T> &a, const C *tw, int sign) {
+template <class T, class F, bool INV>
+__device__ Cx<F> *stockham(Cx<F> *in, Cx<F> *out, const FFTArgs<T> &a, const typename TwOf<F>::type *tw) {
     int Ns = 1;
     for (int s = 0; s < a.nst; ++s) {
         const int R = (int)((a.radices >> (4 * s)) & 15ull);
         switch (R) {
-            case 2: stockham_stage<T, C, 2>(in, out, tw, a.K, a.W, Ns, sign); break;
-            case 3: stockham_stage<T, C, 3>(in, out, tw, a.K, a.W, Ns, sign); break;
-            case 4: stockham_stage<T, C, 4>(in, out, tw, a.K, a.W, Ns, sign); break;
-            case 5: stockham_stage<T, C, 5>(in, out, tw, a.K, a.W, Ns, sign); break;
-            default: stockham_stage<T, C, 8>(in, out, tw, a.K, a.W, Ns, sign); break;
+            case 2: stockham_stage<F, 2, INV>(in, out, tw, a.K, a.W, Ns); break;
+            case 3: stockham_stage<F, 3, INV>(in, out, tw, a.K, a.W, Ns); break;
+            case 4: stockham_stage<F, 4, INV>(in, out, tw, a.K, a.W, Ns); break;
+            case 5: stockham_stage<F, 5, INV>(in, out, tw, a.K, a.W, Ns); break;
+            default: stockham_stage<F, 8, INV>(in, out, tw, a.K, a.W, Ns); break;
         }
         __syncthreads();
-        C *t = in;
+        Cx<F> *t = in;
         in = out;
         out = t;
         Ns *= R;
@@ -397,29 +208,31 @@ __device__ C *stockham(C *in, C *out, const FFTArgs<T> &a, const C *tw, int sign
     return in;
 }
 
-// One 1D FFT pass along the middle axis of [outer][K][inner] (complex); with
-// FUSED the pass is forward, then multiplies by G(k1, k2, k3), then inverse.
-template <class T, bool FUSED>
+// One 1D FFT pass along the middle axis of [outer][K][inner] (values Cx<F>)
+// for the lengths without a compile-time pass; MODE 0 forward, 1 inverse, 2
+// forward, multiplied by G(k1, k2, k3), inverse.
+template <class T, class F, int MODE>
 __global__ void __launch_bounds__(256) k_fft_pass(FFTArgs<T> a) {
-    using C = typename Cplx<T>::type;
+    using C = Cx<F>;
+    using TW = typename TwOf<F>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *b0 = reinterpret_cast<C *>(smem_raw);
+    TW *tw = reinterpret_cast<TW *>(smem_raw);
+    C *b0 = reinterpret_cast<C *>(tw + a.K);
     C *b1 = b0 + a.K * a.W;
-    C *tw = b1 + a.K * a.W;
-    for (int i = threadIdx.x; i < a.K; i += blockDim.x) tw[i] = a.tw[i];
+    for (int i = threadIdx.x; i < a.K; i += blockDim.x) tw_set(tw[i], a.tw[i]);
     const int ncb = (a.inner + a.W - 1) / a.W;
     const size_t outer = blockIdx.x / ncb;
     const int c0 = (int)(blockIdx.x % ncb) * a.W;
     const int wc = min(a.W, a.inner - c0);
-    C *base = a.data + outer * (size_t)a.K * a.inner + c0;
+    C *base = reinterpret_cast<C *>(a.data) + outer * (size_t)a.K * a.inner + c0;
     for (int idx = threadIdx.x; idx < a.K * a.W; idx += blockDim.x) {
         const int row = idx / a.W, col = idx - row * a.W;
-        b0[idx] = col < wc ? base[(size_t)row * a.inner + col] : C{T(0), T(0)};
+        if (col < wc) cst(b0 + idx, cld(base + (size_t)row * a.inner + col));
     }
     __syncthreads();
     C *res;
-    if (FUSED) {
-        res = stockham<T, C>(b0, b1, a, tw, -1);
+    if (MODE == 2) {
+        res = stockham<T, F, false>(b0, b1, a, tw);
         C *other = (res == b0) ? b1 : b0;
         // G index: (outer, row, (c0 + col) / V)
         const T *Gb = a.G + outer * (size_t)a.K * (a.inner / a.V);
@@ -427,19 +240,32 @@ __global__ void __launch_bounds__(256) k_fft_pass(FFTArgs<T> a) {
             const int row = idx / a.W, col = idx - row * a.W;
             if (col < wc) {
                 const T gv = Gb[(size_t)row * (a.inner / a.V) + (c0 + col) / a.V];
-                res[idx].x *= gv;
-                res[idx].y *= gv;
+                res[idx] = {fmulc(res[idx].x, gv), fmulc(res[idx].y, gv)};
             }
         }
         __syncthreads();
-        res = stockham<T, C>(res, other, a, tw, +1);
+        res = stockham<T, F, true>(res, other, a, tw);
     } else {
-        res = stockham<T, C>(b0, b1, a, tw, a.sign);
+        res = stockham<T, F, MODE == 1>(b0, b1, a, tw);
     }
     for (int idx = threadIdx.x; idx < a.K * a.W; idx += blockDim.x) {
         const int row = idx / a.W, col = idx - row * a.W;
-        if (col < wc) base[(size_t)row * a.inner + col] = res[idx];
+        if (col < wc) cst(base + (size_t)row * a.inner + col, cld(res + idx));
     }
+}
+
+// The generic pass over columns of Cx<F> (a.inner, a.V and a.W in that unit);
+// the tile narrows until its two buffers fit in shared memory.
+template <class T, class F> mbd_status launch_fft_generic(FFTArgs<T> a, int mode, unsigned outer, cudaStream_t st) {
+    auto bytes = [&] { return sizeof(typename TwOf<F>::type) * a.K + 2 * sizeof(Cx<F>) * (size_t)a.K * a.W; };
+    while (a.W > 1 && bytes() > 200 * 1024) a.W = (a.W + 1) / 2;
+    auto kern = mode == 0 ? k_fft_pass<T, F, 0> : (mode == 1 ? k_fft_pass<T, F, 1> : k_fft_pass<T, F, 2>);
+    const size_t smem = bytes();
+    if (smem > 48 * 1024)
+        MBD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<(unsigned)((size_t)outer * ((a.inner + a.W - 1) / a.W)), 256, smem, st>>>(a);
+    MBD_LAUNCH_CHECK();
+    return MBD_OK;
 }
 
 // ---------------------------------------------------------------- real space on clusters
@@ -872,53 +698,9 @@ mbd_status launch_exclusive_scan(const int *in, int *out, int n, DevBuf &bsum, c
     return MBD_OK;
 }
 
-template <class T> mbd_status build_pencil_records(mbd_system *s);
-
-template <class T> mbd_status build_spread_matrix(mbd_system *s) {
-    PrecData<T> &P = prec<T>(s);
-    const Geom g = geom_of(s);
-    const size_t npts = (size_t)s->K[0] * s->K[1] * s->K[2];
-    if (npts >= 0x7fffffffULL) return MBD_ERR_UNSUPPORTED;
-    // every atom's stencil covers p^3 distinct points (K >= 2p), so the matrix
-    // has exactly p^3 N records
-    const size_t nnz = (size_t)s->p * s->p * s->p * (size_t)s->N;
-    if (nnz >= 0x7fffffffULL) return MBD_ERR_UNSUPPORTED;
-    MBD_TRY(P.srow.ensure(sizeof(int) * (npts + 1)));
-    MBD_TRY(P.srec.ensure(sizeof(SpreadRec<T>) * std::max<size_t>(1, nnz)));
-    DevBuf &cnt = s->scan_cnt, &bsum = s->scan_bsum;
-    MBD_TRY(cnt.ensure(sizeof(int) * npts));
-    const int threads = 256;
-    const BinView &B = s->bins;
-    const int npb = B.bs1 * B.bs2 * B.bs3;
-    if (B.nc1 * B.nc2 * B.nc3 <= kRowsMaxBins && npb <= 1024) {
-        // a block per brick
-        const unsigned nbricks = (unsigned)(B.nb1 * B.nb2 * B.nb3);
-        const unsigned bt = (unsigned)((npb + 31) / 32 * 32);
-        k_spread_rows_brick<T, false><<<nbricks, bt, 0, s->stream>>>(g, B, s->top_d.as<int>(), s->w64_d.as<double>(),
-                                                                    s->dw64_d.as<double>(), cnt.as<int>(), nullptr);
-        MBD_LAUNCH_CHECK();
-        MBD_TRY(launch_exclusive_scan(cnt.as<int>(), P.srow.template as<int>(), (int)npts, bsum, s->stream));
-        k_spread_rows_brick<T, true><<<nbricks, bt, 0, s->stream>>>(g, B, s->top_d.as<int>(), s->w64_d.as<double>(),
-                                                                   s->dw64_d.as<double>(), P.srow.template as<int>(),
-                                                                   P.srec.template as<SpreadRec<T>>());
-        MBD_LAUNCH_CHECK();
-        return s->p == kPencilOrder ? build_pencil_records<T>(s) : MBD_OK;
-    }
-    const unsigned blocks = (unsigned)((npts + threads - 1) / threads);
-    k_spread_rows<T, false><<<blocks, threads, 0, s->stream>>>(g, s->bins, s->top_d.as<int>(), s->w64_d.as<double>(),
-                                                              s->dw64_d.as<double>(), cnt.as<int>(), nullptr);
-    MBD_LAUNCH_CHECK();
-    MBD_TRY(launch_exclusive_scan(cnt.as<int>(), P.srow.template as<int>(), (int)npts, bsum, s->stream));
-    k_spread_rows<T, true><<<blocks, threads, 0, s->stream>>>(g, s->bins, s->top_d.as<int>(), s->w64_d.as<double>(),
-                                                             s->dw64_d.as<double>(), P.srow.template as<int>(),
-                                                             P.srec.template as<SpreadRec<T>>());
-    MBD_LAUNCH_CHECK();
-    return s->p == kPencilOrder ? build_pencil_records<T>(s) : MBD_OK;
-}
-
-// The pencil records of spline order 6 (the order of the fused pencil
-// spreading): counts, CSR starts, records, and the per-atom k3 stencils.
-template <class T> mbd_status build_pencil_records(mbd_system *s) {
+// The spreading records of the current geometry: counts, CSR starts, records,
+// and the per-atom k3 stencils.
+template <class T> mbd_status build_spread_records(mbd_system *s) {
     PrecData<T> &P = prec<T>(s);
     const Geom g = geom_of(s);
     const size_t npts = (size_t)s->K[0] * s->K[1] * s->K[2];
@@ -926,7 +708,7 @@ template <class T> mbd_status build_pencil_records(mbd_system *s) {
     if (npts >= 0x7fffffffULL || nnz >= 0x7fffffffULL) return MBD_ERR_UNSUPPORTED;
     MBD_TRY(P.prow.ensure(sizeof(int) * (npts + 1)));
     MBD_TRY(P.prec.ensure(sizeof(PencilRec<T>) * std::max<size_t>(1, nnz)));
-    MBD_TRY(P.k3w.ensure(sizeof(T) * 16 * std::max(1, s->N)));
+    MBD_TRY(P.k3w.ensure(sizeof(T) * 2 * s->p * std::max(1, s->N)));
     DevBuf &cnt = s->scan_cnt, &bsum = s->scan_bsum;
     MBD_TRY(cnt.ensure(sizeof(int) * npts));
     const int threads = 256;
@@ -940,27 +722,30 @@ template <class T> mbd_status build_pencil_records(mbd_system *s) {
                                                              P.prec.template as<PencilRec<T>>());
     MBD_LAUNCH_CHECK();
     if (s->N > 0) {
-        k_pencil_k3w<T><<<(16 * s->N + threads - 1) / threads, threads, 0, s->stream>>>(
+        k_pencil_k3w<T><<<(2 * s->p * s->N + threads - 1) / threads, threads, 0, s->stream>>>(
             s->N, s->p, s->w64_d.as<double>(), s->dw64_d.as<double>(), P.k3w.template as<T>());
         MBD_LAUNCH_CHECK();
     }
     return MBD_OK;
 }
 
-template <class T> mbd_status launch_spread(mbd_system *s, const T *d, T *mesh, int R, int ld) {
+template <class T> SpreadArgs<T> spread_args(mbd_system *s, const T *d, T *mesh, int R, int ld) {
     PrecData<T> &P = prec<T>(s);
-    const size_t npts = (size_t)s->K[0] * s->K[1] * s->K[2];
-    const int vec = (sizeof(T) == 4 && ld % 4 == 0 && ld >= 128) ? 4 : ((ld % 2 == 0 && ld >= 64) ? 2 : 1);
-    const unsigned gx = (unsigned)std::min<size_t>((npts + 15) / 16, 152 * 16);
-    dim3 grid(gx, (ld + 32 * vec - 1) / (32 * vec));
-    const int *rowp = P.srow.template as<int>();
-    const SpreadRec<T> *recp = P.srec.template as<SpreadRec<T>>();
-    if (vec == 4) {
-        if constexpr (sizeof(T) == 4) k_spread_csr<T, 4><<<grid, 256, 0, s->stream>>>(d, mesh, R, ld, npts, rowp, recp);
-    } else if (vec == 2) {
-        k_spread_csr<T, 2><<<grid, 256, 0, s->stream>>>(d, mesh, R, ld, npts, rowp, recp);
-    } else {
-        k_spread_csr<T, 1><<<grid, 256, 0, s->stream>>>(d, mesh, R, ld, npts, rowp, recp);
+    return {d, mesh, R, ld, s->K[0], s->K[1], s->K[2], s->p, P.prow.template as<int>(),
+            P.prec.template as<PencilRec<T>>(), P.k3w.template as<T>(),
+            P.tw3.template as<typename Cplx<T>::type>()};
+}
+
+template <class T> mbd_status launch_spread(mbd_system *s, const T *d, T *mesh, int R, int ld) {
+    const SpreadArgs<T> a = spread_args(s, d, mesh, R, ld);
+    const unsigned ncols = (unsigned)((size_t)a.K1 * a.K2 * (ld / 2));
+    const unsigned grid = (ncols + 4 * spread_w<T>() - 1) / (4 * spread_w<T>());
+    switch (s->p) {
+#define MBD_SPREAD_ORDER(P) \
+    case P: k_spread_pencil<T, P><<<grid, 128, 0, s->stream>>>(a, ncols); break;
+        MBD_SPLINE_ORDERS(MBD_SPREAD_ORDER)
+#undef MBD_SPREAD_ORDER
+        default: return MBD_ERR_UNSUPPORTED;
     }
     MBD_LAUNCH_CHECK();
     return MBD_OK;
@@ -969,21 +754,6 @@ template <class T> mbd_status launch_spread(mbd_system *s, const T *d, T *mesh, 
 // Meshes of at most this many bytes (three quarters of the 129 MB L2) launch
 // their FFT passes with programmatic dependence; larger ones plainly.
 constexpr size_t kEarlyFFTMaxBytes = 96u << 20;
-
-// FP32 passes and fused spreading over meshes longer than this use tiles of
-// 16 complex columns instead of 32: half the shared memory per block, twice
-// the resident blocks, which the long (latency-bound) spreading phase needs.
-constexpr int kWideTileMaxK = 96;
-
-// Tile width of the fused spreading + k3 pass for V complex probe-pair
-// columns: whole tiles only (float 32 or 16, double 16), 0 when none fits.
-int sf3_width(const mbd_system *s, int V, int real_bytes) {
-    if (real_bytes == 4) {
-        if (s->tune_sf3_w != 0 && s->tune_ld == 2 * V && V % s->tune_sf3_w == 0) return s->tune_sf3_w;
-        return (V % 32 == 0 && s->K[2] <= kWideTileMaxK) ? 32 : (V % 16 == 0 ? 16 : 0);
-    }
-    return V % 16 == 0 ? 16 : 0;
-}
 
 #define MBD_HAS_CASE(K, ...) case K:
 bool fft_ct_size(int K) {
@@ -1000,59 +770,33 @@ bool fft_ct_size(int K) {
 }
 #undef MBD_HAS_CASE
 
-template <class T> int launch_fft_ct_sized(const FFTArgs<T> &a, bool fused, unsigned grid, cudaStream_t st) {
+template <class T> int launch_fft_ct_sized(const FFTArgs<T> &a, int mode, unsigned outer, cudaStream_t st) {
     int r;
-    if ((r = launch_fft_ct_group0<T>(a, fused, grid, st)) >= 0) return r;
-    if ((r = launch_fft_ct_group1<T>(a, fused, grid, st)) >= 0) return r;
-    if ((r = launch_fft_ct_group2<T>(a, fused, grid, st)) >= 0) return r;
-    if ((r = launch_fft_ct_group3<T>(a, fused, grid, st)) >= 0) return r;
-    if ((r = launch_fft_ct_group4<T>(a, fused, grid, st)) >= 0) return r;
-    return launch_fft_ct_group5<T>(a, fused, grid, st);
+    if ((r = launch_fft_ct_group0<T>(a, mode, outer, st)) >= 0) return r;
+    if ((r = launch_fft_ct_group1<T>(a, mode, outer, st)) >= 0) return r;
+    if ((r = launch_fft_ct_group2<T>(a, mode, outer, st)) >= 0) return r;
+    if ((r = launch_fft_ct_group3<T>(a, mode, outer, st)) >= 0) return r;
+    if ((r = launch_fft_ct_group4<T>(a, mode, outer, st)) >= 0) return r;
+    return launch_fft_ct_group5<T>(a, mode, outer, st);
 }
 
-template <class T>
-int launch_sf3_sized(int K3, int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *row,
-                     const SpreadRec<T> *rec, const typename Cplx<T>::type *tw, cudaStream_t st) {
+template <class T> int launch_spp_sized(const SpreadArgs<T> &a, cudaStream_t st) {
     int r;
-    if ((r = launch_sf3_group0<T>(K3, W, d, mesh, R, ld, K1, K2, row, rec, tw, st)) >= 0) return r;
-    if ((r = launch_sf3_group1<T>(K3, W, d, mesh, R, ld, K1, K2, row, rec, tw, st)) >= 0) return r;
-    if ((r = launch_sf3_group2<T>(K3, W, d, mesh, R, ld, K1, K2, row, rec, tw, st)) >= 0) return r;
-    if ((r = launch_sf3_group3<T>(K3, W, d, mesh, R, ld, K1, K2, row, rec, tw, st)) >= 0) return r;
-    if ((r = launch_sf3_group4<T>(K3, W, d, mesh, R, ld, K1, K2, row, rec, tw, st)) >= 0) return r;
-    return launch_sf3_group5<T>(K3, W, d, mesh, R, ld, K1, K2, row, rec, tw, st);
-}
-
-template <class T>
-int launch_spp_sized(int K3, int W, const T *d, T *mesh, int R, int ld, int K1, int K2, const int *prow,
-                     const PencilRec<T> *prec, const T *k3w, const typename Cplx<T>::type *tw, cudaStream_t st) {
-    int r;
-    if ((r = launch_spp_group0<T>(K3, W, d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st)) >= 0) return r;
-    if ((r = launch_spp_group1<T>(K3, W, d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st)) >= 0) return r;
-    if ((r = launch_spp_group2<T>(K3, W, d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st)) >= 0) return r;
-    if ((r = launch_spp_group3<T>(K3, W, d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st)) >= 0) return r;
-    if ((r = launch_spp_group4<T>(K3, W, d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st)) >= 0) return r;
-    return launch_spp_group5<T>(K3, W, d, mesh, R, ld, K1, K2, prow, prec, k3w, tw, st);
+    if ((r = launch_spp_group0<T>(a, st)) >= 0) return r;
+    if ((r = launch_spp_group1<T>(a, st)) >= 0) return r;
+    if ((r = launch_spp_group2<T>(a, st)) >= 0) return r;
+    if ((r = launch_spp_group3<T>(a, st)) >= 0) return r;
+    if ((r = launch_spp_group4<T>(a, st)) >= 0) return r;
+    return launch_spp_group5<T>(a, st);
 }
 
 // Spreading fused with the first forward FFT pass when the k3 size has a
-// compile-time pass and the probe-pair columns fill whole tiles.
-bool spread_fft3_supported(const mbd_system *s, int ld, int real_bytes) {
-    return fft_ct_size(s->K[2]) && sf3_width(s, ld / 2, real_bytes) > 0;
-}
+// compile-time pass.
+bool spread_fft3_supported(const mbd_system *s) { return fft_ct_size(s->K[2]); }
 
 // Returns MBD_ERR_UNSUPPORTED (nothing launched) when spread_fft3_supported is false.
 template <class T> mbd_status launch_spread_fft3(mbd_system *s, const T *d, T *mesh, int R, int ld) {
-    PrecData<T> &P = prec<T>(s);
-    const int W = sf3_width(s, ld / 2, (int)sizeof(T));
-    if (W == 0) return MBD_ERR_UNSUPPORTED;
-    using C = typename Cplx<T>::type;
-    // spline order 6: spreading by pencil records; other orders by the point records
-    const int r = s->p == kPencilOrder
-                      ? launch_spp_sized<T>(s->K[2], W, d, mesh, R, ld, s->K[0], s->K[1], P.prow.template as<int>(),
-                                            P.prec.template as<PencilRec<T>>(), P.k3w.template as<T>(),
-                                            P.tw3.template as<C>(), s->stream)
-                      : launch_sf3_sized<T>(s->K[2], W, d, mesh, R, ld, s->K[0], s->K[1], P.srow.template as<int>(),
-                                            P.srec.template as<SpreadRec<T>>(), P.tw3.template as<C>(), s->stream);
+    const int r = launch_spp_sized<T>(spread_args(s, d, mesh, R, ld), s->stream);
     if (r < 0) return MBD_ERR_UNSUPPORTED;
     if (r == 0) {
         set_last_error("fused spreading: shared-memory size", cudaGetLastError());
@@ -1067,9 +811,8 @@ template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bo
     PrecData<T> &P = prec<T>(s);
     const int V = ld / 2;
     const int K1 = s->K[0], K2 = s->K[1], K3 = s->K[2];
-    const int Wmax = sizeof(T) == 4 ? 32 : 16;
     const size_t npts_bytes = sizeof(T) * (size_t)K1 * K2 * K3 * ld;
-    auto run = [&](int dim, int outer, int inner, int sign, bool fused) -> mbd_status {
+    auto run = [&](int dim, int outer, int inner, int mode) -> mbd_status {
         FFTArgs<T> a;
         a.data = reinterpret_cast<C *>(mesh);
         a.tw = (dim == 0 ? P.tw1 : (dim == 1 ? P.tw2 : P.tw3)).template as<C>();
@@ -1079,25 +822,14 @@ template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bo
         a.radices = 0ull;
         for (int k = 0; k < a.nst; ++k) a.radices |= (unsigned long long)s->fft[dim].radix[k] << (4 * k);
         a.inner = inner;
-        a.W = inner < Wmax ? inner : Wmax;
         a.V = V;
-        a.sign = sign;
         // early launch of the passes while the mesh fits in three quarters of L2
         a.early = npts_bytes <= kEarlyFFTMaxBytes ? 1 : 0;
         a.sms = s->num_sms;
-        // compile-time pass: float tiles of 32 complex columns (16 for narrow
-        // rows and for long meshes), double tiles of 16; narrower rows are masked
-        FFTArgs<T> c = a;
-        c.W = (sizeof(T) == 4 && (inner < 32 || a.K > kWideTileMaxK)) ? 16 : Wmax;
-        if (sizeof(T) == 4 && s->tune_fft_w != 0 && s->tune_ld == ld) c.W = inner < 32 ? 16 : s->tune_fft_w;
-        // the pass fused with G does twice the arithmetic per element of the
-        // mesh: on meshes of 97 to 128 points it keeps 32-column tiles (128^3,
-        // 128 probes: 474 -> 462 us per pass on average over the four passes);
-        // longer ones do not (192^3: 818 -> 934 us, the tile's shared memory
-        // leaves too few blocks per SM)
-        if (sizeof(T) == 4 && fused && a.K > kWideTileMaxK && a.K <= 128 && inner >= 32) c.W = 32;
-        const int r = launch_fft_ct_sized<T>(c, fused, (unsigned)((size_t)outer * ((inner + c.W - 1) / c.W)),
-                                             s->stream);
+        // wide tiles unless they are too few for four blocks per SM
+        a.W = (size_t)outer * inner >= (size_t)128 * a.sms ? 32 : 16;
+        if (s->tune_fft_w != 0 && tuned_for<T>(s, ld)) a.W = s->tune_fft_w;
+        const int r = launch_fft_ct_sized<T>(a, mode, (unsigned)outer, s->stream);
         if (r == 0) {
             set_last_error("FFT pass: shared-memory size", cudaGetLastError());
             return MBD_ERR_CUDA;
@@ -1106,27 +838,18 @@ template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bo
             MBD_LAUNCH_CHECK();
             return MBD_OK;
         }
-        const size_t smem = sizeof(C) * (2 * (size_t)a.K * a.W + a.K);
-        dim3 grid((unsigned)((size_t)outer * ((inner + a.W - 1) / a.W)));
-        if (fused) {
-            if (smem > 48 * 1024)
-                MBD_CUDA_TRY(cudaFuncSetAttribute(k_fft_pass<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem));
-            k_fft_pass<T, true><<<grid, 256, smem, s->stream>>>(a);
-        } else {
-            if (smem > 48 * 1024)
-                MBD_CUDA_TRY(cudaFuncSetAttribute(k_fft_pass<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)smem));
-            k_fft_pass<T, false><<<grid, 256, smem, s->stream>>>(a);
+        if (sizeof(T) == 4) {
+            a.inner /= 2;
+            a.V /= 2;
         }
-        MBD_LAUNCH_CHECK();
-        return MBD_OK;
+        a.W = std::min(a.inner, 16);
+        return launch_fft_generic<T, typename PackOf<T>::type>(a, mode, (unsigned)outer, s->stream);
     };
-    if (!skip_first) MBD_TRY(run(2, K1 * K2, V, -1, false));   // forward along k3
-    MBD_TRY(run(1, K1, K3 * V, -1, false));            // forward along k2
-    MBD_TRY(run(0, 1, K2 * K3 * V, -1, true));         // forward k1, x G, inverse k1
-    MBD_TRY(run(1, K1, K3 * V, +1, false));            // inverse along k2
-    MBD_TRY(run(2, K1 * K2, V, +1, false));            // inverse along k3
+    if (!skip_first) MBD_TRY(run(2, K1 * K2, V, 0));   // forward along k3
+    MBD_TRY(run(1, K1, K3 * V, 0));            // forward along k2
+    MBD_TRY(run(0, 1, K2 * K3 * V, 2));         // forward k1, x G, inverse k1
+    MBD_TRY(run(1, K1, K3 * V, 1));            // inverse along k2
+    MBD_TRY(run(2, K1 * K2, V, 1));            // inverse along k3
     return MBD_OK;
 }
 
@@ -1288,7 +1011,7 @@ int field_apb(const mbd_system *s, int ld) {
     // leaves no half-empty iteration
     const bool pairs = bytes == 4 && s->p == 6 && real_on_clusters(s, ld, bytes) && (vec == 4 || field_half(ld, bytes));
     int apb;
-    if (s->tune_field_apb > 0 && s->tune_ld == ld) {
+    if (s->tune_field_apb > 0 && (bytes == 4 ? tuned_for<float>(s, ld) : tuned_for<double>(s, ld))) {
         apb = s->tune_field_apb;
     } else {
         const int ych = (ld + 32 * vec - 1) / (32 * vec);
@@ -1303,8 +1026,8 @@ int field_blocks(const mbd_system *s, int ld) {
     return (s->N + apb - 1) / apb;
 }
 
-template mbd_status build_spread_matrix<double>(mbd_system *);
-template mbd_status build_spread_matrix<float>(mbd_system *);
+template mbd_status build_spread_records<double>(mbd_system *);
+template mbd_status build_spread_records<float>(mbd_system *);
 template mbd_status launch_spread<double>(mbd_system *, const double *, double *, int, int);
 template mbd_status launch_spread<float>(mbd_system *, const float *, float *, int, int);
 template mbd_status launch_convolve<double>(mbd_system *, double *, int, bool);

@@ -48,10 +48,10 @@ void set_last_error(const char *where, cudaError_t e);
 
 // Programmatic dependent launch in a Lanczos step: a kernel launched with it
 // may be scheduled while its predecessor in the stream runs its last blocks.
-// The kernels of the step let their successor launch at once
-// (pdl_launch_dependents, their first instruction) and wait for their
-// predecessor's completion and memory (pdl_wait) before they touch global
-// data.  The successor launches only when every block of the predecessor has
+// The kernels of the step wait for their predecessor's completion and memory
+// (pdl_wait) before they touch data that it writes, and then let their
+// successor launch (pdl_launch_dependents), so that one kernel waits at a time.
+// The successor launches only when every block of the predecessor has
 // started, so its early blocks take resources only from the predecessor's
 // tail.  Both instructions are no-ops in a kernel launched without the
 // attribute.  Measured per kernel: early launch helps the fused spreading
@@ -127,7 +127,6 @@ struct NeighborGrid {
 struct BinView {
     int nb1, nb2, nb3;      // bricks (= bins) per dimension
     int bs1, bs2, bs3;      // brick edge (mesh points)
-    int nc1, nc2, nc3;      // candidate bins per dimension for one brick
     const int *start;       // [nbins+1]
     const int *atoms;       // [N] atoms sorted by bin
 };
@@ -213,13 +212,6 @@ __device__ __forceinline__ bool grid_reduce(const double *bval, int nloc, int rb
 // ---------------------------------------------------------------- per-system state
 struct SystemData;
 
-// One nonzero of the transposed stencil matrix: the Cartesian weights
-// dW_j(k)/dR_j of atom j at mesh point k (row = k).  For float the atom index
-// travels in the .w component (bit pattern), for double in a separate word.
-template <class T> struct SpreadRec;
-template <> struct __align__(16) SpreadRec<float> { float w0, w1, w2; int atom; };
-template <> struct __align__(16) SpreadRec<double> { double w0, w1, w2; int atom; int pad; };
-
 // One (pencil, atom) record of the factorised spreading: for the pencil
 // (k1, k2) and an atom j whose stencil covers it (t1 = top1 - k1, t2 = top2 - k2
 // mod K), the weights along the pencil are
@@ -227,6 +219,11 @@ template <> struct __align__(16) SpreadRec<double> { double w0, w1, w2; int atom
 //   e0_alpha = C_{0 alpha} M1'(t1) M2(t2) + C_{1 alpha} M1(t1) M2'(t2),
 //   e1_alpha = C_{2 alpha} M1(t1) M2(t2),   C_{beta alpha} = K_beta a*_{beta alpha}.
 // Records are grouped by the mesh point (k1, k2, top3_j) (CSR over points).
+template <class T> struct __align__(16) PencilRec {
+    T e0[3], e1[3];
+    int atom, top3;
+};
+
 // Clusters of the real-space field: kClusterSize consecutive atoms of the
 // Morton order; a cluster with more than kClusterSortCap pairs in all (more
 // than 256 neighbours per atom on average) sends the system back to the
@@ -241,20 +238,12 @@ template <class T> struct __align__(16) RealPair {
     T a[6];
 };
 
-constexpr int kPencilOrder = 6;   // the spline order the pencil spreading is compiled for
-template <class T> struct __align__(16) PencilRec {
-    T e0[3], e1[3];
-    int atom, top3;
-};
-
 template <class T> struct PrecData {
     DevBuf pairA;       // [nnz][6]
     DevBuf pairdA;      // [nnz][18] dA_ab/dr_c (forces)
-    DevBuf srow;        // [K^3 + 1] CSR row pointers of the spread matrix
-    DevBuf srec;        // [216 N] SpreadRec<T>
-    DevBuf prow;        // [K^3 + 1] CSR over points (k1, k2, top3) of the pencil records (spline order 6)
-    DevBuf prec;        // [36 N] PencilRec<T>
-    DevBuf k3w;         // [N][16] M3(t3) (t3 < p) at 0.., M3'(t3) at 8..
+    DevBuf prow;        // [K^3 + 1] CSR over points (k1, k2, top3) of the pencil records
+    DevBuf prec;        // [p^2 N] PencilRec<T>
+    DevBuf k3w;         // [N][2p] M3(t3), M3'(t3)
     DevBuf w, dw, d2w;  // [N][3][p]
     DevBuf G;           // [K1K2K3] influence function
     DevBuf tw1, tw2, tw3;   // twiddles [K] complex per dimension
@@ -296,7 +285,7 @@ struct mbd_system {
     int num_sms = 1;    // multiprocessors of the device the system lives on
     // launch choices made by mbd_autotune or mbd_set_launch_choices for probe
     // width tune_ld (0: the built-in rules): field-kernel atoms per block, FP32
-    // FFT and fused-spreading tiles
+    // FFT tile, and the fused-spreading tile (recorded only: there is one width)
     int tune_ld = 0, tune_field_apb = 0, tune_fft_w = 0, tune_sf3_w = 0;
     int basis_recompute = 0;    // MBD_BASIS_RECOMPUTE: three basis vectors kept, the forces rerun the recurrence
     cudaStream_t stream;
@@ -367,11 +356,11 @@ template <class T> mbd_status launch_influence(mbd_system *s, const double *bmod
 
 // mesh stages
 template <class T> mbd_status launch_spread(mbd_system *s, const T *d, T *mesh, int R, int ld);
-template <class T> mbd_status build_spread_matrix(mbd_system *s);
+template <class T> mbd_status build_spread_records(mbd_system *s);
 // in place; skip_first: the forward k3 pass was already done (launch_spread_fft3)
 template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bool skip_first = false);
 template <class T> mbd_status launch_spread_fft3(mbd_system *s, const T *d, T *mesh, int R, int ld);
-bool spread_fft3_supported(const mbd_system *s, int ld, int real_bytes);
+bool spread_fft3_supported(const mbd_system *s);
 bool fft_ct_size(int K);        // a compile-time FFT pass exists for this length
 enum FieldMode { kFieldOut = 0, kFieldApply = 1, kFieldLanczos = 2 };
 template <class T> struct FieldOut {
@@ -425,7 +414,15 @@ mbd_status launch_force_gather_t(mbd_system *s, const T *dpq, const T *mesh, int
                                  double *forces);
 
 // misc
-int probe_ld(int R);
+// Padded probe count of arrays of T: even, a multiple of four for float (16-byte
+// rows, probe pairs packed two by two in the FFT passes).
+template <class T> constexpr int probe_ld(int R) {
+    return sizeof(T) == 4 ? (R + 3) / 4 * 4 : R + (R & 1);
+}
+// whether the launch choices set for probe width tune_ld hold at ld
+template <class T> bool tuned_for(const mbd_system *s, int ld) {
+    return s->tune_ld != 0 && probe_ld<T>(s->tune_ld) == ld;
+}
 void prof_begin(mbd_system *s, int stage, cudaEvent_t *e0);
 void prof_end(mbd_system *s, int stage, int n_launches, cudaEvent_t e0);
 void prof_release(mbd_system *s);
