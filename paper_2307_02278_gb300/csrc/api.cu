@@ -405,8 +405,7 @@ template <class T> mbd_status setup_geometry(mbd_system *s) {
     s->n_clusters = (s->N + kClusterSize - 1) / kClusterSize;
     MBD_TRY(s->cl_err.ensure(sizeof(int)));
     MBD_CUDA_TRY(cudaMemsetAsync(s->cl_err.ptr, 0, sizeof(int), s->stream));
-    MBD_TRY(launch_cluster_pairs<T>(s, s->order_d.as<int>(), s->n_clusters, s->cl_ecnt, s->cl_pcnt, s->cl_estart,
-                                    s->cl_pstart, s->cl_entries, prec<T>(s).cA, s->cl_err.as<int>(), s->stream));
+    MBD_TRY(launch_cluster_pairs<T>(s, s->stream));
     int cerr = 0;
     MBD_CUDA_TRY(cudaMemcpyAsync(&cerr, s->cl_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
     MBD_CUDA_TRY(cudaStreamSynchronize(s->stream));

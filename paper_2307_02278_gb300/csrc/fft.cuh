@@ -710,10 +710,13 @@ template <class T, class P> int ct_size(const FFTArgs<T> &a, int mode, unsigned 
 
 // a c + b over the probes of a lane (packed for two floats), scalar c.
 template <class T, int PPL> __device__ __forceinline__ void lane_fma(const T *a, T c, T *b) {
-    if constexpr (PPL == 2 && sizeof(T) == 4) {
-        const float2 r = __ffma2_rn(make_float2(a[0], a[1]), make_float2(c, c), make_float2(b[0], b[1]));
-        b[0] = r.x;
-        b[1] = r.y;
+    if constexpr (PPL % 2 == 0 && sizeof(T) == 4) {
+#pragma unroll
+        for (int e = 0; e < PPL; e += 2) {
+            const float2 r = __ffma2_rn(make_float2(a[e], a[e + 1]), make_float2(c, c), make_float2(b[e], b[e + 1]));
+            b[e] = r.x;
+            b[e + 1] = r.y;
+        }
     } else {
 #pragma unroll
         for (int e = 0; e < PPL; ++e) b[e] += a[e] * c;

@@ -11,8 +11,6 @@ namespace mbd {
 
 namespace {
 
-constexpr int kWarps = 8;          // warps per block in the field kernel
-
 // ---------------------------------------------------------------- spreading
 // The dipole array D(k) = sum_j d_j . grad W_j(k) (Eq. dipolarr) from the
 // pencil records, built once per geometry in a fixed atom order, so every mesh
@@ -272,112 +270,147 @@ template <class T, class F> mbd_status launch_fft_generic(FFTArgs<T> a, int mode
 template <class T> struct RealArgs {
     const T *d;          // [N][3][ld]
     T *out;              // [N][3][ld] E_real
-    int ld, N, nclus;
+    int ld, N;
     const int *order;    // cluster c = atoms order[16c .. 16c + 15]
-    const int *estart;   // [nclus + 1] entry starts
-    const int *pstart;   // [16 nclus + 1] pair starts per (cluster, atom)
-    const int *entries;  // distinct neighbours j of each cluster
-    const RealPair<T> *pairs;
+    const int *pstart, *ecnt, *rcnt, *entries;
+    const RealDuo<T> *recs;
+    int np;              // probes of a chunk (blockIdx.y)
+    int ce;              // entries staged at a time
 };
 
 // The real-space field E_real = sum over pairs A(r) d_j (Eq. fld_ewald with
 // the damping correction) on clusters: a block per cluster of 16 atoms and
-// probe chunk (blockIdx.y, 32 PPL probes), warp w for cluster atom w, lanes
-// over PPL consecutive probes.  The block stages the dipoles of the cluster's
-// distinct neighbours in shared memory, kRealCE entries at a time (coalesced
-// 16-byte loads by all threads), so each neighbour's dipoles come from L2
-// once per cluster.  Each warp reads its atom's pairs (entry index and
-// tensor) 32 at a time into shared memory, one per lane, counts by a ballot
-// those whose entries are staged (entries increase along a batch) and applies
-// them with no test per pair, accumulating in registers: no global load waits
-// inside the pair loop.  An atom's field is the sum over its pairs in
-// (j, image) order: deterministic.
-constexpr int kRealCE = 48;
-template <class T, int PPL>
-__global__ void __launch_bounds__(32 * kClusterSize) k_real_clusters(RealArgs<T> a) {
-    constexpr int NP = 32 * PPL;                   // probes of the block
-    constexpr int U = 16 / (int)sizeof(T);         // values per 16-byte load
-    constexpr int PER_ROW = NP / U;                // 16-byte loads per staged row
-    // dynamic shared memory: the staged dipoles [kRealCE][3][NP], then the
-    // warps' batches of pairs [kClusterSize][32]
+// chunk of np probes, warp w for the cluster's atoms 2w and 2w + 1.  The block
+// stages the dipoles of the cluster's distinct neighbours in shared memory, ce
+// entries at a time (cp.async, 16 bytes per lane), so each neighbour's dipoles
+// come from L2 once per cluster.  A warp walks the records of its two atoms in
+// entry order, in double-buffered batches of 16 (cp.async), and counts by a
+// ballot those whose entries are staged; np / VEC lanes hold the probes, and
+// the S groups of a warp take the records in turn.  A record applies one
+// neighbour's dipoles, read from shared memory once, to both atoms: close atoms
+// share three quarters of their neighbours, and the reads of shared memory and
+// the instructions beside the packed FMAs are what bound the kernel (100,002
+// atoms x 64 probes: 677 -> 559 us per launch; with 64 registers and four
+// blocks per SM it spills, 605 us; batches of 32 records 636 us).
+// An atom's field is a sum in a fixed order (per group, then the groups).
+constexpr int kRealBatch = 16;
+constexpr int kRealStageBytes = 36 * 1024;
+template <class T>
+__global__ void __launch_bounds__(16 * kClusterSize, sizeof(T) == 4 ? 3 : 2) k_real_clusters(RealArgs<T> a) {
+    constexpr int VEC = 16 / (int)sizeof(T), NW = kClusterSize / 2;
+    constexpr int RC = (int)sizeof(RealDuo<T>) / 16;       // 16-byte pieces of a record
     extern __shared__ __align__(16) unsigned char real_smem[];
-    T(*sd)[3][NP] = reinterpret_cast<T(*)[3][NP]>(real_smem);
-    RealPair<T>(*sp)[32] = reinterpret_cast<RealPair<T>(*)[32]>(real_smem + sizeof(T) * kRealCE * 3 * NP);
+    RealDuo<T> *sp = reinterpret_cast<RealDuo<T> *>(real_smem);              // [NW][2][kRealBatch]
+    int *ent = reinterpret_cast<int *>(sp + NW * 2 * kRealBatch);            // [2][ce]
+    T *sd = reinterpret_cast<T *>(real_smem + sizeof(RealDuo<T>) * NW * 2 * kRealBatch + 16 * ((8 * a.ce + 15) / 16));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c = blockIdx.x;
-    const int pb = blockIdx.y * NP;
-    const int r0 = pb + lane * PPL;
-    const bool inld = r0 < a.ld;
-    const bool vec = a.ld % U == 0;
-    const int eb = a.estart[c], ee = a.estart[c + 1];
-    const int slot = c * kClusterSize + warp;
-    const int pe = a.pstart[slot + 1];
-    int bbase = a.pstart[slot], bn = 0, bi = 0;    // the warp's batch of pairs [bbase, bbase + bn), next bi
-    int ev = 0x7fffffff;                           // entry of the batch's pair held by this lane
-    T E[3][PPL];
+    const int c = blockIdx.x, pb = blockIdx.y * a.np, np = min(a.np, a.ld - pb);
+    const int lanes = a.np / VEC, S = 32 / lanes, sub = lane / lanes, lid = lane - sub * lanes;
+    const bool on = sub < S && lid * VEC < np;
+    const int p0 = a.pstart[c * kClusterSize], ne = a.ecnt[c];
+    const int *entries = a.entries + p0;
+    const RealDuo<T> *recs = a.recs + a.pstart[c * kClusterSize + 2 * warp];
+    const int nrec = a.rcnt[c * NW + warp];
+    RealDuo<T> *mine = sp + warp * 2 * kRealBatch;
+    auto fetch_batch = [&](int first, int b) {
+        const int nq = min(kRealBatch, nrec - first) * RC;
+        const float4 *src = reinterpret_cast<const float4 *>(recs + first);
+        float4 *dst = reinterpret_cast<float4 *>(mine + b * kRealBatch);
+        for (int q = lane; q < nq; q += 32) cp_async<16>(dst + q, src + q);
+        cp_async_commit();
+    };
+    if (nrec > 0) fetch_batch(0, 0);
+    for (int q = threadIdx.x; q < min(a.ce, ne); q += blockDim.x) ent[q] = entries[q];
+    int first = -kRealBatch, bn = kRealBatch, bi = kRealBatch, buf = 1;   // current batch: none yet
+    int ev = 0x7fffffff;                           // entry of the batch's record held by this lane
+    T E[2][3][VEC];
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int e = 0; e < PPL; ++e) E[k][e] = T(0);
-    for (int c0 = eb; c0 < ee; c0 += kRealCE) {
-        const int ne = min(kRealCE, ee - c0);
-        __syncthreads();                           // the previous chunk is consumed
-        for (int t = threadIdx.x; t < ne * 3 * PER_ROW; t += blockDim.x) {
-            const int q = t / (3 * PER_ROW), rem = t - q * (3 * PER_ROW), k = rem / PER_ROW, u = rem - k * PER_ROW;
-            const T *src = a.d + (size_t)(3 * a.entries[c0 + q] + k) * a.ld + pb + u * U;
-            T *dst = &sd[q][k][u * U];
-            if (vec && pb + u * U + U <= a.ld) {
-                *reinterpret_cast<float4 *>(dst) = *reinterpret_cast<const float4 *>(src);
-            } else {
+        for (int k = 0; k < 3; ++k)
 #pragma unroll
-                for (int v = 0; v < U; ++v) dst[v] = pb + u * U + v < a.ld ? src[v] : T(0);
-            }
+            for (int v = 0; v < VEC; ++v) E[h][k][v] = T(0);
+    for (int c0 = 0, eb = 0; c0 < ne; c0 += a.ce, eb ^= 1) {
+        const int m = min(a.ce, ne - c0);
+        __syncthreads();                           // the previous chunk is consumed; its successor's entries are there
+        for (int r = warp * S + sub; r < 3 * m && on; r += NW * S) {
+            const int q = r / 3, k = r - 3 * q;
+            cp_async<16>(sd + (size_t)r * a.np + lid * VEC,
+                         a.d + (size_t)(3 * ent[eb * a.ce + q] + k) * a.ld + pb + lid * VEC);
         }
+        for (int q = threadIdx.x; q < min(a.ce, ne - c0 - m); q += blockDim.x)
+            ent[(eb ^ 1) * a.ce + q] = entries[c0 + m + q];
+        cp_async_commit();
+        cp_async_wait<0>();                        // the chunk (and the records on their way)
         __syncthreads();
-        const int lo = c0 - eb, lim = lo + ne;     // entries staged: [lo, lim)
+        const int lim = c0 + m;                    // entries staged: [c0, lim)
         for (;;) {
-            if (bi == bn) {                        // the next 32 pairs of this atom
-                bbase += bn;
-                if (bbase >= pe) break;
-                bn = min(32, pe - bbase);
+            if (bi == bn) {                        // the next batch of records
+                first += bn;
+                if (first >= nrec) {
+                    first = nrec;
+                    bn = bi = 0;
+                    break;
+                }
+                buf ^= 1;
+                bn = min(kRealBatch, nrec - first);
                 bi = 0;
+                cp_async_wait<0>();
                 __syncwarp();
-                if (lane < bn) {
-                    const RealPair<T> r = a.pairs[bbase + lane];
-                    sp[warp][lane] = r;
-                    ev = r.e;
-                } else {
-                    ev = 0x7fffffff;
-                }
-                __syncwarp();
+                ev = lane < bn ? mine[buf * kRealBatch + lane].e : 0x7fffffff;
+                if (first + bn < nrec) fetch_batch(first + bn, buf ^ 1);
             }
-            // the pairs bi .. bi + cnt - 1 of the batch have their entries staged
-            // (entries increase along the batch)
+            // the records bi .. bi + cnt - 1 of the batch have their entries
+            // staged (entries increase along the batch)
             const int cnt = __popc(__ballot_sync(0xffffffffu, lane >= bi && ev < lim));
-            for (int t = 0; t < cnt; ++t) {
-                const RealPair<T> &cur = sp[warp][bi + t];
-                const int q = cur.e - lo;
-                T x[PPL], y[PPL], z[PPL];
-                vload<T, PPL>(&sd[q][0][lane * PPL], x);
-                vload<T, PPL>(&sd[q][1][lane * PPL], y);
-                vload<T, PPL>(&sd[q][2][lane * PPL], z);
-                const T A0 = cur.a[0], A1 = cur.a[1], A2 = cur.a[2], A3 = cur.a[3], A4 = cur.a[4], A5 = cur.a[5];
+            if (on) {
+                for (int t = sub; t < cnt; t += S) {
+                    const RealDuo<T> &cur = mine[buf * kRealBatch + bi + t];
+                    const T *x0 = sd + (size_t)(cur.e - c0) * 3 * a.np + lid * VEC;
+                    T x[VEC], y[VEC], z[VEC], A[12];
+                    vload<T, VEC>(x0, x);
+                    vload<T, VEC>(x0 + a.np, y);
+                    vload<T, VEC>(x0 + 2 * a.np, z);
 #pragma unroll
-                for (int e = 0; e < PPL; ++e) {
-                    E[0][e] += A0 * x[e] + A1 * y[e] + A2 * z[e];
-                    E[1][e] += A1 * x[e] + A3 * y[e] + A4 * z[e];
-                    E[2][e] += A2 * x[e] + A4 * y[e] + A5 * z[e];
+                    for (int q = 0; q < 12; q += VEC) vload<T, VEC>(cur.a + q, A + q);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        // FP64 is bound by its FMAs: tensors that are zero are skipped
+                        if (sizeof(T) == 8 && !(cur.mask & (1 << h))) continue;
+                        const T *B = A + 6 * h;
+                        lane_fma<T, VEC>(x, B[0], E[h][0]);
+                        lane_fma<T, VEC>(y, B[1], E[h][0]);
+                        lane_fma<T, VEC>(z, B[2], E[h][0]);
+                        lane_fma<T, VEC>(x, B[1], E[h][1]);
+                        lane_fma<T, VEC>(y, B[3], E[h][1]);
+                        lane_fma<T, VEC>(z, B[4], E[h][1]);
+                        lane_fma<T, VEC>(x, B[2], E[h][2]);
+                        lane_fma<T, VEC>(y, B[4], E[h][2]);
+                        lane_fma<T, VEC>(z, B[5], E[h][2]);
+                    }
                 }
             }
+            __syncwarp();                          // the batch is read before a later one takes its buffer
             bi += cnt;
-            if (bi < bn) break;                    // the next pair waits for a later chunk
+            if (bi < bn) break;                    // the next record waits for a later chunk
         }
     }
-    const int idx = c * kClusterSize + warp;
-    if (!inld || idx >= a.N) return;
-    const int i = a.order[idx];
+    cp_async_wait<0>();                            // no copy in flight at exit
 #pragma unroll
-    for (int k = 0; k < 3; ++k) vstore<T, PPL>(a.out + (size_t)(3 * i + k) * a.ld + r0, E[k]);
+    for (int h = 0; h < 2; ++h) {
+        const int idx = c * kClusterSize + 2 * warp + h;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            T o[VEC];
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) {
+                o[v] = E[h][k][v];
+                for (int g = 1; g < S; ++g) o[v] += __shfl_sync(0xffffffffu, E[h][k][v], lid + g * lanes);
+            }
+            if (sub == 0 && on && idx < a.N)
+                vstore<T, VEC>(a.out + (size_t)(3 * a.order[idx] + k) * a.ld + pb + lid * VEC, o);
+        }
+    }
 }
 
 // ---------------------------------------------------------------- field
@@ -386,281 +419,409 @@ template <class T> struct FieldArgs {
     const T *mesh;       // [K^3][ld]
     int R, ld;
     Geom g;
-    SplineView<T> sp;
     PairView<T> pr;
-    const int *order;    // atom processing order (spatially sorted)
+    const unsigned char *rec;   // FieldRec of every atom in processing order
     const double *g_at;  // [N] w sqrt(alpha)
     const double *w2;    // [N] w^2
     double self_coef;
-    const T *ereal;      // when set: the real-space field from k_real_clusters [N][3][ld]
+    const T *ereal;      // real-space field from k_real_clusters [N][3][ld] (kernels without the pair loop)
     FieldOut<T> o;
+    int lanes;           // lanes of a warp that share an atom (VEC probes each)
+    int teams;           // atoms that a block works on at once
+    int apb;             // atoms per block
 };
 
-// Field kernel: one block works on `apb` atoms in turn; for each atom its NW
-// warps split the work (warp w takes stencil planes t1 = w, w + NW, ... and,
-// with the pair loop, neighbours nb0 + w, nb0 + w + NW, ...; warp 0 adds the
-// self term, warp NW - 1 the real-space field of the clusters), lanes own VEC
-// consecutive probes.  NW = 8, or NW = p = 6 when the real space comes from
-// the clusters (one warp per stencil plane, none idle).  The 8 partial fields are summed in a fixed order in
-// shared memory and the epilogue selected by o.mode runs with one thread per
-// probe: E* = E^rec + E^dir + E^self (Eqs. ewalddip, spme, fld_ewald,
-// fld_ewald1), l_k = Omega y_k + Diag(g) E*_k and a_k = y_k^T l_k (Eqs. lk3,
-// recurs2).  PC = spline order (0: runtime).
-template <class T, int VEC, int PC, int NW, int LPA = 32>
-__global__ void __launch_bounds__(NW * 32, NW == kWarps ? ((VEC <= 2 && sizeof(T) == 4 && PC > 0) ? 3 : 2)
-                                                        : (LPA == 16 ? 4 : ((VEC <= 2 && sizeof(T) == 4) ? 4 : 2)))
-    k_field(FieldArgs<T> a, int apb) {
-    // atoms per iteration: with six warps (no pair loop) and four probes per
-    // lane, two atoms are gathered together, their loads interleaved, sharing
-    // one barrier (128 probes: 585 -> 527 us per launch at 128^3); with
-    // fewer probes per lane the registers this takes cost a resident block
-    // (64 probes at 192^3: 1236 -> 1369 us).  LPA = 16 (six warps, 64-probe
-    // chunks, four probes per lane): each half-warp gathers its own atom, so a
-    // warp takes two atoms with one atom's registers per lane.
-    constexpr bool HALF = LPA == 16;
-    static_assert(!HALF || (NW != kWarps && VEC == 4), "half-warp atoms: six warps, four probes per lane");
-    constexpr int AIT = HALF ? 2 : ((NW != kWarps && VEC == 4) ? 2 : 1);   // atoms per iteration
-    constexpr int APT = HALF ? 1 : AIT;                                    // atoms per lane
-    constexpr int NLOC = LPA * VEC;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int sub = HALF ? (lane >> 4) : 0;          // the lane's atom of the iteration (half-warp mode)
-    const int lid = HALF ? (lane & 15) : lane;
-    const int rbase = blockIdx.y * NLOC;
-    const int r0 = rbase + lid * VEC;
-    const bool inld = r0 < a.ld;
-    const int p = PC > 0 ? PC : a.g.p;
-    // partial fields of the warps, double-buffered by atom iteration: the
-    // barrier after one iteration's writes also orders the previous epilogue's
-    // reads before the buffer is written again, so one barrier per iteration
-    __shared__ T red[2][AIT][NW][3][NLOC];
-    __shared__ double bsum[NLOC];
-    __shared__ double pcarry[3 * NLOC > NW * 32 ? 3 * NLOC - NW * 32 : 1];
-    __shared__ double pall[3 * NLOC];
-    pdl_launch_dependents();
-    for (int k = threadIdx.x; k < (3 * NLOC > NW * 32 ? 3 * NLOC - NW * 32 : 1); k += blockDim.x)
-        pcarry[k] = 0.0;
-    pdl_wait();
-    double part = 0.0;                          // y.l of the (component, probe) this thread owns
-    for (int ai = 0; ai < apb; ai += AIT) {
-        const int rb = (ai / AIT) & 1;
-        int iat[AIT];
-        bool val[AIT];
+// What the field kernel reads of an atom, in processing order (Morton order of
+// the bricks): {atom, top1, top2, top3}, then M1, M1', M2, M2', M3, M3' (P values each).
+template <class T, int P> constexpr int field_rec_bytes() { return 16 + 6 * P * (int)sizeof(T); }
+template <class T>
+__global__ void k_field_rec(int N, int p, const int *__restrict__ order, const int *__restrict__ top,
+                            const double *__restrict__ w64, const double *__restrict__ dw64,
+                            unsigned char *__restrict__ rec) {
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x, per = 6 * p + 4;
+    if (idx >= N * per) return;
+    const int pos = idx / per, k = idx - pos * per, i = order[pos];
+    unsigned char *r = rec + (size_t)pos * (16 + 6 * p * sizeof(T));
+    if (k < 4) {
+        reinterpret_cast<int *>(r)[k] = k == 0 ? i : top[3 * i + k - 1];
+    } else {
+        const int dim = (k - 4) / (2 * p), t = (k - 4) % (2 * p);
+        reinterpret_cast<T *>(r + 16)[k - 4] =
+            T(t < p ? w64[(size_t)(3 * i + dim) * p + t] : dw64[(size_t)(3 * i + dim) * p + t - p]);
+    }
+}
+
+// Warps of a field block: as many as divide the p^2 pencils of a stencil evenly.
+template <int P> constexpr int field_warps() { return P == 6 ? 6 : (P == 10 ? 10 : 8); }
+template <class T> constexpr int field_vec() { return 16 / (int)sizeof(T); }
+
+// The epilogue of one iteration of the field kernels, one thread per (atom,
+// component, probe) slot: the warps' partial fields red[NW][OUT] summed in
+// order, then the output selected by o.mode; part: y.l of the thread's slots.
+template <class T, int NW, int OUT, int OPT>
+__device__ __forceinline__ void field_epilogue(const FieldArgs<T> &a, const T *red, int rec_bytes, int nloc, int nout,
+                                               int rbase, int ib, int i1, double *part) {
 #pragma unroll
-        for (int aa = 0; aa < AIT; ++aa) {
-            const int idx = blockIdx.x * apb + ai + aa;
-            val[aa] = ai + aa < apb && idx < a.g.N;
-            iat[aa] = val[aa] ? a.order[idx] : 0;
-        }
-        if (!val[0]) break;
-        // the lane's own atom in half-warp mode (a select, not an indexed array)
-        const int my_i = (HALF && sub) ? iat[AIT - 1] : iat[0];
-        const bool my_v = (HALF && sub) ? val[AIT - 1] : val[0];
-        T E0[APT][VEC], E1[APT][VEC], E2[APT][VEC];
+    for (int k = 0; k < OPT; ++k) {
+        const int slot = threadIdx.x + k * NW * 32;
+        if (slot >= nout) break;
+        const int tc = slot / nloc, t = slot - tc * nloc, tm = tc / 3, c = tc - 3 * tm;
+        const int r = rbase + t;
+        if (r >= a.ld || ib + tm >= i1) continue;
+        const int i = *reinterpret_cast<const int *>(a.rec + (size_t)(ib + tm) * rec_bytes);
+        T sum = T(0);
 #pragma unroll
-        for (int aa = 0; aa < APT; ++aa)
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) E0[aa][v] = E1[aa][v] = E2[aa][v] = T(0);
-        if (inld) {
-            if (a.o.terms & MBD_TERM_RECIP) {
-                T f0[APT][VEC], f1[APT][VEC], f2[APT][VEC];
-                int top1[APT], top2[APT], top3[APT];
-                const T *w[APT], *dw[APT];
-#pragma unroll
-                for (int aa = 0; aa < APT; ++aa) {
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) f0[aa][v] = f1[aa][v] = f2[aa][v] = T(0);
-                    const int i = HALF ? my_i : iat[aa];
-                    top1[aa] = a.sp.top[3 * i];
-                    top2[aa] = a.sp.top[3 * i + 1];
-                    top3[aa] = a.sp.top[3 * i + 2];
-                    w[aa] = a.sp.w + (size_t)3 * p * i;
-                    dw[aa] = a.sp.dw + (size_t)3 * p * i;
-                }
-                for (int t1 = warp; t1 < p; t1 += NW) {
-                    int k1[APT];
-                    T wa[APT], da[APT];
-#pragma unroll
-                    for (int aa = 0; aa < APT; ++aa) {
-                        k1[aa] = top1[aa] - t1;
-                        if (k1[aa] < 0) k1[aa] += a.g.K1;
-                        wa[aa] = w[aa][t1];
-                        da[aa] = dw[aa][t1];
-                    }
-#pragma unroll
-                    for (int t2 = 0; t2 < (PC > 0 ? PC : kMaxOrder); ++t2) {
-                        if (t2 >= p) break;
-                        const T *rowp[APT];
-                        T ab[APT], Ab[APT], aB[APT];
-#pragma unroll
-                        for (int aa = 0; aa < APT; ++aa) {
-                            int k2 = top2[aa] - t2;
-                            if (k2 < 0) k2 += a.g.K2;
-                            const T wb = w[aa][p + t2], db = dw[aa][p + t2];
-                            ab[aa] = wa[aa] * wb;
-                            Ab[aa] = da[aa] * wb;
-                            aB[aa] = wa[aa] * db;
-                            rowp[aa] = a.mesh + ((size_t)k1[aa] * a.g.K2 + k2) * a.g.K3 * a.ld + r0;
-                        }
-#pragma unroll
-                        for (int t3 = 0; t3 < (PC > 0 ? PC : kMaxOrder); ++t3) {
-                            if (t3 >= p) break;
-                            T phi[APT][VEC];
-#pragma unroll
-                            for (int aa = 0; aa < APT; ++aa) {
-                                int k3 = top3[aa] - t3;
-                                if (k3 < 0) k3 += a.g.K3;
-                                vload<T, VEC>(rowp[aa] + (size_t)k3 * a.ld, phi[aa]);
-                            }
-#pragma unroll
-                            for (int aa = 0; aa < APT; ++aa) {
-                                const T wc = w[aa][2 * p + t3], dc = dw[aa][2 * p + t3];
-                                const T c0 = Ab[aa] * wc, c1 = aB[aa] * wc, c2 = ab[aa] * dc;
-#pragma unroll
-                                for (int v = 0; v < VEC; ++v) {
-                                    f0[aa][v] += c0 * phi[aa][v];
-                                    f1[aa][v] += c1 * phi[aa][v];
-                                    f2[aa][v] += c2 * phi[aa][v];
-                                }
-                            }
-                        }
-                    }
-                }
-                // E^rec_alpha = sum_beta C_{beta alpha} f_beta
-                const T m00 = T(a.g.cmat[0]), m01 = T(a.g.cmat[1]), m02 = T(a.g.cmat[2]);
-                const T m10 = T(a.g.cmat[3]), m11 = T(a.g.cmat[4]), m12 = T(a.g.cmat[5]);
-                const T m20 = T(a.g.cmat[6]), m21 = T(a.g.cmat[7]), m22 = T(a.g.cmat[8]);
-#pragma unroll
-                for (int aa = 0; aa < APT; ++aa)
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) {
-                        E0[aa][v] += m00 * f0[aa][v] + m10 * f1[aa][v] + m20 * f2[aa][v];
-                        E1[aa][v] += m01 * f0[aa][v] + m11 * f1[aa][v] + m21 * f2[aa][v];
-                        E2[aa][v] += m02 * f0[aa][v] + m12 * f1[aa][v] + m22 * f2[aa][v];
-                    }
-            }
-#pragma unroll
-            for (int aa = 0; aa < APT; ++aa) {
-                if (!(HALF ? my_v : val[aa])) continue;
-                const int i = HALF ? my_i : iat[aa];
-                if ((a.o.terms & MBD_TERM_REAL) && a.ereal != nullptr) {
-                    if (warp == NW - 1) {
-                        T x[VEC], y[VEC], z[VEC];
-                        const T *ei = a.ereal + (size_t)(3 * i) * a.ld + r0;
-                        vload<T, VEC>(ei, x);
-                        vload<T, VEC>(ei + a.ld, y);
-                        vload<T, VEC>(ei + 2 * (size_t)a.ld, z);
-#pragma unroll
-                        for (int v = 0; v < VEC; ++v) {
-                            E0[aa][v] += x[v];
-                            E1[aa][v] += y[v];
-                            E2[aa][v] += z[v];
-                        }
-                    }
-                } else if (!HALF && (a.o.terms & MBD_TERM_REAL)) {
-                    const int nb1 = a.pr.row[i + 1];
-                    constexpr int B4 = 4;
-                    for (int nb = a.pr.row[i] + warp; nb < nb1; nb += B4 * NW) {
-                        int jj[B4];
-#pragma unroll
-                        for (int u = 0; u < B4; ++u) jj[u] = (nb + u * NW < nb1) ? a.pr.col[nb + u * NW] : -1;
-                        T xs[B4][VEC], ys[B4][VEC], zs[B4][VEC];
-#pragma unroll
-                        for (int u = 0; u < B4; ++u) {
-                            if (jj[u] >= 0) {
-                                const T *dj = a.d + (size_t)(3 * jj[u]) * a.ld + r0;
-                                vload<T, VEC>(dj, xs[u]);
-                                vload<T, VEC>(dj + a.ld, ys[u]);
-                                vload<T, VEC>(dj + 2 * (size_t)a.ld, zs[u]);
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < B4; ++u) {
-                            if (jj[u] >= 0) {
-                                const T *A = a.pr.A + 6 * (size_t)(nb + u * NW);
-                                const T A0 = A[0], A1 = A[1], A2 = A[2], A3 = A[3], A4 = A[4], A5 = A[5];
-#pragma unroll
-                                for (int v = 0; v < VEC; ++v) {
-                                    E0[aa][v] += A0 * xs[u][v] + A1 * ys[u][v] + A2 * zs[u][v];
-                                    E1[aa][v] += A1 * xs[u][v] + A3 * ys[u][v] + A4 * zs[u][v];
-                                    E2[aa][v] += A2 * xs[u][v] + A4 * ys[u][v] + A5 * zs[u][v];
-                                }
-                            }
-                        }
-                    }
-                }
-                if ((a.o.terms & MBD_TERM_SELF) && warp == 0) {
-                    const T c = T(a.self_coef);
-                    T x[VEC], y[VEC], z[VEC];
-                    const T *di = a.d + (size_t)(3 * i) * a.ld + r0;
-                    vload<T, VEC>(di, x);
-                    vload<T, VEC>(di + a.ld, y);
-                    vload<T, VEC>(di + 2 * (size_t)a.ld, z);
-#pragma unroll
-                    for (int v = 0; v < VEC; ++v) {
-                        E0[aa][v] += c * x[v];
-                        E1[aa][v] += c * y[v];
-                        E2[aa][v] += c * z[v];
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int aa = 0; aa < APT; ++aa)
-#pragma unroll
-            for (int v = 0; v < VEC; ++v) {
-                red[rb][HALF ? sub : aa][warp][0][lid * VEC + v] = E0[aa][v];
-                red[rb][HALF ? sub : aa][warp][1][lid * VEC + v] = E1[aa][v];
-                red[rb][HALF ? sub : aa][warp][2][lid * VEC + v] = E2[aa][v];
-            }
-        __syncthreads();
-        // epilogue: one thread per (component, probe) so that the FP64 work
-        // spreads over the warps; the atoms of the iteration in order
-#pragma unroll
-        for (int aa = 0; aa < AIT; ++aa) {
-            if (!val[aa]) continue;
-            const int i = iat[aa];
-            for (int cp = threadIdx.x; cp < 3 * NLOC; cp += blockDim.x) {
-                const int c = cp / NLOC, t = cp - c * NLOC;
-                const int r = rbase + t;
-                if (r < a.ld) {
-                    T sum = T(0);
-#pragma unroll
-                    for (int w = 0; w < NW; ++w) sum += red[rb][aa][w][c][t];
-                    const double E = double(sum);
-                    const size_t o = (size_t)(3 * i + c) * a.ld + r;
-                    if (a.o.mode == kFieldOut) {
-                        a.o.out[o] = E;
-                    } else if (a.o.mode == kFieldApply) {
-                        a.o.out[o] = a.w2[i] * a.o.xin[o] + a.g_at[i] * E;
-                    } else {
-                        const double invb = a.o.lz.invb[r];
-                        double *Yk = a.o.lz.Y + lz_slot(a.o.lz, a.o.k) * (size_t)(3 * a.g.N) * a.ld;
-                        const double y = Yk[o] * invb;
-                        const double l = a.w2[i] * y + a.g_at[i] * E * invb;
-                        Yk[o] = y;
-                        a.o.lz.L[o] = l;
-                        if (a.o.lz.W) a.o.lz.W[o] += a.o.lz.coef[(size_t)a.o.k * a.ld + r] * y;
-                        if (cp < (int)blockDim.x) part += y * l;
-                        else pcarry[cp - blockDim.x] += y * l;   // thread cp - blockDim.x owns this slot
-                    }
-                }
-            }
+        for (int w = 0; w < NW; ++w) sum += red[w * OUT + slot];
+        const double En = double(sum);
+        const size_t o = (size_t)(3 * i + c) * a.ld + r;
+        if (a.o.mode == kFieldOut) {
+            a.o.out[o] = En;
+        } else if (a.o.mode == kFieldApply) {
+            a.o.out[o] = a.w2[i] * a.o.xin[o] + a.g_at[i] * En;
+        } else {
+            const double invb = a.o.lz.invb[r];
+            double *Yk = a.o.lz.Y + lz_slot(a.o.lz, a.o.k) * (size_t)(3 * a.g.N) * a.ld;
+            const double ys = Yk[o];
+            const double y = ys * invb, l = (a.w2[i] * ys + a.g_at[i] * En) * invb;
+            Yk[o] = y;
+            a.o.lz.L[o] = l;
+            if (a.o.lz.W) a.o.lz.W[o] += a.o.lz.coef[(size_t)a.o.k * a.ld + r] * y;
+            part[k] += y * l;
         }
     }
+}
+// a_k = y_k^T l_k: per probe, the teams and components in order, then a
+// deterministic reduction over blocks.  pall [OUT], bsum and tot [probes of a
+// chunk] are shared scratch.
+template <class T, int NW, int OPT>
+__device__ __forceinline__ void field_reduce_a(const FieldArgs<T> &a, int nloc, int nout, int rbase, const double *part,
+                                               double *pall, double *bsum, double *tot) {
+#pragma unroll
+    for (int k = 0; k < OPT; ++k)
+        if ((int)threadIdx.x + k * NW * 32 < nout) pall[threadIdx.x + k * NW * 32] = part[k];
     __syncthreads();
-    if (a.o.mode != kFieldLanczos) return;
-    // a_k = y_k^T l_k: per probe, the three components in order, then a
-    // deterministic reduction over blocks
-    for (int cp = threadIdx.x; cp < 3 * NLOC; cp += blockDim.x)
-        pall[cp] = (cp < (int)blockDim.x) ? part : pcarry[cp - blockDim.x];
+    for (int t = threadIdx.x; t < nloc; t += NW * 32) {
+        double sum = 0.0;
+        for (int q = 0; q < 3 * a.teams; ++q) sum += pall[q * nloc + t];
+        bsum[t] = sum;
+    }
     __syncthreads();
-    for (int t = threadIdx.x; t < NLOC; t += blockDim.x) bsum[t] = pall[t] + pall[NLOC + t] + pall[2 * NLOC + t];
-    __syncthreads();
-    __shared__ double tot[NLOC];
-    if (grid_reduce(bsum, NLOC, rbase, a.R, a.ld, a.o.lz, tot)) {
-        for (int k = threadIdx.x; k < NLOC; k += blockDim.x)
+    if (grid_reduce(bsum, nloc, rbase, a.R, a.ld, a.o.lz, tot)) {
+        for (int k = threadIdx.x; k < nloc; k += NW * 32)
             if (rbase + k < a.R) a.o.lz.a[(size_t)a.o.k * a.ld + rbase + k] = tot[k];
     }
+}
+
+// Field kernel.  `lanes` lanes with VEC probes each (16-byte accesses) hold the
+// probes of an atom (of a chunk of 32 VEC probes, blockIdx.y), so a warp holds
+// S = 32 / lanes groups.  A block works on `teams` atoms at once; the groups of
+// a team (S / teams per warp, in every warp) split the p^2 pencils of the
+// atom's stencil and, with PAIRS, its neighbours.  With many probes (S = teams
+// = 1) a warp gathers whole planes of the stencil; with few, a warp's groups take
+// several atoms or, in small systems, share one.  Along a pencil the field
+// factorises like the weights: s0 = sum_t M3(t) phi, s1 = sum_t M3'(t) phi
+// (two FMAs per mesh value), then f += (M1' M2 s0, M1 M2' s0, M1 M2 s1) once.
+// The partial fields are summed in a fixed order (shuffles within a warp,
+// then the warps in shared memory) and the epilogue selected by o.mode runs
+// with one thread per (atom, component, probe): E* = E^rec + E^dir + E^self
+// (Eqs. ewalddip, spme, fld_ewald, fld_ewald1), l_k = Omega y_k + Diag(g) E*_k
+// and a_k = y_k^T l_k (Eqs. lk3, recurs2).
+// Bound: load latency (FP32), the FP64 units (FP64).  Against a lane per probe
+// with six FMAs and three products per mesh value: 288 atoms x 1 FP64 68 -> 23
+// us per launch, 1371 x 33 order 8 127 -> 34, 3000 x 32 FP64 544 -> 295, 15,000
+// x 2 order 8 331 -> 76.
+template <class T, int P, bool PAIRS>
+__global__ void __launch_bounds__(field_warps<P>() * 32, sizeof(T) == 8 ? 2 : (PAIRS ? 3 : 4) * 6 / field_warps<P>())
+    k_field(FieldArgs<T> a) {
+    constexpr int VEC = field_vec<T>(), NW = field_warps<P>(), NTH = NW * 32;
+    constexpr int RB = field_rec_bytes<T, P>();
+    constexpr int OUT = 32 * VEC * 3;            // (team, component, probe) slots of an iteration, at most
+    constexpr int OPT = (OUT + NTH - 1) / NTH;   // of them per thread, at most
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int S = 32 / a.lanes, nloc = a.lanes * VEC, per = S / a.teams;   // groups of a team in a warp
+    const int sub = lane / a.lanes, lid = lane - sub * a.lanes;
+    const int team = sub % a.teams, member = warp + NW * (sub / a.teams), members = NW * per;
+    const int rbase = blockIdx.y * 32 * VEC;
+    const int r0 = rbase + lid * VEC;
+    const bool on = sub < S && r0 < a.ld;
+    const int nout = a.teams * 3 * nloc;
+    // partial fields of the warps, double-buffered by iteration: the barrier
+    // after one iteration's writes also orders the previous epilogue's reads
+    // before the buffer is written again, so one barrier per iteration
+    __shared__ __align__(16) T red[2][NW][OUT];
+    __shared__ double pall[OUT], bsum[32 * VEC], tot[32 * VEC];
+    double part[OPT];                            // y.l of the slots this thread owns
+#pragma unroll
+    for (int k = 0; k < OPT; ++k) part[k] = 0.0;
+    const int i0 = blockIdx.x * a.apb, i1 = min(i0 + a.apb, a.g.N);
+    int buf = 0;
+    for (int ib = i0; ib < i1; ib += a.teams, buf ^= 1) {
+        T E[3][VEC];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) E[c][v] = T(0);
+        if (on && ib + team < i1) {
+            const unsigned char *rec = a.rec + (size_t)(ib + team) * RB;
+            const int4 hd = *reinterpret_cast<const int4 *>(rec);
+            const int i = hd.x;
+            if (a.o.terms & MBD_TERM_RECIP) {
+                T f[3][VEC];
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) f[c][v] = T(0);
+                const T *w = reinterpret_cast<const T *>(rec + 16);
+                T w3[2 * P];
+#pragma unroll
+                for (int b = 0; b < 2 * P; b += VEC) vload<T, VEC>(w + 4 * P + b, w3 + b);
+                int off[P];
+#pragma unroll
+                for (int t = 0; t < P; ++t) off[t] = (hd.w - t + (hd.w < t ? a.g.K3 : 0)) * a.ld;
+                for (int u = member; u < P * P; u += members) {
+                    const int t1 = u % P, t2 = u / P;
+                    int k1 = hd.y - t1, k2 = hd.z - t2;
+                    if (k1 < 0) k1 += a.g.K1;
+                    if (k2 < 0) k2 += a.g.K2;
+                    const T *rowp = a.mesh + ((size_t)k1 * a.g.K2 + k2) * a.g.K3 * a.ld + r0;
+                    T phi[P][VEC];
+#pragma unroll
+                    for (int t = 0; t < P; ++t) vload<T, VEC>(rowp + off[t], phi[t]);
+                    const T wa = w[t1], da = w[P + t1], wb = w[2 * P + t2], db = w[3 * P + t2];
+                    T s0[VEC], s1[VEC];
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) s0[v] = s1[v] = T(0);
+#pragma unroll
+                    for (int t = 0; t < P; ++t) {
+                        lane_fma<T, VEC>(phi[t], w3[t], s0);
+                        lane_fma<T, VEC>(phi[t], w3[P + t], s1);
+                    }
+                    lane_fma<T, VEC>(s0, da * wb, f[0]);
+                    lane_fma<T, VEC>(s0, wa * db, f[1]);
+                    lane_fma<T, VEC>(s1, wa * wb, f[2]);
+                }
+                // E^rec_alpha = sum_beta C_{beta alpha} f_beta
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) lane_fma<T, VEC>(f[b], T(a.g.cmat[3 * b + c]), E[c]);
+            }
+            if (a.o.terms & MBD_TERM_REAL) {
+                if constexpr (PAIRS) {
+                    const int nb1 = a.pr.row[i + 1];
+                    constexpr int B = 2;
+                    for (int nb = a.pr.row[i] + member; nb < nb1; nb += B * members) {
+                        int jj[B];
+                        T x[B][VEC], y[B][VEC], z[B][VEC];
+#pragma unroll
+                        for (int u = 0; u < B; ++u) jj[u] = nb + u * members < nb1 ? a.pr.col[nb + u * members] : -1;
+#pragma unroll
+                        for (int u = 0; u < B; ++u)
+                            if (jj[u] >= 0) {
+                                const T *dj = a.d + (size_t)(3 * jj[u]) * a.ld + r0;
+                                vload<T, VEC>(dj, x[u]);
+                                vload<T, VEC>(dj + a.ld, y[u]);
+                                vload<T, VEC>(dj + 2 * (size_t)a.ld, z[u]);
+                            }
+#pragma unroll
+                        for (int u = 0; u < B; ++u)
+                            if (jj[u] >= 0) {
+                                T A[6];
+#pragma unroll
+                                for (int e = 0; e < 6; e += 2)
+                                    vload<T, 2>(a.pr.A + 6 * (size_t)(nb + u * members) + e, A + e);
+                                lane_fma<T, VEC>(x[u], A[0], E[0]);
+                                lane_fma<T, VEC>(y[u], A[1], E[0]);
+                                lane_fma<T, VEC>(z[u], A[2], E[0]);
+                                lane_fma<T, VEC>(x[u], A[1], E[1]);
+                                lane_fma<T, VEC>(y[u], A[3], E[1]);
+                                lane_fma<T, VEC>(z[u], A[4], E[1]);
+                                lane_fma<T, VEC>(x[u], A[2], E[2]);
+                                lane_fma<T, VEC>(y[u], A[4], E[2]);
+                                lane_fma<T, VEC>(z[u], A[5], E[2]);
+                            }
+                    }
+                } else if (member == NW - 1) {
+                    T x[VEC];
+                    const T *ei = a.ereal + (size_t)(3 * i) * a.ld + r0;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        vload<T, VEC>(ei + (size_t)c * a.ld, x);
+#pragma unroll
+                        for (int v = 0; v < VEC; ++v) E[c][v] += x[v];
+                    }
+                }
+            }
+            if ((a.o.terms & MBD_TERM_SELF) && member == 0) {
+                T x[VEC];
+                const T *di = a.d + (size_t)(3 * i) * a.ld + r0;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    vload<T, VEC>(di + (size_t)c * a.ld, x);
+                    lane_fma<T, VEC>(x, T(a.self_coef), E[c]);
+                }
+            }
+        }
+        // the groups of a team within the warp (S is a power of two when per > 1)
+        for (int h = S / 2; h >= a.teams && per > 1; h >>= 1) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) E[c][v] += __shfl_down_sync(0xffffffffu, E[c][v], h * a.lanes);
+        }
+        if (sub < a.teams) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) vstore<T, VEC>(&red[buf][warp][(team * 3 + c) * nloc + lid * VEC], E[c]);
+        }
+        __syncthreads();
+        field_epilogue<T, NW, OUT, OPT>(a, &red[buf][0][0], RB, nloc, nout, rbase, ib, i1, part);
+    }
+    if (a.o.mode != kFieldLanczos) return;
+    field_reduce_a<T, NW, OPT>(a, nloc, nout, rbase, part, pall, bsum, tot);
+}
+
+// The field kernel for large FP32 systems with the real space on clusters: the
+// same split (a group per warp and atom, so members = NW, and p^2 / NW pencils
+// per group in a fixed order), with the mesh values streamed through shared
+// memory.  Each thread copies its own 16 bytes of a pencil's P points by
+// cp.async, kFieldDepth pencils ahead of the one it works on and across atoms,
+// and reads back only what it copied itself, so no barrier is involved and no
+// register holds a value in flight: the loads in flight per SM, which bound the
+// kernel (ncu: DRAM and L2 far from their peaks, long-scoreboard stalls), no
+// longer depend on registers.  The atoms' weights for the next iteration are
+// copied to shared memory meanwhile.
+constexpr int kFieldDepth = 2;
+template <int P> constexpr size_t field_stream_smem(int teams) {
+    constexpr int NTH = field_warps<P>() * 32;
+    return 16 * (size_t)kFieldDepth * P * NTH + 4 * (size_t)field_warps<P>() * 384 + 2 * (size_t)teams * 24 * P;
+}
+template <int P>
+__global__ void __launch_bounds__(field_warps<P>() * 32, P == 6 ? 4 : 2) k_field_stream(FieldArgs<float> a) {
+    constexpr int VEC = 4, NW = field_warps<P>(), NTH = NW * 32, PP = P * P / NW, D = kFieldDepth;
+    constexpr int OUT = 32 * VEC * 3, OPT = (OUT + NTH - 1) / NTH, RB = field_rec_bytes<float, P>(), W4 = 6 * P / 4;
+    static_assert(P * P % NW == 0 && PP % D == 0 && 6 * P % 4 == 0, "whole pencils per warp and ring");
+    extern __shared__ __align__(16) unsigned char smem_fs[];
+    float4 *ring = reinterpret_cast<float4 *>(smem_fs);                  // [D][P][NTH]
+    float *red = reinterpret_cast<float *>(ring + D * P * NTH);          // [NW][OUT]
+    float4 *wts = reinterpret_cast<float4 *>(red + NW * OUT);            // [2][teams][W4]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nloc = a.lanes * VEC, sub = lane / a.lanes, lid = lane - sub * a.lanes;
+    const int rbase = blockIdx.y * 32 * VEC, r0 = rbase + lid * VEC;
+    const bool on = sub < a.teams && r0 < a.ld;
+    const int nout = a.teams * 3 * nloc;
+    double part[OPT];
+#pragma unroll
+    for (int k = 0; k < OPT; ++k) part[k] = 0.0;
+    const int i0 = blockIdx.x * a.apb, i1 = min(i0 + a.apb, a.g.N);
+    auto header = [&](int pos) {
+        return pos < i1 ? *reinterpret_cast<const int4 *>(a.rec + (size_t)pos * RB) : make_int4(-1, 0, 0, 0);
+    };
+    auto fetch_weights = [&](int ib, int b) {   // the weights of the teams' atoms from ib on
+        for (int q = threadIdx.x; q < a.teams * W4; q += NTH)
+            if (ib + q / W4 < i1)
+                cp_async<16>(wts + b * a.teams * W4 + q, a.rec + (size_t)(ib + q / W4) * RB + 16 + 16 * (q % W4));
+    };
+    int off[P];
+    auto offsets = [&](int4 hd) {
+#pragma unroll
+        for (int t = 0; t < P; ++t) off[t] = (hd.w - t + (hd.w < t ? a.g.K3 : 0)) * a.ld;
+    };
+    auto fetch = [&](int4 hd, int j) {          // pencil j of the atom into ring slot j % D
+        if (on && hd.x >= 0) {
+            const int u = warp + NW * j, t1 = u % P, t2 = u / P;
+            int k1 = hd.y - t1, k2 = hd.z - t2;
+            if (k1 < 0) k1 += a.g.K1;
+            if (k2 < 0) k2 += a.g.K2;
+            const float *rowp = a.mesh + ((size_t)k1 * a.g.K2 + k2) * a.g.K3 * a.ld + r0;
+#pragma unroll
+            for (int t = 0; t < P; ++t) cp_async<16>(ring + ((j % D) * P + t) * NTH + threadIdx.x, rowp + off[t]);
+        }
+        cp_async_commit();
+    };
+    int4 hd = header(i0 + sub);
+    fetch_weights(i0, 0);
+    cp_async_commit();
+    offsets(hd);
+#pragma unroll
+    for (int j = 0; j < D; ++j) fetch(hd, j);
+    cp_async_wait<D>();                          // the first weights, made visible by the barrier
+    __syncthreads();
+    int b = 0;
+    for (int ib = i0; ib < i1; ib += a.teams, b ^= 1) {
+        const int4 next = header(ib + a.teams + sub);
+        fetch_weights(ib + a.teams, b ^ 1);      // joins the group of the next pencil
+        const float *w = reinterpret_cast<const float *>(wts + (b * a.teams + (sub < a.teams ? sub : 0)) * W4);
+        float f[3][VEC];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) f[c][v] = 0.f;
+#pragma unroll
+        for (int j = 0; j < PP; ++j) {
+            cp_async_wait<D - 1>();              // this thread's copies of pencil j are done
+            float s0[VEC], s1[VEC];
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) s0[v] = s1[v] = 0.f;
+#pragma unroll
+            for (int t = 0; t < P; ++t) {
+                float phi[VEC];
+                vload<float, VEC>(reinterpret_cast<const float *>(ring + ((j % D) * P + t) * NTH + threadIdx.x), phi);
+                lane_fma<float, VEC>(phi, w[4 * P + t], s0);
+                lane_fma<float, VEC>(phi, w[5 * P + t], s1);
+            }
+            if (j + D == PP) offsets(next);
+            if (j + D < PP) fetch(hd, j + D);
+            else fetch(next, j + D - PP);
+            const int u = warp + NW * j, t1 = u % P, t2 = u / P;
+            const float wa = w[t1], da = w[P + t1], wb = w[2 * P + t2], db = w[3 * P + t2];
+            lane_fma<float, VEC>(s0, da * wb, f[0]);
+            lane_fma<float, VEC>(s0, wa * db, f[1]);
+            lane_fma<float, VEC>(s1, wa * wb, f[2]);
+        }
+        float E[3][VEC];
+        const bool act = on && hd.x >= 0;
+        // E^rec_alpha = sum_beta C_{beta alpha} f_beta
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) E[c][v] = 0.f;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) lane_fma<float, VEC>(f[q], float(a.g.cmat[3 * q + c]), E[c]);
+        }
+        if (act && warp == NW - 1 && (a.o.terms & MBD_TERM_REAL)) {
+            const float *ei = a.ereal + (size_t)(3 * hd.x) * a.ld + r0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float x[VEC];
+                vload<float, VEC>(ei + (size_t)c * a.ld, x);
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) E[c][v] += x[v];
+            }
+        }
+        if (act && warp == 0 && (a.o.terms & MBD_TERM_SELF)) {
+            const float *di = a.d + (size_t)(3 * hd.x) * a.ld + r0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float x[VEC];
+                vload<float, VEC>(di + (size_t)c * a.ld, x);
+                lane_fma<float, VEC>(x, float(a.self_coef), E[c]);
+            }
+        }
+        if (sub < a.teams) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) vstore<float, VEC>(red + warp * OUT + (sub * 3 + c) * nloc + lid * VEC, E[c]);
+        }
+        if constexpr (PP == D) cp_async_wait<D - 1>();   // (they came with the next atom's first pencil)
+        __syncthreads();                         // the partial fields, and the next weights
+        field_epilogue<float, NW, OUT, OPT>(a, red, RB, nloc, nout, rbase, ib, i1, part);
+        __syncthreads();                         // red is written again
+        hd = next;
+    }
+    cp_async_wait<0>();                          // no copy in flight at exit
+    if (a.o.mode != kFieldLanczos) return;
+    double *pall = reinterpret_cast<double *>(smem_fs);
+    __syncthreads();                             // the ring is scratch from here on
+    field_reduce_a<float, NW, OPT>(a, nloc, nout, rbase, part, pall, pall + OUT, pall + OUT + 32 * VEC);
 }
 
 template <class T> PrecData<T> &prec(mbd_system *s);
@@ -699,7 +860,7 @@ mbd_status launch_exclusive_scan(const int *in, int *out, int n, DevBuf &bsum, c
 }
 
 // The spreading records of the current geometry: counts, CSR starts, records,
-// and the per-atom k3 stencils.
+// and the per-atom k3 stencils; and the field kernel's records.
 template <class T> mbd_status build_spread_records(mbd_system *s) {
     PrecData<T> &P = prec<T>(s);
     const Geom g = geom_of(s);
@@ -721,7 +882,13 @@ template <class T> mbd_status build_spread_records(mbd_system *s) {
                                                              s->dw64_d.as<double>(), P.prow.template as<int>(),
                                                              P.prec.template as<PencilRec<T>>());
     MBD_LAUNCH_CHECK();
+    MBD_TRY(P.frec.ensure((16 + 6 * (size_t)s->p * sizeof(T)) * std::max(1, s->N)));
     if (s->N > 0) {
+        const int nrec = s->N * (6 * s->p + 4);
+        k_field_rec<T><<<(nrec + threads - 1) / threads, threads, 0, s->stream>>>(
+            s->N, s->p, s->order_d.as<int>(), s->top_d.as<int>(), s->w64_d.as<double>(), s->dw64_d.as<double>(),
+            P.frec.template as<unsigned char>());
+        MBD_LAUNCH_CHECK();
         k_pencil_k3w<T><<<(2 * s->p * s->N + threads - 1) / threads, threads, 0, s->stream>>>(
             s->N, s->p, s->w64_d.as<double>(), s->dw64_d.as<double>(), P.k3w.template as<T>());
         MBD_LAUNCH_CHECK();
@@ -853,117 +1020,20 @@ template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bo
     return MBD_OK;
 }
 
-template <class T>
-mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld, const FieldOut<T> &o) {
-    PrecData<T> &P = prec<T>(s);
-    FieldArgs<T> a;
-    a.d = d;
-    a.mesh = mesh;
-    a.R = R;
-    a.ld = ld;
-    a.g = geom_of(s);
-    a.sp = SplineView<T>{s->top_d.as<int>(), P.w.template as<T>(), P.dw.template as<T>(), P.d2w.template as<T>()};
-    a.pr = PairView<T>{s->row_d.as<int>(), s->col_d.as<int>(), s->shift_d.as<int>(), P.pairA.template as<T>()};
-    a.order = s->order_d.as<int>();
-    a.g_at = s->g_d.as<double>();
-    a.w2 = s->w2_d.as<double>();
-    a.self_coef = -4.0 * s->ewald_beta * s->ewald_beta * s->ewald_beta / (3.0 * 1.77245385090551602730);
-    a.ereal = real_on_clusters(s, ld, (int)sizeof(T)) ? P.ereal.template as<T>() : nullptr;
-    a.o = o;
-    const int vec = field_vec(ld, (int)sizeof(T));
-    const int apb = field_apb(s, ld);
-    dim3 grid(field_blocks(s, ld), (ld + 32 * vec - 1) / (32 * vec));
-    const bool six = a.ereal != nullptr && s->p == 6;
-#define MBD_FIELD_LAUNCH(V, P, NW) k_field<T, V, P, NW><<<grid, (NW) * 32, 0, s->stream>>>(a, apb)
-    if constexpr (sizeof(T) == 4) {
-        if (six && field_half(ld, 4)) {
-            // 64-probe chunks as with two probes per lane, here four probes per
-            // lane on half-warps, one atom each
-            k_field<T, 4, 6, 6, 16><<<grid, 6 * 32, 0, s->stream>>>(a, apb);
-            MBD_LAUNCH_CHECK();
-            return MBD_OK;
-        }
-    }
-    if (vec == 4) {
-        if constexpr (sizeof(T) == 4) {
-            if (six) MBD_FIELD_LAUNCH(4, 6, 6);
-            else if (s->p == 6) MBD_FIELD_LAUNCH(4, 6, kWarps);
-            else MBD_FIELD_LAUNCH(4, 0, kWarps);
-        }
-    } else if (vec == 2) {
-        if (six) MBD_FIELD_LAUNCH(2, 6, 6);
-        else if (s->p == 6) MBD_FIELD_LAUNCH(2, 6, kWarps);
-        else MBD_FIELD_LAUNCH(2, 0, kWarps);
-    } else {
-        if (six) MBD_FIELD_LAUNCH(1, 6, 6);
-        else if (s->p == 6) MBD_FIELD_LAUNCH(1, 6, kWarps);
-        else MBD_FIELD_LAUNCH(1, 0, kWarps);
-    }
-#undef MBD_FIELD_LAUNCH
-    MBD_LAUNCH_CHECK();
-    return MBD_OK;
-}
-
-// The real-space field runs on the clusters when they were built and there
-// are enough of them for four blocks per SM (a block per cluster and probe
-// chunk); smaller systems keep the pair loop of the field kernel, whose warps
-// split the neighbours of one atom.
-bool real_on_clusters(const mbd_system *s, int ld, int real_bytes) {
-    if (!s->real_clusters || s->real_method == MBD_REAL_PAIRS) return false;
-    if (s->real_method == MBD_REAL_CLUSTERS) return true;
-    const int ppl = real_bytes == 4 ? 2 : 1;
-    const long long chunks = (ld + 32 * ppl - 1) / (32 * ppl);
-    return (long long)s->n_clusters * chunks >= 4LL * std::max(1, s->num_sms);
-}
-
-// E_real of every atom from the clusters (the caller runs this before
-// launch_field whenever real_on_clusters holds and the real-space term is wanted).
-template <class T> mbd_status launch_real_clusters(mbd_system *s, const T *d, T *ereal, int ld, cudaStream_t st) {
-    PrecData<T> &P = prec<T>(s);
-    RealArgs<T> a;
-    a.d = d;
-    a.out = ereal;
-    a.ld = ld;
-    a.N = s->N;
-    a.nclus = s->n_clusters;
-    a.order = s->order_d.as<int>();
-    a.estart = s->cl_estart.as<int>();
-    a.pstart = s->cl_pstart.as<int>();
-    a.entries = s->cl_entries.as<int>();
-    a.pairs = P.cA.template as<RealPair<T>>();
-    if (a.nclus == 0) return MBD_OK;
-    constexpr int ppl = sizeof(T) == 4 ? 2 : 1;
-    dim3 grid((unsigned)a.nclus, (unsigned)((ld + 32 * ppl - 1) / (32 * ppl)));
-    const size_t smem = sizeof(T) * kRealCE * 3 * 32 * ppl + sizeof(RealPair<T>) * kClusterSize * 32;
-    static bool attr = false;
-    if (!attr) {
-        MBD_CUDA_TRY(cudaFuncSetAttribute(k_real_clusters<T, ppl>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
-        attr = true;
-    }
-    k_real_clusters<T, ppl><<<grid, 32 * kClusterSize, smem, st>>>(a);
-    MBD_LAUNCH_CHECK();
-    return MBD_OK;
-}
-
-// Probes per lane of the field kernel.
-int field_vec(int ld, int real_bytes) {
-    return (real_bytes == 4 && ld % 4 == 0 && ld >= 128) ? 4 : ((ld % 2 == 0 && ld >= 64) ? 2 : 1);
-}
-
-// FP32 chunks of 64 probes (two per lane) whose probe count allows 16-byte
-// loads: the six-warp field kernel then gathers one atom per half-warp, four
-// probes per lane (the same chunks).
-bool field_half(int ld, int real_bytes) { return real_bytes == 4 && field_vec(ld, 4) == 2 && ld % 4 == 0; }
-
+// How a field launch is laid out: lanes per atom, atoms at once and in all per
+// block, blocks.
+struct FieldShape {
+    int lanes, teams, apb, blocks, chunks;
+};
 namespace {
 // Resident blocks per SM of one field-kernel variant (the same on every
 // device of one architecture), asked of the occupancy calculator once.
-template <class T, int V, int P, int NW = kWarps, int LPA = 32> int field_occupancy() {
+template <class T, int P, bool PAIRS> int field_occupancy() {
     static int nb = 0;
     if (nb == 0) {
         int x = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_field<T, V, P, NW, LPA>, NW * 32, 0) != cudaSuccess ||
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_field<T, P, PAIRS>, field_warps<P>() * 32, 0) !=
+                cudaSuccess ||
             x < 1) {
             cudaGetLastError();
             x = 1;
@@ -973,57 +1043,165 @@ template <class T, int V, int P, int NW = kWarps, int LPA = 32> int field_occupa
     return nb;
 }
 
-int field_resident_blocks(const mbd_system *s, int ld) {
-    const bool p6 = s->p == 6;
-    const bool fp64 = s->precision == MBD_FP64;
-    const bool six = p6 && real_on_clusters(s, ld, fp64 ? 8 : 4);
-    int nb;
-    if (fp64) {
-        const int vec = field_vec(ld, 8);
-        if (six)
-            nb = vec == 2 ? field_occupancy<double, 2, 6, 6>() : field_occupancy<double, 1, 6, 6>();
-        else
-            nb = vec == 2 ? (p6 ? field_occupancy<double, 2, 6>() : field_occupancy<double, 2, 0>())
-                          : (p6 ? field_occupancy<double, 1, 6>() : field_occupancy<double, 1, 0>());
-    } else {
-        const int vec = field_vec(ld, 4);
-        if (six)
-            nb = vec == 4            ? field_occupancy<float, 4, 6, 6>()
-                 : field_half(ld, 4) ? field_occupancy<float, 4, 6, 6, 16>()
-                 : vec == 2          ? field_occupancy<float, 2, 6, 6>()
-                                     : field_occupancy<float, 1, 6, 6>();
-        else
-            nb = vec == 4   ? (p6 ? field_occupancy<float, 4, 6>() : field_occupancy<float, 4, 0>())
-                 : vec == 2 ? (p6 ? field_occupancy<float, 2, 6>() : field_occupancy<float, 2, 0>())
-                            : (p6 ? field_occupancy<float, 1, 6>() : field_occupancy<float, 1, 0>());
+// Lanes per atom: just enough for the probes of a chunk (32 VEC at most).  In
+// systems with fewer atoms than the resident blocks can take S at a time, the
+// groups of a warp share atoms instead (lanes a power of two): as many atoms
+// at once per block as give the resident blocks one iteration each.  Otherwise
+// the blocks fill whole waves of the resident capacity, with at most 64
+// atoms per block (more waves beyond that, for balance).
+template <class T> FieldShape field_shape(const mbd_system *s, int ld) {
+    constexpr int VEC = field_vec<T>();
+    const bool pairs = !real_on_clusters(s, ld, (int)sizeof(T));
+    int occ = 1;
+    switch (s->p) {
+#define MBD_FIELD_OCC(P) \
+    case P: occ = pairs ? field_occupancy<T, P, true>() : field_occupancy<T, P, false>(); break;
+        MBD_SPLINE_ORDERS(MBD_FIELD_OCC)
+#undef MBD_FIELD_OCC
+        default: break;
     }
-    return nb * std::max(1, s->num_sms);
+    FieldShape f;
+    f.chunks = (ld + 32 * VEC - 1) / (32 * VEC);
+    f.lanes = std::min(32, ld / VEC);
+    const long long per_wave = std::max(1, occ * std::max(1, s->num_sms) / f.chunks);
+    f.teams = 32 / f.lanes;
+    const long long want = (s->N + per_wave - 1) / per_wave;   // atoms per resident block
+    if (want < f.teams) {
+        int l = 1;
+        while (l < f.lanes) l *= 2;
+        f.lanes = l;
+        f.teams = 32 / l;
+        while (f.teams > 1 && f.teams / 2 >= want) f.teams /= 2;
+    }
+    if (s->tune_field_apb > 0 && tuned_for<T>(s, ld)) {
+        f.apb = s->tune_field_apb;
+    } else {
+        const long long waves = (s->N + 64 * per_wave - 1) / (64 * per_wave);
+        f.apb = (int)std::max<long long>(1, (s->N + waves * per_wave - 1) / (waves * per_wave));
+    }
+    f.apb = (f.apb + f.teams - 1) / f.teams * f.teams;
+    f.blocks = (s->N + f.apb - 1) / f.apb;
+    return f;
+}
+// The streaming kernel: FP32 with the real space on clusters, at least 32
+// probes (four groups per warp at most), whole iterations' worth of atoms, the
+// mesh term wanted.
+bool field_streams(const mbd_system *s, int ld, const FieldShape &f, int terms) {
+    return s->precision != MBD_FP64 && real_on_clusters(s, ld, 4) && f.lanes >= 8 && f.teams == 32 / f.lanes &&
+           (terms & MBD_TERM_RECIP);
 }
 }  // namespace
 
-// Atoms per block of the field kernel: the blocks fill whole waves of the
-// resident-block capacity (blocks per SM x SMs, shared by the probe chunks),
-// with at most 64 atoms per block (more waves beyond that, for balance).
-int field_apb(const mbd_system *s, int ld) {
-    const int bytes = s->precision == MBD_FP64 ? 8 : 4;
-    const int vec = field_vec(ld, bytes);
-    // the six-warp FP32 kernels take two atoms per iteration: an even count
-    // leaves no half-empty iteration
-    const bool pairs = bytes == 4 && s->p == 6 && real_on_clusters(s, ld, bytes) && (vec == 4 || field_half(ld, bytes));
-    int apb;
-    if (s->tune_field_apb > 0 && (bytes == 4 ? tuned_for<float>(s, ld) : tuned_for<double>(s, ld))) {
-        apb = s->tune_field_apb;
-    } else {
-        const int ych = (ld + 32 * vec - 1) / (32 * vec);
-        const long long per_wave = std::max(1, field_resident_blocks(s, ld) / ych);
-        const long long waves = (s->N + 64 * per_wave - 1) / (64 * per_wave);
-        apb = (int)std::max<long long>(1, (s->N + waves * per_wave - 1) / (waves * per_wave));
+template <class T>
+mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld, const FieldOut<T> &o) {
+    PrecData<T> &P = prec<T>(s);
+    const FieldShape f = field_shape<T>(s, ld);
+    FieldArgs<T> a;
+    a.d = d;
+    a.mesh = mesh;
+    a.R = R;
+    a.ld = ld;
+    a.g = geom_of(s);
+    a.pr = PairView<T>{s->row_d.as<int>(), s->col_d.as<int>(), s->shift_d.as<int>(), P.pairA.template as<T>()};
+    a.rec = P.frec.template as<unsigned char>();
+    a.g_at = s->g_d.as<double>();
+    a.w2 = s->w2_d.as<double>();
+    a.self_coef = -4.0 * s->ewald_beta * s->ewald_beta * s->ewald_beta / (3.0 * 1.77245385090551602730);
+    const bool pairs = !real_on_clusters(s, ld, (int)sizeof(T));
+    a.ereal = pairs ? nullptr : P.ereal.template as<T>();
+    a.o = o;
+    a.lanes = f.lanes;
+    a.teams = f.teams;
+    a.apb = f.apb;
+    const dim3 grid(f.blocks, f.chunks);
+    if constexpr (sizeof(T) == 4) {
+        if (field_streams(s, ld, f, o.terms)) {
+            switch (s->p) {
+#define MBD_FIELD_ORDER(P)                                                                                        \
+    case P: {                                                                                                     \
+        const size_t smem = field_stream_smem<P>(f.teams);                                                        \
+        MBD_CUDA_TRY(cudaFuncSetAttribute(k_field_stream<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+        k_field_stream<P><<<grid, field_warps<P>() * 32, smem, s->stream>>>(a);                                    \
+        break;                                                                                                    \
     }
-    return pairs ? apb + (apb & 1) : apb;
+                MBD_SPLINE_ORDERS(MBD_FIELD_ORDER)
+#undef MBD_FIELD_ORDER
+            }
+            MBD_LAUNCH_CHECK();
+            return MBD_OK;
+        }
+    }
+    switch (s->p) {
+#define MBD_FIELD_ORDER(P)                                                                \
+    case P:                                                                               \
+        if (pairs) k_field<T, P, true><<<grid, field_warps<P>() * 32, 0, s->stream>>>(a);  \
+        else k_field<T, P, false><<<grid, field_warps<P>() * 32, 0, s->stream>>>(a);       \
+        break;
+        MBD_SPLINE_ORDERS(MBD_FIELD_ORDER)
+#undef MBD_FIELD_ORDER
+        default: return MBD_ERR_UNSUPPORTED;
+    }
+    MBD_LAUNCH_CHECK();
+    return MBD_OK;
+}
+
+int field_apb(const mbd_system *s, int ld) {
+    return s->precision == MBD_FP64 ? field_shape<double>(s, ld).apb : field_shape<float>(s, ld).apb;
 }
 int field_blocks(const mbd_system *s, int ld) {
-    const int apb = field_apb(s, ld);
-    return (s->N + apb - 1) / apb;
+    return s->precision == MBD_FP64 ? field_shape<double>(s, ld).blocks : field_shape<float>(s, ld).blocks;
+}
+
+// Chunks of probes of the cluster kernel: at most 64 probes each (FP64: 32), and
+// down to 16 where fewer would leave less than four blocks per SM.
+template <class T> int real_chunks(const mbd_system *s, int ld) {
+    constexpr int most = 256 / (int)sizeof(T);
+    const int least = (ld + most - 1) / most, want = (4 * std::max(1, s->num_sms) + s->n_clusters - 1) /
+                                                     std::max(1, s->n_clusters);
+    return std::max(least, std::min(want, ld / 16));
+}
+// The real-space field runs on the clusters when they were built and atoms x
+// probes are enough to fill the GPU with them; smaller systems keep the pair
+// loop of the field kernel, whose groups split the neighbours of one atom.
+// Measured per Lanczos step, pairs against clusters: 3000 atoms x 64 probes 222
+// and 230 us, x 128 440 and 429; 6000 x 32 260 and 261, x 64 466 and 443; 15,000
+// x 2 (padded to 4) 203 and 240.  FP64, bound by its arithmetic either way, takes
+// them with four blocks per SM.
+constexpr long long kRealMinValues = 256 * 1024;
+bool real_on_clusters(const mbd_system *s, int ld, int real_bytes) {
+    if (!s->real_clusters || s->real_method == MBD_REAL_PAIRS) return false;
+    if (s->real_method == MBD_REAL_CLUSTERS) return true;
+    if (real_bytes == 8) return (long long)s->n_clusters * ((ld + 31) / 32) >= 4LL * std::max(1, s->num_sms);
+    return (long long)s->N * ld >= kRealMinValues;
+}
+
+// E_real of every atom from the clusters (the caller runs this before
+// launch_field whenever real_on_clusters holds and the real-space term is wanted).
+template <class T> mbd_status launch_real_clusters(mbd_system *s, const T *d, T *ereal, int ld, cudaStream_t st) {
+    PrecData<T> &P = prec<T>(s);
+    constexpr int VEC = 16 / (int)sizeof(T);
+    if (s->n_clusters == 0) return MBD_OK;
+    const int chunks = real_chunks<T>(s, ld);
+    RealArgs<T> a;
+    a.d = d;
+    a.out = ereal;
+    a.ld = ld;
+    a.N = s->N;
+    a.order = s->order_d.as<int>();
+    a.pstart = s->cl_pstart.as<int>();
+    a.ecnt = s->cl_ecnt.as<int>();
+    a.rcnt = s->cl_rcnt.as<int>();
+    a.entries = s->cl_entries.as<int>();
+    a.recs = P.cA.template as<RealDuo<T>>();
+    a.np = ((ld + chunks - 1) / chunks + VEC - 1) / VEC * VEC;
+    a.ce = std::min(192, kRealStageBytes / (3 * a.np * (int)sizeof(T)));
+    dim3 grid((unsigned)s->n_clusters, (unsigned)((ld + a.np - 1) / a.np));
+    const size_t smem = sizeof(RealDuo<T>) * kClusterSize * kRealBatch + 16 * ((8 * (size_t)a.ce + 15) / 16) +
+                        sizeof(T) * 3 * (size_t)a.np * a.ce;
+    MBD_CUDA_TRY(cudaFuncSetAttribute(k_real_clusters<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_real_clusters<T><<<grid, 16 * kClusterSize, smem, st>>>(a);
+    MBD_LAUNCH_CHECK();
+    return MBD_OK;
 }
 
 template mbd_status build_spread_records<double>(mbd_system *);

@@ -426,13 +426,15 @@ __global__ void k_morton_fill(unsigned mtotal, BinView B, const int *__restrict_
 
 // ---------------------------------------------------------------- clusters of the real-space field
 // Cluster c is the atoms order[16c .. 16c + 15] (consecutive in the Morton order
-// of the bricks, so close in space).  Its entries are the distinct neighbours
-// j of its atoms (over all images), in increasing j; its pairs are grouped by
-// the cluster atom il (pair starts per (c, il)) and, within an atom, ordered
-// by (j, image), each carrying the index of its entry and its pair tensor.
-// A block per cluster sorts the cluster's pairs in shared memory (bitonic,
-// keys (j, image, il), il in the low 4 bits); COUNT = true counts entries and pairs, COUNT = false
-// writes them at the scanned starts.
+// of the bricks, so close in space), in eight pairs of consecutive atoms
+// ("duos").  Its entries are the distinct neighbours j of its atoms (over all
+// images), in increasing j.  A duo's records (RealDuo) are its atoms' pairs in
+// the order (j, image): the k-th pair of each atom with the same j share a
+// record, which carries the index of the entry and both pair tensors (zero
+// where an atom has none).  A block per cluster sorts the cluster's pairs in
+// shared memory once (bitonic, keys (j, image, il), il in the low 4 bits);
+// entries and records go to regions sized by the pair counts (starts: the
+// scanned pair counts of the cluster atoms), with their own counts.
 __device__ __forceinline__ void bitonic_sort_smem(unsigned long long *key, int n) {
     for (int k = 2; k <= n; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
@@ -452,48 +454,49 @@ __device__ __forceinline__ void bitonic_sort_smem(unsigned long long *key, int n
     }
 }
 
-template <class T, bool COUNT>
-__global__ void __launch_bounds__(256) k_cluster_pairs(int N, int nclus, const int *__restrict__ order,
-                                                       const int *__restrict__ row, const int *__restrict__ col,
-                                                       const int *__restrict__ shift, const double *__restrict__ pos,
-                                                       const double *__restrict__ rvdw, Geom g, double beta,
-                                                       double r_cut, double damp_cut, double damp_beta, double damp_d,
-                                                       int *__restrict__ ecnt, int *__restrict__ pcnt,
-                                                       int *__restrict__ entries, RealPair<T> *__restrict__ pairs,
-                                                       int *__restrict__ err) {
-    extern __shared__ __align__(16) unsigned char cl_smem[];   // kClusterSortCap keys, entry indices, slots
+// Pairs of the cluster atoms in processing order (0 past the last atom).
+__global__ void k_cluster_slots(int N, int nslots, const int *__restrict__ order, const int *__restrict__ row,
+                                int *__restrict__ cnt) {
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= nslots) return;
+    const int i = idx < N ? order[idx] : -1;
+    cnt[idx] = i >= 0 ? row[i + 1] - row[i] : 0;
+}
+
+constexpr int kClusterThreads = 512;
+template <class T>
+__global__ void __launch_bounds__(kClusterThreads)
+    k_cluster_pairs(int N, const int *__restrict__ order, const int *__restrict__ row, const int *__restrict__ col,
+                    const int *__restrict__ shift, const double *__restrict__ pos, const double *__restrict__ rvdw,
+                    Geom g, double beta, double r_cut, double damp_cut, double damp_beta, double damp_d,
+                    const int *__restrict__ pstart, int *__restrict__ ecnt, int *__restrict__ rcnt,
+                    int *__restrict__ entries, RealDuo<T> *__restrict__ recs, int *__restrict__ err) {
+    constexpr int ND = kClusterSize / 2, NT = kClusterThreads, NC = kClusterSortCap / 32;
+    extern __shared__ __align__(16) unsigned char cl_smem[];   // kClusterSortCap keys and record slots
     unsigned long long *key = reinterpret_cast<unsigned long long *>(cl_smem);
-    int *eidx = reinterpret_cast<int *>(key + kClusterSortCap);
-    int *slot = eidx + kClusterSortCap;
-    __shared__ int at[kClusterSize], rb[kClusterSize + 1], ilstart[kClusterSize];
-    __shared__ int s_total;
-    const int c = blockIdx.x;
-    if (c >= nclus) return;
+    int *slot = reinterpret_cast<int *>(key + kClusterSortCap);
+    __shared__ int at[kClusterSize], rb[kClusterSize + 1];
+    __shared__ int base[NC][ND + 1];               // owners of each duo (and entries) before each 32 sorted pairs
+    const int c = blockIdx.x, lane = threadIdx.x & 31;
     if (threadIdx.x < kClusterSize) {
         const int idx = c * kClusterSize + threadIdx.x;
         at[threadIdx.x] = idx < N ? order[idx] : -1;
+        rb[threadIdx.x] = pstart[idx] - pstart[c * kClusterSize];
     }
+    if (threadIdx.x == 0) rb[kClusterSize] = pstart[(c + 1) * kClusterSize] - pstart[c * kClusterSize];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        rb[0] = 0;
-        for (int l = 0; l < kClusterSize; ++l) rb[l + 1] = rb[l] + (at[l] >= 0 ? row[at[l] + 1] - row[at[l]] : 0);
-        s_total = rb[kClusterSize];
-    }
-    __syncthreads();
-    const int total = s_total;
+    const int total = rb[kClusterSize];
     if (total > kClusterSortCap) {                 // the caller falls back to per-atom pairs
         if (threadIdx.x == 0) {
             atomicOr(err, 1);
-            if (COUNT) {
-                ecnt[c] = 0;
-                for (int l = 0; l < kClusterSize; ++l) pcnt[c * kClusterSize + l] = 0;
-            }
+            ecnt[c] = 0;
         }
+        if (threadIdx.x < ND) rcnt[c * ND + threadIdx.x] = 0;
         return;
     }
-    int n = 1;
+    int n = 32;
     while (n < total) n <<= 1;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    for (int k = threadIdx.x; k < n; k += NT) {
         unsigned long long kv = ~0ull;
         if (k < total) {
             int l = 0;
@@ -506,31 +509,74 @@ __global__ void __launch_bounds__(256) k_cluster_pairs(int N, int nclus, const i
     }
     __syncthreads();
     bitonic_sort_smem(key, n);
-    // entry index of every pair (a new entry at each new j) and its slot
-    // among the pairs of its atom (order of the sorted keys)
-    if (threadIdx.x == 0) {   // serial (at most kClusterSortCap pairs; setup only)
-        int ne = 0, cnt[kClusterSize];
-        for (int l = 0; l < kClusterSize; ++l) cnt[l] = 0;
-        for (int k = 0; k < total; ++k) {
-            if (k == 0 || (key[k] >> 28) != (key[k - 1] >> 28)) ++ne;
-            eidx[k] = ne - 1;
-            const int l = (int)(key[k] & 15ull);
-            slot[k] = cnt[l]++;
+    // the record of every sorted pair: the pair itself when its atom is the
+    // first of the duo or the first has no pair of this rank with j (the pair
+    // then "owns" the record), else the first atom's pair; rank: the pair's
+    // number among those of its atom with j
+    for (int k = threadIdx.x; k < n; k += NT) {
+        const unsigned long long kv = key[k];
+        const int il = (int)(kv & 15ull);
+        int own = k, first = 0;
+        if (k < total) {
+            int g0 = k;
+            while (g0 > 0 && (key[g0 - 1] >> 28) == (kv >> 28)) --g0;
+            first = g0 == k;
+            if (il & 1) {
+                int rank = 0;
+                for (int q = g0; q < k; ++q) rank += (int)(key[q] & 15ull) == il;
+                for (int q = g0; q < total && (key[q] >> 28) == (kv >> 28); ++q)
+                    if ((int)(key[q] & 15ull) == il - 1 && rank-- == 0) {
+                        own = q;
+                        break;
+                    }
+            }
         }
-        int acc = 0;
-        for (int l = 0; l < kClusterSize; ++l) {
-            ilstart[l] = acc;
-            acc += cnt[l];
-            if (COUNT) pcnt[c * kClusterSize + l] = cnt[l];
+        const bool owner = k < total && own == k;
+        for (int d = 0; d < ND; ++d) {
+            const unsigned m = __ballot_sync(0xffffffffu, owner && (il >> 1) == d);
+            if (lane == d) base[k >> 5][d] = __popc(m);
         }
-        if (COUNT) ecnt[c] = ne;
+        const unsigned m = __ballot_sync(0xffffffffu, first);
+        if (lane == ND) base[k >> 5][ND] = __popc(m);
+        slot[k] = own | (first << 16);             // own < 4096
     }
     __syncthreads();
-    if (COUNT) return;
-    const int e0 = ecnt[c], p0 = pcnt[c * kClusterSize];   // scanned starts
-    for (int k = threadIdx.x; k < total; k += blockDim.x) {
-        const int il = (int)(key[k] & 15ull), j = (int)(key[k] >> 28), sh = (int)((key[k] >> 4) & 0xffffff);
-        if (k == 0 || eidx[k] != eidx[k - 1]) entries[e0 + eidx[k]] = j;
+    if (threadIdx.x <= ND) {                       // running counts over the groups of 32 (128 at most)
+        int acc = 0;
+        for (int q = 0; q < n / 32; ++q) {
+            const int v = base[q][threadIdx.x];
+            base[q][threadIdx.x] = acc;
+            acc += v;
+        }
+        if (threadIdx.x < ND) rcnt[c * ND + threadIdx.x] = acc;
+        else ecnt[c] = acc;
+    }
+    __syncthreads();
+    // slot of each owner's record within its duo (bits 0..15 of the second half
+    // of the keys' scratch is not needed any more: kept beside own in slot's
+    // place through a second pass)
+    const int p0 = pstart[c * kClusterSize];
+    int *rslot = reinterpret_cast<int *>(slot + kClusterSortCap);   // [kClusterSortCap] record slot of owners
+    int *eidx = rslot + kClusterSortCap;                             // [kClusterSortCap] entry index
+    for (int k = threadIdx.x; k < n; k += NT) {
+        const int il = (int)(key[k] & 15ull), d = il >> 1;
+        const bool owner = k < total && (slot[k] & 0xffff) == k;
+        const unsigned below = (1u << lane) - 1u;
+        int before = 0;
+        for (int q = 0; q < ND; ++q) {
+            const unsigned m = __ballot_sync(0xffffffffu, owner && d == q);
+            if (d == q) before = __popc(m & below);
+        }
+        const unsigned me = __ballot_sync(0xffffffffu, k < total && (slot[k] >> 16));
+        rslot[k] = base[k >> 5][d] + before;
+        eidx[k] = base[k >> 5][ND] + __popc(me & (below | (1u << lane))) - 1;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < total; k += NT) {
+        const unsigned long long kv = key[k];
+        const int il = (int)(kv & 15ull), j = (int)(kv >> 28), sh = (int)((kv >> 4) & 0xffffff);
+        const int own = slot[k] & 0xffff;
+        if (slot[k] >> 16) entries[p0 + eidx[k]] = j;
         // the pair tensor of atom il and (j, image), FP64 from the positions
         const int i = at[il];
         const double n1 = double((sh & 255) - 128), n2 = double(((sh >> 8) & 255) - 128),
@@ -540,16 +586,31 @@ __global__ void __launch_bounds__(256) k_cluster_pairs(int N, int nclus, const i
         const double rz = pos[3 * i + 2] - pos[3 * j + 2] - (n1 * g.cell[2] + n2 * g.cell[5] + n3 * g.cell[8]);
         const PairRadial pr = pair_radial(rx * rx + ry * ry + rz * rz, rvdw[i] + rvdw[j], beta, r_cut, damp_cut,
                                           damp_beta, damp_d);
-        RealPair<T> rp;
-        rp.e = eidx[k];
-        rp.pad = 0;
-        rp.a[0] = T(pr.cid - pr.crr * rx * rx);
-        rp.a[1] = T(-pr.crr * rx * ry);
-        rp.a[2] = T(-pr.crr * rx * rz);
-        rp.a[3] = T(pr.cid - pr.crr * ry * ry);
-        rp.a[4] = T(-pr.crr * ry * rz);
-        rp.a[5] = T(pr.cid - pr.crr * rz * rz);
-        pairs[(size_t)p0 + ilstart[il] + slot[k]] = rp;
+        RealDuo<T> &r = recs[(size_t)p0 + rb[il & ~1] + rslot[own]];
+        T *h = r.a + 6 * (il & 1);
+        h[0] = T(pr.cid - pr.crr * rx * rx);
+        h[1] = T(-pr.crr * rx * ry);
+        h[2] = T(-pr.crr * rx * rz);
+        h[3] = T(pr.cid - pr.crr * ry * ry);
+        h[4] = T(-pr.crr * ry * rz);
+        h[5] = T(pr.cid - pr.crr * rz * rz);
+        if (own == k) {
+            // shared with the other atom of the duo?  Only a first atom's pair can be.
+            bool both = false;
+            if (!(il & 1))
+                for (int q = k + 1; q < total && (key[q] >> 28) == (kv >> 28) && !both; ++q)
+                    both = (slot[q] & 0xffff) == k;
+            // the second atom's pair of a shared record may come before it in the order of images
+            if (!(il & 1))
+                for (int q = k - 1; q >= 0 && (key[q] >> 28) == (kv >> 28) && !both; --q)
+                    both = (slot[q] & 0xffff) == k;
+            r.e = eidx[k];
+            r.mask = both ? 3 : 1 << (il & 1);
+            if (!both) {
+                T *o = r.a + 6 * ((il & 1) ^ 1);
+                for (int q = 0; q < 6; ++q) o[q] = T(0);
+            }
+        }
     }
 }
 }  // namespace
@@ -577,45 +638,37 @@ mbd_status launch_morton_order(const BinView &B, int N, int *order, DevBuf &cnt,
     return MBD_OK;
 }
 
-// The clusters of the real-space field (k_cluster_pairs): counts, scans of
-// the entry starts (per cluster) and pair starts (per cluster atom), then
-// entries and pairs.  err (device int) gets bit 1 when a cluster has more
-// than kClusterSortCap pairs.
-template <class T>
-mbd_status launch_cluster_pairs(mbd_system *s, const int *order, int nclus, DevBuf &ecnt, DevBuf &pcnt,
-                                DevBuf &estart, DevBuf &pstart, DevBuf &entries, DevBuf &A, int *err,
-                                cudaStream_t st) {
+// The clusters of the real-space field: the pair starts of the cluster atoms
+// (pstart), then entries and records with their counts (k_cluster_pairs).  err
+// (device int) gets bit 1 when a cluster has more than kClusterSortCap pairs.
+template <class T> mbd_status launch_cluster_pairs(mbd_system *s, cudaStream_t st) {
     const Geom g = make_geom(s);
-    const int nslots = nclus * kClusterSize;
-    MBD_TRY(ecnt.ensure(sizeof(int) * std::max(1, nclus)));
-    MBD_TRY(pcnt.ensure(sizeof(int) * std::max(1, nslots)));
-    MBD_TRY(estart.ensure(sizeof(int) * (nclus + 1)));
-    MBD_TRY(pstart.ensure(sizeof(int) * (nslots + 1)));
+    const int nclus = s->n_clusters, nslots = nclus * kClusterSize;
+    MBD_TRY(s->cl_ecnt.ensure(sizeof(int) * std::max(1, nclus)));
+    MBD_TRY(s->cl_rcnt.ensure(sizeof(int) * std::max(1, nslots / 2)));
+    MBD_TRY(s->cl_pcnt.ensure(sizeof(int) * std::max(1, nslots)));
+    MBD_TRY(s->cl_pstart.ensure(sizeof(int) * (nslots + 1)));
     const size_t cap = (size_t)std::max<long long>(1, s->nb_cap);
-    MBD_TRY(entries.ensure(sizeof(int) * cap));
-    MBD_TRY(A.ensure(sizeof(RealPair<T>) * cap));
+    DevBuf &recs = (sizeof(T) == 8 ? s->f64.cA : s->f32.cA);
+    MBD_TRY(s->cl_entries.ensure(sizeof(int) * cap));
+    MBD_TRY(recs.ensure(sizeof(RealDuo<T>) * cap));
     if (nclus == 0) return MBD_OK;
-    const size_t smem = (size_t)kClusterSortCap * (sizeof(unsigned long long) + 2 * sizeof(int));
-    MBD_CUDA_TRY(cudaFuncSetAttribute(k_cluster_pairs<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    MBD_CUDA_TRY(cudaFuncSetAttribute(k_cluster_pairs<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_cluster_pairs<T, true><<<nclus, 256, smem, st>>>(
-        s->N, nclus, order, s->row_d.as<int>(), s->col_d.as<int>(), s->shift_d.as<int>(), s->pos_d.as<double>(),
-        s->rvdw_d.as<double>(), g, s->ewald_beta, s->r_cut, s->damp_cut, s->damp_beta, s->damp_d, ecnt.as<int>(),
-        pcnt.as<int>(), nullptr, (RealPair<T> *)nullptr, err);
+    k_cluster_slots<<<(nslots + 255) / 256, 256, 0, st>>>(s->N, nslots, s->order_d.as<int>(), s->row_d.as<int>(),
+                                                          s->cl_pcnt.as<int>());
     MBD_LAUNCH_CHECK();
-    MBD_TRY(launch_exclusive_scan(ecnt.as<int>(), estart.as<int>(), nclus, s->scan_bsum, st));
-    MBD_TRY(launch_exclusive_scan(pcnt.as<int>(), pstart.as<int>(), nslots, s->scan_bsum, st));
-    k_cluster_pairs<T, false><<<nclus, 256, smem, st>>>(
-        s->N, nclus, order, s->row_d.as<int>(), s->col_d.as<int>(), s->shift_d.as<int>(), s->pos_d.as<double>(),
-        s->rvdw_d.as<double>(), g, s->ewald_beta, s->r_cut, s->damp_cut, s->damp_beta, s->damp_d,
-        estart.as<int>(), pstart.as<int>(), entries.as<int>(), A.template as<RealPair<T>>(), err);
+    MBD_TRY(launch_exclusive_scan(s->cl_pcnt.as<int>(), s->cl_pstart.as<int>(), nslots, s->scan_bsum, st));
+    const size_t smem = (size_t)kClusterSortCap * (sizeof(unsigned long long) + 3 * sizeof(int));
+    MBD_CUDA_TRY(cudaFuncSetAttribute(k_cluster_pairs<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_cluster_pairs<T><<<nclus, kClusterThreads, smem, st>>>(
+        s->N, s->order_d.as<int>(), s->row_d.as<int>(), s->col_d.as<int>(), s->shift_d.as<int>(),
+        s->pos_d.as<double>(), s->rvdw_d.as<double>(), g, s->ewald_beta, s->r_cut, s->damp_cut, s->damp_beta,
+        s->damp_d, s->cl_pstart.as<int>(), s->cl_ecnt.as<int>(), s->cl_rcnt.as<int>(), s->cl_entries.as<int>(),
+        recs.as<RealDuo<T>>(), s->cl_err.as<int>());
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }
-template mbd_status launch_cluster_pairs<double>(mbd_system *, const int *, int, DevBuf &, DevBuf &, DevBuf &,
-                                                 DevBuf &, DevBuf &, DevBuf &, int *, cudaStream_t);
-template mbd_status launch_cluster_pairs<float>(mbd_system *, const int *, int, DevBuf &, DevBuf &, DevBuf &,
-                                                DevBuf &, DevBuf &, DevBuf &, int *, cudaStream_t);
+template mbd_status launch_cluster_pairs<double>(mbd_system *, cudaStream_t);
+template mbd_status launch_cluster_pairs<float>(mbd_system *, cudaStream_t);
 
 mbd_status launch_bin_atoms(int N, const int *top, const BinView &B, int *bin_of, int *cnt, int *start,
                             int *cursor, int *atoms, DevBuf &bsum, cudaStream_t st) {

@@ -230,12 +230,13 @@ template <class T> struct __align__(16) PencilRec {
 // per-atom pair loop of the field kernel.
 constexpr int kClusterSize = 16;
 constexpr int kClusterSortCap = 4096;
-// One real-space pair of a cluster atom: the index of the neighbour entry
-// within the cluster and the pair tensor A (xx xy xz yy yz zz).
-template <class T> struct __align__(16) RealPair {
-    int e;
-    int pad;
-    T a[6];
+// One real-space record of two consecutive cluster atoms: the index of the
+// neighbour entry within the cluster, which of the two atoms have it (bits),
+// and their pair tensors A (xx xy xz yy yz zz of the first, then of the second).
+template <class T> struct __align__(16) RealDuo {
+    int e, mask;
+    int pad[2];
+    T a[12];
 };
 
 template <class T> struct PrecData {
@@ -244,10 +245,11 @@ template <class T> struct PrecData {
     DevBuf prow;        // [K^3 + 1] CSR over points (k1, k2, top3) of the pencil records
     DevBuf prec;        // [p^2 N] PencilRec<T>
     DevBuf k3w;         // [N][2p] M3(t3), M3'(t3)
+    DevBuf frec;        // [N] field records in processing order: atom, top, weights
     DevBuf w, dw, d2w;  // [N][3][p]
     DevBuf G;           // [K1K2K3] influence function
     DevBuf tw1, tw2, tw3;   // twiddles [K] complex per dimension
-    DevBuf cA;          // [nnz] RealPair<T>: per (cluster, atom), sorted by entry (real-space clusters)
+    DevBuf cA;          // [pair capacity] RealDuo<T>: per (cluster, two atoms), sorted by entry (real-space clusters)
     DevBuf ereal;       // [N][3][ld] real-space field of the current dipoles (cluster kernel output)
     DevBuf d;           // dipoles [N][3][ld]
     DevBuf mesh;        // [K1K2K3][ld]
@@ -302,9 +304,10 @@ struct mbd_system {
     mbd::DevBuf bin_start_d, bin_atoms_d, order_d;  // spread bins; field atom order
     mbd::DevBuf bin_of_d, bin_cursor_d;             // [N] brick of each atom, [nbins] fill cursors
     mbd::DevBuf morton_cnt, morton_start;           // Morton order of the bricks (setup scratch)
-    // real-space clusters: the distinct neighbours j of each cluster (CSR by
-    // cluster) and the pair starts per (cluster, atom) [8 nclus + 1]
-    mbd::DevBuf cl_ecnt, cl_pcnt, cl_estart, cl_pstart, cl_entries, cl_err;
+    // real-space clusters: pairs and pair starts of the cluster atoms [16 nclus (+ 1)],
+    // the distinct neighbours j of each cluster (from pstart[16 c], ecnt[c] of them) and
+    // the record counts of its eight pairs of atoms (records from pstart[16 c + 2 d])
+    mbd::DevBuf cl_pcnt, cl_pstart, cl_ecnt, cl_rcnt, cl_entries, cl_err;
     int n_clusters = 0;
     bool real_clusters = false;                     // the clusters of the last geometry were built
     int real_method = MBD_REAL_AUTO;                // mbd_set_real_space_method
@@ -343,10 +346,7 @@ mbd_status launch_exclusive_scan(const int *in, int *out, int n, DevBuf &bsum, c
 template <class T> mbd_status launch_pair_tensors(mbd_system *s, cudaStream_t st);
 mbd_status launch_morton_order(const BinView &B, int N, int *order, DevBuf &cnt, DevBuf &start, DevBuf &bsum,
                                cudaStream_t st);
-template <class T>
-mbd_status launch_cluster_pairs(mbd_system *s, const int *order, int nclus, DevBuf &ecnt, DevBuf &pcnt,
-                                DevBuf &estart, DevBuf &pstart, DevBuf &entries, DevBuf &A, int *err,
-                                cudaStream_t st);
+template <class T> mbd_status launch_cluster_pairs(mbd_system *s, cudaStream_t st);
 // whether this call's real-space field runs on the clusters (probe width ld)
 bool real_on_clusters(const mbd_system *s, int ld, int real_bytes);
 // E_real = sum over real-space pairs A d_j of the clusters (T [N][3][ld])
@@ -388,8 +388,6 @@ mbd_status launch_energy_reduce(const double *q, int R, int dim, double omega_su
 mbd_status launch_probes(uint64_t seed, int first, int R, int dim, double *v, cudaStream_t st);
 mbd_status launch_dense_step(const double *c, int dim, const LanczosView &lz, int k, int R, int ld, int nblk,
                              cudaStream_t st);
-int field_vec(int ld, int real_bytes);
-bool field_half(int ld, int real_bytes);
 int field_apb(const mbd_system *s, int ld);
 int field_blocks(const mbd_system *s, int ld);
 
