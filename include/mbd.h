@@ -279,11 +279,12 @@ mbd_status mbd_set_basis_storage(mbd_system *sys, int32_t mode);
  * MBD_REAL_PAIRS: inside the field kernel, each atom's neighbours split over
  *   the warps of a block (every neighbour's dipoles loaded once per pair).
  * MBD_REAL_CLUSTERS: a kernel of its own over clusters of 16 atoms that are
- *   consecutive in the Morton order of the mesh bricks: a warp loads each
- *   distinct neighbour (j, image) of the cluster once and applies it to every
- *   cluster atom that has it, then the field kernel adds the result.
- * MBD_REAL_AUTO (default): clusters when there are at least four per SM
- *   (and probe chunk of 64 FP32 or 32 FP64 probes), else pairs.
+ *   consecutive in the Morton order of the mesh bricks: the dipoles of each
+ *   distinct neighbour of the cluster are staged once, and a warp applies them
+ *   to two atoms at a time, then the field kernel adds the result.
+ * MBD_REAL_AUTO (default): clusters when atoms x (padded) probes are at least
+ *   160 x 1024 (MBD_MIXED), or when there are four clusters per SM and chunk of
+ *   32 probes (MBD_FP64), else pairs.
  * The two evaluations sum the same pairs in different orders (results agree
  * to rounding).  MBD_ERR_UNSUPPORTED for MBD_REAL_CLUSTERS when a cluster has
  * more than 4096 pairs (more than 256 neighbours per atom on average); the

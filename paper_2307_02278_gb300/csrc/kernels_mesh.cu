@@ -284,16 +284,16 @@ template <class T> struct RealArgs {
 // stages the dipoles of the cluster's distinct neighbours in shared memory, ce
 // entries at a time (cp.async, 16 bytes per lane), so each neighbour's dipoles
 // come from L2 once per cluster.  A warp walks the records of its two atoms in
-// entry order, in double-buffered batches of 16 (cp.async), and counts by a
+// entry order, in double-buffered batches of 32 (cp.async), and counts by a
 // ballot those whose entries are staged; np / VEC lanes hold the probes, and
 // the S groups of a warp take the records in turn.  A record applies one
 // neighbour's dipoles, read from shared memory once, to both atoms: close atoms
 // share three quarters of their neighbours, and the reads of shared memory and
 // the instructions beside the packed FMAs are what bound the kernel (100,002
 // atoms x 64 probes: 677 -> 559 us per launch; with 64 registers and four
-// blocks per SM it spills, 605 us; batches of 32 records 636 us).
+// blocks per SM it spills, 605 us).
 // An atom's field is a sum in a fixed order (per group, then the groups).
-constexpr int kRealBatch = 16;
+constexpr int kRealBatch = 32;
 constexpr int kRealStageBytes = 36 * 1024;
 template <class T>
 __global__ void __launch_bounds__(16 * kClusterSize, sizeof(T) == 4 ? 3 : 2) k_real_clusters(RealArgs<T> a) {
@@ -1153,21 +1153,21 @@ int field_blocks(const mbd_system *s, int ld) {
 }
 
 // Chunks of probes of the cluster kernel: at most 64 probes each (FP64: 32), and
-// down to 16 where fewer would leave less than four blocks per SM.
+// down to 16 where fewer would leave less than two blocks per SM.
 template <class T> int real_chunks(const mbd_system *s, int ld) {
     constexpr int most = 256 / (int)sizeof(T);
-    const int least = (ld + most - 1) / most, want = (4 * std::max(1, s->num_sms) + s->n_clusters - 1) /
+    const int least = (ld + most - 1) / most, want = (2 * std::max(1, s->num_sms) + s->n_clusters - 1) /
                                                      std::max(1, s->n_clusters);
     return std::max(least, std::min(want, ld / 16));
 }
 // The real-space field runs on the clusters when they were built and atoms x
 // probes are enough to fill the GPU with them; smaller systems keep the pair
 // loop of the field kernel, whose groups split the neighbours of one atom.
-// Measured per Lanczos step, pairs against clusters: 3000 atoms x 64 probes 222
-// and 230 us, x 128 440 and 429; 6000 x 32 260 and 261, x 64 466 and 443; 15,000
-// x 2 (padded to 4) 203 and 240.  FP64, bound by its arithmetic either way, takes
+// Measured per Lanczos step, pairs against clusters: 1200 atoms x 128 probes 188
+// and 195 us; 3000 x 32 122 and 131, x 64 224 and 210; 6000 x 16 156 and 157, x 32
+// 260 and 240; 15,000 x 2 (padded to 4) 203 and 240.  FP64, bound by its arithmetic either way, takes
 // them with four blocks per SM.
-constexpr long long kRealMinValues = 256 * 1024;
+constexpr long long kRealMinValues = 160 * 1024;
 bool real_on_clusters(const mbd_system *s, int ld, int real_bytes) {
     if (!s->real_clusters || s->real_method == MBD_REAL_PAIRS) return false;
     if (s->real_method == MBD_REAL_CLUSTERS) return true;

@@ -157,16 +157,24 @@ struct LanczosView {
 };
 __host__ __device__ inline size_t lz_slot(const LanczosView &lz, int k) { return (size_t)(k % lz.yslots); }
 
-// Deterministic two-level reduction across the blocks of a grid row
-// (blockIdx.y = probe chunk).  Each block contributes bval[t] for the probes
-// rbase + t (t < nloc); blocks are grouped by kRedGroup; the last block of a
-// group sums its group in block order, the last group finisher sums the groups
-// in group order.  Returns true (block-uniformly) in exactly one block, whose
-// out[t] then holds the grid totals.  Counters reset themselves.
+// Deterministic reduction across the blocks of a grid row (blockIdx.y = probe
+// chunk).  Each block contributes bval[t] for the probes rbase + t (t < nloc).
+// Small grids (at most kRedDirect values) take one level: the last block sums
+// all of them, its threads split into up to 16 slices of the blocks, the
+// slices in order.  Larger ones take two: blocks are grouped by kRedGroup; the
+// last block of a group sums its group in block order, the last group finisher
+// sums the groups in group order.  Returns true (block-uniformly) in exactly one
+// block, whose out[t] then holds the grid totals.  Counters reset themselves.
+// The second level's fence, counter and dependent FP64 additions cost about
+// 2 us per launch, a fifth of a small system's prologue.
 constexpr int kRedGroup = 16;
+constexpr unsigned kRedDirect = 4096;
+constexpr int kRedSlices = 16;
+constexpr int kRedThreads = 320;          // threads of the largest block that reduces
 __device__ __forceinline__ bool grid_reduce(const double *bval, int nloc, int rbase, int R, int ld,
                                             const LanczosView &lz, double *out) {
     __shared__ bool s_last;
+    __shared__ double s_slice[kRedThreads];
     const int t = threadIdx.x + threadIdx.y * blockDim.x;
     const int nthr = blockDim.x * blockDim.y;
     const unsigned nblk = gridDim.x;
@@ -176,6 +184,38 @@ __device__ __forceinline__ bool grid_reduce(const double *bval, int nloc, int rb
         if (rbase + k < R) lz.partial[(size_t)blockIdx.x * ld + rbase + k] = bval[k];
     __threadfence();
     __syncthreads();
+    if (nblk * (unsigned)nloc <= kRedDirect) {
+        if (t == 0) s_last = (atomicAdd(&cnt[ngroups], 1u) == nblk - 1);
+        __syncthreads();
+        if (!s_last) return false;
+        __threadfence();
+        const int slices = nloc >= nthr ? 1 : min(kRedSlices, nthr / nloc);
+        for (int k0 = 0; k0 < nloc; k0 += nthr / slices) {      // one pass unless nloc > nthr
+            const int k = k0 + t % (nthr / slices), sl = t / (nthr / slices);
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+            if (k < nloc && sl < slices && rbase + k < R) {
+                const double *p = lz.partial + rbase + k;
+                unsigned b = sl;
+                for (; b + 3 * slices < nblk; b += 4 * slices) {
+                    s0 += __ldcg(p + (size_t)b * ld);
+                    s1 += __ldcg(p + (size_t)(b + slices) * ld);
+                    s2 += __ldcg(p + (size_t)(b + 2 * slices) * ld);
+                    s3 += __ldcg(p + (size_t)(b + 3 * slices) * ld);
+                }
+                for (; b < nblk; b += slices) s0 += __ldcg(p + (size_t)b * ld);
+            }
+            s_slice[t] = (s0 + s1) + (s2 + s3);
+            __syncthreads();
+            if (sl == 0 && k < nloc) {
+                double s = 0.0;
+                for (int q = 0; q < slices; ++q) s += s_slice[q * (nthr / slices) + t];
+                out[k] = s;
+            }
+            __syncthreads();
+        }
+        if (t == 0) cnt[ngroups] = 0u;
+        return true;
+    }
     const unsigned g = blockIdx.x / kRedGroup;
     const unsigned gsize = min((unsigned)kRedGroup, nblk - g * kRedGroup);
     if (t == 0) s_last = (atomicAdd(&cnt[g], 1u) == gsize - 1);
