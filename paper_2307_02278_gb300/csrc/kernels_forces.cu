@@ -8,7 +8,9 @@
 // and grad_i = sum_k H_i(k) [p_i phi_q(k) + q_i phi_p(k)] with H_i the Hessian
 // of the stencil weight W_i(k) wrt R_i; the real-space part contracts the
 // derivative of the pair tensor, dA_ab/dr_c, with p_i q_j + p_j q_i.
-#include "mbd_internal.cuh"
+#include "fft.cuh"
+
+#include <algorithm>
 
 namespace mbd {
 
@@ -50,126 +52,156 @@ template <class T> struct ForceArgs {
     const T *mesh;       // [K^3][ld2] (phi_p, phi_q) interleaved
     int R, ld2;
     Geom g;
+    const int *order;    // atoms in the Morton order of the bricks
     const int *top;
     const T *w, *dw, *d2w;
     const int *row, *col;
     const T *dA;         // [nnz][18] dA_ab/dr_c of the real-space pair tensor
     double scale;
     double *forces;      // [N][3] FP64
+    int lanes;           // lanes that hold a chunk of 32 VEC values of a row (or all of it)
+    int wpa;             // warps per atom
 };
 
-// WPA warps per atom: they share out the stencil planes t1 and the
-// neighbours, and their partial gradients are summed in warp order.
-template <class T, int WPA>
-__global__ void __launch_bounds__(kWarps * 32) k_force_gather(ForceArgs<T> a) {
-    static_assert(kWarps % WPA == 0, "whole atoms per block");
+// One atom's force, wpa warps each: `lanes` lanes with 16-byte accesses hold the
+// probes' (p, q) values (chunks of 32 VEC of them, one after another), and the
+// groups of the atom's warps share out the p^2 pencils of its stencil and its
+// neighbours.  Along a pencil the Hessian of the weight factorises like the
+// weight: s_n = sum_t M3^(n)(t) phi, n = 0, 1, 2 (three FMAs per mesh value), and
+// six sums over the pencils, G_ab = sum H_ab phi, take two products of M1, M2 and
+// their derivatives times s_n each; the dipoles enter once per atom, h_a = sum_b
+// (G^q_ab e_p,b + G^p_ab e_q,b).  Partial gradients are summed in FP64 in a fixed
+// order (lanes, then warps).
+// Bound: load latency (FP32), the FP64 units (FP64).  100,002 atoms x 64 probes
+// 6.4 -> 3.1 ms per launch, 3000 x 64 258 -> 135 us, 501 x 7 FP64 391 -> 86 us, 64
+// x 16 FP64 124 -> 25 us against the Hessian per mesh value and a lane per probe.
+template <class T, int P>
+__global__ void __launch_bounds__(kWarps * 32, 2) k_force_gather(ForceArgs<T> a) {
+    constexpr int VEC = 16 / (int)sizeof(T);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = blockIdx.x * (kWarps / WPA) + warp / WPA, sub = warp % WPA;
-    const bool valid = i < a.g.N;
+    const int idx = blockIdx.x * (kWarps / a.wpa) + warp / a.wpa;
+    const int S = 32 / a.lanes, sub = lane / a.lanes, lid = lane - sub * a.lanes;
+    const int member = (warp % a.wpa) * S + sub, members = a.wpa * S;
+    const bool valid = idx < a.g.N;
     __shared__ double part[kWarps][3];
     double gx = 0.0, gy = 0.0, gz = 0.0;
-    if (valid) {
-    const int p = a.g.p;
-    const double *cm = a.g.cmat;
-    // ---- SPME: acc_beta = sum_k sum_l H_u(k)_{beta gamma} (e_p,gamma phi_q + e_q,gamma phi_p)
-    double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0;
-    {
+    const int i = valid ? a.order[idx] : 0;
+    if (valid && sub < S) {
+        const double *cm = a.g.cmat;
         const int top1 = a.top[3 * i], top2 = a.top[3 * i + 1], top3 = a.top[3 * i + 2];
-        const T *w = a.w + (size_t)3 * p * i, *dw = a.dw + (size_t)3 * p * i, *d2w = a.d2w + (size_t)3 * p * i;
-        for (int l = lane; l < a.R; l += 32) {
-            // scaled-fractional components e = C x of p_i and q_i
-            T pc[3], qc[3];
+        const T *w = a.w + (size_t)3 * P * i, *dw = a.dw + (size_t)3 * P * i, *d2w = a.d2w + (size_t)3 * P * i;
+        T w3[3][P];
+#pragma unroll
+        for (int t = 0; t < P; t += 2) {
+            vload<T, 2>(w + 2 * P + t, w3[0] + t);
+            vload<T, 2>(dw + 2 * P + t, w3[1] + t);
+            vload<T, 2>(d2w + 2 * P + t, w3[2] + t);
+        }
+        T g[3] = {T(0), T(0), T(0)};
+        double acc[3] = {0.0, 0.0, 0.0};
+        const int nb0 = a.row[i], nb1 = a.row[i + 1];
+        for (int c0 = 0; c0 < a.ld2; c0 += 32 * VEC) {
+            const int r0 = c0 + lid * VEC;
+            if (r0 >= a.ld2) break;
+            // the lane's own dipoles; values past the last probe are zero
+            T own[3][VEC];
+#pragma unroll
             for (int c = 0; c < 3; ++c) {
-                pc[c] = a.dpq[(size_t)(3 * i + c) * a.ld2 + 2 * l];
-                qc[c] = a.dpq[(size_t)(3 * i + c) * a.ld2 + 2 * l + 1];
+                vload<T, VEC>(a.dpq + (size_t)(3 * i + c) * a.ld2 + r0, own[c]);
+#pragma unroll
+                for (int v = 0; v < VEC; ++v)
+                    if (r0 + v >= 2 * a.R) own[c][v] = T(0);
             }
-            T ep[3], eq[3];
-            for (int b = 0; b < 3; ++b) {
-                ep[b] = T(cm[3 * b]) * pc[0] + T(cm[3 * b + 1]) * pc[1] + T(cm[3 * b + 2]) * pc[2];
-                eq[b] = T(cm[3 * b]) * qc[0] + T(cm[3 * b + 1]) * qc[1] + T(cm[3 * b + 2]) * qc[2];
-            }
-            T h0 = T(0), h1 = T(0), h2 = T(0);
-            for (int t1 = sub; t1 < p; t1 += WPA) {
-                int k1 = top1 - t1;
+            // ---- SPME: G_ab (00, 11, 22, 01, 02, 12) of this member's pencils
+            T G[6][VEC];
+#pragma unroll
+            for (int q = 0; q < 6; ++q)
+#pragma unroll
+                for (int v = 0; v < VEC; ++v) G[q][v] = T(0);
+            for (int u = member; u < P * P; u += members) {
+                const int t1 = u % P, t2 = u / P;
+                int k1 = top1 - t1, k2 = top2 - t2;
                 if (k1 < 0) k1 += a.g.K1;
-                const T wa = w[t1], da = dw[t1], ea = d2w[t1];
-                for (int t2 = 0; t2 < p; ++t2) {
-                    int k2 = top2 - t2;
-                    if (k2 < 0) k2 += a.g.K2;
-                    const T wb = w[p + t2], db = dw[p + t2], eb = d2w[p + t2];
-                    const size_t rowbase = ((size_t)k1 * a.g.K2 + k2) * a.g.K3;
-                    for (int t3 = 0; t3 < p; ++t3) {
-                        int k3 = top3 - t3;
-                        if (k3 < 0) k3 += a.g.K3;
-                        const T wc = w[2 * p + t3], dc = dw[2 * p + t3], ec = d2w[2 * p + t3];
-                        const size_t o = (rowbase + k3) * a.ld2 + 2 * l;
-                        const T fp = a.mesh[o], fq = a.mesh[o + 1];
-                        const T u0 = ep[0] * fq + eq[0] * fp;
-                        const T u1 = ep[1] * fq + eq[1] * fp;
-                        const T u2 = ep[2] * fq + eq[2] * fp;
-                        const T H00 = ea * wb * wc, H11 = wa * eb * wc, H22 = wa * wb * ec;
-                        const T H01 = da * db * wc, H02 = da * wb * dc, H12 = wa * db * dc;
-                        h0 += H00 * u0 + H01 * u1 + H02 * u2;
-                        h1 += H01 * u0 + H11 * u1 + H12 * u2;
-                        h2 += H02 * u0 + H12 * u1 + H22 * u2;
-                    }
+                if (k2 < 0) k2 += a.g.K2;
+                const T *rowp = a.mesh + ((size_t)k1 * a.g.K2 + k2) * a.g.K3 * a.ld2 + r0;
+                T phi[P][VEC], s[3][VEC];
+#pragma unroll
+                for (int t = 0; t < P; ++t)
+                    vload<T, VEC>(rowp + (size_t)(top3 - t + (top3 < t ? a.g.K3 : 0)) * a.ld2, phi[t]);
+                const T wa = w[t1], da = dw[t1], ea = d2w[t1], wb = w[P + t2], db = dw[P + t2], eb = d2w[P + t2];
+#pragma unroll
+                for (int n = 0; n < 3; ++n) {
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v) s[n][v] = T(0);
+#pragma unroll
+                    for (int t = 0; t < P; ++t) lane_fma<T, VEC>(phi[t], w3[n][t], s[n]);
                 }
+                lane_fma<T, VEC>(s[0], ea * wb, G[0]);
+                lane_fma<T, VEC>(s[0], wa * eb, G[1]);
+                lane_fma<T, VEC>(s[2], wa * wb, G[2]);
+                lane_fma<T, VEC>(s[0], da * db, G[3]);
+                lane_fma<T, VEC>(s[1], da * wb, G[4]);
+                lane_fma<T, VEC>(s[1], wa * db, G[5]);
             }
-            acc0 += double(h0);
-            acc1 += double(h1);
-            acc2 += double(h2);
-        }
-    }
-    // Cartesian: grad_alpha = sum_beta C_{beta alpha} acc_beta
-    gx = cm[0] * acc0 + cm[3] * acc1 + cm[6] * acc2;
-    gy = cm[1] * acc0 + cm[4] * acc1 + cm[7] * acc2;
-    gz = cm[2] * acc0 + cm[5] * acc1 + cm[8] * acc2;
-    // ---- real space: sum_j dA_ab/dr_c sum_l (p_ia q_jb + p_ja q_ib), dA precomputed per pair
-    {
-        T g0 = T(0), g1 = T(0), g2 = T(0);
-        for (int nb = a.row[i] + sub; nb < a.row[i + 1]; nb += WPA) {
-            const int j = a.col[nb];
-            T M[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-            for (int l = lane; l < a.R; l += 32) {
-                T pi_[3], qi_[3], pj_[3], qj_[3];
+            // scaled-fractional components e = C x of p_i and q_i, and h
+#pragma unroll
+            for (int v = 0; v < VEC; v += 2) {
+                T ep[3], eq[3];
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    ep[b] = T(cm[3 * b]) * own[0][v] + T(cm[3 * b + 1]) * own[1][v] + T(cm[3 * b + 2]) * own[2][v];
+                    eq[b] = T(cm[3 * b]) * own[0][v + 1] + T(cm[3 * b + 1]) * own[1][v + 1] +
+                            T(cm[3 * b + 2]) * own[2][v + 1];
+                }
+                auto h = [&](int x, int y, int z) {   // row of G against the other probe vector's components
+                    return G[x][v + 1] * ep[0] + G[x][v] * eq[0] + G[y][v + 1] * ep[1] + G[y][v] * eq[1] +
+                           G[z][v + 1] * ep[2] + G[z][v] * eq[2];
+                };
+                acc[0] += double(h(0, 3, 4));
+                acc[1] += double(h(3, 1, 5));
+                acc[2] += double(h(4, 5, 2));
+            }
+            // ---- real space: sum_j dA_ab/dr_c sum_l (p_ia q_jb + p_ja q_ib), dA precomputed per pair
+            for (int nb = nb0 + member; nb < nb1; nb += members) {
+                const int j = a.col[nb];
+                T o[3][VEC], M[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+#pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    pi_[c] = a.dpq[(size_t)(3 * i + c) * a.ld2 + 2 * l];
-                    qi_[c] = a.dpq[(size_t)(3 * i + c) * a.ld2 + 2 * l + 1];
-                    pj_[c] = a.dpq[(size_t)(3 * j + c) * a.ld2 + 2 * l];
-                    qj_[c] = a.dpq[(size_t)(3 * j + c) * a.ld2 + 2 * l + 1];
+                    vload<T, VEC>(a.dpq + (size_t)(3 * j + c) * a.ld2 + r0, o[c]);
+#pragma unroll
+                    for (int v = 0; v < VEC; ++v)
+                        if (r0 + v >= 2 * a.R) o[c][v] = T(0);
                 }
-                int o = 0;
-                for (int x = 0; x < 3; ++x)
-                    for (int y = x; y < 3; ++y) {
-                        T v = pi_[x] * qj_[y] + pj_[x] * qi_[y];
-                        if (x != y) v += pi_[y] * qj_[x] + pj_[y] * qi_[x];
-                        M[o++] += v;
-                    }
-            }
-            const T *dA = a.dA + 18 * (size_t)nb;
-            for (int ab = 0; ab < 6; ++ab) {
-                g0 += dA[3 * ab] * M[ab];
-                g1 += dA[3 * ab + 1] * M[ab];
-                g2 += dA[3 * ab + 2] * M[ab];
+                T dA[18];
+#pragma unroll
+                for (int q = 0; q < 18; q += 2) vload<T, 2>(a.dA + 18 * (size_t)nb + q, dA + q);
+#pragma unroll
+                for (int v = 0; v < VEC; v += 2) {
+                    int e = 0;
+#pragma unroll
+                    for (int x = 0; x < 3; ++x)
+#pragma unroll
+                        for (int y = x; y < 3; ++y) {
+                            T m = own[x][v] * o[y][v + 1] + o[x][v] * own[y][v + 1];
+                            if (x != y) m += own[y][v] * o[x][v + 1] + o[y][v] * own[x][v + 1];
+                            M[e++] += m;
+                        }
+                }
+#pragma unroll
+                for (int ab = 0; ab < 6; ++ab)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) g[c] += dA[3 * ab + c] * M[ab];
             }
         }
-        gx += double(g0);
-        gy += double(g1);
-        gz += double(g2);
-    }
+        // Cartesian: grad_alpha = sum_beta C_{beta alpha} acc_beta
+        gx = cm[0] * acc[0] + cm[3] * acc[1] + cm[6] * acc[2] + double(g[0]);
+        gy = cm[1] * acc[0] + cm[4] * acc[1] + cm[7] * acc[2] + double(g[1]);
+        gz = cm[2] * acc[0] + cm[5] * acc[1] + cm[8] * acc[2] + double(g[2]);
     }
     for (int off = 16; off > 0; off >>= 1) {
         gx += __shfl_down_sync(0xffffffffu, gx, off);
         gy += __shfl_down_sync(0xffffffffu, gy, off);
         gz += __shfl_down_sync(0xffffffffu, gz, off);
-    }
-    if (WPA == 1) {
-        if (valid && lane == 0) {
-            a.forces[3 * i] = -a.scale * gx;
-            a.forces[3 * i + 1] = -a.scale * gy;
-            a.forces[3 * i + 2] = -a.scale * gz;
-        }
-        return;
     }
     if (lane == 0) {
         part[warp][0] = gx;
@@ -177,9 +209,9 @@ __global__ void __launch_bounds__(kWarps * 32) k_force_gather(ForceArgs<T> a) {
         part[warp][2] = gz;
     }
     __syncthreads();
-    if (valid && sub == 0 && lane < 3) {
+    if (valid && warp % a.wpa == 0 && lane < 3) {
         double t = 0.0;
-        for (int w = 0; w < WPA; ++w) t += part[warp + w][lane];
+        for (int q = 0; q < a.wpa; ++q) t += part[warp + q][lane];
         a.forces[3 * i + lane] = -a.scale * t;
     }
 }
@@ -238,16 +270,21 @@ mbd_status launch_force_gather_t(mbd_system *s, const T *dpq, const T *mesh, int
     a.dA = P.pairdA.template as<T>();
     a.scale = scale;
     a.forces = forces;
+    constexpr int VEC = 16 / (int)sizeof(T);
+    a.order = s->order_d.as<int>();
+    a.lanes = std::min(32, ld2 / VEC);
     // warps per atom: more for small systems, whose one warp per atom would
-    // leave most of the SMs' warp slots empty (3000 atoms: 272 -> 234 us with 4;
-    // 24000 atoms: 2606 -> 2548 us with 2)
-    const int wpa = s->N <= 8192 ? 4 : (s->N <= 65536 ? 2 : 1);
-    if (wpa == 2)
-        k_force_gather<T, 2><<<(s->N + kWarps / 2 - 1) / (kWarps / 2), kWarps * 32, 0, s->stream>>>(a);
-    else if (wpa == 4)
-        k_force_gather<T, 4><<<(s->N + kWarps / 4 - 1) / (kWarps / 4), kWarps * 32, 0, s->stream>>>(a);
-    else
-        k_force_gather<T, 1><<<(s->N + kWarps - 1) / kWarps, kWarps * 32, 0, s->stream>>>(a);
+    // leave most of the SMs' warp slots empty
+    a.wpa = s->N <= 2048 ? 8 : (s->N <= 8192 ? 4 : (s->N <= 65536 ? 2 : 1));
+    const int per = kWarps / a.wpa;
+    const unsigned grid = (unsigned)((s->N + per - 1) / per);
+    switch (s->p) {
+#define MBD_FORCE_ORDER(P) \
+    case P: k_force_gather<T, P><<<grid, kWarps * 32, 0, s->stream>>>(a); break;
+        MBD_SPLINE_ORDERS(MBD_FORCE_ORDER)
+#undef MBD_FORCE_ORDER
+        default: return MBD_ERR_UNSUPPORTED;
+    }
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }
