@@ -219,62 +219,49 @@ mbd_status build_neighbors(mbd_system *s) {
         ng.kk[a] = (int)std::ceil(rmax * ng.nc[a] / width - 1e-12);
         if (ng.kk[a] > 120) return MBD_ERR_INVALID_ARG;
     }
-    // cell binning on the host (O(N)), the pair search on the device
     const int ncell = ng.nc[0] * ng.nc[1] * ng.nc[2];
-    std::vector<int> bin(N), cstart(ncell + 1, 0), catoms(N), cidx(3 * (size_t)N);
-    for (int i = 0; i < N; ++i) {
-        int b[3];
-        for (int a = 0; a < 3; ++a) {
-            double f = s->recip[3 * a] * s->pos[3 * i] + s->recip[3 * a + 1] * s->pos[3 * i + 1] +
-                       s->recip[3 * a + 2] * s->pos[3 * i + 2];
-            f -= std::floor(f);
-            b[a] = std::min(ng.nc[a] - 1, std::max(0, (int)std::floor(f * ng.nc[a])));
-            cidx[3 * i + a] = b[a];
-        }
-        bin[i] = (b[0] * ng.nc[1] + b[1]) * ng.nc[2] + b[2];
-        cstart[bin[i] + 1]++;
-    }
-    for (int c = 0; c < ncell; ++c) cstart[c + 1] += cstart[c];
-    {
-        std::vector<int> fill(cstart.begin(), cstart.end() - 1);
-        for (int i = 0; i < N; ++i) catoms[fill[bin[i]]++] = i;
-    }
     MBD_TRY(s->cell_start_d.ensure(sizeof(int) * (ncell + 1)));
-    MBD_TRY(s->cell_atoms_d.ensure(sizeof(int) * std::max(1, N)));
+    MBD_TRY(s->cell_atoms_d.ensure(sizeof(float4) * std::max(1, N)));
     MBD_TRY(s->cell_idx_d.ensure(sizeof(int) * 3 * std::max<size_t>(1, N)));
-    MBD_TRY(s->nb_err_d.ensure(sizeof(int)));
     MBD_TRY(s->row_d.ensure(sizeof(int) * (N + 1)));
-    MBD_CUDA_TRY(cudaMemcpyAsync(s->cell_start_d.ptr, cstart.data(), sizeof(int) * (ncell + 1),
-                                 cudaMemcpyHostToDevice, s->stream));
-    MBD_CUDA_TRY(cudaMemcpyAsync(s->cell_atoms_d.ptr, catoms.data(), sizeof(int) * N, cudaMemcpyHostToDevice,
-                                 s->stream));
-    MBD_CUDA_TRY(cudaMemcpyAsync(s->cell_idx_d.ptr, cidx.data(), sizeof(int) * 3 * N, cudaMemcpyHostToDevice,
-                                 s->stream));
-    MBD_CUDA_TRY(cudaMemsetAsync(s->nb_err_d.ptr, 0, sizeof(int), s->stream));
+    MBD_TRY(s->bin_of_d.ensure(sizeof(int) * std::max(1, N)));
+    MBD_TRY(s->bin_cursor_d.ensure(sizeof(int) * ncell));
+    MBD_TRY(s->bin_atoms_d.ensure(sizeof(int) * std::max(1, N)));
+    MBD_TRY(s->scan_cnt.ensure(sizeof(int) * std::max(std::max(1, N), ncell)));
     ng.start = s->cell_start_d.as<int>();
-    ng.atoms = s->cell_atoms_d.as<int>();
+    ng.atoms = s->cell_atoms_d.as<float4>();
     ng.cidx = s->cell_idx_d.as<int>();
-    for (int k = 0; k < 9; ++k) ng.cell[k] = s->cell[k];
+    // the FP32 distance test: coordinates and image shifts of at most `most`
+    // bohr are off by a few 2^-24 of it each, the distance by as much
+    double most = 0.0;
+    for (int k = 0; k < 9; ++k) {
+        ng.cell[k] = s->cell[k];
+        ng.cellf[k] = (float)s->cell[k];
+        ng.recip[k] = s->recip[k];
+        most += std::fabs(s->cell[k]) * (2.0 + ng.kk[k / 3] / (double)ng.nc[k / 3]);
+    }
     ng.r2max = rmax * rmax;
+    const double near = rmax * (1.0 + 1e-5) + 32.0 * std::ldexp(most, -24);
+    ng.r2near = (float)(near * near * (1.0 + 1e-6));
     s->ngrid = ng;
-    MBD_TRY(s->scan_cnt.ensure(sizeof(int) * std::max(1, N)));
-    MBD_TRY(launch_neighbors(ng, s->pos_d.as<double>(), s->scan_cnt.as<int>(), nullptr, nullptr,
-                             s->nb_err_d.as<int>(), false, 0, s->stream));
+    MBD_TRY(launch_cells(ng, s->pos_d.as<double>(), s->cell_idx_d.as<int>(), s->bin_of_d.as<int>(),
+                         s->scan_cnt.as<int>(), s->cell_start_d.as<int>(), s->bin_cursor_d.as<int>(),
+                         s->bin_atoms_d.as<int>(), s->cell_atoms_d.as<float4>(), s->scan_bsum, s->stream));
+    MBD_TRY(launch_neighbors(ng, s->pos_d.as<double>(), s->scan_cnt.as<int>(), nullptr, nullptr, false, 0,
+                             s->stream));
     MBD_TRY(launch_exclusive_scan(s->scan_cnt.as<int>(), s->row_d.as<int>(), N, s->scan_bsum, s->stream));
     if (s->nb_cap == 0) {
         // first build: the list is sized from its count (with room to grow)
-        int head[2] = {0, 0};
-        MBD_CUDA_TRY(cudaMemcpyAsync(&head[0], s->row_d.as<int>() + N, sizeof(int), cudaMemcpyDeviceToHost,
-                                     s->stream));
-        MBD_CUDA_TRY(cudaMemcpyAsync(&head[1], s->nb_err_d.ptr, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+        int head = 0;
+        MBD_CUDA_TRY(cudaMemcpyAsync(&head, s->row_d.as<int>() + N, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
         MBD_CUDA_TRY(cudaStreamSynchronize(s->stream));
-        if (head[0] < 0 || head[1] != 0) return MBD_ERR_INVALID_ARG;
-        MBD_TRY(size_pair_buffers(s, head[0]));
+        if (head < 0) return MBD_ERR_INVALID_ARG;
+        MBD_TRY(size_pair_buffers(s, head));
     }
     // later builds keep the buffers and find out at the end whether the list
     // still fits them (setup_geometry)
     return launch_neighbors(ng, s->pos_d.as<double>(), s->row_d.as<int>(), s->col_d.as<int>(),
-                            s->shift_d.as<int>(), s->nb_err_d.as<int>(), true, s->nb_cap, s->stream);
+                            s->shift_d.as<int>(), true, s->nb_cap, s->stream);
 }
 
 // Bricks of the mesh for deterministic spreading; atoms are binned by the
@@ -387,17 +374,15 @@ template <class T> mbd_status setup_geometry(mbd_system *s) {
     MBD_TRY(launch_splines<T>(s, s->stream));
     MBD_TRY(build_bins(s));
     MBD_TRY(build_spread_records<T>(s));
-    int head[2] = {0, 0};
-    MBD_CUDA_TRY(cudaMemcpyAsync(&head[0], s->row_d.as<int>() + s->N, sizeof(int), cudaMemcpyDeviceToHost,
-                                 s->stream));
-    MBD_CUDA_TRY(cudaMemcpyAsync(&head[1], s->nb_err_d.ptr, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+    int head = 0;
+    MBD_CUDA_TRY(cudaMemcpyAsync(&head, s->row_d.as<int>() + s->N, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
     MBD_CUDA_TRY(cudaStreamSynchronize(s->stream));
-    if (head[0] < 0 || head[1] != 0) return MBD_ERR_INVALID_ARG;
-    s->nnz = head[0];
+    if (head < 0) return MBD_ERR_INVALID_ARG;
+    s->nnz = head;
     if (s->nnz > s->nb_cap) {
         MBD_TRY(size_pair_buffers(s, s->nnz));
         MBD_TRY(launch_neighbors(s->ngrid, s->pos_d.as<double>(), s->row_d.as<int>(), s->col_d.as<int>(),
-                                 s->shift_d.as<int>(), s->nb_err_d.as<int>(), true, s->nb_cap, s->stream));
+                                 s->shift_d.as<int>(), true, s->nb_cap, s->stream));
         MBD_TRY(launch_pair_tensors<T>(s, s->stream));
     }
     // the clusters of the real-space field, from the final neighbour list

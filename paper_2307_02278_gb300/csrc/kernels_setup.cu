@@ -220,23 +220,92 @@ Geom make_geom(const mbd_system *s) {
     return g;
 }
 
-// Real-space neighbour list over a cell grid (cells of width >= rmax along
-// each reciprocal direction, kk cells searched each way).  A warp per atom i
-// visits the cells c = cidx(i) + o, o in [-kk, kk]^3, with their lattice
-// image n; the lanes take the atoms of each cell 32 at a time, and a ballot
-// keeps the hits in cell order, then atom order.  FILL = false counts, FILL =
-// true writes (j, packed n) for the pairs below cap.  The order is fixed, so
-// the list is the same on every run.  err bit 1: an image index beyond +-127.
+// Cell of each atom (cells of width >= rmax along each reciprocal direction)
+// and the atoms per cell.
+__global__ void k_cell_count(NeighborGrid ng, const double *__restrict__ pos, int *__restrict__ cidx,
+                             int *__restrict__ bin_of, int *__restrict__ cnt) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= ng.N) return;
+    int b[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        double f = ng.recip[3 * a] * pos[3 * i] + ng.recip[3 * a + 1] * pos[3 * i + 1] +
+                   ng.recip[3 * a + 2] * pos[3 * i + 2];
+        f -= floor(f);
+        b[a] = min(ng.nc[a] - 1, max(0, (int)floor(f * ng.nc[a])));
+        cidx[3 * i + a] = b[a];
+    }
+    const int c = (b[0] * ng.nc[1] + b[1]) * ng.nc[2] + b[2];
+    bin_of[i] = c;
+    atomicAdd(&cnt[c], 1);
+}
+// The atoms of each cell in increasing index, whatever the order they arrived
+// in (a warp per cell ranks them), with their positions in FP32.
+__global__ void k_cell_sort(int ncell, const int *__restrict__ start, const int *__restrict__ tmp,
+                            const double *__restrict__ pos, float4 *__restrict__ out) {
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (c >= ncell) return;
+    const int q0 = start[c], n = start[c + 1] - q0;
+    for (int a = lane; a < n; a += 32) {
+        const int v = tmp[q0 + a];
+        int rank = 0;
+        for (int b = 0; b < n; ++b) rank += tmp[q0 + b] < v;
+        out[q0 + rank] = make_float4(float(pos[3 * v]), float(pos[3 * v + 1]), float(pos[3 * v + 2]),
+                                     __int_as_float(v));
+    }
+}
+
+// Real-space neighbour list over the cell grid (kk cells searched each way).  A
+// warp per atom i visits the cells c = cidx(i) + o, o in [-kk, kk]^3, with their
+// lattice image n; the lanes take the atoms of each cell 32 at a time.  Those
+// within the cutoff by their FP32 distance, with room for its rounding, queue up
+// in shared memory; 32 at a time they take the FP64 test, and a ballot keeps the
+// hits in cell order, then atom order.  FILL = false counts, FILL = true writes
+// (j, packed n) for the pairs below cap.  The order is fixed, so the list is the
+// same on every run.  An image index fits its byte: kk <= 120.
+// Bound: the FP64 units, which see one candidate in seven (12,000 atoms: 478
+// -> 100 us per pass).
 template <bool FILL>
 __global__ void __launch_bounds__(128) k_neighbors(NeighborGrid ng, const double *__restrict__ pos,
                                                    int *__restrict__ cnt_or_row, int *__restrict__ col,
-                                                   int *__restrict__ shift, int *__restrict__ err, long long cap) {
-    const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
+                                                   int *__restrict__ shift, long long cap) {
+    __shared__ int2 queue[4][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = blockIdx.x * 4 + warp;
     if (i >= ng.N) return;
     const double px = pos[3 * i], py = pos[3 * i + 1], pz = pos[3 * i + 2];
-    int c = 0;
+    const float fx = float(px), fy = float(py), fz = float(pz);
+    int2 *mine = queue[warp];
+    int c = 0, qn = 0;
     const int base = FILL ? cnt_or_row[i] : 0;
+    auto test = [&](int m) {                       // the first m of the queue
+        __syncwarp();
+        bool hit = false;
+        int2 e = make_int2(0, 0);
+        if (lane < m) {
+            e = mine[lane];
+            const double n0 = double((e.y & 255) - 128), n1 = double(((e.y >> 8) & 255) - 128),
+                         n2 = double(((e.y >> 16) & 255) - 128);
+            const double rx = px - pos[3 * e.x] - (n0 * ng.cell[0] + n1 * ng.cell[3] + n2 * ng.cell[6]);
+            const double ry = py - pos[3 * e.x + 1] - (n0 * ng.cell[1] + n1 * ng.cell[4] + n2 * ng.cell[7]);
+            const double rz = pz - pos[3 * e.x + 2] - (n0 * ng.cell[2] + n1 * ng.cell[5] + n2 * ng.cell[8]);
+            const double r2 = rx * rx + ry * ry + rz * rz;
+            hit = r2 < ng.r2max && r2 > 0.0;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, hit);
+        if (FILL && hit) {
+            const int at = base + c + __popc(bal & ((1u << lane) - 1u));
+            if (at < cap) {
+                col[at] = e.x;
+                shift[at] = e.y;
+            }
+        }
+        c += __popc(bal);
+        const int2 rest = lane < qn - m ? mine[m + lane] : make_int2(0, 0);
+        __syncwarp();
+        if (lane < qn - m) mine[lane] = rest;
+        qn -= m;
+    };
     for (int o0 = -ng.kk[0]; o0 <= ng.kk[0]; ++o0) {
         const int t0 = ng.cidx[3 * i] + o0;
         const int n0 = t0 >= 0 ? t0 / ng.nc[0] : -((-t0 + ng.nc[0] - 1) / ng.nc[0]);
@@ -250,36 +319,29 @@ __global__ void __launch_bounds__(128) k_neighbors(NeighborGrid ng, const double
                 const int n2 = t2 >= 0 ? t2 / ng.nc[2] : -((-t2 + ng.nc[2] - 1) / ng.nc[2]);
                 const int b2 = t2 - n2 * ng.nc[2];
                 const int cell = (b0 * ng.nc[1] + b1) * ng.nc[2] + b2;
-                const double sx = n0 * ng.cell[0] + n1 * ng.cell[3] + n2 * ng.cell[6];
-                const double sy = n0 * ng.cell[1] + n1 * ng.cell[4] + n2 * ng.cell[7];
-                const double sz = n0 * ng.cell[2] + n1 * ng.cell[5] + n2 * ng.cell[8];
-                const bool far = abs(n0) > 127 || abs(n1) > 127 || abs(n2) > 127;
-                const int q0 = ng.start[cell], q1 = ng.start[cell + 1];
-                for (int qb = q0; qb < q1; qb += 32) {
+                const float sx = n0 * ng.cellf[0] + n1 * ng.cellf[3] + n2 * ng.cellf[6];
+                const float sy = n0 * ng.cellf[1] + n1 * ng.cellf[4] + n2 * ng.cellf[7];
+                const float sz = n0 * ng.cellf[2] + n1 * ng.cellf[5] + n2 * ng.cellf[8];
+                const int packed = (n0 + 128) | ((n1 + 128) << 8) | ((n2 + 128) << 16);
+                const int q1 = ng.start[cell + 1];
+                for (int qb = ng.start[cell]; qb < q1; qb += 32) {
                     const int q = qb + lane;
-                    bool hit = false;
-                    int j = 0;
+                    bool near = false;
+                    float4 at = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (q < q1) {
-                        j = ng.atoms[q];
-                        const double rx = px - pos[3 * j] - sx, ry = py - pos[3 * j + 1] - sy,
-                                     rz = pz - pos[3 * j + 2] - sz;
-                        const double r2 = rx * rx + ry * ry + rz * rz;
-                        hit = r2 < ng.r2max && r2 > 0.0;
+                        at = ng.atoms[q];
+                        const float rx = fx - at.x - sx, ry = fy - at.y - sy, rz = fz - at.z - sz;
+                        near = !(rx * rx + ry * ry + rz * rz > ng.r2near);   // not finite: to the exact test
                     }
-                    const unsigned bal = __ballot_sync(0xffffffffu, hit);
-                    if (hit && far && !FILL) atomicOr(err, 1);
-                    if (FILL && hit && !far) {
-                        const int at = base + c + __popc(bal & ((1u << lane) - 1u));
-                        if (at < cap) {
-                            col[at] = j;
-                            shift[at] = (n0 + 128) | ((n1 + 128) << 8) | ((n2 + 128) << 16);
-                        }
-                    }
-                    c += __popc(bal);
+                    const unsigned bal = __ballot_sync(0xffffffffu, near);
+                    if (near) mine[qn + __popc(bal & ((1u << lane) - 1u))] = make_int2(__float_as_int(at.w), packed);
+                    qn += __popc(bal);
+                    if (qn >= 32) test(32);
                 }
             }
         }
     }
+    while (qn > 0) test(min(qn, 32));
     if (!FILL && lane == 0) cnt_or_row[i] = c;
 }
 
@@ -341,13 +403,13 @@ template <class T> mbd_status launch_influence(mbd_system *s, const double *bmod
 }
 
 mbd_status launch_neighbors(const NeighborGrid &ng, const double *pos, int *cnt_or_row, int *col, int *shift,
-                            int *err, bool fill, long long cap, cudaStream_t st) {
+                            bool fill, long long cap, cudaStream_t st) {
     const unsigned blocks = (unsigned)((ng.N + 3) / 4);   // a warp per atom
     if (ng.N == 0) return MBD_OK;
     if (fill)
-        k_neighbors<true><<<blocks, 128, 0, st>>>(ng, pos, cnt_or_row, col, shift, err, cap);
+        k_neighbors<true><<<blocks, 128, 0, st>>>(ng, pos, cnt_or_row, col, shift, cap);
     else
-        k_neighbors<false><<<blocks, 128, 0, st>>>(ng, pos, cnt_or_row, col, shift, err, cap);
+        k_neighbors<false><<<blocks, 128, 0, st>>>(ng, pos, cnt_or_row, col, shift, cap);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }
@@ -432,7 +494,8 @@ __global__ void k_morton_fill(unsigned mtotal, BinView B, const int *__restrict_
 // the order (j, image): the k-th pair of each atom with the same j share a
 // record, which carries the index of the entry and both pair tensors (zero
 // where an atom has none).  A block per cluster sorts the cluster's pairs in
-// shared memory once (bitonic, keys (j, image, il), il in the low 4 bits);
+// shared memory once (bitonic, keys (j, image, pair), the pair's number within the
+// cluster in the low 12 bits, so its atom and its tensor are at hand);
 // entries and records go to regions sized by the pair counts (starts: the
 // scanned pair counts of the cluster atoms), with their own counts.
 __device__ __forceinline__ void bitonic_sort_smem(unsigned long long *key, int n) {
@@ -467,14 +530,13 @@ constexpr int kClusterThreads = 512;
 template <class T>
 __global__ void __launch_bounds__(kClusterThreads)
     k_cluster_pairs(int N, const int *__restrict__ order, const int *__restrict__ row, const int *__restrict__ col,
-                    const int *__restrict__ shift, const double *__restrict__ pos, const double *__restrict__ rvdw,
-                    Geom g, double beta, double r_cut, double damp_cut, double damp_beta, double damp_d,
-                    const int *__restrict__ pstart, int *__restrict__ ecnt, int *__restrict__ rcnt,
+                    const int *__restrict__ shift, const T *__restrict__ pairA, const int *__restrict__ pstart, int *__restrict__ ecnt, int *__restrict__ rcnt,
                     int *__restrict__ entries, RealDuo<T> *__restrict__ recs, int *__restrict__ err) {
     constexpr int ND = kClusterSize / 2, NT = kClusterThreads, NC = kClusterSortCap / 32;
-    extern __shared__ __align__(16) unsigned char cl_smem[];   // kClusterSortCap keys and record slots
+    extern __shared__ __align__(16) unsigned char cl_smem[];   // kClusterSortCap each: keys, three words, atoms
     unsigned long long *key = reinterpret_cast<unsigned long long *>(cl_smem);
     int *slot = reinterpret_cast<int *>(key + kClusterSortCap);
+    unsigned char *ilof = reinterpret_cast<unsigned char *>(slot + 3 * kClusterSortCap);   // cluster atom of a pair
     __shared__ int at[kClusterSize], rb[kClusterSize + 1];
     __shared__ int base[NC][ND + 1];               // owners of each duo (and entries) before each 32 sorted pairs
     const int c = blockIdx.x, lane = threadIdx.x & 31;
@@ -501,9 +563,10 @@ __global__ void __launch_bounds__(kClusterThreads)
         if (k < total) {
             int l = 0;
             while (rb[l + 1] <= k) ++l;
+            ilof[k] = (unsigned char)l;
             const int q = row[at[l]] + (k - rb[l]);
-            kv = ((unsigned long long)col[q] << 28) | ((unsigned long long)(shift[q] & 0xffffff) << 4) |
-                 (unsigned long long)l;
+            kv = ((unsigned long long)col[q] << 36) | ((unsigned long long)(shift[q] & 0xffffff) << 12) |
+                 (unsigned long long)k;
         }
         key[k] = kv;
     }
@@ -515,17 +578,17 @@ __global__ void __launch_bounds__(kClusterThreads)
     // number among those of its atom with j
     for (int k = threadIdx.x; k < n; k += NT) {
         const unsigned long long kv = key[k];
-        const int il = (int)(kv & 15ull);
+        const int il = k < total ? ilof[kv & 4095ull] : 0;
         int own = k, first = 0;
         if (k < total) {
             int g0 = k;
-            while (g0 > 0 && (key[g0 - 1] >> 28) == (kv >> 28)) --g0;
+            while (g0 > 0 && (key[g0 - 1] >> 36) == (kv >> 36)) --g0;
             first = g0 == k;
             if (il & 1) {
                 int rank = 0;
-                for (int q = g0; q < k; ++q) rank += (int)(key[q] & 15ull) == il;
-                for (int q = g0; q < total && (key[q] >> 28) == (kv >> 28); ++q)
-                    if ((int)(key[q] & 15ull) == il - 1 && rank-- == 0) {
+                for (int q = g0; q < k; ++q) rank += ilof[key[q] & 4095ull] == il;
+                for (int q = g0; q < total && (key[q] >> 36) == (kv >> 36); ++q)
+                    if (ilof[key[q] & 4095ull] == il - 1 && rank-- == 0) {
                         own = q;
                         break;
                     }
@@ -552,14 +615,12 @@ __global__ void __launch_bounds__(kClusterThreads)
         else ecnt[c] = acc;
     }
     __syncthreads();
-    // slot of each owner's record within its duo (bits 0..15 of the second half
-    // of the keys' scratch is not needed any more: kept beside own in slot's
-    // place through a second pass)
+    // slot of each owner's record within its duo, and every pair's entry
     const int p0 = pstart[c * kClusterSize];
     int *rslot = reinterpret_cast<int *>(slot + kClusterSortCap);   // [kClusterSortCap] record slot of owners
     int *eidx = rslot + kClusterSortCap;                             // [kClusterSortCap] entry index
     for (int k = threadIdx.x; k < n; k += NT) {
-        const int il = (int)(key[k] & 15ull), d = il >> 1;
+        const int il = k < total ? ilof[key[k] & 4095ull] : 0, d = il >> 1;
         const bool owner = k < total && (slot[k] & 0xffff) == k;
         const unsigned below = (1u << lane) - 1u;
         int before = 0;
@@ -574,35 +635,23 @@ __global__ void __launch_bounds__(kClusterThreads)
     __syncthreads();
     for (int k = threadIdx.x; k < total; k += NT) {
         const unsigned long long kv = key[k];
-        const int il = (int)(kv & 15ull), j = (int)(kv >> 28), sh = (int)((kv >> 4) & 0xffffff);
+        const int pk = (int)(kv & 4095ull), il = ilof[pk], j = (int)(kv >> 36);
         const int own = slot[k] & 0xffff;
         if (slot[k] >> 16) entries[p0 + eidx[k]] = j;
-        // the pair tensor of atom il and (j, image), FP64 from the positions
-        const int i = at[il];
-        const double n1 = double((sh & 255) - 128), n2 = double(((sh >> 8) & 255) - 128),
-                     n3 = double(((sh >> 16) & 255) - 128);
-        const double rx = pos[3 * i] - pos[3 * j] - (n1 * g.cell[0] + n2 * g.cell[3] + n3 * g.cell[6]);
-        const double ry = pos[3 * i + 1] - pos[3 * j + 1] - (n1 * g.cell[1] + n2 * g.cell[4] + n3 * g.cell[7]);
-        const double rz = pos[3 * i + 2] - pos[3 * j + 2] - (n1 * g.cell[2] + n2 * g.cell[5] + n3 * g.cell[8]);
-        const PairRadial pr = pair_radial(rx * rx + ry * ry + rz * rz, rvdw[i] + rvdw[j], beta, r_cut, damp_cut,
-                                          damp_beta, damp_d);
         RealDuo<T> &r = recs[(size_t)p0 + rb[il & ~1] + rslot[own]];
+        const T *src = pairA + 6 * ((size_t)row[at[il]] + (pk - rb[il]));
         T *h = r.a + 6 * (il & 1);
-        h[0] = T(pr.cid - pr.crr * rx * rx);
-        h[1] = T(-pr.crr * rx * ry);
-        h[2] = T(-pr.crr * rx * rz);
-        h[3] = T(pr.cid - pr.crr * ry * ry);
-        h[4] = T(-pr.crr * ry * rz);
-        h[5] = T(pr.cid - pr.crr * rz * rz);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) h[q] = src[q];
         if (own == k) {
             // shared with the other atom of the duo?  Only a first atom's pair can be.
             bool both = false;
             if (!(il & 1))
-                for (int q = k + 1; q < total && (key[q] >> 28) == (kv >> 28) && !both; ++q)
+                for (int q = k + 1; q < total && (key[q] >> 36) == (kv >> 36) && !both; ++q)
                     both = (slot[q] & 0xffff) == k;
             // the second atom's pair of a shared record may come before it in the order of images
             if (!(il & 1))
-                for (int q = k - 1; q >= 0 && (key[q] >> 28) == (kv >> 28) && !both; --q)
+                for (int q = k - 1; q >= 0 && (key[q] >> 36) == (kv >> 36) && !both; --q)
                     both = (slot[q] & 0xffff) == k;
             r.e = eidx[k];
             r.mask = both ? 3 : 1 << (il & 1);
@@ -642,14 +691,14 @@ mbd_status launch_morton_order(const BinView &B, int N, int *order, DevBuf &cnt,
 // (pstart), then entries and records with their counts (k_cluster_pairs).  err
 // (device int) gets bit 1 when a cluster has more than kClusterSortCap pairs.
 template <class T> mbd_status launch_cluster_pairs(mbd_system *s, cudaStream_t st) {
-    const Geom g = make_geom(s);
     const int nclus = s->n_clusters, nslots = nclus * kClusterSize;
+    PrecData<T> &P = prec<T>(s);
     MBD_TRY(s->cl_ecnt.ensure(sizeof(int) * std::max(1, nclus)));
     MBD_TRY(s->cl_rcnt.ensure(sizeof(int) * std::max(1, nslots / 2)));
     MBD_TRY(s->cl_pcnt.ensure(sizeof(int) * std::max(1, nslots)));
     MBD_TRY(s->cl_pstart.ensure(sizeof(int) * (nslots + 1)));
     const size_t cap = (size_t)std::max<long long>(1, s->nb_cap);
-    DevBuf &recs = (sizeof(T) == 8 ? s->f64.cA : s->f32.cA);
+    DevBuf &recs = P.cA;
     MBD_TRY(s->cl_entries.ensure(sizeof(int) * cap));
     MBD_TRY(recs.ensure(sizeof(RealDuo<T>) * cap));
     if (nclus == 0) return MBD_OK;
@@ -657,12 +706,11 @@ template <class T> mbd_status launch_cluster_pairs(mbd_system *s, cudaStream_t s
                                                           s->cl_pcnt.as<int>());
     MBD_LAUNCH_CHECK();
     MBD_TRY(launch_exclusive_scan(s->cl_pcnt.as<int>(), s->cl_pstart.as<int>(), nslots, s->scan_bsum, st));
-    const size_t smem = (size_t)kClusterSortCap * (sizeof(unsigned long long) + 3 * sizeof(int));
+    const size_t smem = (size_t)kClusterSortCap * (sizeof(unsigned long long) + 3 * sizeof(int) + 1);
     MBD_CUDA_TRY(cudaFuncSetAttribute(k_cluster_pairs<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_cluster_pairs<T><<<nclus, kClusterThreads, smem, st>>>(
         s->N, s->order_d.as<int>(), s->row_d.as<int>(), s->col_d.as<int>(), s->shift_d.as<int>(),
-        s->pos_d.as<double>(), s->rvdw_d.as<double>(), g, s->ewald_beta, s->r_cut, s->damp_cut, s->damp_beta,
-        s->damp_d, s->cl_pstart.as<int>(), s->cl_ecnt.as<int>(), s->cl_rcnt.as<int>(), s->cl_entries.as<int>(),
+        P.pairA.template as<T>(), s->cl_pstart.as<int>(), s->cl_ecnt.as<int>(), s->cl_rcnt.as<int>(), s->cl_entries.as<int>(),
         recs.as<RealDuo<T>>(), s->cl_err.as<int>());
     MBD_LAUNCH_CHECK();
     return MBD_OK;
@@ -684,6 +732,25 @@ mbd_status launch_bin_atoms(int N, const int *top, const BinView &B, int *bin_of
         k_bin_fill<<<(N + 255) / 256, 256, 0, st>>>(N, bin_of, cursor, atoms);
         MBD_LAUNCH_CHECK();
         k_bin_sort<<<(nbins + 255) / 256, 256, 0, st>>>(nbins, start, atoms);
+        MBD_LAUNCH_CHECK();
+    }
+    return MBD_OK;
+}
+
+mbd_status launch_cells(const NeighborGrid &ng, const double *pos, int *cidx, int *bin_of, int *cnt, int *start,
+                        int *cursor, int *tmp, float4 *atoms, DevBuf &bsum, cudaStream_t st) {
+    const int ncell = ng.nc[0] * ng.nc[1] * ng.nc[2];
+    MBD_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int) * ncell, st));
+    if (ng.N > 0) {
+        k_cell_count<<<(ng.N + 255) / 256, 256, 0, st>>>(ng, pos, cidx, bin_of, cnt);
+        MBD_LAUNCH_CHECK();
+    }
+    MBD_TRY(launch_exclusive_scan(cnt, start, ncell, bsum, st));
+    MBD_CUDA_TRY(cudaMemcpyAsync(cursor, start, sizeof(int) * ncell, cudaMemcpyDeviceToDevice, st));
+    if (ng.N > 0) {
+        k_bin_fill<<<(ng.N + 255) / 256, 256, 0, st>>>(ng.N, bin_of, cursor, tmp);
+        MBD_LAUNCH_CHECK();
+        k_cell_sort<<<(ncell + 7) / 8, 256, 0, st>>>(ncell, start, tmp, pos, atoms);
         MBD_LAUNCH_CHECK();
     }
     return MBD_OK;

@@ -113,15 +113,17 @@ template <class T> struct SplineView {
     const T *d2w;       // [N][3][p] (forces only)
 };
 
-// Cell grid of the neighbour search (built on the host, searched on the device).
+// Cell grid of the neighbour search.
 struct NeighborGrid {
     int N;
     int nc[3], kk[3];       // cells per direction; cells searched each way
     const int *start;       // [ncell + 1]
-    const int *atoms;       // [N] atoms by cell
+    const float4 *atoms;    // [N] FP32 position and index (bits), by cell, in increasing index
     const int *cidx;        // [N][3] cell coordinates of each atom
-    double cell[9];
+    double cell[9], recip[9];
+    float cellf[9];
     double r2max;
+    float r2near;           // FP32 squared distance beyond which no pair is within r2max
 };
 
 struct BinView {
@@ -338,7 +340,7 @@ struct mbd_system {
     // common device data
     mbd::DevBuf pos_d, g_d, w2_d, rvdw_d;            // [N][3], [N], [N], [N]
     mbd::DevBuf row_d, col_d, shift_d;              // CSR
-    mbd::DevBuf cell_start_d, cell_atoms_d, cell_idx_d, nb_err_d;   // neighbour-search cell grid
+    mbd::DevBuf cell_start_d, cell_atoms_d, cell_idx_d;   // neighbour-search cell grid
     mbd::DevBuf top_d;                              // [N][3]
     mbd::DevBuf w64_d, dw64_d;                      // [N][3][p] FP64 stencil weights (setup)
     mbd::DevBuf bin_start_d, bin_atoms_d, order_d;  // spread bins; field atom order
@@ -379,9 +381,12 @@ namespace mbd {
 // increasing atom index within a brick: counts, starts [nbins + 1], atoms [N].
 mbd_status launch_bin_atoms(int N, const int *top, const BinView &B, int *bin_of, int *cnt, int *start,
                             int *cursor, int *atoms, DevBuf &bsum, cudaStream_t st);
+// cells of the atoms: coordinates [N][3], starts [ncell + 1], atoms by cell
+mbd_status launch_cells(const NeighborGrid &ng, const double *pos, int *cidx, int *bin_of, int *cnt, int *start,
+                        int *cursor, int *tmp, float4 *atoms, DevBuf &bsum, cudaStream_t st);
 // fill: writes the pairs below cap only (the caller compares row[N] with cap)
 mbd_status launch_neighbors(const NeighborGrid &ng, const double *pos, int *cnt_or_row, int *col, int *shift,
-                            int *err, bool fill, long long cap, cudaStream_t st);
+                            bool fill, long long cap, cudaStream_t st);
 mbd_status launch_exclusive_scan(const int *in, int *out, int n, DevBuf &bsum, cudaStream_t st);
 template <class T> mbd_status launch_pair_tensors(mbd_system *s, cudaStream_t st);
 mbd_status launch_morton_order(const BinView &B, int N, int *order, DevBuf &cnt, DevBuf &start, DevBuf &bsum,
