@@ -56,40 +56,52 @@ __device__ __forceinline__ PairRadial pair_radial(double r2, double rsum, double
 
 // dA_ab / dr_c = cid_p r_c delta_ab - crr_p r_c r_a r_b - c_rr (delta_ac r_b + delta_bc r_a),
 // (ab) over the 6 upper-triangle entries, c = x, y, z.
-__device__ __forceinline__ void pair_tensor_grad(double rx, double ry, double rz, const PairRadial &pr,
+__device__ __forceinline__ void pair_tensor_grad(double x, double y, double z, const PairRadial &pr,
                                                  double out[18]) {
-    const double rv[3] = {rx, ry, rz};
-    int o = 0;
-    for (int ab = 0; ab < 6; ++ab) {
-        const int ia = ab < 3 ? 0 : (ab < 5 ? 1 : 2);
-        const int ib = ab < 3 ? ab : (ab < 5 ? ab - 2 : 2);
-        for (int c = 0; c < 3; ++c) {
-            double v = -pr.crr_p * rv[c] * rv[ia] * rv[ib];
-            if (ia == ib) v += pr.cid_p * rv[c];
-            if (ia == c) v -= pr.crr * rv[ib];
-            if (ib == c) v -= pr.crr * rv[ia];
-            out[o++] = v;
-        }
-    }
+    // s_abc = crr_p r_a r_b r_c is symmetric: ten values; u = cid_p r, m = crr r
+    const double qxx = pr.crr_p * x * x, qxy = pr.crr_p * x * y, qyy = pr.crr_p * y * y, qzz = pr.crr_p * z * z;
+    const double xxy = qxx * y, xxz = qxx * z, xyy = qxy * y, xyz = qxy * z, xzz = qzz * x, yyz = qyy * z,
+                 yzz = qzz * y;
+    const double mx = pr.crr * x, my = pr.crr * y, mz = pr.crr * z;
+    const double ux = pr.cid_p * x, uy = pr.cid_p * y, uz = pr.cid_p * z;
+    out[0] = ux - qxx * x - 2.0 * mx;   // xx: x, y, z
+    out[1] = uy - xxy;
+    out[2] = uz - xxz;
+    out[3] = -xxy - my;                 // xy
+    out[4] = -xyy - mx;
+    out[5] = -xyz;
+    out[6] = -xxz - mz;                 // xz
+    out[7] = -xyz;
+    out[8] = -xzz - mx;
+    out[9] = ux - xyy;                  // yy
+    out[10] = uy - qyy * y - 2.0 * my;
+    out[11] = uz - yyz;
+    out[12] = -xyz;                     // yz
+    out[13] = -yyz - mz;
+    out[14] = -yzz - my;
+    out[15] = ux - xzz;                 // zz
+    out[16] = uy - yzz;
+    out[17] = uz - qzz * z - 2.0 * mz;
 }
 
 // Real-space pair tensor of E^dir with the damping correction (Eq. fld_ewald):
 //   A(r) = [|r| < r_cut] (B1 I - B2 r r^T) - [|r| < damp_cut] (1 - s(|r|)) T(r)
 // with Smith's erfc-screened B1, B2 and the bare T(r) = (r^2 I - 3 r r^T)/r^5,
 // and its derivative dA/dr (forces).  FP64 from positions and the image shift,
-// stored in T; a warp per atom, lanes over its neighbours.
+// stored in T; `parts` warps per atom, lanes over its neighbours.  Bound: the
+// FP64 units.
 template <class T>
 __global__ void k_pair_tensors(int N, const double *__restrict__ pos, const double *__restrict__ rvdw,
                                const int *__restrict__ row, const int *__restrict__ col,
                                const int *__restrict__ shift, Geom g, double beta, double r_cut,
                                double damp_cut, double damp_beta, double damp_d, T *__restrict__ A,
-                               T *__restrict__ dA, long long cap) {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+                               T *__restrict__ dA, long long cap, int parts) {
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int i = w / parts, sub = w - i * parts, lane = threadIdx.x & 31;
     if (i >= N) return;
     const double xi = pos[3 * i], yi = pos[3 * i + 1], zi = pos[3 * i + 2];
     const int nb1 = (int)min((long long)row[i + 1], cap);   // pairs beyond the buffers: rebuilt by the caller
-    for (int nb = row[i] + lane; nb < nb1; nb += 32) {
+    for (int nb = row[i] + 32 * sub + lane; nb < nb1; nb += 32 * parts) {
         const int j = col[nb];
         const int sh = shift[nb];
         const double n1 = double((sh & 255) - 128), n2 = double(((sh >> 8) & 255) - 128),
@@ -358,12 +370,14 @@ template <class T> mbd_status launch_pair_tensors(mbd_system *s, cudaStream_t st
     MBD_TRY(P.pairdA.ensure(sizeof(T) * 18 * cap));
     const Geom g = make_geom(s);
     const int threads = 256;
-    const int blocks = (int)(((long long)s->N * 32 + threads - 1) / threads);
+    // enough warps for every scheduler: up to four per atom
+    const int parts = std::max(1, std::min(4, 16 * std::max(1, s->num_sms) / std::max(1, s->N)));
+    const int blocks = (int)(((long long)s->N * 32 * parts + threads - 1) / threads);
     k_pair_tensors<T><<<blocks, threads, 0, st>>>(s->N, s->pos_d.as<double>(), s->rvdw_d.as<double>(),
                                                   s->row_d.as<int>(), s->col_d.as<int>(), s->shift_d.as<int>(), g,
                                                   s->ewald_beta, s->r_cut, s->damp_cut, s->damp_beta, s->damp_d,
                                                   P.pairA.template as<T>(), P.pairdA.template as<T>(),
-                                                  (long long)cap);
+                                                  (long long)cap, parts);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }
