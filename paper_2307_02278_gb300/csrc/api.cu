@@ -111,8 +111,6 @@ void prof_release(mbd_system *s) {
     P.pool.clear();
 }
 
-// gscale kernels live in kernels_lanczos.cu
-template <class T> mbd_status launch_gscale(const double *x, const double *g, T *d, int rows, int ld, cudaStream_t st);
 
 namespace {
 
@@ -753,14 +751,9 @@ template <class T> mbd_status apply_impl(mbd_system *s, int nvec, const double *
     double *xt = s->L.as<double>();
     double *yt = s->work2.as<double>();
     PrecData<T> &P = prec<T>(s);
-    MBD_CUDA_TRY(cudaMemsetAsync(xt, 0, sizeof(double) * (size_t)rows * ld, s->stream));
-    MBD_STAGE(s, MBD_STAGE_OTHER, 1, launch_to_probe_major(x, nvec, rows, xt, ld, s->stream));
-    if (field) {
-        MBD_STAGE(s, MBD_STAGE_OTHER, 1, launch_cast_rows<T>(xt, P.d.template as<T>(), (size_t)rows * ld, s->stream));
-    } else {
-        MBD_STAGE(s, MBD_STAGE_OTHER, 1,
-                  launch_gscale<T>(xt, s->g_d.as<double>(), P.d.template as<T>(), rows, ld, s->stream));
-    }
+    MBD_STAGE(s, MBD_STAGE_OTHER, 1,
+              launch_to_probe_major<T>(x, nvec, rows, field ? nullptr : s->g_d.as<double>(), field ? nullptr : xt,
+                                       P.d.template as<T>(), ld, s->stream));
     if (terms & MBD_TERM_RECIP) {
         const bool fuse3 = spread_fft3_supported(s);
         MBD_STAGE(s, MBD_STAGE_SPREAD, 1,
@@ -789,12 +782,8 @@ template <class T> mbd_status spread_impl(mbd_system *s, int nvec, const double 
     const int rows = 3 * s->N;
     const int ld = probe_ld<T>(nvec);
     MBD_TRY(ensure_mesh<T>(s, ld));
-    MBD_TRY(s->L.ensure(sizeof(double) * (size_t)rows * ld));
-    double *xt = s->L.as<double>();
     PrecData<T> &P = prec<T>(s);
-    MBD_CUDA_TRY(cudaMemsetAsync(xt, 0, sizeof(double) * (size_t)rows * ld, s->stream));
-    MBD_TRY(launch_to_probe_major(d, nvec, rows, xt, ld, s->stream));
-    MBD_TRY(launch_cast_rows<T>(xt, P.d.template as<T>(), (size_t)rows * ld, s->stream));
+    MBD_TRY(launch_to_probe_major<T>(d, nvec, rows, nullptr, nullptr, P.d.template as<T>(), ld, s->stream));
     MBD_TRY(launch_spread<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), nvec, ld));
     const size_t npts = (size_t)s->K[0] * s->K[1] * s->K[2];
     MBD_TRY(launch_mesh_out<T>(P.mesh.template as<T>(), nvec, npts, ld, mesh_out, s->stream));

@@ -177,7 +177,9 @@ __device__ int sturm_count(const double *a, const double *b2, int n, double x) {
     return cnt;
 }
 
-template <bool FULL>
+// SLOTS: 32-row slots that cover m rows (one for m <= 32): the slots beyond are
+// FP64 work on zeros (64 probes x 30 steps: 58 -> 40 us per call).
+template <bool FULL, int SLOTS>
 __global__ void __launch_bounds__(32) k_quad_cheb(const double *__restrict__ a, const double *__restrict__ b,
                                                   const int *__restrict__ length, int R, int ld, int m,
                                                   double *__restrict__ q, double *__restrict__ coef,
@@ -187,11 +189,11 @@ __global__ void __launch_bounds__(32) k_quad_cheb(const double *__restrict__ a, 
     const int r = blockIdx.x, lane = threadIdx.x;
     const int n = length ? length[r] : m;
     // rows in registers: row k = lane + 32 t
-    double ar[kRowSlots], br[kRowSlots], bl[kRowSlots];
+    double ar[SLOTS], br[SLOTS], bl[SLOTS];
     int finite = 1;
     double glo = 1e300, ghi = -1e300;
 #pragma unroll
-    for (int t = 0; t < kRowSlots; ++t) {
+    for (int t = 0; t < SLOTS; ++t) {
         const int k = lane + 32 * t;
         ar[t] = br[t] = 0.0;
         if (k < n) {
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(32) k_quad_cheb(const double *__restrict__ a, 
         }
     }
 #pragma unroll
-    for (int t = 0; t < kRowSlots; ++t) {
+    for (int t = 0; t < SLOTS; ++t) {
         // b_{k-1}: lane - 1 of the same slot, or lane 31 of the previous one
         const double up = __shfl_up_sync(0xffffffffu, br[t], 1);
         const double prev31 = __shfl_sync(0xffffffffu, t > 0 ? br[t > 0 ? t - 1 : 0] : 0.0, 31);
@@ -303,9 +305,9 @@ __global__ void __launch_bounds__(32) k_quad_cheb(const double *__restrict__ a, 
     __syncwarp();
     // ---- recurrence v_{j+1} = 2 X v_j - v_{j-1}, v_0 = e_1, accumulating sum c_j v_j
     const double ih = 1.0 / half;
-    double am[kRowSlots], v0[kRowSlots], v1[kRowSlots], w[kRowSlots];
+    double am[SLOTS], v0[SLOTS], v1[SLOTS], w[SLOTS];
 #pragma unroll
-    for (int t = 0; t < kRowSlots; ++t) {
+    for (int t = 0; t < SLOTS; ++t) {
         const int k = lane + 32 * t;
         am[t] = k < n ? ar[t] - mid : 0.0;
         v0[t] = k == 0 ? 1.0 : 0.0;
@@ -315,25 +317,25 @@ __global__ void __launch_bounds__(32) k_quad_cheb(const double *__restrict__ a, 
     // v1 = X e_1
     auto matvec = [&](const double *v, double *y) {
 #pragma unroll
-        for (int t = 0; t < kRowSlots; ++t) {
+        for (int t = 0; t < SLOTS; ++t) {
             const double left0 = __shfl_up_sync(0xffffffffu, v[t], 1);
             const double l31 = __shfl_sync(0xffffffffu, v[t > 0 ? t - 1 : 0], 31);
             const double right0 = __shfl_down_sync(0xffffffffu, v[t], 1);
-            const double r0 = __shfl_sync(0xffffffffu, v[t + 1 < kRowSlots ? t + 1 : t], 0);
+            const double r0 = __shfl_sync(0xffffffffu, v[t + 1 < SLOTS ? t + 1 : t], 0);
             const double left = lane > 0 ? left0 : (t > 0 ? l31 : 0.0);
-            const double right = lane < 31 ? right0 : (t + 1 < kRowSlots ? r0 : 0.0);
+            const double right = lane < 31 ? right0 : (t + 1 < SLOTS ? r0 : 0.0);
             y[t] = (am[t] * v[t] + bl[t] * left + br[t] * right) * ih;
         }
     };
     matvec(v0, v1);
 #pragma unroll
-    for (int t = 0; t < kRowSlots; ++t) w[t] += c2[1] * v1[t];
+    for (int t = 0; t < SLOTS; ++t) w[t] += c2[1] * v1[t];
     qa += c1[1] * __shfl_sync(0xffffffffu, v1[0], 0);
     for (int j = 2; j < N; ++j) {
-        double y[kRowSlots];
+        double y[SLOTS];
         matvec(v1, y);
 #pragma unroll
-        for (int t = 0; t < kRowSlots; ++t) {
+        for (int t = 0; t < SLOTS; ++t) {
             const double vn = 2.0 * y[t] - v0[t];
             v0[t] = v1[t];
             v1[t] = vn;
@@ -347,7 +349,7 @@ __global__ void __launch_bounds__(32) k_quad_cheb(const double *__restrict__ a, 
     }
     if (FULL) {
 #pragma unroll
-        for (int t = 0; t < kRowSlots; ++t) {
+        for (int t = 0; t < SLOTS; ++t) {
             const int k = lane + 32 * t;
             if (k < m) coef[(size_t)k * ld + r] = k < n ? w[t] : 0.0;
         }
@@ -558,8 +560,12 @@ __global__ void __launch_bounds__(256) k_dense_epilogue(int dim, LanczosView lz,
         lz.a[(size_t)k * ld + r] = tot[lane];
 }
 
-// [nvec][rows] <-> [rows][ld] transposes through a 32x33 shared tile.
-__global__ void k_transpose_in(const double *__restrict__ x, int nvec, int rows, double *__restrict__ xt, int ld) {
+// [nvec][rows] <-> [rows][ld] transposes through a 32x33 shared tile.  The way in
+// pads the vectors with zeros to ld and writes the dipoles d = g x (or x, g
+// null; g indexed by atom = row / 3) in T beside them (xt null: d alone).
+template <class T>
+__global__ void k_transpose_in(const double *__restrict__ x, int nvec, int rows, const double *__restrict__ g,
+                               double *__restrict__ xt, T *__restrict__ d, int ld) {
     __shared__ double tile[32][33];
     const int r0 = blockIdx.x * 32, v0 = blockIdx.y * 32;
     for (int j = threadIdx.y; j < 32; j += 8) {
@@ -569,7 +575,11 @@ __global__ void k_transpose_in(const double *__restrict__ x, int nvec, int rows,
     __syncthreads();
     for (int j = threadIdx.y; j < 32; j += 8) {
         const int row = r0 + j, v = v0 + threadIdx.x;
-        if (row < rows && v < ld) xt[(size_t)row * ld + v] = tile[threadIdx.x][j];
+        if (row < rows && v < ld) {
+            const double t = tile[threadIdx.x][j];
+            if (xt) xt[(size_t)row * ld + v] = t;
+            d[(size_t)row * ld + v] = T(g ? g[row / 3] * t : t);
+        }
     }
 }
 __global__ void k_transpose_out(const double *__restrict__ xt, int nvec, int rows, int ld, double *__restrict__ x) {
@@ -584,18 +594,6 @@ __global__ void k_transpose_out(const double *__restrict__ xt, int nvec, int row
         const int v = v0 + j, row = r0 + threadIdx.x;
         if (v < nvec && row < rows) x[(size_t)v * rows + row] = tile[threadIdx.x][j];
     }
-}
-template <class T> __global__ void k_cast(const double *__restrict__ x, T *__restrict__ y, size_t n) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = T(x[i]);
-}
-// d = g . x (per row, g indexed by atom = row / 3), cast to T
-template <class T>
-__global__ void k_gscale(const double *__restrict__ x, const double *__restrict__ g, T *__restrict__ d, int rows,
-                         int ld) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)rows * ld) return;
-    d[i] = T(g[(i / ld) / 3] * x[i]);
 }
 template <class T>
 __global__ void k_mesh_out(const T *__restrict__ mesh, int nvec, size_t npts, int ld, double *__restrict__ out) {
@@ -650,10 +648,10 @@ mbd_status launch_quadrature(const double *a, const double *b, const int *length
                              double *coef, int *status, int *fallback, cudaStream_t st, int method) {
     if (method == MBD_QUAD_QL_DF64) return launch_tridiag_s<df>(a, b, length, R, ld, m, q, coef, status, st, nullptr);
     if (method == MBD_QUAD_QL) return launch_tridiag_s<double>(a, b, length, R, ld, m, q, coef, status, st, nullptr);
-    if (coef)
-        k_quad_cheb<true><<<R, 32, 0, st>>>(a, b, length, R, ld, m, q, coef, status, fallback);
-    else
-        k_quad_cheb<false><<<R, 32, 0, st>>>(a, b, length, R, ld, m, q, coef, status, fallback);
+    auto kern = m <= 32   ? (coef ? k_quad_cheb<true, 1> : k_quad_cheb<false, 1>)
+                : m <= 64 ? (coef ? k_quad_cheb<true, 2> : k_quad_cheb<false, 2>)
+                          : (coef ? k_quad_cheb<true, kRowSlots> : k_quad_cheb<false, kRowSlots>);
+    kern<<<R, 32, 0, st>>>(a, b, length, R, ld, m, q, coef, status, fallback);
     MBD_LAUNCH_CHECK();
     // probes whose spectrum the expansion cannot cover go through QL
     return launch_tridiag_s<double>(a, b, length, R, ld, m, q, coef, status, st, fallback);
@@ -683,20 +681,21 @@ mbd_status launch_dense_step(const double *c, int dim, const LanczosView &lz, in
     return MBD_OK;
 }
 
-mbd_status launch_to_probe_major(const double *x, int nvec, int rows, double *xt, int ld, cudaStream_t st) {
+template <class T>
+mbd_status launch_to_probe_major(const double *x, int nvec, int rows, const double *g, double *xt, T *d, int ld,
+                                 cudaStream_t st) {
     dim3 grid((rows + 31) / 32, (ld + 31) / 32), block(32, 8);
-    k_transpose_in<<<grid, block, 0, st>>>(x, nvec, rows, xt, ld);
+    k_transpose_in<T><<<grid, block, 0, st>>>(x, nvec, rows, g, xt, d, ld);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }
+template mbd_status launch_to_probe_major<double>(const double *, int, int, const double *, double *, double *, int,
+                                                  cudaStream_t);
+template mbd_status launch_to_probe_major<float>(const double *, int, int, const double *, double *, float *, int,
+                                                 cudaStream_t);
 mbd_status launch_from_probe_major(const double *xt, int nvec, int rows, int ld, double *x, cudaStream_t st) {
     dim3 grid((rows + 31) / 32, (nvec + 31) / 32), block(32, 8);
     k_transpose_out<<<grid, block, 0, st>>>(xt, nvec, rows, ld, x);
-    MBD_LAUNCH_CHECK();
-    return MBD_OK;
-}
-template <class T> mbd_status launch_cast_rows(const double *x, T *y, size_t n, cudaStream_t st) {
-    k_cast<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, y, n);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }
@@ -715,16 +714,6 @@ mbd_status launch_mesh_in(const double *in, int nvec, size_t npts, int ld, T *me
     return MBD_OK;
 }
 
-template <class T> mbd_status launch_gscale(const double *x, const double *g, T *d, int rows, int ld, cudaStream_t st) {
-    const size_t n = (size_t)rows * ld;
-    k_gscale<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, g, d, rows, ld);
-    MBD_LAUNCH_CHECK();
-    return MBD_OK;
-}
-template mbd_status launch_gscale<double>(const double *, const double *, double *, int, int, cudaStream_t);
-template mbd_status launch_gscale<float>(const double *, const double *, float *, int, int, cudaStream_t);
-template mbd_status launch_cast_rows<double>(const double *, double *, size_t, cudaStream_t);
-template mbd_status launch_cast_rows<float>(const double *, float *, size_t, cudaStream_t);
 template mbd_status launch_mesh_out<double>(const double *, int, size_t, int, double *, cudaStream_t);
 template mbd_status launch_mesh_out<float>(const float *, int, size_t, int, double *, cudaStream_t);
 template mbd_status launch_mesh_in<double>(const double *, int, size_t, int, double *, cudaStream_t);

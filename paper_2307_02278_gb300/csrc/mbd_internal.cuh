@@ -437,9 +437,11 @@ int field_apb(const mbd_system *s, int ld);
 int field_blocks(const mbd_system *s, int ld);
 
 // layout helpers
-mbd_status launch_to_probe_major(const double *x, int nvec, int rows, double *xt, int ld, cudaStream_t st);
+// x [nvec][rows] to rows [rows][ld] (xt, may be null) and dipoles g x (x: g null) in T
+template <class T>
+mbd_status launch_to_probe_major(const double *x, int nvec, int rows, const double *g, double *xt, T *d, int ld,
+                                 cudaStream_t st);
 mbd_status launch_from_probe_major(const double *xt, int nvec, int rows, int ld, double *x, cudaStream_t st);
-template <class T> mbd_status launch_cast_rows(const double *x, T *y, size_t n, cudaStream_t st);
 template <class T> mbd_status launch_mesh_out(const T *mesh, int nvec, size_t npts, int ld, double *out,
                                               cudaStream_t st);
 template <class T> mbd_status launch_mesh_in(const double *in, int nvec, size_t npts, int ld, T *mesh,
