@@ -43,6 +43,7 @@ template <class T> struct SpreadArgs {
     const PencilRec<T> *prec;
     const T *k3w;        // [N][2p] M3, M3'
     const typename Cplx<T>::type *tw;   // twiddles of k3
+    int sms;             // multiprocessors
 };
 // Spreading fused with the forward transform along k3; same return values.
 template <class T> int launch_spp_sized(const SpreadArgs<T> &a, cudaStream_t st);
@@ -787,21 +788,31 @@ __device__ __forceinline__ void pencil_walk(const T *__restrict__ d, int ld, con
 // Probes per lane and complex columns per tile (a warp's width) of the spreading.
 template <class T> constexpr int spread_ppl() { return sizeof(T) == 4 ? 2 : 1; }
 template <class T> constexpr int spread_w() { return 16 * spread_ppl<T>(); }
-// Warps of a block: segments of at least P - 1 rows, at most 8.
-template <int K, int P> constexpr int spread_segs() { return K / (P - 1) < 8 ? K / (P - 1) : 8; }
+// Warps of a block: one per segment of the pencil, each at least P - 1 rows.  Few
+// long segments waste less on the halos and balance their records better, as
+// long as the blocks' warps fill the SM (short pencils: many blocks); long
+// pencils have fewer blocks in shared memory and take more warps per block.  us
+// per launch with 4, 5, 6 and 8 segments: 64^3 x 64 probes 41, 43, 46, 49; 108^3 x
+// 64 177, 171, 187, 198; 128^3 x 128 589, 539, 552, 614; 160^3 x 64 807, 684, 636,
+// 659; 192^3 x 64 1646, 1468, 1284, 1139.  Grids of few tiles are bound by a
+// warp's own chain of records: 8 (40^3 x 8: 12.4, 12.0, 10.7, 10.3).
+template <int K, int P> constexpr int spread_segs(bool few_tiles) {
+    constexpr int want = K <= 96 ? 4 : (K <= 112 ? 5 : (K <= 160 ? 6 : 8)), most = K / (P - 1);
+    return (few_tiles ? 8 : want) < most ? (few_tiles ? 8 : want) : most;
+}
 
 // Shared memory of a block whose tile touches `pens` pencils, and the blocks
 // per SM asked of the compiler: 32 warps (64 registers) in float and 24 in
 // double as far as shared memory holds them (128^3 x 128 probes: 663 -> 618 us
 // per launch against the compiler's own 92 registers; 192^3, where it holds
 // three blocks, 1139 us with 80 registers and 1255 with 64).
-template <class T, int K, int P> constexpr size_t spread_smem(int pens) {
+template <class T, int K, int P, int NSEG> constexpr size_t spread_smem(int pens) {
     return sizeof(typename TwOf<typename PackOf<T>::type>::type) * K +
-           sizeof(T) * 2 * (size_t)spread_w<T>() * (K + spread_segs<K, P>() * (P - 1)) +
+           sizeof(T) * 2 * (size_t)spread_w<T>() * (K + NSEG * (P - 1)) +
            sizeof(int) * ((size_t)pens * K + 1);
 }
-template <class T, int K, int P> constexpr int spread_blocks() {
-    constexpr int by_smem = (int)(227 * 1024 / (spread_smem<T, K, P>(2) + 1024)), by_regs = (sizeof(T) == 4 ? 32 : 24) / spread_segs<K, P>();
+template <class T, int K, int P, int NSEG> constexpr int spread_blocks() {
+    constexpr int by_smem = (int)(227 * 1024 / (spread_smem<T, K, P, NSEG>(2) + 1024)), by_regs = (sizeof(T) == 4 ? 32 : 24) / NSEG;
     return by_smem < by_regs ? by_smem : by_regs;
 }
 
@@ -815,14 +826,14 @@ template <class T, int K, int P> constexpr int spread_blocks() {
 // warp adds after a barrier.  Then the block transforms the tile and writes it.
 // Probes >= R are zero.
 // Bound: instruction issue and the latency of the dipole loads (L2).
-template <class T, class PL, int P>
-__global__ void __launch_bounds__(32 * spread_segs<PL::K, P>(), spread_blocks<T, PL::K, P>())
+template <class T, class PL, int P, int NSEG>
+__global__ void __launch_bounds__(32 * NSEG, (spread_blocks<T, PL::K, P, NSEG>()))
     k_spread_pencil_fft3(const T *__restrict__ d, T *__restrict__ mesh, int R, int ld, unsigned ncols,
                          const int *__restrict__ prow, const PencilRec<T> *__restrict__ prec,
                          const T *__restrict__ k3w, const typename Cplx<T>::type *__restrict__ twg) {
     using F = typename PackOf<T>::type;
     using C = Cx<F>;
-    constexpr int K = PL::K, PPL = spread_ppl<T>(), W = spread_w<T>(), NSEG = spread_segs<K, P>(), NT = 32 * NSEG;
+    constexpr int K = PL::K, PPL = spread_ppl<T>(), W = spread_w<T>(), NT = 32 * NSEG;
     constexpr int WF = W * 2 * (int)sizeof(T) / (int)sizeof(C);
     static_assert(NT % WF == 0 && NSEG >= 2, "whole rows of threads, two segments at least");
     extern __shared__ __align__(16) unsigned char smem_spp[];
@@ -878,13 +889,13 @@ __global__ void __launch_bounds__(32 * spread_segs<PL::K, P>(), spread_blocks<T,
                                        VF, valid);
 }
 
-template <class T, class PL, int P>
-int launch_spp(const SpreadArgs<T> &a, cudaStream_t st) {
-    constexpr int K = PL::K, W = spread_w<T>(), NSEG = spread_segs<K, P>();
-    auto kern = k_spread_pencil_fft3<T, PL, P>;
+template <class T, class PL, int P, int NSEG>
+int launch_spp_segs(const SpreadArgs<T> &a, cudaStream_t st) {
+    constexpr int K = PL::K, W = spread_w<T>();
+    auto kern = k_spread_pencil_fft3<T, PL, P, NSEG>;
     const int V = a.ld / 2;
     const int pens = (W - 1) / V + 2;              // pencils that a tile can touch
-    const size_t smem = spread_smem<T, K, P>(pens);
+    const size_t smem = spread_smem<T, K, P, NSEG>(pens);
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return 0;
@@ -892,6 +903,12 @@ int launch_spp(const SpreadArgs<T> &a, cudaStream_t st) {
     launch_pdl(true, kern, dim3((ncols + W - 1) / W), dim3(32 * NSEG), smem, st, a.d, a.mesh, a.R, a.ld, ncols, a.prow,
                a.prec, a.k3w, a.tw);
     return 1;
+}
+template <class T, class PL, int P> int launch_spp(const SpreadArgs<T> &a, cudaStream_t st) {
+    constexpr int many = spread_segs<PL::K, P>(false), few = spread_segs<PL::K, P>(true);
+    const size_t tiles = (size_t)a.K1 * a.K2 * (a.ld / 2) / spread_w<T>();
+    if (many != few && tiles < 8 * (size_t)a.sms) return launch_spp_segs<T, PL, P, few>(a, st);
+    return launch_spp_segs<T, PL, P, many>(a, st);
 }
 template <class T, class PL> int spp_size(const SpreadArgs<T> &a, cudaStream_t st) {
 #define MBD_SPP_ORDER(P) \

@@ -900,7 +900,7 @@ template <class T> SpreadArgs<T> spread_args(mbd_system *s, const T *d, T *mesh,
     PrecData<T> &P = prec<T>(s);
     return {d, mesh, R, ld, s->K[0], s->K[1], s->K[2], s->p, P.prow.template as<int>(),
             P.prec.template as<PencilRec<T>>(), P.k3w.template as<T>(),
-            P.tw3.template as<typename Cplx<T>::type>()};
+            P.tw3.template as<typename Cplx<T>::type>(), std::max(1, s->num_sms)};
 }
 
 template <class T> mbd_status launch_spread(mbd_system *s, const T *d, T *mesh, int R, int ld) {
