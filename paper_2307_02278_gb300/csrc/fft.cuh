@@ -725,33 +725,33 @@ template <class T, int PPL> __device__ __forceinline__ void lane_fma(const T *a,
 }
 
 // A lane's walk along one pencil (k1, k2) for its PPL probes (d: the dipole
-// rows at those probes): the records of the points (k1, k2, t) for t = t0 ..
-// t1 - 1 in CSR order (record q0 up to q1; ends(t) the end of point t's
-// records), each adding M3(j) (e0 . d) + M3'(j) (e1 . d) to the rows t - j,
-// j < P.  Row t - P + 1 is complete after point t and goes to row_done; the
-// walk ends with the P - 1 rows still open after the last point.  The window
-// of P open rows is a register array whose origin moves with t, unrolled by P
-// so that it never shifts; each row is a sum in a fixed order.  The next
-// record is loaded one ahead.
-template <class T, int P, int PPL, class Ends, class Done>
+// rows at those probes): the records of the points (k1, k2, t) for t = t1 - 1
+// down to t0 (records q0 .. q1 - 1, begins(t) the first of point t), each adding
+// M3(j) (e0 . d) + M3'(j) (e1 . d) to the rows t - j, j < P.  Row t is complete
+// after point t and goes to row_done; the P - 1 rows below t0 stay in
+// registers and go to tail after between() (a barrier where they belong to
+// another warp).  The window of P open rows is a register array whose origin
+// moves with t, unrolled by P so that it never shifts; each row is a sum in a
+// fixed order.  The next record is loaded one ahead.
+template <class T, int P, int PPL, class Begins, class Done, class Between, class Tail>
 __device__ __forceinline__ void pencil_walk(const T *__restrict__ d, int ld, const PencilRec<T> *__restrict__ prec,
-                                            const T *__restrict__ k3w, int t0, int t1, int q0, int q1, Ends &&ends,
-                                            Done &&row_done) {
-    T acc[P][PPL];
+                                            const T *__restrict__ k3w, int t0, int t1, int q0, int q1, Begins &&begins,
+                                            Done &&row_done, Between &&between, Tail &&tail) {
+    T acc[P][PPL];                              // row r in slot (t1 - 1 - r) mod P
 #pragma unroll
     for (int j = 0; j < P; ++j)
 #pragma unroll
         for (int e = 0; e < PPL; ++e) acc[j][e] = T(0);
-    int q = q0;
+    int q = q1 - 1;
     PencilRec<T> rc{};
-    if (q < q1) rc = prec[q];
-    for (int tb = t0; tb < t1 + P - 1; tb += P) {
+    if (q >= q0) rc = prec[q];
+    const int n = t1 - t0;
+    for (int sb = 0; sb < n; sb += P) {
 #pragma unroll
         for (int u = 0; u < P; ++u) {
-            const int t = tb + u;
-            if (t >= t1 + P - 1) break;
-            const int qe = t < t1 ? ends(t) : q;
-            while (q < qe) {
+            if (sb + u >= n) break;
+            const int t = t1 - 1 - sb - u, qb = begins(t);
+            while (q >= qb) {
                 T x[PPL], y[PPL], z[PPL], w[2 * P];
                 const T *dj = d + (size_t)(3 * rc.atom) * ld;
                 vload<T, PPL>(dj, x);
@@ -770,49 +770,53 @@ __device__ __forceinline__ void pencil_walk(const T *__restrict__ d, int ld, con
                 lane_fma<T, PPL>(x, rc.e1[0], fv);
                 lane_fma<T, PPL>(y, rc.e1[1], fv);
                 lane_fma<T, PPL>(z, rc.e1[2], fv);
-                if (++q < q1) rc = prec[q];
+                if (--q >= q0) rc = prec[q];
 #pragma unroll
                 for (int j = 0; j < P; ++j) {
-                    lane_fma<T, PPL>(fu, w[j], acc[(u - j + P) % P]);
-                    lane_fma<T, PPL>(fv, w[P + j], acc[(u - j + P) % P]);
+                    lane_fma<T, PPL>(fu, w[j], acc[(u + j) % P]);
+                    lane_fma<T, PPL>(fv, w[P + j], acc[(u + j) % P]);
                 }
             }
-            T *done = acc[(u + 1) % P];
-            row_done(t - P + 1, done);
+            row_done(t, acc[u]);
 #pragma unroll
-            for (int e = 0; e < PPL; ++e) done[e] = T(0);
+            for (int e = 0; e < PPL; ++e) acc[u][e] = T(0);
         }
     }
+    between();
+    const int phase = n % P;                    // slot of row t0 - 1
+#pragma unroll
+    for (int k = 0; k < 2 * P - 2; ++k)
+        if (k >= phase && k < phase + P - 1) tail(t0 - 1 - (k - phase), acc[k % P]);
 }
 
 // Probes per lane and complex columns per tile (a warp's width) of the spreading.
 template <class T> constexpr int spread_ppl() { return sizeof(T) == 4 ? 2 : 1; }
 template <class T> constexpr int spread_w() { return 16 * spread_ppl<T>(); }
 // Warps of a block: one per segment of the pencil, each at least P - 1 rows.  Few
-// long segments waste less on the halos and balance their records better, as
+// long segments add fewer rows twice and balance their records better, as
 // long as the blocks' warps fill the SM (short pencils: many blocks); long
 // pencils have fewer blocks in shared memory and take more warps per block.  us
-// per launch with 4, 5, 6 and 8 segments: 64^3 x 64 probes 41, 43, 46, 49; 108^3 x
-// 64 177, 171, 187, 198; 128^3 x 128 589, 539, 552, 614; 160^3 x 64 807, 684, 636,
-// 659; 192^3 x 64 1646, 1468, 1284, 1139.  Grids of few tiles are bound by a
-// warp's own chain of records: 8 (40^3 x 8: 12.4, 12.0, 10.7, 10.3).
+// per launch: 120^3 x 64 probes 207 with 4 segments and 221 with 6, 128^3 x 128
+// 490 and 498; 144^3 x 64 363 with 6 and 379 with 5, 160^3 x 64 547 and 556; 192^3
+// x 64 921 with 8, 986 with 6 and 1012 with 10.  Grids of few tiles are bound by a
+// warp's own chain of records: 8 (40^3 x 8: 9.9 against 10.3).
 template <int K, int P> constexpr int spread_segs(bool few_tiles) {
-    constexpr int want = K <= 96 ? 4 : (K <= 112 ? 5 : (K <= 160 ? 6 : 8)), most = K / (P - 1);
+    constexpr int want = K <= 128 ? 4 : (K <= 160 ? 6 : 8), most = K / (P - 1);
     return (few_tiles ? 8 : want) < most ? (few_tiles ? 8 : want) : most;
 }
 
 // Shared memory of a block whose tile touches `pens` pencils, and the blocks
 // per SM asked of the compiler: 32 warps (64 registers) in float and 24 in
-// double as far as shared memory holds them (128^3 x 128 probes: 663 -> 618 us
-// per launch against the compiler's own 92 registers; 192^3, where it holds
-// three blocks, 1139 us with 80 registers and 1255 with 64).
-template <class T, int K, int P, int NSEG> constexpr size_t spread_smem(int pens) {
+// double as far as shared memory holds them (resident warps hide the latency
+// of the dipole loads: loading them one record ahead takes the registers of a
+// third of the warps, 64^3 x 64 probes 49 -> 62 us).
+template <class T, int K> constexpr size_t spread_smem(int pens) {
     return sizeof(typename TwOf<typename PackOf<T>::type>::type) * K +
-           sizeof(T) * 2 * (size_t)spread_w<T>() * (K + NSEG * (P - 1)) +
+           sizeof(T) * 2 * (size_t)spread_w<T>() * K +
            sizeof(int) * ((size_t)pens * K + 1);
 }
-template <class T, int K, int P, int NSEG> constexpr int spread_blocks() {
-    constexpr int by_smem = (int)(227 * 1024 / (spread_smem<T, K, P, NSEG>(2) + 1024)), by_regs = (sizeof(T) == 4 ? 32 : 24) / NSEG;
+template <class T, int K, int NSEG> constexpr int spread_blocks() {
+    constexpr int by_smem = (int)(227 * 1024 / (spread_smem<T, K>(2) + 1024)), by_regs = (sizeof(T) == 4 ? 32 : 24) / NSEG;
     return by_smem < by_regs ? by_smem : by_regs;
 }
 
@@ -821,13 +825,17 @@ template <class T, int K, int P, int NSEG> constexpr int spread_blocks() {
 // when the probes fill a warp, several pencils' otherwise; lane l holds the
 // tile's probes l PPL .. and so its own pencil.  The K points of the pencil
 // are cut into one segment per warp; a warp walks the records of its segment's
-// points once, its rows go to the shared tile, and the P - 1 rows below its
-// segment, which belong to the warp before (cyclically), to a halo that this
-// warp adds after a barrier.  Then the block transforms the tile and writes it.
-// Probes >= R are zero.
-// Bound: instruction issue and the latency of the dipole loads (L2).
+// points once, its rows go to the shared tile, and after a barrier it adds the
+// P - 1 rows below its segment, which belong to the warp before (cyclically).
+// Then the block transforms the tile and writes it.  Probes >= R are zero.
+// Bound: instruction issue and the latency of the dipole loads (L2).  Walking
+// every record that reaches a warp's rows, and a second buffer for the
+// transform: 192^3 x 64 probes 1507 us per launch; each record once, the rows
+// below a segment through a halo in shared memory: 1139; those rows kept in
+// registers (the walk runs downwards), one block more per SM: 921.  128^3 x 128:
+// 862, 552 and 490; 64^3 x 64: 56, 41 and 37.
 template <class T, class PL, int P, int NSEG>
-__global__ void __launch_bounds__(32 * NSEG, (spread_blocks<T, PL::K, P, NSEG>()))
+__global__ void __launch_bounds__(32 * NSEG, (spread_blocks<T, PL::K, NSEG>()))
     k_spread_pencil_fft3(const T *__restrict__ d, T *__restrict__ mesh, int R, int ld, unsigned ncols,
                          const int *__restrict__ prow, const PencilRec<T> *__restrict__ prec,
                          const T *__restrict__ k3w, const typename Cplx<T>::type *__restrict__ twg) {
@@ -839,8 +847,7 @@ __global__ void __launch_bounds__(32 * NSEG, (spread_blocks<T, PL::K, P, NSEG>()
     extern __shared__ __align__(16) unsigned char smem_spp[];
     auto *tw = reinterpret_cast<typename TwOf<F>::type *>(smem_spp);
     T *tile = reinterpret_cast<T *>(tw + K);          // [K][2W] reals
-    T *halo = tile + 2 * (size_t)K * W;               // [NSEG][P - 1][2W]
-    int *rp = reinterpret_cast<int *>(halo + 2 * (size_t)NSEG * (P - 1) * W);   // record starts of the tile's pencils
+    int *rp = reinterpret_cast<int *>(tile + 2 * (size_t)K * W);   // record starts of the tile's pencils
     const int V = ld / 2;
     const unsigned c0 = blockIdx.x * W;
     const unsigned pen0 = c0 / V, pen1 = min(c0 + W, ncols) - 1;   // first pencil, last column
@@ -856,29 +863,24 @@ __global__ void __launch_bounds__(32 * NSEG, (spread_blocks<T, PL::K, P, NSEG>()
     const unsigned pen = cl / V;
     const int pr0 = 2 * (int)(cl - pen * V) + (lane * PPL & 1);   // its first probe
     const int *rpp = rp + (pen - pen0) * K;
-    T *mine = tile + lane * PPL, *hmine = halo + (size_t)warp * (P - 1) * 2 * W + lane * PPL;
+    T *mine = tile + lane * PPL;
     pencil_walk<T, P, PPL>(
-        d + pr0, ld, prec, k3w, r0, r1, rpp[r0], rpp[r1], [&](int t) { return rpp[t + 1]; },
+        d + pr0, ld, prec, k3w, r0, r1, rpp[r0], rpp[r1], [&](int t) { return rpp[t]; },
         [&](int row, const T *v) {
             T o[PPL];
 #pragma unroll
             for (int e = 0; e < PPL; ++e) o[e] = pr0 + e < R ? v[e] : T(0);
-            vstore<T, PPL>(row >= r0 ? mine + row * 2 * W : hmine + (row - r0 + P - 1) * 2 * W, o);
+            vstore<T, PPL>(mine + row * 2 * W, o);
+        },
+        [] { __syncthreads(); },
+        [&](int row, const T *v) {
+            T *o = mine + (row < 0 ? row + K : row) * 2 * W;
+            T y[PPL];
+            vload<T, PPL>(o, y);
+#pragma unroll
+            for (int e = 0; e < PPL; ++e) y[e] += pr0 + e < R ? v[e] : T(0);
+            vstore<T, PPL>(o, y);
         });
-    __syncthreads();
-    {
-        const T *h = halo + (size_t)((warp + 1) % NSEG) * (P - 1) * 2 * W + lane * PPL;
-        T *o = mine + (r1 - (P - 1)) * 2 * W;
-#pragma unroll
-        for (int j = 0; j < P - 1; ++j) {
-            T x[PPL], y[PPL];
-            vload<T, PPL>(h + j * 2 * W, x);
-            vload<T, PPL>(o + j * 2 * W, y);
-#pragma unroll
-            for (int e = 0; e < PPL; ++e) y[e] += x[e];
-            vstore<T, PPL>(o + j * 2 * W, y);
-        }
-    }
     __syncthreads();
     const unsigned VF = (unsigned)((size_t)ld * sizeof(T) / sizeof(C)), nf = ncols / V * VF;
     const unsigned cg = blockIdx.x * WF + threadIdx.x % WF;
@@ -895,7 +897,7 @@ int launch_spp_segs(const SpreadArgs<T> &a, cudaStream_t st) {
     auto kern = k_spread_pencil_fft3<T, PL, P, NSEG>;
     const int V = a.ld / 2;
     const int pens = (W - 1) / V + 2;              // pencils that a tile can touch
-    const size_t smem = spread_smem<T, K, P, NSEG>(pens);
+    const size_t smem = spread_smem<T, K>(pens);
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return 0;

@@ -126,12 +126,11 @@ __global__ void k_scan_add(int *__restrict__ out, const int *__restrict__ bsum, 
 
 // The spreading alone, for mesh lengths without a fused pass and for the
 // stage-level call: a warp per tile of W complex columns, each lane walking its
-// pencil from top3 = 0 to K3 - 1.  The P - 1 rows below the first point are
-// kept in shared memory and added to the last rows, which they are.
+// pencil from top3 = K3 - 1 to 0 and adding the P - 1 rows below the first point
+// to the last rows, which they are.
 template <class T, int P>
 __global__ void __launch_bounds__(128) k_spread_pencil(SpreadArgs<T> a, unsigned ncols) {
     constexpr int PPL = spread_ppl<T>(), W = spread_w<T>();
-    __shared__ __align__(16) T halo[4][P - 1][2 * W];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, K = a.K3, V = a.ld / 2;
     const unsigned c = (blockIdx.x * 4 + warp) * W + lane * PPL / 2;
     if (c >= ncols) return;
@@ -140,22 +139,21 @@ __global__ void __launch_bounds__(128) k_spread_pencil(SpreadArgs<T> a, unsigned
     const int *rp = a.prow + (size_t)pen * K;
     T *out = a.mesh + (size_t)pen * K * a.ld + pr0;
     pencil_walk<T, P, PPL>(
-        a.d + pr0, a.ld, a.prec, a.k3w, 0, K, rp[0], rp[K], [&](int t) { return rp[t + 1]; },
+        a.d + pr0, a.ld, a.prec, a.k3w, 0, K, rp[0], rp[K], [&](int t) { return rp[t]; },
         [&](int row, const T *v) {
             T o[PPL];
 #pragma unroll
             for (int e = 0; e < PPL; ++e) o[e] = pr0 + e < a.R ? v[e] : T(0);
-            if (row < 0) {
-                vstore<T, PPL>(&halo[warp][row + P - 1][lane * PPL], o);
-                return;
-            }
-            if (row >= K - (P - 1)) {
-                T h[PPL];
-                vload<T, PPL>(&halo[warp][row - (K - (P - 1))][lane * PPL], h);
-#pragma unroll
-                for (int e = 0; e < PPL; ++e) o[e] += h[e];
-            }
             vstore<T, PPL>(out + (size_t)row * a.ld, o);
+        },
+        [] {},
+        [&](int row, const T *v) {
+            T *o = out + (size_t)(row + K) * a.ld;
+            T y[PPL];
+            vload<T, PPL>(o, y);
+#pragma unroll
+            for (int e = 0; e < PPL; ++e) y[e] += pr0 + e < a.R ? v[e] : T(0);
+            vstore<T, PPL>(o, y);
         });
 }
 
