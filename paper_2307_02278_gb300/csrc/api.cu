@@ -599,10 +599,13 @@ mbd_status enqueue_steps(mbd_system *s, int R, int m, uint64_t seed, const uint6
     fo.lz = z.v;
     const bool fuse3 = spread_fft3_supported(s);
     const bool real_cl = real_on_clusters(s, z.ld, (int)sizeof(T));
+    const bool early = step_early(s, z.ld, (int)sizeof(T));
     for (int k = 0; k < m; ++k) {
+        const bool behind_field = k > 1 || (k == 1 && !v0);   // else a memset or a copy comes before
         MBD_STAGE(s, MBD_STAGE_PROLOGUE, 1,
                   launch_prologue_t(s->stream, z.v, k, m, seed, R, z.ld, rows, s->g_d.as<double>(), P.d.ptr,
-                                    (int)sizeof(T), z.nblk, seed_dev));
+                                    (int)sizeof(T), z.nblk, seed_dev,
+                                    behind_field && early));
         MBD_STAGE(s, MBD_STAGE_SPREAD, 1,
                   fuse3 ? launch_spread_fft3<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), R, z.ld)
                         : launch_spread<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), R, z.ld));

@@ -614,16 +614,16 @@ __global__ void k_mesh_in(const double *__restrict__ in, int nvec, size_t npts, 
 
 mbd_status launch_prologue_t(cudaStream_t st, const LanczosView &lz, int k, int m, uint64_t seed, int R, int ld,
                              int rows, const double *g, void *dout, int dtype_bytes, int nblk,
-                             const uint64_t *seed_dev) {
+                             const uint64_t *seed_dev, bool early) {
     // blocks with no row of their own would only lengthen the reduction
     const int per = 8 * row_lanes(R).rows;
     dim3 block(32, 8), grid(std::min(nblk, (rows + per - 1) / per), (R + 31) / 32);
     if (dtype_bytes == 8)
-        k_prologue<double><<<grid, block, 0, st>>>(lz, k, m, seed, seed_dev, R, ld, rows, g,
-                                                   static_cast<double *>(dout));
+        launch_pdl(early, k_prologue<double>, grid, block, 0, st, lz, k, m, seed, seed_dev, R, ld, rows, g,
+                   static_cast<double *>(dout));
     else
-        k_prologue<float><<<grid, block, 0, st>>>(lz, k, m, seed, seed_dev, R, ld, rows, g,
-                                                  static_cast<float *>(dout));
+        launch_pdl(early, k_prologue<float>, grid, block, 0, st, lz, k, m, seed, seed_dev, R, ld, rows, g,
+                   static_cast<float *>(dout));
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }

@@ -535,6 +535,8 @@ __global__ void __launch_bounds__(field_warps<P>() * 32, sizeof(T) == 8 ? 2 : (P
     constexpr int RB = field_rec_bytes<T, P>();
     constexpr int OUT = 32 * VEC * 3;            // (team, component, probe) slots of an iteration, at most
     constexpr int OPT = (OUT + NTH - 1) / NTH;   // of them per thread, at most
+    pdl_wait();
+    pdl_launch_dependents();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int S = 32 / a.lanes, nloc = a.lanes * VEC, per = S / a.teams;   // groups of a team in a warp
     const int sub = lane / a.lanes, lid = lane - sub * a.lanes;
@@ -698,6 +700,8 @@ __global__ void __launch_bounds__(field_warps<P>() * 32, P == 6 ? 4 : 2) k_field
     constexpr int VEC = 4, NW = field_warps<P>(), NTH = NW * 32, PP = P * P / NW, D = kFieldDepth;
     constexpr int OUT = 32 * VEC * 3, OPT = (OUT + NTH - 1) / NTH, RB = field_rec_bytes<float, P>(), W4 = 6 * P / 4;
     static_assert(P * P % NW == 0 && PP % D == 0 && 6 * P % 4 == 0, "whole pencils per warp and ring");
+    pdl_wait();
+    pdl_launch_dependents();
     extern __shared__ __align__(16) unsigned char smem_fs[];
     float4 *ring = reinterpret_cast<float4 *>(smem_fs);                  // [D][P][NTH]
     float *red = reinterpret_cast<float *>(ring + D * P * NTH);          // [NW][OUT]
@@ -1018,6 +1022,18 @@ template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bo
     return MBD_OK;
 }
 
+// On small meshes the field kernel and the prologue are launched before the
+// kernel in front of them has ended: their own launch then hides behind it, and
+// a step of 36 us (96 atoms, 24^3, 1 probe) takes 31, one of 45 (1,200 atoms,
+// 45^3, 4 probes) 42, one of 76.5 (32 probes, 12 MB) 73.8.  With longer kernels
+// their waiting blocks hold registers and shared memory that the running one
+// has a use for: nothing is gained at 23 MB, and 64^3 x 32 probes (34 MB) goes
+// from 111 to 118 us.
+constexpr size_t kEarlyStepMaxBytes = 16u << 20;
+bool step_early(const mbd_system *s, int ld, int real_bytes) {
+    return (size_t)real_bytes * s->K[0] * s->K[1] * s->K[2] * ld <= kEarlyStepMaxBytes;
+}
+
 // How a field launch is laid out: lanes per atom, atoms at once and in all per
 // block, blocks.
 struct FieldShape {
@@ -1112,6 +1128,7 @@ mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld,
     a.teams = f.teams;
     a.apb = f.apb;
     const dim3 grid(f.blocks, f.chunks);
+    const bool early = step_early(s, ld, (int)sizeof(T));
     if constexpr (sizeof(T) == 4) {
         if (field_streams(s, ld, f, o.terms)) {
             switch (s->p) {
@@ -1119,7 +1136,7 @@ mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld,
     case P: {                                                                                                     \
         const size_t smem = field_stream_smem<P>(f.teams);                                                        \
         MBD_CUDA_TRY(cudaFuncSetAttribute(k_field_stream<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-        k_field_stream<P><<<grid, field_warps<P>() * 32, smem, s->stream>>>(a);                                    \
+        launch_pdl(early, k_field_stream<P>, grid, dim3(field_warps<P>() * 32), smem, s->stream, a);               \
         break;                                                                                                    \
     }
                 MBD_SPLINE_ORDERS(MBD_FIELD_ORDER)
@@ -1132,8 +1149,8 @@ mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld,
     switch (s->p) {
 #define MBD_FIELD_ORDER(P)                                                                \
     case P:                                                                               \
-        if (pairs) k_field<T, P, true><<<grid, field_warps<P>() * 32, 0, s->stream>>>(a);  \
-        else k_field<T, P, false><<<grid, field_warps<P>() * 32, 0, s->stream>>>(a);       \
+        launch_pdl(early, pairs ? k_field<T, P, true> : k_field<T, P, false>, grid,       \
+                   dim3(field_warps<P>() * 32), 0, s->stream, a);                         \
         break;
         MBD_SPLINE_ORDERS(MBD_FIELD_ORDER)
 #undef MBD_FIELD_ORDER

@@ -55,9 +55,8 @@ void set_last_error(const char *where, cudaError_t e);
 // started, so its early blocks take resources only from the predecessor's
 // tail.  Both instructions are no-ops in a kernel launched without the
 // attribute.  Measured per kernel: early launch helps the fused spreading
-// (after the prologue) and the FFT passes while the mesh fits in L2; it slows
-// the FFT passes on meshes beyond L2, and the prologue and field kernels at
-// every size, which are therefore launched plainly.
+// (after the prologue) at every size, the FFT passes while the mesh fits in L2,
+// and the field kernel and the prologues on small meshes only (step_early).
 __device__ __forceinline__ void pdl_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -422,7 +421,7 @@ template <class T> mbd_status launch_field(mbd_system *s, const T *d, const T *m
 // Lanczos
 mbd_status launch_prologue_t(cudaStream_t st, const LanczosView &lz, int k, int m, uint64_t seed, int R, int ld,
                              int rows, const double *g, void *dout, int dtype_bytes, int nblk,
-                             const uint64_t *seed_dev = nullptr);
+                             const uint64_t *seed_dev = nullptr, bool early = false);
 // Quadrature of every probe's tridiagonal, q [R] and, when coef != nullptr,
 // c = Delta^{-1/2} e_1 as coef [m][ld]: MBD_QUAD_CHEBYSHEV (default) runs the
 // Chebyshev kernel and QL for the probes it flags in fallback [ld]; the QL methods
@@ -433,6 +432,8 @@ mbd_status launch_energy_reduce(const double *q, int R, int dim, double omega_su
 mbd_status launch_probes(uint64_t seed, int first, int R, int dim, double *v, cudaStream_t st);
 mbd_status launch_dense_step(const double *c, int dim, const LanczosView &lz, int k, int R, int ld, int nblk,
                              cudaStream_t st);
+// whether the field kernel and the prologues of a run are launched early (launch_pdl)
+bool step_early(const mbd_system *s, int ld, int real_bytes);
 int field_apb(const mbd_system *s, int ld);
 int field_blocks(const mbd_system *s, int ld);
 
