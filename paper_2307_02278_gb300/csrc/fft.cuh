@@ -49,15 +49,22 @@ template <class T> struct SpreadArgs {
 template <class T> int launch_spp_sized(const SpreadArgs<T> &a, cudaStream_t st);
 
 // Sizes with a compile-time pass and their radices (first stage first), in
-// groups of one translation unit each.
-#define MBD_FFT_GROUP0(X) X(16, 4, 4) X(18, 6, 3) X(20, 5, 4) X(24, 6, 4) X(25, 5, 5) X(27, 9, 3) X(30, 6, 5)
-#define MBD_FFT_GROUP1(X) X(32, 8, 4) X(36, 6, 6) X(40, 8, 5) X(45, 9, 5) X(48, 8, 6) X(50, 10, 5) X(54, 9, 6)
-#define MBD_FFT_GROUP2(X) X(60, 10, 6) X(64, 8, 8) X(72, 9, 8) X(75, 15, 5) X(80, 10, 8) X(81, 9, 9) X(90, 10, 9)
-#define MBD_FFT_GROUP3(X) X(96, 12, 8) X(100, 10, 10) X(108, 12, 9) X(120, 12, 10) X(125, 5, 5, 5) X(128, 16, 8) \
-    X(135, 15, 9)
-#define MBD_FFT_GROUP4(X) X(144, 12, 12) X(150, 15, 10) X(160, 16, 10) X(162, 9, 6, 3) X(180, 15, 12) \
-    X(192, 16, 12) X(200, 10, 5, 4)
-#define MBD_FFT_GROUP5(X) X(216, 6, 6, 6) X(225, 15, 15) X(240, 16, 15) X(243, 9, 9, 3) X(250, 10, 5, 5) \
+// groups of one translation unit each.  The largest radix comes last: the last
+// stage has no twiddles to multiply by, and the stages before it keep more
+// threads busy.  us per pass (mean of the four of a convolution), largest first
+// and largest last: 192^3 x 64 probes 661 and 640, 162^3 x 16 122 and 107, 75^3 x 32
+// 24.2 and 20.5, 60^3 x 64 17.6 and 16.8, 40^3 x 16 in double 35.3 and 32.1; spreading
+// with its k3 transform at 180^3 x 64 793 and 708.  45, 72, 80, 108 and 150 are
+// the other way round: in double 72^3 x 16 takes 166 and 173, the spreading at 45^3 x 8 49 and
+// 55; the others differ by less than 1 %, in favour of this order.
+#define MBD_FFT_GROUP0(X) X(16, 4, 4) X(18, 3, 6) X(20, 4, 5) X(24, 4, 6) X(25, 5, 5) X(27, 3, 9) X(30, 5, 6)
+#define MBD_FFT_GROUP1(X) X(32, 4, 8) X(36, 6, 6) X(40, 5, 8) X(45, 9, 5) X(48, 6, 8) X(50, 5, 10) X(54, 6, 9)
+#define MBD_FFT_GROUP2(X) X(60, 6, 10) X(64, 8, 8) X(72, 9, 8) X(75, 5, 15) X(80, 10, 8) X(81, 9, 9) X(90, 9, 10)
+#define MBD_FFT_GROUP3(X) X(96, 8, 12) X(100, 10, 10) X(108, 12, 9) X(120, 10, 12) X(125, 5, 5, 5) X(128, 8, 16) \
+    X(135, 9, 15)
+#define MBD_FFT_GROUP4(X) X(144, 12, 12) X(150, 15, 10) X(160, 10, 16) X(162, 3, 6, 9) X(180, 12, 15) \
+    X(192, 12, 16) X(200, 4, 5, 10)
+#define MBD_FFT_GROUP5(X) X(216, 6, 6, 6) X(225, 15, 15) X(240, 15, 16) X(243, 3, 9, 9) X(250, 5, 5, 10) \
     X(256, 16, 16)
 #define MBD_FFT_NUM_GROUPS 6
 
@@ -798,7 +805,7 @@ template <class T> constexpr int spread_w() { return 16 * spread_ppl<T>(); }
 // pencils have fewer blocks in shared memory and take more warps per block.  us
 // per launch: 120^3 x 64 probes 207 with 4 segments and 221 with 6, 128^3 x 128
 // 490 and 498; 144^3 x 64 363 with 6 and 379 with 5, 160^3 x 64 547 and 556; 192^3
-// x 64 921 with 8, 986 with 6 and 1012 with 10.  Grids of few tiles are bound by a
+// x 64 921 with 8, 986 with 6 and 1012 with 10 (before the order of the radices).  Grids of few tiles are bound by a
 // warp's own chain of records: 8 (40^3 x 8: 9.9 against 10.3).
 template <int K, int P> constexpr int spread_segs(bool few_tiles) {
     constexpr int want = K <= 128 ? 4 : (K <= 160 ? 6 : 8), most = K / (P - 1);
@@ -832,8 +839,8 @@ template <class T, int K, int NSEG> constexpr int spread_blocks() {
 // every record that reaches a warp's rows, and a second buffer for the
 // transform: 192^3 x 64 probes 1507 us per launch; each record once, the rows
 // below a segment through a halo in shared memory: 1139; those rows kept in
-// registers (the walk runs downwards), one block more per SM: 921.  128^3 x 128:
-// 862, 552 and 490; 64^3 x 64: 56, 41 and 37.
+// registers (the walk runs downwards), one block more per SM: 921, and 900 with
+// the largest radix last.  128^3 x 128: 862, 552 and 490; 64^3 x 64: 56, 41 and 37.
 template <class T, class PL, int P, int NSEG>
 __global__ void __launch_bounds__(32 * NSEG, (spread_blocks<T, PL::K, NSEG>()))
     k_spread_pencil_fft3(const T *__restrict__ d, T *__restrict__ mesh, int R, int ld, unsigned ncols,
