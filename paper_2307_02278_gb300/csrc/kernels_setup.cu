@@ -233,7 +233,10 @@ Geom make_geom(const mbd_system *s) {
 }
 
 // Cell of each atom (cells of width >= rmax along each reciprocal direction)
-// and the atoms per cell.
+// and the atoms per cell.  The positions are wrapped: their fractions lie in
+// [0, 1) up to rounding, which the clamp takes care of.  Wrapping them again
+// would put an atom on a face of a non-orthogonal cell, whose fraction comes
+// back as a residue below zero, into the last cell, away from its position.
 __global__ void k_cell_count(NeighborGrid ng, const double *__restrict__ pos, int *__restrict__ cidx,
                              int *__restrict__ bin_of, int *__restrict__ cnt) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -241,9 +244,8 @@ __global__ void k_cell_count(NeighborGrid ng, const double *__restrict__ pos, in
     int b[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        double f = ng.recip[3 * a] * pos[3 * i] + ng.recip[3 * a + 1] * pos[3 * i + 1] +
-                   ng.recip[3 * a + 2] * pos[3 * i + 2];
-        f -= floor(f);
+        const double f = ng.recip[3 * a] * pos[3 * i] + ng.recip[3 * a + 1] * pos[3 * i + 1] +
+                         ng.recip[3 * a + 2] * pos[3 * i + 2];
         b[a] = min(ng.nc[a] - 1, max(0, (int)floor(f * ng.nc[a])));
         cidx[3 * i + a] = b[a];
     }
