@@ -1090,7 +1090,8 @@ template <class T> FieldShape field_shape(const mbd_system *s, int ld) {
     if (s->tune_field_apb > 0 && tuned_for<T>(s, ld)) {
         f.apb = s->tune_field_apb;
     } else {
-        const long long waves = (s->N + 64 * per_wave - 1) / (64 * per_wave);
+        // at most 64 in whole iterations of `teams` atoms (launch choices hold no more)
+        const long long most = 64 / f.teams * f.teams * per_wave, waves = (s->N + most - 1) / most;
         f.apb = (int)std::max<long long>(1, (s->N + waves * per_wave - 1) / (waves * per_wave));
     }
     f.apb = (f.apb + f.teams - 1) / f.teams * f.teams;
