@@ -5,6 +5,7 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 
 #include "mbd_internal.cuh"
 
@@ -667,23 +668,21 @@ template <class T, class F, class P, int MODE, int W> int launch_ct(const FFTArg
     constexpr int NT = ct_threads<P, W>();
     auto kern = k_fft_ct<T, F, P, MODE, W, NT>;
     const size_t tile = sizeof(Cx<F>) * (size_t)P::K * W, fixed = sizeof(typename TwOf<F>::type) * P::K;
-    static int per_sm[2] = {-1, -1};          // resident blocks per SM with one and two buffers (one architecture)
-    for (int k = 0; k < 2; ++k)
-        if (per_sm[k] < 0) {
-            const size_t smem = fixed + (k + 1) * tile;
-            int x = 0;
-            if ((smem > 48 * 1024 &&
-                 cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) ||
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, kern, NT, smem) != cudaSuccess)
-                x = 0;
-            cudaGetLastError();
-            per_sm[k] = x;
-        }
+    if (allow_smem(kern, fixed + 2 * tile) != cudaSuccess) return 0;
+    static std::atomic<int> per_sm[2];        // resident blocks per SM with one and two buffers (one architecture)
+    int resident[2];
+    for (int k = 0; k < 2; ++k) {
+        resident[k] = per_sm[k].load(std::memory_order_relaxed);
+        if (resident[k] > 0) continue;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident[k], kern, NT, fixed + (k + 1) * tile) != cudaSuccess ||
+            resident[k] < 1)
+            return 0;
+        per_sm[k].store(resident[k], std::memory_order_relaxed);
+    }
     const unsigned ncols = outer * (unsigned)a.inner, ntiles = (ncols + W - 1) / W;
     const unsigned sms = (unsigned)std::max(1, a.sms);
-    if (per_sm[0] < 1 || per_sm[1] < 1) return 0;
-    const bool once = ntiles <= per_sm[0] * sms;
-    const unsigned grid = once ? ntiles : std::min(ntiles, per_sm[1] * sms);
+    const bool once = ntiles <= resident[0] * sms;
+    const unsigned grid = once ? ntiles : std::min(ntiles, resident[1] * sms);
     const size_t smem = fixed + (once ? 1 : 2) * tile;
     // double passes of a few blocks per SM are bound by the FP64 units: blocks
     // launched early land unevenly on the SMs (64 atoms, 32^3 x 16 probes: 4.2 ms
