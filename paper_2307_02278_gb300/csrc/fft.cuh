@@ -902,11 +902,10 @@ int launch_spp_segs(const SpreadArgs<T> &a, cudaStream_t st) {
     constexpr int K = PL::K, W = spread_w<T>();
     auto kern = k_spread_pencil_fft3<T, PL, P, NSEG>;
     const int V = a.ld / 2;
-    const int pens = (W - 1) / V + 2;              // pencils that a tile can touch
+    const int pens = (W - 1) / V + 2;              // pencils that a tile can touch; most at the smallest V
     const size_t smem = spread_smem<T, K>(pens);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return 0;
+    constexpr int vmin = probe_ld<T>(1) / 2;
+    if (allow_smem(kern, spread_smem<T, K>((W - 1) / vmin + 2)) != cudaSuccess) return 0;
     const unsigned ncols = (unsigned)((size_t)a.K1 * a.K2 * V);
     launch_pdl(true, kern, dim3((ncols + W - 1) / W), dim3(32 * NSEG), smem, st, a.d, a.mesh, a.R, a.ld, ncols, a.prow,
                a.prec, a.k3w, a.tw);

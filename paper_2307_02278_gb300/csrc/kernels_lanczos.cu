@@ -632,10 +632,10 @@ template <class S>
 mbd_status launch_tridiag_s(const double *a, const double *b, const int *length, int R, int ld, int m, double *q,
                             double *coef, int *status, cudaStream_t st, const int *only) {
     const bool full = coef != nullptr;
-    const size_t smem = sizeof(S) * (size_t)(6 * m + (full ? m * (m + 1) : m + 1));
+    auto bytes = [full](int n) { return sizeof(S) * (size_t)(6 * n + (full ? n * (n + 1) : n + 1)); };
+    const size_t smem = bytes(m);
     if (full) {
-        if (smem > 48 * 1024)
-            MBD_CUDA_TRY(cudaFuncSetAttribute(k_tridiag<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        MBD_CUDA_TRY(allow_smem(k_tridiag<S, true>, bytes(kMaxSteps)));
         k_tridiag<S, true><<<R, 64, smem, st>>>(a, b, length, R, ld, m, q, coef, status, only);
     } else {
         k_tridiag<S, false><<<R, 64, smem, st>>>(a, b, length, R, ld, m, q, nullptr, status, only);

@@ -252,13 +252,13 @@ __global__ void __launch_bounds__(256) k_fft_pass(FFTArgs<T> a) {
 
 // The generic pass over columns of Cx<F> (a.inner, a.V and a.W in that unit);
 // the tile narrows until its two buffers fit in shared memory.
+constexpr size_t kGenericPassSmem = 200 * 1024;
 template <class T, class F> mbd_status launch_fft_generic(FFTArgs<T> a, int mode, unsigned outer, cudaStream_t st) {
     auto bytes = [&] { return sizeof(typename TwOf<F>::type) * a.K + 2 * sizeof(Cx<F>) * (size_t)a.K * a.W; };
-    while (a.W > 1 && bytes() > 200 * 1024) a.W = (a.W + 1) / 2;
+    while (a.W > 1 && bytes() > kGenericPassSmem) a.W = (a.W + 1) / 2;
     auto kern = mode == 0 ? k_fft_pass<T, F, 0> : (mode == 1 ? k_fft_pass<T, F, 1> : k_fft_pass<T, F, 2>);
     const size_t smem = bytes();
-    if (smem > 48 * 1024)
-        MBD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MBD_CUDA_TRY(allow_smem(kern, kGenericPassSmem));
     kern<<<(unsigned)((size_t)outer * ((a.inner + a.W - 1) / a.W)), 256, smem, st>>>(a);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
@@ -293,6 +293,7 @@ template <class T> struct RealArgs {
 // An atom's field is a sum in a fixed order (per group, then the groups).
 constexpr int kRealBatch = 32;
 constexpr int kRealStageBytes = 36 * 1024;
+constexpr int kRealMaxEntries = 192;      // staged at a time
 template <class T>
 __global__ void __launch_bounds__(16 * kClusterSize, sizeof(T) == 4 ? 3 : 2) k_real_clusters(RealArgs<T> a) {
     constexpr int VEC = 16 / (int)sizeof(T), NW = kClusterSize / 2;
@@ -1043,18 +1044,18 @@ namespace {
 // Resident blocks per SM of one field-kernel variant (the same on every
 // device of one architecture), asked of the occupancy calculator once.
 template <class T, int P, bool PAIRS> int field_occupancy() {
-    static int nb = 0;
-    if (nb == 0) {
-        int x = 0;
+    static std::atomic<int> nb;
+    int x = nb.load(std::memory_order_relaxed);
+    if (x == 0) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&x, k_field<T, P, PAIRS>, field_warps<P>() * 32, 0) !=
                 cudaSuccess ||
             x < 1) {
             cudaGetLastError();
-            x = 1;
+            return 1;
         }
-        nb = x;
+        nb.store(x, std::memory_order_relaxed);
     }
-    return nb;
+    return x;
 }
 
 // Lanes per atom: just enough for the probes of a chunk (32 VEC at most).  In
@@ -1101,8 +1102,9 @@ template <class T> FieldShape field_shape(const mbd_system *s, int ld) {
 // The streaming kernel: FP32 with the real space on clusters, at least 32
 // probes (four groups per warp at most), whole iterations' worth of atoms, the
 // mesh term wanted.
+constexpr int kFieldStreamLanes = 8;
 bool field_streams(const mbd_system *s, int ld, const FieldShape &f, int terms) {
-    return s->precision != MBD_FP64 && real_on_clusters(s, ld, 4) && f.lanes >= 8 && f.teams == 32 / f.lanes &&
+    return s->precision != MBD_FP64 && real_on_clusters(s, ld, 4) && f.lanes >= kFieldStreamLanes && f.teams == 32 / f.lanes &&
            (terms & MBD_TERM_RECIP);
 }
 }  // namespace
@@ -1136,7 +1138,7 @@ mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld,
 #define MBD_FIELD_ORDER(P)                                                                                        \
     case P: {                                                                                                     \
         const size_t smem = field_stream_smem<P>(f.teams);                                                        \
-        MBD_CUDA_TRY(cudaFuncSetAttribute(k_field_stream<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+        MBD_CUDA_TRY(allow_smem(k_field_stream<P>, field_stream_smem<P>(32 / kFieldStreamLanes)));                \
         launch_pdl(early, k_field_stream<P>, grid, dim3(field_warps<P>() * 32), smem, s->stream, a);               \
         break;                                                                                                    \
     }
@@ -1210,11 +1212,13 @@ template <class T> mbd_status launch_real_clusters(mbd_system *s, const T *d, T 
     a.entries = s->cl_entries.as<int>();
     a.recs = P.cA.template as<RealDuo<T>>();
     a.np = ((ld + chunks - 1) / chunks + VEC - 1) / VEC * VEC;
-    a.ce = std::min(192, kRealStageBytes / (3 * a.np * (int)sizeof(T)));
+    a.ce = std::min(kRealMaxEntries, kRealStageBytes / (3 * a.np * (int)sizeof(T)));
     dim3 grid((unsigned)s->n_clusters, (unsigned)((ld + a.np - 1) / a.np));
-    const size_t smem = sizeof(RealDuo<T>) * kClusterSize * kRealBatch + 16 * ((8 * (size_t)a.ce + 15) / 16) +
-                        sizeof(T) * 3 * (size_t)a.np * a.ce;
-    MBD_CUDA_TRY(cudaFuncSetAttribute(k_real_clusters<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    auto bytes = [](size_t ce, size_t dipoles) {
+        return sizeof(RealDuo<T>) * kClusterSize * kRealBatch + 16 * ((8 * ce + 15) / 16) + dipoles;
+    };
+    const size_t smem = bytes(a.ce, sizeof(T) * 3 * (size_t)a.np * a.ce);
+    MBD_CUDA_TRY(allow_smem(k_real_clusters<T>, bytes(kRealMaxEntries, kRealStageBytes)));
     k_real_clusters<T><<<grid, 16 * kClusterSize, smem, st>>>(a);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
