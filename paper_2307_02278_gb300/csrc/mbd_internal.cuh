@@ -77,12 +77,13 @@ inline cudaError_t launch_pdl(bool early, void (*kern)(KArgs...), dim3 grid, dim
     cfg.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<Args &&>(args)...);
 }
-// Dynamic shared memory above 48 KB is allowed per kernel and device.  Asked for at
-// every launch, and always for `most`, the largest size that any launch of the
-// kernel uses: a process may hold systems on several devices, and host threads with
-// a system each launch the same kernel with different sizes.
+// Shared memory above 48 KB has to be allowed per kernel and device: asked for at
+// every launch, and always for `most`, the largest dynamic size that any launch of
+// the kernel uses, because a process may hold systems on several devices and host
+// threads with a system each launch the same kernel with different sizes.  From
+// 44 KB on, as the kernel's own arrays count too (grid_reduce's 2.6 KB).
 template <class Kern> inline cudaError_t allow_smem(Kern kern, size_t most) {
-    if (most <= 48 * 1024) return cudaSuccess;
+    if (most <= 44 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 #define MBD_TRY(expr)                       \
