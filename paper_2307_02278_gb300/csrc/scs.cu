@@ -688,12 +688,12 @@ mbd_status screen(mbd_system *s, int n_freq, double tol, int max_iter, double *a
         MBD_LAUNCH_CHECK();
         iters += n;
         MBD_TRY(read());
+        if (h.flag[0]) return MBD_ERR_NOT_POSITIVE_DEFINITE;   // a stalled column need never converge
         if (h.flag[1]) break;
     }
     k_scs_finish<<<(N + 127) / 128, 128, 0, st>>>(N, ncol, d_x, a.alpha, a.rvdw, d_wq, d_out, d_aiu, d_flag);
     MBD_LAUNCH_CHECK();
     MBD_TRY(read());
-    if (h.flag[0]) return MBD_ERR_NOT_POSITIVE_DEFINITE;
     if (h.flag[3]) return MBD_ERR_NONFINITE;
     double *const to[4] = {alpha_out, omega_out, rvdw_out, c6_out};
     for (int q = 0; q < 4; ++q)
