@@ -738,8 +738,9 @@ template <class T, int PPL> __device__ __forceinline__ void lane_fma(const T *a,
 // registers and go to tail after between() (a barrier where they belong to
 // another warp).  The window of P open rows is a register array whose origin
 // moves with t, unrolled by P so that it never shifts; each row is a sum in a
-// fixed order.  The next record is loaded one ahead.
-template <class T, int P, int PPL, class Begins, class Done, class Between, class Tail>
+// fixed order.  The next record is loaded one ahead.  STARTS: the record starts of
+// P points are loaded together (where they come from global memory).
+template <class T, int P, int PPL, bool STARTS, class Begins, class Done, class Between, class Tail>
 __device__ __forceinline__ void pencil_walk(const T *__restrict__ d, int ld, const PencilRec<T> *__restrict__ prec,
                                             const T *__restrict__ k3w, int t0, int t1, int q0, int q1, Begins &&begins,
                                             Done &&row_done, Between &&between, Tail &&tail) {
@@ -753,10 +754,15 @@ __device__ __forceinline__ void pencil_walk(const T *__restrict__ d, int ld, con
     if (q >= q0) rc = prec[q];
     const int n = t1 - t0;
     for (int sb = 0; sb < n; sb += P) {
+        int starts[P];
+        if constexpr (STARTS) {
+#pragma unroll
+            for (int u = 0; u < P; ++u) starts[u] = begins(max(t0, t1 - 1 - sb - u));
+        }
 #pragma unroll
         for (int u = 0; u < P; ++u) {
             if (sb + u >= n) break;
-            const int t = t1 - 1 - sb - u, qb = begins(t);
+            const int t = t1 - 1 - sb - u, qb = STARTS ? starts[u] : begins(t);
             while (q >= qb) {
                 T x[PPL], y[PPL], z[PPL], w[2 * P];
                 const T *dj = d + (size_t)(3 * rc.atom) * ld;
@@ -870,7 +876,7 @@ __global__ void __launch_bounds__(32 * NSEG, (spread_blocks<T, PL::K, NSEG>()))
     const int pr0 = 2 * (int)(cl - pen * V) + (lane * PPL & 1);   // its first probe
     const int *rpp = rp + (pen - pen0) * K;
     T *mine = tile + lane * PPL;
-    pencil_walk<T, P, PPL>(
+    pencil_walk<T, P, PPL, false>(
         d + pr0, ld, prec, k3w, r0, r1, rpp[r0], rpp[r1], [&](int t) { return rpp[t]; },
         [&](int row, const T *v) {
             T o[PPL];

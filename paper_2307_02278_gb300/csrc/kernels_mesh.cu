@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256) k_spread_pencil(SpreadArgs<T> a, unsigned
     const int pr0 = on ? 2 * (int)(c - pen * V) + (lane * PPL & 1) : 0;
     const int *rp = a.prow + (size_t)pen * K;
     T *out = a.mesh + (size_t)pen * K * a.ld + pr0;
-    pencil_walk<T, P, PPL>(
+    pencil_walk<T, P, PPL, true>(
         a.d + pr0, a.ld, a.prec, a.k3w, r0, r1, rp[r0], rp[r1], [&](int t) { return rp[t]; },
         [&](int row, const T *v) {
             T o[PPL];
@@ -211,9 +211,11 @@ __device__ Cx<F> *stockham(Cx<F> *in, Cx<F> *out, const FFTArgs<T> &a, const typ
 
 // One 1D FFT pass along the middle axis of [outer][K][inner] (values Cx<F>)
 // for the lengths without a compile-time pass; MODE 0 forward, 1 inverse, 2
-// forward, multiplied by G(k1, k2, k3), inverse.
+// forward, multiplied by G(k1, k2, k3), inverse.  A tile is W columns of one
+// outer slab or, where a slab has fewer than W (one or two probes along k3), the
+// whole columns of `slabs` slabs, which are contiguous.
 template <class T, class F, int MODE>
-__global__ void __launch_bounds__(256) k_fft_pass(FFTArgs<T> a) {
+__global__ void __launch_bounds__(256) k_fft_pass(FFTArgs<T> a, unsigned outer, int slabs) {
     using C = Cx<F>;
     using TW = typename TwOf<F>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -221,50 +223,57 @@ __global__ void __launch_bounds__(256) k_fft_pass(FFTArgs<T> a) {
     C *b0 = reinterpret_cast<C *>(tw + a.K);
     C *b1 = b0 + a.K * a.W;
     for (int i = threadIdx.x; i < a.K; i += blockDim.x) tw_set(tw[i], a.tw[i]);
-    const int ncb = (a.inner + a.W - 1) / a.W;
-    const size_t outer = blockIdx.x / ncb;
+    const int ncb = slabs > 1 ? 1 : (a.inner + a.W - 1) / a.W;
+    const size_t o0 = (size_t)(blockIdx.x / ncb) * slabs;
     const int c0 = (int)(blockIdx.x % ncb) * a.W;
-    const int wc = min(a.W, a.inner - c0);
-    C *base = reinterpret_cast<C *>(a.data) + outer * (size_t)a.K * a.inner + c0;
-    for (int idx = threadIdx.x; idx < a.K * a.W; idx += blockDim.x) {
-        const int row = idx / a.W, col = idx - row * a.W;
-        if (col < wc) cst(b0 + idx, cld(base + (size_t)row * a.inner + col));
-    }
+    const int wc = min(a.W, a.inner - c0), ns = (int)min((size_t)slabs, outer - o0);   // columns of a slab, slabs
+    C *base = reinterpret_cast<C *>(a.data) + o0 * (size_t)a.K * a.inner + c0;
+    // element e of the tile: column e % wc, row, slab
+    auto each = [&](auto &&f) {
+        for (int e = threadIdx.x; e < ns * a.K * wc; e += blockDim.x) {
+            const int q = e / wc, col = e - q * wc, sl = slabs > 1 ? q / a.K : 0, row = q - sl * a.K;
+            f(row * a.W + sl * wc + col, base + ((size_t)sl * a.K + row) * a.inner + col, row, col);
+        }
+    };
+    each([&](int t, const C *g, int, int) { cst(b0 + t, cld(g)); });
     __syncthreads();
     C *res;
     if (MODE == 2) {
         res = stockham<T, F, false>(b0, b1, a, tw);
         C *other = (res == b0) ? b1 : b0;
-        // G index: (outer, row, (c0 + col) / V)
-        const T *Gb = a.G + outer * (size_t)a.K * (a.inner / a.V);
-        for (int idx = threadIdx.x; idx < a.K * a.W; idx += blockDim.x) {
-            const int row = idx / a.W, col = idx - row * a.W;
-            if (col < wc) {
-                const T gv = Gb[(size_t)row * (a.inner / a.V) + (c0 + col) / a.V];
-                res[idx] = {fmulc(res[idx].x, gv), fmulc(res[idx].y, gv)};
-            }
-        }
+        // one slab; G index: (row, (c0 + col) / V)
+        each([&](int t, const C *, int row, int col) {
+            const T gv = a.G[(size_t)row * (a.inner / a.V) + (c0 + col) / a.V];
+            res[t] = {fmulc(res[t].x, gv), fmulc(res[t].y, gv)};
+        });
         __syncthreads();
         res = stockham<T, F, true>(res, other, a, tw);
     } else {
         res = stockham<T, F, MODE == 1>(b0, b1, a, tw);
     }
-    for (int idx = threadIdx.x; idx < a.K * a.W; idx += blockDim.x) {
-        const int row = idx / a.W, col = idx - row * a.W;
-        if (col < wc) cst(base + (size_t)row * a.inner + col, cld(res + idx));
-    }
+    each([&](int t, C *g, int, int) { cst(g, cld(res + t)); });
 }
 
-// The generic pass over columns of Cx<F> (a.inner, a.V and a.W in that unit);
-// the tile narrows until its two buffers fit in shared memory.
-constexpr size_t kGenericPassSmem = 200 * 1024;
+// The generic pass over columns of Cx<F> (a.inner, a.V and a.W in that unit).  The
+// tile narrows until two blocks fit an SM (one block of 16 columns left it at eight
+// warps); slabs narrower than a tile are taken together up to four blocks per SM, as
+// far as that leaves two blocks for each.  us for the five passes of 288^3: FP32,
+// up to 4 probes 4236 -> 2439, 8 probes 7239 -> 4913; FP64, 2 probes 10840 -> 8084.
+constexpr size_t kGenericPassSmem = 100 * 1024;
 template <class T, class F> mbd_status launch_fft_generic(FFTArgs<T> a, int mode, unsigned outer, cudaStream_t st) {
-    auto bytes = [&] { return sizeof(typename TwOf<F>::type) * a.K + 2 * sizeof(Cx<F>) * (size_t)a.K * a.W; };
-    while (a.W > 1 && bytes() > kGenericPassSmem) a.W = (a.W + 1) / 2;
+    auto bytes = [&](int w) { return sizeof(typename TwOf<F>::type) * a.K + 2 * sizeof(Cx<F>) * (size_t)a.K * w; };
+    a.W = std::min(a.inner, 16);
+    while (a.W > 1 && bytes(a.W) > kGenericPassSmem) a.W = (a.W + 1) / 2;
+    int slabs = 1;
+    if (a.W == a.inner && mode != 2) {
+        slabs = (int)std::max(1u, std::min(16u / a.W, outer / (2u * (unsigned)std::max(1, a.sms))));
+        while (slabs > 1 && bytes(slabs * a.W) > kGenericPassSmem / 2) --slabs;
+        a.W *= slabs;
+    }
     auto kern = mode == 0 ? k_fft_pass<T, F, 0> : (mode == 1 ? k_fft_pass<T, F, 1> : k_fft_pass<T, F, 2>);
-    const size_t smem = bytes();
+    const unsigned grid = slabs > 1 ? (outer + slabs - 1) / slabs : outer * (unsigned)((a.inner + a.W - 1) / a.W);
     MBD_CUDA_TRY(allow_smem(kern, kGenericPassSmem));
-    kern<<<(unsigned)((size_t)outer * ((a.inner + a.W - 1) / a.W)), 256, smem, st>>>(a);
+    kern<<<grid, 256, bytes(a.W), st>>>(a, outer, slabs);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }
@@ -1021,7 +1030,6 @@ template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bo
             a.inner /= 2;
             a.V /= 2;
         }
-        a.W = std::min(a.inner, 16);
         return launch_fft_generic<T, typename PackOf<T>::type>(a, mode, (unsigned)outer, s->stream);
     };
     if (!skip_first) MBD_TRY(run(2, K1 * K2, V, 0));   // forward along k3
