@@ -668,13 +668,14 @@ template <class T, class F, class P, int MODE, int W> int launch_ct(const FFTArg
     constexpr int NT = ct_threads<P, W>();
     auto kern = k_fft_ct<T, F, P, MODE, W, NT>;
     const size_t tile = sizeof(Cx<F>) * (size_t)P::K * W, fixed = sizeof(typename TwOf<F>::type) * P::K;
-    if (allow_smem(kern, fixed + 2 * tile) != cudaSuccess) return 0;
+    const size_t most = fixed + 2 * tile;
     static std::atomic<int> per_sm[2];        // resident blocks per SM with one and two buffers (one architecture)
     int resident[2];
     for (int k = 0; k < 2; ++k) {
         resident[k] = per_sm[k].load(std::memory_order_relaxed);
         if (resident[k] > 0) continue;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident[k], kern, NT, fixed + (k + 1) * tile) != cudaSuccess ||
+        if (allow_smem(kern, most, most) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident[k], kern, NT, fixed + (k + 1) * tile) != cudaSuccess ||
             resident[k] < 1)
             return 0;
         per_sm[k].store(resident[k], std::memory_order_relaxed);
@@ -684,6 +685,7 @@ template <class T, class F, class P, int MODE, int W> int launch_ct(const FFTArg
     const bool once = ntiles <= resident[0] * sms;
     const unsigned grid = once ? ntiles : std::min(ntiles, resident[1] * sms);
     const size_t smem = fixed + (once ? 1 : 2) * tile;
+    if (allow_smem(kern, smem, most) != cudaSuccess) return 0;
     // double passes of a few blocks per SM are bound by the FP64 units: blocks
     // launched early land unevenly on the SMs (64 atoms, 32^3 x 16 probes: 4.2 ms
     // per energy + forces against 3.6); one block per SM or persistent blocks
@@ -911,7 +913,7 @@ int launch_spp_segs(const SpreadArgs<T> &a, cudaStream_t st) {
     const int pens = (W - 1) / V + 2;              // pencils that a tile can touch; most at the smallest V
     const size_t smem = spread_smem<T, K>(pens);
     constexpr int vmin = probe_ld<T>(1) / 2;
-    if (allow_smem(kern, spread_smem<T, K>((W - 1) / vmin + 2)) != cudaSuccess) return 0;
+    if (allow_smem(kern, smem, spread_smem<T, K>((W - 1) / vmin + 2)) != cudaSuccess) return 0;
     const unsigned ncols = (unsigned)((size_t)a.K1 * a.K2 * V);
     launch_pdl(true, kern, dim3((ncols + W - 1) / W), dim3(32 * NSEG), smem, st, a.d, a.mesh, a.R, a.ld, ncols, a.prow,
                a.prec, a.k3w, a.tw);

@@ -635,7 +635,7 @@ mbd_status launch_tridiag_s(const double *a, const double *b, const int *length,
     auto bytes = [full](int n) { return sizeof(S) * (size_t)(6 * n + (full ? n * (n + 1) : n + 1)); };
     const size_t smem = bytes(m);
     if (full) {
-        MBD_CUDA_TRY(allow_smem(k_tridiag<S, true>, bytes(kMaxSteps)));
+        MBD_CUDA_TRY(allow_smem(k_tridiag<S, true>, smem, bytes(kMaxSteps)));
         k_tridiag<S, true><<<R, 64, smem, st>>>(a, b, length, R, ld, m, q, coef, status, only);
     } else {
         k_tridiag<S, false><<<R, 64, smem, st>>>(a, b, length, R, ld, m, q, nullptr, status, only);

@@ -272,7 +272,7 @@ template <class T, class F> mbd_status launch_fft_generic(FFTArgs<T> a, int mode
     }
     auto kern = mode == 0 ? k_fft_pass<T, F, 0> : (mode == 1 ? k_fft_pass<T, F, 1> : k_fft_pass<T, F, 2>);
     const unsigned grid = slabs > 1 ? (outer + slabs - 1) / slabs : outer * (unsigned)((a.inner + a.W - 1) / a.W);
-    MBD_CUDA_TRY(allow_smem(kern, kGenericPassSmem));
+    MBD_CUDA_TRY(allow_smem(kern, bytes(a.W), kGenericPassSmem));
     kern<<<grid, 256, bytes(a.W), st>>>(a, outer, slabs);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
@@ -1155,7 +1155,7 @@ mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld,
 #define MBD_FIELD_ORDER(P)                                                                                        \
     case P: {                                                                                                     \
         const size_t smem = field_stream_smem<P>(f.teams);                                                        \
-        MBD_CUDA_TRY(allow_smem(k_field_stream<P>, field_stream_smem<P>(32 / kFieldStreamLanes)));                \
+        MBD_CUDA_TRY(allow_smem(k_field_stream<P>, smem, field_stream_smem<P>(32 / kFieldStreamLanes)));          \
         launch_pdl(early, k_field_stream<P>, grid, dim3(field_warps<P>() * 32), smem, s->stream, a);               \
         break;                                                                                                    \
     }
@@ -1235,7 +1235,7 @@ template <class T> mbd_status launch_real_clusters(mbd_system *s, const T *d, T 
         return sizeof(RealDuo<T>) * kClusterSize * kRealBatch + 16 * ((8 * ce + 15) / 16) + dipoles;
     };
     const size_t smem = bytes(a.ce, sizeof(T) * 3 * (size_t)a.np * a.ce);
-    MBD_CUDA_TRY(allow_smem(k_real_clusters<T>, bytes(kRealMaxEntries, kRealStageBytes)));
+    MBD_CUDA_TRY(allow_smem(k_real_clusters<T>, smem, bytes(kRealMaxEntries, kRealStageBytes)));
     k_real_clusters<T><<<grid, 16 * kClusterSize, smem, st>>>(a);
     MBD_LAUNCH_CHECK();
     return MBD_OK;

@@ -723,7 +723,7 @@ template <class T> mbd_status launch_cluster_pairs(mbd_system *s, cudaStream_t s
     MBD_LAUNCH_CHECK();
     MBD_TRY(launch_exclusive_scan(s->cl_pcnt.as<int>(), s->cl_pstart.as<int>(), nslots, s->scan_bsum, st));
     const size_t smem = (size_t)kClusterSortCap * (sizeof(unsigned long long) + 3 * sizeof(int) + 1);
-    MBD_CUDA_TRY(allow_smem(k_cluster_pairs<T>, smem));
+    MBD_CUDA_TRY(allow_smem(k_cluster_pairs<T>, smem, smem));
     k_cluster_pairs<T><<<nclus, kClusterThreads, smem, st>>>(
         s->N, s->order_d.as<int>(), s->row_d.as<int>(), s->col_d.as<int>(), s->shift_d.as<int>(),
         P.pairA.template as<T>(), s->cl_pstart.as<int>(), s->cl_ecnt.as<int>(), s->cl_rcnt.as<int>(), s->cl_entries.as<int>(),

@@ -78,12 +78,12 @@ inline cudaError_t launch_pdl(bool early, void (*kern)(KArgs...), dim3 grid, dim
     return cudaLaunchKernelEx(&cfg, kern, static_cast<Args &&>(args)...);
 }
 // Shared memory above 48 KB has to be allowed per kernel and device: asked for at
-// every launch, and always for `most`, the largest dynamic size that any launch of
-// the kernel uses, because a process may hold systems on several devices and host
-// threads with a system each launch the same kernel with different sizes.  From
-// 44 KB on, as the kernel's own arrays count too (grid_reduce's 2.6 KB).
-template <class Kern> inline cudaError_t allow_smem(Kern kern, size_t most) {
-    if (most <= 44 * 1024) return cudaSuccess;
+// every launch that needs it, and always for `most`, the largest dynamic size that
+// any launch of the kernel uses, because a process may hold systems on several devices
+// and host threads with a system each launch the same kernel with different sizes.
+// From 44 KB on, as the kernel's own arrays count too (grid_reduce's 2.6 KB).
+template <class Kern> inline cudaError_t allow_smem(Kern kern, size_t need, size_t most) {
+    if (need <= 44 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 #define MBD_TRY(expr)                       \
