@@ -21,7 +21,7 @@ template <class T> struct FFTArgs {
     int nst;
     unsigned long long radices;   // stage s radix = (radices >> 4 s) & 15
     int V;               // complex probe pairs per mesh point (fused pass: G index = e / V)
-    int early;           // compile-time passes: programmatic dependent launch (1) or plain (0)
+    int early;           // compile-time passes: programmatic dependent launch (1; 2: of every double pass too) or plain (0)
     int sms;             // multiprocessors
 };
 
@@ -690,7 +690,7 @@ template <class T, class F, class P, int MODE, int W> int launch_ct(const FFTArg
     // launched early land unevenly on the SMs (64 atoms, 32^3 x 16 probes: 4.2 ms
     // per energy + forces against 3.6); one block per SM or persistent blocks
     // are even in any case
-    const bool early = a.early != 0 && (sizeof(T) == 4 || !once || grid <= sms);
+    const bool early = a.early == 2 || (a.early == 1 && (sizeof(T) == 4 || !once || grid <= sms));
     launch_pdl(early, kern, dim3(grid), dim3(NT), smem, st, a, ncols, ntiles);
     return 1;
 }

@@ -942,6 +942,10 @@ template <class T> mbd_status launch_spread(mbd_system *s, const T *d, T *mesh, 
 // Meshes of at most this many bytes (three quarters of the 129 MB L2) launch
 // their FFT passes with programmatic dependence; larger ones plainly.
 constexpr size_t kEarlyFFTMaxBytes = 96u << 20;
+// A convolution on its own launches its double passes early as well while the mesh is
+// small: us per mbd_convolve, plain and early, 16^3 x 32 probes 64 and 49, 20^3 x 32 80
+// and 69, 32^3 x 16 104 and 90, 40^3 x 16 (8 MB) 193 and 209.
+constexpr size_t kEarlyAloneMaxBytes = 4u << 20;
 
 #define MBD_HAS_CASE(K, ...) case K:
 bool fft_ct_size(int K) {
@@ -994,7 +998,7 @@ template <class T> mbd_status launch_spread_fft3(mbd_system *s, const T *d, T *m
     return MBD_OK;
 }
 
-template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bool skip_first) {
+template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bool skip_first, bool alone) {
     using C = typename Cplx<T>::type;
     PrecData<T> &P = prec<T>(s);
     const int V = ld / 2;
@@ -1012,7 +1016,7 @@ template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bo
         a.inner = inner;
         a.V = V;
         // early launch of the passes while the mesh fits in three quarters of L2
-        a.early = npts_bytes <= kEarlyFFTMaxBytes ? 1 : 0;
+        a.early = npts_bytes > kEarlyFFTMaxBytes ? 0 : (alone && npts_bytes <= kEarlyAloneMaxBytes ? 2 : 1);
         a.sms = s->num_sms;
         // wide tiles unless they are too few for four blocks per SM
         a.W = (size_t)outer * inner >= (size_t)128 * a.sms ? 32 : 16;
@@ -1245,8 +1249,8 @@ template mbd_status build_spread_records<double>(mbd_system *);
 template mbd_status build_spread_records<float>(mbd_system *);
 template mbd_status launch_spread<double>(mbd_system *, const double *, double *, int, int);
 template mbd_status launch_spread<float>(mbd_system *, const float *, float *, int, int);
-template mbd_status launch_convolve<double>(mbd_system *, double *, int, bool);
-template mbd_status launch_convolve<float>(mbd_system *, float *, int, bool);
+template mbd_status launch_convolve<double>(mbd_system *, double *, int, bool, bool);
+template mbd_status launch_convolve<float>(mbd_system *, float *, int, bool, bool);
 template mbd_status launch_spread_fft3<double>(mbd_system *, const double *, double *, int, int);
 template mbd_status launch_spread_fft3<float>(mbd_system *, const float *, float *, int, int);
 template mbd_status launch_field<double>(mbd_system *, const double *, const double *, int, int,

@@ -410,8 +410,10 @@ template <class T> mbd_status launch_influence(mbd_system *s, const double *bmod
 // mesh stages
 template <class T> mbd_status launch_spread(mbd_system *s, const T *d, T *mesh, int R, int ld);
 template <class T> mbd_status build_spread_records(mbd_system *s);
-// in place; skip_first: the forward k3 pass was already done (launch_spread_fft3)
-template <class T> mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bool skip_first = false);
+// in place; skip_first: the forward k3 pass was already done (launch_spread_fft3);
+// alone: not between the kernels of a product
+template <class T>
+mbd_status launch_convolve(mbd_system *s, T *mesh, int ld, bool skip_first = false, bool alone = false);
 template <class T> mbd_status launch_spread_fft3(mbd_system *s, const T *d, T *mesh, int R, int ld);
 bool spread_fft3_supported(const mbd_system *s);
 bool fft_ct_size(int K);        // a compile-time FFT pass exists for this length
