@@ -83,7 +83,13 @@ __global__ void k_pencil_k3w(int N, int p, const double *__restrict__ w64, const
     k3w[idx] = T(t < p ? w64[(size_t)(3 * j + 2) * p + t] : dw64[(size_t)(3 * j + 2) * p + t - p]);
 }
 
-// Exclusive scan of n counts (blocks of 4096), the block sums, and the fix-up.
+// Exclusive scan of n counts (blocks of 4096), the block sums, and the fix-up.  Sums
+// stop at 2^31 - 1 instead of wrapping to negative starts: kernels may read the
+// starts of a scan that has overflowed before the host sees its total, -1.
+__device__ __forceinline__ int sat_add(int a, int b) {   // a, b >= 0
+    const unsigned s = (unsigned)a + (unsigned)b;
+    return s > 0x7fffffffu ? 0x7fffffff : (int)s;
+}
 __global__ void __launch_bounds__(1024) k_scan_block(const int *__restrict__ in, int *__restrict__ out,
                                                      int *__restrict__ bsum, int n) {
     __shared__ int sh[1024];
@@ -92,20 +98,20 @@ __global__ void __launch_bounds__(1024) k_scan_block(const int *__restrict__ in,
     int v[4], tsum = 0;
     for (int k = 0; k < 4; ++k) {
         v[k] = (base + k < n) ? in[base + k] : 0;
-        tsum += v[k];
+        tsum = sat_add(tsum, v[k]);
     }
     sh[tid] = tsum;
     __syncthreads();
     for (int off = 1; off < 1024; off <<= 1) {
         const int t = tid >= off ? sh[tid - off] : 0;
         __syncthreads();
-        sh[tid] += t;
+        sh[tid] = sat_add(sh[tid], t);
         __syncthreads();
     }
-    int excl = sh[tid] - tsum;
+    int excl = tid > 0 ? sh[tid - 1] : 0;
     for (int k = 0; k < 4; ++k) {
         if (base + k < n) out[base + k] = excl;
-        excl += v[k];
+        excl = sat_add(excl, v[k]);
     }
     if (tid == 1023) bsum[blockIdx.x] = sh[1023];
 }
@@ -114,14 +120,14 @@ __global__ void k_scan_sums(int *__restrict__ bsum, int nb, int *__restrict__ to
     long long acc = 0;
     for (int b = 0; b < nb; ++b) {
         const int t = bsum[b];
-        bsum[b] = (int)acc;
+        bsum[b] = (int)min(acc, 0x7fffffffLL);
         acc += t;
     }
-    *total = acc > 0x7fffffffLL ? -1 : (int)acc;
+    *total = acc >= 0x7fffffffLL ? -1 : (int)acc;
 }
 __global__ void k_scan_add(int *__restrict__ out, const int *__restrict__ bsum, int n) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] += bsum[i / 4096];
+    if (i < n) out[i] = sat_add(out[i], bsum[i / 4096]);
 }
 
 // The spreading alone, for mesh lengths without a fused pass and for the

@@ -100,8 +100,8 @@ __global__ void k_pair_tensors(int N, const double *__restrict__ pos, const doub
     const int i = w / parts, sub = w - i * parts, lane = threadIdx.x & 31;
     if (i >= N) return;
     const double xi = pos[3 * i], yi = pos[3 * i + 1], zi = pos[3 * i + 2];
-    const int nb1 = (int)min((long long)row[i + 1], cap);   // pairs beyond the buffers: rebuilt by the caller
-    for (int nb = row[i] + 32 * sub + lane; nb < nb1; nb += 32 * parts) {
+    const long long nb1 = min((long long)row[i + 1], cap);   // pairs beyond the buffers: rebuilt by the caller
+    for (long long nb = row[i] + 32LL * sub + lane; nb < nb1; nb += 32 * parts) {
         const int j = col[nb];
         const int sh = shift[nb];
         const double n1 = double((sh & 255) - 128), n2 = double(((sh >> 8) & 255) - 128),
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(128) k_neighbors(NeighborGrid ng, const double
         }
         const unsigned bal = __ballot_sync(0xffffffffu, hit);
         if (FILL && hit) {
-            const int at = base + c + __popc(bal & ((1u << lane) - 1u));
+            const long long at = (long long)base + c + __popc(bal & ((1u << lane) - 1u));
             if (at < cap) {
                 col[at] = e.x;
                 shift[at] = e.y;
