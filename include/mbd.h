@@ -118,7 +118,10 @@ mbd_status mbd_create_system(const mbd_system_desc *desc, void *cuda_stream, mbd
 void mbd_destroy_system(mbd_system *sys);
 
 /* New positions (host [N][3], bohr) for the same atoms and cell; rebuilds the
- * neighbour list and spline stencils. */
+ * neighbour list and spline stencils.  Positions that are not finite are refused
+ * and change nothing.  After any other error (MBD_ERR_OOM, or MBD_ERR_INVALID_ARG
+ * for 2^31 - 1 pairs or more) the system has no geometry: calls that need one
+ * return MBD_ERR_INVALID_ARG until an update succeeds. */
 mbd_status mbd_update_positions(mbd_system *sys, const double *pos);
 
 /* y = C x for a block of vectors (Eqs. ccd, lk3): x_dev, y_dev are device

@@ -198,6 +198,7 @@ void wrap_positions(mbd_system *s, const double *pos) {
 // room so that small changes of the list between steps need no reallocation.
 mbd_status size_pair_buffers(mbd_system *s, long long nnz) {
     const long long cap = std::max<long long>(1, nnz + nnz / 4 + 32);
+    s->nb_cap = 0;                              // should one of them fail, the next build sizes both again
     MBD_TRY(s->col_d.ensure(sizeof(int) * (size_t)cap));
     MBD_TRY(s->shift_d.ensure(sizeof(int) * (size_t)cap));
     s->nb_cap = cap;
@@ -363,8 +364,11 @@ template <class T> mbd_status upload_twiddles(mbd_system *s) {
 // Positions to neighbour list, pair tensors, splines, bricks and spreading
 // matrix, all queued on the stream; one readback at the end gives the pair
 // count and the error flags.  A list that outgrew its buffers is filled again
-// into larger ones, with its pair tensors.
+// into larger ones, with its pair tensors.  After a failure part of the lists are of
+// the new positions, and a buffer may be gone: check_geometry refuses the calls that
+// read them until an update succeeds.
 template <class T> mbd_status setup_geometry(mbd_system *s) {
+    s->geometry_ok = false;
     MBD_CUDA_TRY(cudaMemcpyAsync(s->pos_d.ptr, s->pos.data(), sizeof(double) * 3 * s->N, cudaMemcpyHostToDevice,
                                  s->stream));
     MBD_TRY(build_neighbors(s));
@@ -393,6 +397,7 @@ template <class T> mbd_status setup_geometry(mbd_system *s) {
     MBD_CUDA_TRY(cudaMemcpyAsync(&cerr, s->cl_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
     MBD_CUDA_TRY(cudaStreamSynchronize(s->stream));
     s->real_clusters = cerr == 0;
+    s->geometry_ok = true;
     return MBD_OK;
 }
 
@@ -993,10 +998,16 @@ template <class T> mbd_status autotune_impl(mbd_system *s, int R, int32_t *out) 
 mbd_status check_run_args(mbd_system *s, int R, int m, double *energy) {
     if (!s || !energy) return MBD_ERR_INVALID_ARG;
     if (R < 1 || R > (1 << 20) || m < 1 || m > kMaxSteps) return MBD_ERR_INVALID_ARG;
-    return MBD_OK;
+    return check_geometry(s);
 }
 
 }  // namespace
+
+mbd_status check_geometry(const mbd_system *s) {
+    if (s->geometry_ok) return MBD_OK;
+    g_last_error = "the last mbd_update_positions of this system failed";
+    return MBD_ERR_INVALID_ARG;
+}
 }  // namespace mbd
 
 using namespace mbd;
@@ -1159,6 +1170,7 @@ mbd_status mbd_batch_get_info(const mbd_batch *b, mbd_batch_info *info) {
 
 mbd_status mbd_autotune(mbd_system *s, int32_t n_probes, int32_t choices[4]) {
     if (!s || n_probes < 1 || n_probes > (1 << 20)) return MBD_ERR_INVALID_ARG;
+    MBD_TRY(check_geometry(s));
     if (s->precision == MBD_FP64) return autotune_impl<double>(s, n_probes, choices);
     return autotune_impl<float>(s, n_probes, choices);
 }
@@ -1196,6 +1208,7 @@ mbd_status mbd_update_positions(mbd_system *s, const double *pos) {
 
 mbd_status mbd_apply_C(mbd_system *s, int32_t nvec, const double *x_dev, double *y_dev) {
     if (!s || !x_dev || !y_dev || nvec < 1 || nvec > (1 << 20) || x_dev == y_dev) return MBD_ERR_INVALID_ARG;
+    MBD_TRY(check_geometry(s));
     if (s->precision == MBD_FP64) return apply_impl<double>(s, nvec, x_dev, y_dev, MBD_TERM_ALL, false);
     return apply_impl<float>(s, nvec, x_dev, y_dev, MBD_TERM_ALL, false);
 }
@@ -1203,12 +1216,14 @@ mbd_status mbd_apply_C(mbd_system *s, int32_t nvec, const double *x_dev, double 
 mbd_status mbd_field(mbd_system *s, int32_t nvec, const double *d_dev, double *e_dev, int32_t terms) {
     if (!s || !d_dev || !e_dev || nvec < 1 || nvec > (1 << 20) || d_dev == e_dev) return MBD_ERR_INVALID_ARG;
     if (terms < 0 || terms > MBD_TERM_ALL) return MBD_ERR_INVALID_ARG;
+    MBD_TRY(check_geometry(s));
     if (s->precision == MBD_FP64) return apply_impl<double>(s, nvec, d_dev, e_dev, terms, true);
     return apply_impl<float>(s, nvec, d_dev, e_dev, terms, true);
 }
 
 mbd_status mbd_spread(mbd_system *s, int32_t nvec, const double *d_dev, double *mesh_dev) {
     if (!s || !d_dev || !mesh_dev || nvec < 1 || nvec > (1 << 16)) return MBD_ERR_INVALID_ARG;
+    MBD_TRY(check_geometry(s));
     if (s->precision == MBD_FP64) return spread_impl<double>(s, nvec, d_dev, mesh_dev);
     return spread_impl<float>(s, nvec, d_dev, mesh_dev);
 }

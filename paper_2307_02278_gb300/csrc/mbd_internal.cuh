@@ -362,6 +362,7 @@ struct mbd_system {
     bool real_clusters = false;                     // the clusters of the last geometry were built
     int real_method = MBD_REAL_AUTO;                // mbd_set_real_space_method
     mbd::DevBuf scan_cnt, scan_bsum;                // count / scan scratch of the geometry setup
+    bool geometry_ok = false;   // the lists and records below are those of the positions (setup_geometry)
     long long nb_cap = 0;   // pairs col_d, shift_d and the pair tensors hold (0: not sized yet)
     mbd::NeighborGrid ngrid{};   // the last neighbour search's grid
     mbd::BinView bins;
@@ -471,6 +472,7 @@ mbd_status launch_force_gather_t(mbd_system *s, const T *dpq, const T *mesh, int
                                  double *forces);
 
 // misc
+mbd_status check_geometry(const mbd_system *s);   // MBD_ERR_INVALID_ARG after a failed update
 // Padded probe count of arrays of T: even, a multiple of four for float (16-byte
 // rows, probe pairs packed two by two in the FFT passes).
 template <class T> constexpr int probe_ld(int R) {

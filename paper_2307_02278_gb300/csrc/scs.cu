@@ -714,6 +714,7 @@ extern "C" mbd_status mbd_scs_screen(mbd_system *s, int32_t n_freq, double tol, 
     if (!s || !alpha_out || !omega_out || !r_vdw_out) return MBD_ERR_INVALID_ARG;
     if (n_freq < 1 || n_freq > 31 || !(tol > 0.0) || !std::isfinite(tol) || max_iter < 0 || max_iter > 100000)
         return MBD_ERR_INVALID_ARG;
+    MBD_TRY(mbd::check_geometry(s));
     if (s->precision == MBD_FP64)
         return mbd::screen<double>(s, n_freq, tol, max_iter, alpha_out, omega_out, r_vdw_out, c6_out, alpha_iu_out,
                                    iterations, residual);
