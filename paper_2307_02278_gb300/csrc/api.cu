@@ -778,7 +778,8 @@ template <class T> mbd_status apply_impl(mbd_system *s, int nvec, const double *
     std::memset(&fo.lz, 0, sizeof(fo.lz));
     if (real_on_clusters(s, ld, (int)sizeof(T)) && (terms & MBD_TERM_REAL))
         MBD_STAGE(s, MBD_STAGE_REAL, 1,
-                  launch_real_clusters<T>(s, P.d.template as<T>(), P.ereal.template as<T>(), ld, s->stream));
+                  launch_real_clusters<T>(s, P.d.template as<T>(), P.ereal.template as<T>(), ld, s->stream,
+                                          !(terms & MBD_TERM_RECIP)));
     MBD_STAGE(s, MBD_STAGE_FIELD, 1, launch_field<T>(s, P.d.template as<T>(), P.mesh.template as<T>(), nvec, ld, fo));
     MBD_STAGE(s, MBD_STAGE_OTHER, 1, launch_from_probe_major(yt, nvec, rows, ld, y, s->stream));
     MBD_CUDA_TRY(cudaStreamSynchronize(s->stream));

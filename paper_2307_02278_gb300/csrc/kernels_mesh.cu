@@ -314,7 +314,12 @@ template <class T> struct RealArgs {
 constexpr int kRealBatch = 32;
 constexpr int kRealStageBytes = 36 * 1024;
 constexpr int kRealMaxEntries = 192;      // staged at a time
-template <class T>
+// MASKED: an atom that has no pair with the neighbour of a record is left out.  FP64 is
+// bound by its FMAs and gains by it.  FP32 gives it the record's zero tensor, which
+// is quicker (24,000 atoms x 64 probes 147 against 174 us), but not the same when the
+// neighbour's dipole is not finite: only right where one such dipole reaches
+// every atom anyway, by the mesh.
+template <class T, bool MASKED>
 __global__ void __launch_bounds__(16 * kClusterSize, sizeof(T) == 4 ? 3 : 2) k_real_clusters(RealArgs<T> a) {
     constexpr int VEC = 16 / (int)sizeof(T), NW = kClusterSize / 2;
     constexpr int RC = (int)sizeof(RealDuo<T>) / 16;       // 16-byte pieces of a record
@@ -394,8 +399,7 @@ __global__ void __launch_bounds__(16 * kClusterSize, sizeof(T) == 4 ? 3 : 2) k_r
                     for (int q = 0; q < 12; q += VEC) vload<T, VEC>(cur.a + q, A + q);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        // FP64 is bound by its FMAs: tensors that are zero are skipped
-                        if (sizeof(T) == 8 && !(cur.mask & (1 << h))) continue;
+                        if (MASKED && !(cur.mask & (1 << h))) continue;
                         const T *B = A + 6 * h;
                         lane_fma<T, VEC>(x, B[0], E[h][0]);
                         lane_fma<T, VEC>(y, B[1], E[h][0]);
@@ -1222,7 +1226,8 @@ bool real_on_clusters(const mbd_system *s, int ld, int real_bytes) {
 
 // E_real of every atom from the clusters (the caller runs this before
 // launch_field whenever real_on_clusters holds and the real-space term is wanted).
-template <class T> mbd_status launch_real_clusters(mbd_system *s, const T *d, T *ereal, int ld, cudaStream_t st) {
+template <class T>
+mbd_status launch_real_clusters(mbd_system *s, const T *d, T *ereal, int ld, cudaStream_t st, bool local) {
     PrecData<T> &P = prec<T>(s);
     constexpr int VEC = 16 / (int)sizeof(T);
     if (s->n_clusters == 0) return MBD_OK;
@@ -1245,8 +1250,9 @@ template <class T> mbd_status launch_real_clusters(mbd_system *s, const T *d, T 
         return sizeof(RealDuo<T>) * kClusterSize * kRealBatch + 16 * ((8 * ce + 15) / 16) + dipoles;
     };
     const size_t smem = bytes(a.ce, sizeof(T) * 3 * (size_t)a.np * a.ce);
-    MBD_CUDA_TRY(allow_smem(k_real_clusters<T>, smem, bytes(kRealMaxEntries, kRealStageBytes)));
-    k_real_clusters<T><<<grid, 16 * kClusterSize, smem, st>>>(a);
+    auto kern = sizeof(T) == 8 || local ? k_real_clusters<T, true> : k_real_clusters<T, sizeof(T) == 8>;
+    MBD_CUDA_TRY(allow_smem(kern, smem, bytes(kRealMaxEntries, kRealStageBytes)));
+    kern<<<grid, 16 * kClusterSize, smem, st>>>(a);
     MBD_LAUNCH_CHECK();
     return MBD_OK;
 }
@@ -1263,7 +1269,7 @@ template mbd_status launch_field<double>(mbd_system *, const double *, const dou
                                          const FieldOut<double> &);
 template mbd_status launch_field<float>(mbd_system *, const float *, const float *, int, int,
                                         const FieldOut<float> &);
-template mbd_status launch_real_clusters<double>(mbd_system *, const double *, double *, int, cudaStream_t);
-template mbd_status launch_real_clusters<float>(mbd_system *, const float *, float *, int, cudaStream_t);
+template mbd_status launch_real_clusters<double>(mbd_system *, const double *, double *, int, cudaStream_t, bool);
+template mbd_status launch_real_clusters<float>(mbd_system *, const float *, float *, int, cudaStream_t, bool);
 
 }  // namespace mbd

@@ -403,8 +403,10 @@ mbd_status launch_morton_order(const BinView &B, int N, int *order, DevBuf &cnt,
 template <class T> mbd_status launch_cluster_pairs(mbd_system *s, cudaStream_t st);
 // whether this call's real-space field runs on the clusters (probe width ld)
 bool real_on_clusters(const mbd_system *s, int ld, int real_bytes);
-// E_real = sum over real-space pairs A d_j of the clusters (T [N][3][ld])
-template <class T> mbd_status launch_real_clusters(mbd_system *s, const T *d, T *ereal, int ld, cudaStream_t st);
+// E_real = sum over real-space pairs A d_j of the clusters (T [N][3][ld]); local: no mesh
+// term in the call, so a dipole that is not finite must reach its neighbours only
+template <class T>
+mbd_status launch_real_clusters(mbd_system *s, const T *d, T *ereal, int ld, cudaStream_t st, bool local = false);
 template <class T> mbd_status launch_splines(mbd_system *s, cudaStream_t st);
 template <class T> mbd_status launch_influence(mbd_system *s, const double *bmod_host, cudaStream_t st);
 
