@@ -86,7 +86,6 @@ namespace {
 
 // Vector loads/stores of VEC consecutive values (VEC in {1, 2, 4}).
 template <class T, int VEC> struct VecT;
-template <> struct VecT<float, 1> { using type = float; };
 template <> struct VecT<float, 2> { using type = float2; };
 template <> struct VecT<float, 4> { using type = float4; };
 template <> struct VecT<double, 1> { using type = double; };
@@ -140,8 +139,8 @@ template <class T, int VEC> __device__ __forceinline__ void vstore(T *p, const T
 }
 
 // ---------------------------------------------------------------- FFT
-// Complex values Cx<F>: F = float or double holds one complex probe pair, F =
-// float2 two of them, (x0, x1) in x and (y0, y1) in y, on which every
+// Complex values Cx<F>: F = double holds one complex probe pair, F = float2 two of
+// them, (x0, x1) in x and (y0, y1) in y, on which every
 // operation is one packed instruction (add, multiply, FMA of two floats).
 // FP32 meshes hold a multiple of four probes per point, and four consecutive
 // probes p0 .. p3 are read as the two complex pairs p0 + i p2 and p1 + i p3,
@@ -157,17 +156,13 @@ template <> struct PackOf<float> { using type = float2; };
 template <class F> struct Scal { using type = F; };
 template <> struct Scal<float2> { using type = float; };
 
-__device__ __forceinline__ float fadd(float a, float b) { return a + b; }
 __device__ __forceinline__ double fadd(double a, double b) { return a + b; }
 __device__ __forceinline__ float2 fadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float fsub(float a, float b) { return a - b; }
 __device__ __forceinline__ double fsub(double a, double b) { return a - b; }
 __device__ __forceinline__ float2 fsub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ float fmulc(float a, float c) { return a * c; }
 __device__ __forceinline__ double fmulc(double a, double c) { return a * c; }
 __device__ __forceinline__ float2 fmulc(float2 a, float c) { return __fmul2_rn(a, make_float2(c, c)); }
 // a c + b with a scalar c
-__device__ __forceinline__ float fmac(float a, float c, float b) { return fmaf(a, c, b); }
 __device__ __forceinline__ double fmac(double a, double c, double b) { return fma(a, c, b); }
 __device__ __forceinline__ float2 fmac(float2 a, float c, float2 b) { return __ffma2_rn(a, make_float2(c, c), b); }
 
@@ -351,14 +346,9 @@ template <class F, bool INV> struct Dft<F, 16, INV> {
 // packed form with each component doubled.
 template <class F> struct TwOf { using type = Cx<F>; };
 template <> struct TwOf<float2> { using type = float4; };
-__device__ __forceinline__ void tw_set(Cx<float> &t, float2 w) { t = {w.x, w.y}; }
 __device__ __forceinline__ void tw_set(Cx<double> &t, double2 w) { t = {w.x, w.y}; }
 __device__ __forceinline__ void tw_set(float4 &t, float2 w) { t = make_float4(w.x, w.x, w.y, w.y); }
 // v times the twiddle (its conjugate for INV)
-template <bool INV> __device__ __forceinline__ Cx<float> ctw(Cx<float> v, Cx<float> w) {
-    const float wy = INV ? -w.y : w.y;
-    return {fmaf(v.x, w.x, -(v.y * wy)), fmaf(v.x, wy, v.y * w.x)};
-}
 template <bool INV> __device__ __forceinline__ Cx<double> ctw(Cx<double> v, Cx<double> w) {
     const double wy = INV ? -w.y : w.y;
     return {fma(v.x, w.x, -(v.y * wy)), fma(v.x, wy, v.y * w.x)};
@@ -367,29 +357,21 @@ template <bool INV> __device__ __forceinline__ Cx<float2> ctw(Cx<float2> v, floa
     const float2 wx = make_float2(w.x, w.y), wy = make_float2(w.z, w.w), nwy = make_float2(-w.z, -w.w);
     return {__ffma2_rn(v.x, wx, __fmul2_rn(v.y, INV ? wy : nwy)), __ffma2_rn(v.x, INV ? nwy : wy, __fmul2_rn(v.y, wx))};
 }
+// A complex value in one 16-byte access.
+template <class F> union CxBits {
+    float4 v;
+    Cx<F> c;
+};
 template <class F> __device__ __forceinline__ Cx<F> cld(const Cx<F> *p) {
-    if constexpr (sizeof(Cx<F>) == 16) {
-        union {
-            float4 v;
-            Cx<F> c;
-        } u;
-        u.v = *reinterpret_cast<const float4 *>(p);
-        return u.c;
-    } else {
-        return *p;
-    }
+    static_assert(sizeof(Cx<F>) == 16, "one pair in double, two in float");
+    CxBits<F> u;
+    u.v = *reinterpret_cast<const float4 *>(p);
+    return u.c;
 }
 template <class F> __device__ __forceinline__ void cst(Cx<F> *p, Cx<F> c) {
-    if constexpr (sizeof(Cx<F>) == 16) {
-        union {
-            float4 v;
-            Cx<F> c;
-        } u;
-        u.c = c;
-        *reinterpret_cast<float4 *>(p) = u.v;
-    } else {
-        *p = c;
-    }
+    CxBits<F> u;
+    u.c = c;
+    *reinterpret_cast<float4 *>(p) = u.v;
 }
 
 // ---------------------------------------------------------------- compile-time passes

@@ -2,9 +2,10 @@
 // gradients as the next step); with alpha and omega position-independent,
 //   dE/dR = (1/4) Tr(C^{-1/2} dC/dR) ~ (1/4)(D/R) sum_l grad_R [p_l^T T'(R) q_l],
 // p_l = g . w_l, q_l = g . v_l, w_l = C^{-1/2} v_l = sum_k c_{lk} y_{lk}.
-// The probes' p and q are interleaved as one complex probe pair, so the SPME
-// part reuses the spread and FFT convolution kernels with 2R "probes":
-//   phi_p + i phi_q = F^-1[G F[D_p + i D_q]],
+// The probes' p and q are interleaved as 2R "probes" (p_l, q_l in columns 2l, 2l + 1),
+// so the SPME part reuses the spread and FFT convolution kernels, which transform
+// pairs of them as one complex vector (G is real and even: any pairing is exact):
+//   phi_p = F^-1[G F[D_p]], phi_q = F^-1[G F[D_q]],
 // and grad_i = sum_k H_i(k) [p_i phi_q(k) + q_i phi_p(k)] with H_i the Hessian
 // of the stencil weight W_i(k) wrt R_i; the real-space part contracts the
 // derivative of the pair tensor, dA_ab/dr_c, with p_i q_j + p_j q_i.

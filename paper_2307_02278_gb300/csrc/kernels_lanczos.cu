@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) k_prologue(LanczosView lz, int k, int m, 
         const double bk2 = k >= 2 ? lz.b[(size_t)(k - 2) * ld + r] : 0.0;
         const double *Yk1 = k >= 1 ? lz.Y + lz_slot(lz, k - 1) * stride : nullptr;
         const double *Yk2 = k >= 2 ? lz.Y + lz_slot(lz, k - 2) * stride : nullptr;
-        const double inv0 = k == 0 ? sqrt((double)rows) : 0.0;
+        const double norm0 = k == 0 ? sqrt((double)rows) : 0.0;
         // four rows per iteration, all their loads issued before any use, so
         // that enough bytes are in flight to stream the FP64 vectors from HBM
         constexpr int UR = 4;
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(256) k_prologue(LanczosView lz, int k, int m, 
                     const size_t o = (size_t)row * ld + r;
                     double ys;
                     if (k == 0) {
-                        ys = rademacher(seed, (uint64_t)r, (uint64_t)row) / inv0;
+                        ys = rademacher(seed, (uint64_t)r, (uint64_t)row) / norm0;
                     } else {
                         ys = lv[u] - ak1 * y1[u];
                         if (k >= 2) ys -= bk2 * y2[u];

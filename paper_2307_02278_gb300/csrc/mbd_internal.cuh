@@ -1,13 +1,15 @@
 // Internal declarations shared by the translation units of libmbd.
 //
-// Data layout on the device (probe-innermost, "ld" = padded probe count, even):
+// Data layout on the device (probe-innermost, "ld" = padded probe count, a multiple of
+// two in double and of four in float):
 //   Lanczos vectors (FP64)      [3N][ld]           row (3i + alpha), column = probe
 //   dipoles d, fields E (T)     [N][3][ld]         same indexing as above
-//   SPME mesh (T)               [K1][K2][K3][ld]   = complex [K1][K2][K3][ld/2]:
-//                               probes (2v, 2v+1) form the real/imaginary parts
-//                               of one complex vector; since the influence
-//                               function is real and even, one complex FFT
-//                               convolution serves two probes exactly.
+//   SPME mesh (T)               [K1][K2][K3][ld]   pairs of probes form the real and
+//                               imaginary parts of one complex vector, (2v, 2v+1) in
+//                               double, (4v, 4v+2) and (4v+1, 4v+3) in float (packed
+//                               two by two); since the influence function is real and
+//                               even, one complex FFT convolution serves two probes
+//                               exactly, whichever they are.
 //   spline stencil (T)          w, dw [N][3][p]    M_p(frac(u) + t), M_p'(...), t = 0..p-1
 //                               for mesh points top - t (mod K) per dimension
 //   real-space pairs            CSR over atoms i: col j, packed image shift,
