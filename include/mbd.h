@@ -286,7 +286,7 @@ mbd_status mbd_set_basis_storage(mbd_system *sys, int32_t mode);
  *   distinct neighbour of the cluster are staged once, and a warp applies them
  *   to two atoms at a time, then the field kernel adds the result.
  * MBD_REAL_AUTO (default): clusters when atoms x (padded) probes are at least
- *   160 x 1024 (MBD_MIXED), or when there are four clusters per SM and chunk of
+ *   160 x 1024 (MBD_MIXED; 512 x 1024 in mbd_field without the mesh term), or when there are four clusters per SM and chunk of
  *   32 probes (MBD_FP64), else pairs.
  * The two evaluations sum the same pairs in different orders (results agree
  * to rounding).  MBD_ERR_UNSUPPORTED for MBD_REAL_CLUSTERS when a cluster has

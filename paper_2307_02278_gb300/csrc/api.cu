@@ -776,7 +776,7 @@ template <class T> mbd_status apply_impl(mbd_system *s, int nvec, const double *
     fo.xin = xt;
     fo.k = 0;
     std::memset(&fo.lz, 0, sizeof(fo.lz));
-    if (real_on_clusters(s, ld, (int)sizeof(T)) && (terms & MBD_TERM_REAL))
+    if (real_on_clusters(s, ld, (int)sizeof(T), terms) && (terms & MBD_TERM_REAL))
         MBD_STAGE(s, MBD_STAGE_REAL, 1,
                   launch_real_clusters<T>(s, P.d.template as<T>(), P.ereal.template as<T>(), ld, s->stream,
                                           !(terms & MBD_TERM_RECIP)));

@@ -1095,9 +1095,9 @@ template <class T, int P, bool PAIRS> int field_occupancy() {
 // at once per block as give the resident blocks one iteration each.  Otherwise
 // the blocks fill whole waves of the resident capacity, with at most 64
 // atoms per block (more waves beyond that, for balance).
-template <class T> FieldShape field_shape(const mbd_system *s, int ld) {
+template <class T> FieldShape field_shape(const mbd_system *s, int ld, int terms = MBD_TERM_ALL) {
     constexpr int VEC = field_vec<T>();
-    const bool pairs = !real_on_clusters(s, ld, (int)sizeof(T));
+    const bool pairs = !real_on_clusters(s, ld, (int)sizeof(T), terms);
     int occ = 1;
     switch (s->p) {
 #define MBD_FIELD_OCC(P) \
@@ -1135,7 +1135,7 @@ template <class T> FieldShape field_shape(const mbd_system *s, int ld) {
 // mesh term wanted.
 constexpr int kFieldStreamLanes = 8;
 bool field_streams(const mbd_system *s, int ld, const FieldShape &f, int terms) {
-    return s->precision != MBD_FP64 && real_on_clusters(s, ld, 4) && f.lanes >= kFieldStreamLanes && f.teams == 32 / f.lanes &&
+    return s->precision != MBD_FP64 && real_on_clusters(s, ld, 4, terms) && f.lanes >= kFieldStreamLanes && f.teams == 32 / f.lanes &&
            (terms & MBD_TERM_RECIP);
 }
 }  // namespace
@@ -1143,7 +1143,7 @@ bool field_streams(const mbd_system *s, int ld, const FieldShape &f, int terms) 
 template <class T>
 mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld, const FieldOut<T> &o) {
     PrecData<T> &P = prec<T>(s);
-    const FieldShape f = field_shape<T>(s, ld);
+    const FieldShape f = field_shape<T>(s, ld, o.terms);
     FieldArgs<T> a;
     a.d = d;
     a.mesh = mesh;
@@ -1155,7 +1155,7 @@ mbd_status launch_field(mbd_system *s, const T *d, const T *mesh, int R, int ld,
     a.g_at = s->g_d.as<double>();
     a.w2 = s->w2_d.as<double>();
     a.self_coef = -4.0 * s->ewald_beta * s->ewald_beta * s->ewald_beta / (3.0 * 1.77245385090551602730);
-    const bool pairs = !real_on_clusters(s, ld, (int)sizeof(T));
+    const bool pairs = !real_on_clusters(s, ld, (int)sizeof(T), o.terms);
     a.ereal = pairs ? nullptr : P.ereal.template as<T>();
     a.o = o;
     a.lanes = f.lanes;
@@ -1214,14 +1214,17 @@ template <class T> int real_chunks(const mbd_system *s, int ld) {
 // loop of the field kernel, whose groups split the neighbours of one atom.
 // Measured per Lanczos step, pairs against clusters: 1200 atoms x 128 probes 188
 // and 195 us; 3000 x 32 122 and 131, x 64 224 and 210; 6000 x 16 156 and 157, x 32
-// 260 and 240; 15,000 x 2 (padded to 4) 203 and 240.  FP64, bound by its arithmetic either way, takes
-// them with four blocks per SM.
-constexpr long long kRealMinValues = 160 * 1024;
-bool real_on_clusters(const mbd_system *s, int ld, int real_bytes) {
+// 260 and 240; 15,000 x 2 (padded to 4) 203 and 240.  Without the mesh term the pair loop
+// has the kernel to itself and keeps up for longer (us per mbd_field of the real space,
+// r_cut 9: 1500 x 128 52 and 62, 3000 x 128 66 and 76, 12,000 x 32 68 and 81, x 64 128 and 115,
+// 24,000 x 32 145 and 136).  FP64, bound by its arithmetic either way, takes them with
+// four blocks per SM.
+constexpr long long kRealMinValues = 160 * 1024, kRealMinValuesLocal = 512 * 1024;
+bool real_on_clusters(const mbd_system *s, int ld, int real_bytes, int terms) {
     if (!s->real_clusters || s->real_method == MBD_REAL_PAIRS) return false;
     if (s->real_method == MBD_REAL_CLUSTERS) return true;
     if (real_bytes == 8) return (long long)s->n_clusters * ((ld + 31) / 32) >= 4LL * std::max(1, s->num_sms);
-    return (long long)s->N * ld >= kRealMinValues;
+    return (long long)s->N * ld >= (terms & MBD_TERM_RECIP ? kRealMinValues : kRealMinValuesLocal);
 }
 
 // E_real of every atom from the clusters (the caller runs this before

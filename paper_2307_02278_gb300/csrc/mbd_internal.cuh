@@ -403,8 +403,8 @@ template <class T> mbd_status launch_pair_tensors(mbd_system *s, cudaStream_t st
 mbd_status launch_morton_order(const BinView &B, int N, int *order, DevBuf &cnt, DevBuf &start, DevBuf &bsum,
                                cudaStream_t st);
 template <class T> mbd_status launch_cluster_pairs(mbd_system *s, cudaStream_t st);
-// whether this call's real-space field runs on the clusters (probe width ld)
-bool real_on_clusters(const mbd_system *s, int ld, int real_bytes);
+// whether this call's real-space field runs on the clusters (probe width ld, field terms)
+bool real_on_clusters(const mbd_system *s, int ld, int real_bytes, int terms = MBD_TERM_ALL);
 // E_real = sum over real-space pairs A d_j of the clusters (T [N][3][ld]); local: no mesh
 // term in the call, so a dipole that is not finite must reach its neighbours only
 template <class T>
