@@ -27,6 +27,7 @@
  *     every call returns after that work has finished (it synchronises the
  *     stream), so host outputs are valid on return.
  *   - A system handle is not thread-safe: one handle per host thread/stream.
+ *     Threads with a handle each may call at the same time.
  *   - Probe rule (part of the ABI, so that any implementation draws the same
  *     probes): u_{l,i} = +1 when the top bit of SplitMix64(seed + (l << 32) + i)
  *     is 0, else -1; v_l = u_l / sqrt(3N) (Eq. dds).  SplitMix64(x) is the first
@@ -60,6 +61,11 @@ typedef enum {
  * real-space field).  The Lanczos vectors, dot products, the quadrature of
  * the tridiagonal and the trace sum are always FP64. */
 enum { MBD_FP64 = 0, MBD_MIXED = 1 /* FP32 operator, FP64 Lanczos */ };
+/* Arrays over probes (mesh, dipoles, Lanczos vectors and basis) are padded to a
+ * multiple of four probes with MBD_MIXED and of two with MBD_FP64: one or two mixed
+ * probes take the memory of four.  A system keeps, beside its pair list and tensors,
+ * 64 (MBD_MIXED) or 112 (MBD_FP64) bytes per neighbour pair of records for the
+ * cluster evaluation of the real space, used or not, all with a quarter more room. */
 
 /* Evaluation of each probe's Gauss quadrature (Eqs. tridiag2, sl3):
  * q_l = sum_k U_1k^2 sqrt(theta_k) = e_1^T Delta^{1/2} e_1, and for the forces
@@ -269,7 +275,7 @@ mbd_status mbd_batch_get_info(const mbd_batch *batch, mbd_batch_info *info);
 /* ---- storage of the Lanczos basis ----
  * The force estimator needs w_l = sum_k c_lk y_lk, which takes all m basis
  * vectors of every probe.  MBD_BASIS_STORE (the default) keeps them,
- * m x 3N x R FP64.  MBD_BASIS_RECOMPUTE keeps three and, in
+ * m x 3N x R FP64 (R padded).  MBD_BASIS_RECOMPUTE keeps three and, in
  * mbd_energy_forces, reruns the recurrence after the quadrature.  The rerun uses
  * the same kernels in the same order, so it gives the same y_k, and it adds
  * c_k y_k into w as each y_k is completed.  That costs about twice the
@@ -286,8 +292,9 @@ mbd_status mbd_set_basis_storage(mbd_system *sys, int32_t mode);
  *   distinct neighbour of the cluster are staged once, and a warp applies them
  *   to two atoms at a time, then the field kernel adds the result.
  * MBD_REAL_AUTO (default): clusters when atoms x (padded) probes are at least
- *   160 x 1024 (MBD_MIXED; 512 x 1024 in mbd_field without the mesh term), or when there are four clusters per SM and chunk of
- *   32 probes (MBD_FP64), else pairs.
+ *   160 x 1024 (MBD_MIXED; 512 x 1024 in mbd_field without the mesh term), or
+ *   when there are four clusters per SM and chunk of 32 probes (MBD_FP64), else
+ *   pairs.
  * The two evaluations sum the same pairs in different orders (results agree
  * to rounding).  MBD_ERR_UNSUPPORTED for MBD_REAL_CLUSTERS when a cluster has
  * more than 4096 pairs (more than 256 neighbours per atom on average); the
